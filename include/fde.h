@@ -329,9 +329,9 @@ void fde_nop_destroy(fde_nop* n);
 
 /* ---- step-level entry points (the same kernels the solver runs) ---------- */
 
-/* y = M z (eq. (1.10), u_0 eliminated) in FP64 on the device: the band of A and B
- * along time and J applied to all s time columns through the FFT of the Toeplitz
- * circulant embedding (Sec. 2.1).  z, y: device, length s*m, must not alias.
+/* y = M z (eq. (1.10), u_0 eliminated) on the device: the band of A and B along time in
+ * FP64 and J applied to all s time columns through the FFT of the Toeplitz circulant
+ * embedding (Sec. 2.1), in 64-bit block floating point (rounding below FP64's).  z, y: device, length s*m, must not alias.
  * Requires bvm_assemble.  Errors: FDE_ERR_STATE, FDE_ERR_CUDA. */
 int fde_matvec(fde_problem* p, const double* z, double* y);
 

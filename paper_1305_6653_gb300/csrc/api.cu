@@ -587,7 +587,8 @@ int fde_problem_create(const fde_problem_desc* d, void* stream, fde_problem** ou
     TRY(dalloc(&P.d_g, m + 2));
     TRY(dalloc(&P.d_twL, (size_t)P.L + 1));
     TRY(dalloc(&P.d_twL32, (size_t)P.L + 1));
-    TRY(dalloc(&P.d_sym, (size_t)P.L));
+    TRY(dalloc(&P.d_twq, (size_t)P.L + P.L / 2));
+    TRY(dalloc(&P.d_kap, (size_t)P.L));
     TRY(dalloc(&P.d_sym32, (size_t)P.L));
     TRY(dalloc(&P.d_tws, (size_t)P.s / 2 + 1));
     TRY(dalloc(&P.d_tws32, (size_t)P.s / 2 + 1));
@@ -652,7 +653,7 @@ void fde_problem_destroy(fde_problem* h) {
     if (P.lu_x) cudaStreamSynchronize(P.lu_x);
     free_workspace(P);
     void* bufs[] = {P.d_start, P.d_a, P.d_b, P.d_dplus, P.d_dminus, P.d_u0, P.d_f, P.d_g, P.d_twL, P.d_twL32,
-                    P.d_sym, P.d_sym32, P.d_tws, P.d_tws32, P.d_phi, P.d_psi, P.d_b_rhs, P.d_work, P.d_rhat,
+                    P.d_twq, P.d_kap, P.d_sym32, P.d_tws, P.d_tws32, P.d_phi, P.d_psi, P.d_b_rhs, P.d_work, P.d_rhat,
                     P.d_fac, P.d_dinv, P.d_info, P.d_err, P.d_pack, P.d_tinv, P.d_dtile, P.d_strips, P.d_scal, P.d_partial,
                     P.d_counter, P.d_bccb_K64, P.d_bccb_K32, P.d_rhat_b, P.d_dplus_t, P.d_dminus_t,
                     P.d_jz, P.d_xsol};
@@ -736,8 +737,8 @@ int bvm_assemble(fde_problem* h) {
     if ((rc = launch_grunwald(P.alpha, P.m + 2, P.d_g, P.stream))) return rc;
     if ((rc = launch_twiddles(P.L, P.L, P.d_twL, P.d_twL32, P.stream))) return rc;      // L + 1 allocated
     if ((rc = launch_twiddles(P.s, P.s / 2, P.d_tws, P.d_tws32, P.stream))) return rc;  // s/2 + 1 allocated
-    if ((rc = launch_toeplitz_symbol(P.d_g, P.m, P.L, P.dxa, P.d_twL, P.d_sym, P.d_sym32, nullptr, P.stream)))
-        return rc;
+    if ((rc = launch_bfp_twiddles(P.L, P.d_twq, P.stream))) return rc;
+    if ((rc = launch_toeplitz_symbol(P.d_g, P.m, P.L, P.dxa, P.d_twq, P.d_kap, P.d_sym32, P.stream))) return rc;
     // main-formula coefficients for the Strang symbols
     if ((rc = dalloc(&d_main, 2 * (FDE_MAX_MU + 1)))) return rc;
     double hm[2 * (FDE_MAX_MU + 1)];

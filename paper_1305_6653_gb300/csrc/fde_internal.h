@@ -10,6 +10,7 @@
 #include <vector>
 
 #include "../../include/fde.h"
+#include "bfp_fft.cuh"
 
 namespace fde {
 
@@ -58,8 +59,9 @@ struct InstDev {
     const double* B;
     const double* dplus;
     const double* dminus;
-    const double2* sym;
-    const double2* twL;
+    const bfp::Tw* twq;    // as Problem::d_twq, d_kap
+    const bfp::Q61* kap;
+    double jfac;           // toeplitz_scale
     const float2* tws32;
     const double2* tws;
     void* rhat;
@@ -112,8 +114,10 @@ struct Problem;
 int launch_grunwald(double alpha, int count, double* g, cudaStream_t st);
 // tw[k] = exp(-2 pi i k / L) for k < count (count = the table's length)
 int launch_twiddles(int L, int count, double2* tw64, float2* tw32, cudaStream_t st);
-int launch_toeplitz_symbol(const double* g, int m, int L, double scale, const double2* tw, double2* sym64,
-                           float2* sym32, double2* work, cudaStream_t st);
+// twq: L + L/2 entries (Problem::d_twq)
+int launch_bfp_twiddles(int L, bfp::Tw* twq, cudaStream_t st);
+int launch_toeplitz_symbol(const double* g, int m, int L, double scale, const bfp::Tw* twq, bfp::Q61* kap,
+                           float2* sym32, cudaStream_t st);
 int launch_strang_symbols(const double* a_main, const double* b_main, int mu, int nu, int s, double2* phi,
                           double2* psi, cudaStream_t st);
 int launch_rhs(const Problem& P, const double* Ju0, cudaStream_t st);
@@ -188,8 +192,11 @@ struct Problem {
     double* d_g = nullptr;      // m+2 Grunwald weights
     double2* d_twL = nullptr;   // L twiddles exp(-2 pi i k / L), FP64
     float2* d_twL32 = nullptr;  // same, FP32
-    double2* d_sym = nullptr;   // L: (lambda + i conj(lambda)) / L, lambda = FFT of the circulant embedding of G
-    float2* d_sym32 = nullptr;
+    // block floating-point form (bfp_fft.cuh): twiddles exp(-2 pi i k / L), k < L, followed by
+    // the first L/2 in bit-reversed order; the symbol kap in bit-reversed order, units 2^-58
+    bfp::Tw* d_twq = nullptr;
+    bfp::Q61* d_kap = nullptr;
+    float2* d_sym32 = nullptr;  // L: (lambda + i conj(lambda)) / L, lambda = FFT of the circulant embedding of G
     double2* d_tws = nullptr;   // s/2 twiddles exp(-2 pi i k / s)
     float2* d_tws32 = nullptr;
     double2* d_phi = nullptr;   // s/2+1
@@ -278,6 +285,10 @@ struct Problem {
     double prof_acc_ms[FDE_NUM_STAGES] = {};
     int prof_acc_n[FDE_NUM_STAGES] = {};
 };
+
+// scale of the block floating-point J apply: dx^-alpha / L, one half for the unhalved
+// split and 2^3 for kap's units
+inline double toeplitz_scale(const Problem& P) { return 4.0 * P.dxa / P.L; }
 
 // preconditioner in use by pgmres_solve / fde_precond_apply
 constexpr int FDE_PRECOND_STRANG = 0;         // block-circulant S (eq. 1.11), block LU

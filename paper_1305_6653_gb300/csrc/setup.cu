@@ -2,6 +2,7 @@
 // circulant embedding of the shifted-Grunwald Toeplitz matrix G (eq. (1.5)), the
 // Strang symbols phi_k / psi_k (Sec. 3.1) and the right-hand side of eq. (1.10).
 #include "fde_internal.h"
+#include "bfp_device.cuh"
 #include "fft_device.cuh"
 
 namespace fde {
@@ -43,32 +44,45 @@ __global__ void twiddle_kernel(int L, int count, double2* __restrict__ tw64, flo
     if (tw32) tw32[k] = make_float2((float)cs, (float)sn);
 }
 
+// The block floating-point twiddles: exp(-2 pi i k / L), k < L, then the first L/2 of them
+// in bit-reversed order.
+__global__ void bfp_twiddle_kernel(int logL, bfp::Tw* __restrict__ twq) {
+    const int L = 1 << logL, k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k < L) twq[k] = bfp::twiddle(k, logL);
+    else if (k < L + L / 2) twq[k] = bfp::twiddle(bitrev(k - L, logL - 1), logL);
+}
+
 // First column of the L-periodic circulant C that embeds G (G[i][j] = g_{i-j+1}
 // for j <= i+1): c[k] = g_{k+1} for 0 <= k < m, c[L-1] = g_0, zero elsewhere.
-// lambda = FFT_L(c); the symbol stored is scale * (lambda + i conj(lambda)) / L so
-// that one inverse FFT of sym * FFT(z) returns (G z) + i (G^T z) for real z
-// (C^T has eigenvalues conj(lambda) in the same Fourier basis).
-__global__ void toeplitz_symbol_kernel(const double* __restrict__ g, int m, int logL, double scale,
-                                       const double2* __restrict__ tw, double2* __restrict__ sym64,
-                                       float2* __restrict__ sym32) {
-    extern __shared__ double2 sbuf[];
+// lambda = FFT_L(c); (lambda + i conj(lambda)) = (lr + li)(1 + i), so with kap = lr + li one
+// inverse FFT of kap FFT(z), rotated by 1 + i, returns (G z) + i (G^T z) for real z
+// (C^T has eigenvalues conj(lambda) in the same Fourier basis).  kap is stored in the
+// bit-reversed order in which the transform leaves it; |kap| <= sqrt 2 sum |g| < 5.7.
+// sym32 keeps scale / L times the complex symbol in natural order, in FP32.
+__global__ void __launch_bounds__(512)
+toeplitz_symbol_kernel(const double* __restrict__ g, int m, int logL, double scale, const bfp::Tw* __restrict__ tw,
+                       bfp::Q61* __restrict__ kap, float2* __restrict__ sym32) {
+    extern __shared__ __align__(16) unsigned char sym_smem[];
+    bfp::I2* buf = reinterpret_cast<bfp::I2*>(sym_smem);
+    __shared__ uint32_t red[4];
     const int L = 1 << logL;
+    constexpr int EMAX = 1024;  // |g_k| < 2
+    if (threadIdx.x < 4) red[threadIdx.x] = 0u;
+    __syncthreads();
     for (int k = threadIdx.x; k < L; k += blockDim.x) {
-        double v = 0.0;
-        if (k < m) v = g[k + 1];
-        else if (k == L - 1) v = g[0];
-        sbuf[bitrev(k, logL)] = make_double2(v, 0.0);
+        const double v = k < m ? g[k + 1] : k == L - 1 ? g[0] : 0.0;
+        buf[bfp::slot(k)] = bfp::I2{bfp::to_fixed(v, EMAX), 0};
     }
     __syncthreads();
-    fft_dit<double2, false>(sbuf, logL, 1, L, tw);
-    const double inv = scale / (double)L;
-    for (int k = threadIdx.x; k < L; k += blockDim.x) {
-        double2 l = sbuf[k];
-        // lambda + i conj(lambda) = (lr + i li) + (li + i lr) = (lr + li) (1 + i)
-        const double kap = (l.x + l.y) * inv;
-        double2 v = make_double2(kap, kap);
-        if (sym64) sym64[k] = v;
-        if (sym32) sym32[k] = make_float2((float)v.x, (float)v.y);
+    bfp::RowBits bits{red};
+    int shifts = 0;
+    bfp::transform(buf, logL, false, 0, tw, logL, false, bits, 0u, &shifts);
+    for (int p = threadIdx.x; p < L; p += blockDim.x) {
+        const bfp::I2 v = buf[bfp::slot(p)];
+        const long long s = v.x + v.y;  // units of 2^(shifts - 56)
+        kap[p] = bfp::q61((long long)((unsigned long long)s << (2 + shifts)));
+        const float f = (float)(scalbn(bfp::to_double(s), shifts - (bfp::BITS - 1 + 1023 - EMAX)) * (scale / L));
+        sym32[bitrev(p, logL)] = make_float2(f, f);
     }
 }
 
@@ -123,16 +137,20 @@ int launch_twiddles(int L, int count, double2* tw64, float2* tw32, cudaStream_t 
     return FDE_OK;
 }
 
-int launch_toeplitz_symbol(const double* g, int m, int L, double scale, const double2* tw, double2* sym64,
-                           float2* sym32, double2* /*work*/, cudaStream_t st) {
-    size_t smem = (size_t)L * sizeof(double2);
-    static bool attr = false;
-    if (!attr) {
-        FDE_CUDA_TRY(cudaFuncSetAttribute(toeplitz_symbol_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          227 * 1024));
-        attr = true;
-    }
-    toeplitz_symbol_kernel<<<1, 1024, smem, st>>>(g, m, ilog2(L), scale, tw, sym64, sym32);
+int launch_bfp_twiddles(int L, bfp::Tw* twq, cudaStream_t st) {
+    const int n = L + L / 2;
+    bfp_twiddle_kernel<<<(n + 255) / 256, 256, 0, st>>>(ilog2(L), twq);
+    FDE_LAUNCH_CHECK("bfp_twiddle_kernel");
+    return FDE_OK;
+}
+
+int launch_toeplitz_symbol(const double* g, int m, int L, double scale, const bfp::Tw* twq, bfp::Q61* kap,
+                           float2* sym32, cudaStream_t st) {
+    const size_t smem = (size_t)L * sizeof(bfp::I2);
+    FDE_CUDA_TRY(cudaFuncSetAttribute(toeplitz_symbol_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      226 * 1024));
+    const int threads = L / 8 > 512 ? 512 : L / 8 < 64 ? 64 : L / 8;
+    toeplitz_symbol_kernel<<<1, threads, smem, st>>>(g, m, ilog2(L), scale, twq, kap, sym32);
     FDE_LAUNCH_CHECK("toeplitz_symbol_kernel");
     return FDE_OK;
 }
