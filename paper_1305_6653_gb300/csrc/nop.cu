@@ -26,128 +26,188 @@
 
 namespace fde {
 
-constexpr int CV_TCO = 16;   // output channels per CTA
-constexpr int CV_TX = 128;   // positions per CTA
-constexpr int CV_CI = 16;    // input channels per shared-memory chunk
 constexpr int CV_KMAX = 7;
+constexpr int CV_TP = 16;        // output channels per CTA
+constexpr int CV_WARPS = 8;      // warps per CTA, which share the input channels of a chunk
+constexpr int CV_LDW = CV_TP + 1;
 
 __device__ __forceinline__ float ldf(const float* p) { return *p; }
 __device__ __forceinline__ float ldf(const __half* p) { return __half2float(*p); }
 __device__ __forceinline__ void stf(float* p, float v) { *p = v; }
 __device__ __forceinline__ void stf(__half* p, float v) { *p = __float2half_rn(v); }
 
+// Places of a tile's positions: flattened positions n = b m + x of the batch, so that a tile
+// is full whatever the number of modes; every sample's piece of the tile is staged with a halo
+// of h zeros or neighbours on either side.
+__device__ __forceinline__ int cv_place(int n, int n0, int m, int h) { return n - n0 + (n / m - n0 / m) * 2 * h; }
+// length of a staged row for the positions [n0, n1)
+__host__ __device__ __forceinline__ int cv_length(int n0, int n1, int m, int h) {
+    return n1 - n0 + ((n1 - 1) / m - n0 / m + 1) * 2 * h;
+}
+// offset of slot t's sample row and point, (b Q) m + x for channel 0, or -1 for a zero
+__device__ __forceinline__ int cv_source(int Q, int n0, int m, int h, int t) {
+    const int b0 = n0 / m, head = m - (n0 - b0 * m) + 2 * h;  // slots of the first sample's piece
+    int b = b0, xx = n0 - b0 * m - h + t;
+    if (t >= head) {
+        const int u = t - head, w = m + 2 * h;
+        b = b0 + 1 + u / w;
+        xx = u - (u / w) * w - h;
+    }
+    return xx >= 0 && xx < m ? b * Q * m + xx : -1;
+}
+// stage channels q0 .. q0 + nq - 1 of x: one warp a channel, lanes along the slots (whose
+// sources do not depend on the channel)
+template <typename TI>
+__device__ __forceinline__ void cv_stage(const TI* __restrict__ x, int Q, int q0, int nq, int nmax, int n0, int m,
+                                         int h, int len, float* s, int ld) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    for (int t = lane; t < len; t += 32) {
+        const int src = cv_source(Q, n0, m, h, t);
+#pragma unroll 4
+        for (int c = warp; c < nmax; c += CV_WARPS)
+            s[c * ld + t] = src >= 0 && c < nq ? ldf(x + src + (size_t)(q0 + c) * m) : 0.f;
+    }
+}
+
 // y[b][p][x] = bias[p] + sum_q sum_k Wacc(p,q,k) x[b][q][x + k - K/2]
 //   TRANS = false: Wacc(p,q,k) = W[p][q][k]            (W: P x Q x K)
 //   TRANS = true : Wacc(p,q,k) = W[q][p][K-1-k]        (W: Q x P x K; gradient w.r.t. the input)
 // relu: apply max(., 0); mask: multiply by (mask[b][p][x] > 0) (backward through a ReLU).
-template <typename TI, typename TW, typename TO, bool TRANS>
-__global__ void __launch_bounds__(256)
-conv_kernel(const TI* __restrict__ x, int Q, const TW* __restrict__ W, const float* __restrict__ bias, int P, int K,
-            int m, int relu, const float* __restrict__ mask, TO* __restrict__ y) {
-    __shared__ float s_in[CV_CI][CV_TX + CV_KMAX - 1];
-    __shared__ float s_w[CV_TCO][CV_CI][CV_KMAX];
-    const int b = blockIdx.z;
-    const int p0 = blockIdx.y * CV_TCO;
-    const int x0 = blockIdx.x * CV_TX;
-    const int h = K / 2;
-    const int pl = threadIdx.x / 16, xg = threadIdx.x % 16;
-    float acc[CV_TX / 16];
+//
+// The layers are small (64 channels, 16 modes, 32 samples: 21 MFLOP), so a launch is bound by
+// latency and by how many SMs it reaches.  A CTA takes 16 channels x 4 NL positions of the
+// flattened batch; its eight warps split the input channels of a chunk and their partial sums
+// are added in a fixed order.  Per layer at that size 9 us forward and 13 backward against 51
+// and 45 for a tile of 128 positions of one sample, seven eighths of which were padding.
+// KT: the kernel size, or 0 to take it from K (a known size makes the weights' indices cheap).
+template <typename TI, typename TW, typename TO, bool TRANS, int NL, int KT>
+__global__ void __launch_bounds__(32 * CV_WARPS)
+conv_kernel(const TI* __restrict__ x, int Q, const TW* __restrict__ W, const float* __restrict__ bias, int P, int Kr,
+            int m, int N, int relu, const float* __restrict__ mask, TO* __restrict__ y, int ld) {
+    const int K = KT ? KT : Kr;
+    constexpr int TN = 4 * NL, QW = NL == 4 ? 8 : 4, QC = QW * CV_WARPS;  // QW: channels per warp and chunk
+    extern __shared__ float cv_smem[];
+    float* s_in = cv_smem;            // [QC][ld]
+    float* s_w = cv_smem + QC * ld;   // [QC][K][CV_LDW]
+    const int p0 = blockIdx.y * CV_TP, n0 = blockIdx.x * TN, n1 = min(n0 + TN, N);
+    const int h = K / 2, len = cv_length(n0, n1, m, h);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, pl = lane >> 2, nl = lane & 3;
+    float acc[2][NL];
+    int at[NL];
 #pragma unroll
-    for (int j = 0; j < CV_TX / 16; ++j) acc[j] = 0.f;
-    const TI* xb = x + (size_t)b * Q * m;
-    for (int q0 = 0; q0 < Q; q0 += CV_CI) {
-        for (int e = threadIdx.x; e < CV_CI * (CV_TX + K - 1); e += blockDim.x) {
-            const int c = e / (CV_TX + K - 1), t = e % (CV_TX + K - 1);
-            const int xx = x0 - h + t;
-            s_in[c][t] = (q0 + c < Q && xx >= 0 && xx < m) ? ldf(xb + (size_t)(q0 + c) * m + xx) : 0.f;
-        }
-        for (int e = threadIdx.x; e < CV_TCO * CV_CI * K; e += blockDim.x) {
-            const int o = e / (CV_CI * K), r = e % (CV_CI * K), c = r / K, k = r % K;
-            float v = 0.f;
-            if (p0 + o < P && q0 + c < Q) {
-                v = TRANS ? ldf(W + ((size_t)(q0 + c) * P + (p0 + o)) * K + (K - 1 - k))
-                          : ldf(W + ((size_t)(p0 + o) * Q + (q0 + c)) * K + k);
-            }
-            s_w[o][c][k] = v;
+    for (int j = 0; j < NL; ++j) {
+        acc[0][j] = acc[1][j] = 0.f;
+        at[j] = cv_place(min(n0 + nl + 4 * j, n1 - 1), n0, m, h);
+    }
+    for (int q0 = 0; q0 < Q; q0 += QC) {
+        const int nq = min(QC, Q - q0);
+        cv_stage(x, Q, q0, nq, nq, n0, m, h, len, s_in, ld);
+        // 16 threads a row of weights: channel o's (TRANS = false) or input channel c's
+        const int row = tid >> 4;
+        if (TRANS) {
+#pragma unroll 2
+            for (int c = row; c < nq; c += 2 * CV_WARPS)
+                for (int r = tid & 15; r < CV_TP * K; r += 16) {
+                    const int o = r / K, k = r - o * K;
+                    s_w[(c * K + K - 1 - k) * CV_LDW + o] =
+                        p0 + o < P ? ldf(W + ((size_t)(q0 + c) * P + p0) * K + r) : 0.f;
+                }
+        } else {
+            const TW* wr = W + ((size_t)(p0 + row) * Q + q0) * K;
+#pragma unroll 8
+            for (int r = tid & 15; r < nq * K; r += 16) s_w[r * CV_LDW + row] = p0 + row < P ? ldf(wr + r) : 0.f;
         }
         __syncthreads();
-        for (int c = 0; c < CV_CI; ++c)
-            for (int k = 0; k < K; ++k) {
-                const float w = s_w[pl][c][k];
+        for (int c = warp; c < nq; c += CV_WARPS) {
+            const float* in = s_in + c * ld;
+            const float* w = s_w + c * K * CV_LDW + 2 * pl;
 #pragma unroll
-                for (int j = 0; j < CV_TX / 16; ++j) acc[j] += w * s_in[c][xg + 16 * j + k];
+            for (int k = 0; k < (KT ? KT : CV_KMAX); ++k) {
+                if (!KT && k >= K) break;
+                const float w0 = w[k * CV_LDW], w1 = w[k * CV_LDW + 1];
+#pragma unroll
+                for (int j = 0; j < NL; ++j) {
+                    const float v = in[at[j] + k];
+                    acc[0][j] += w0 * v;
+                    acc[1][j] += w1 * v;
+                }
             }
+        }
         __syncthreads();
     }
-    const int p = p0 + pl;
-    if (p >= P) return;
-    const float bb = bias ? bias[p] : 0.f;
+    // add the warps' partial sums: red[warp][channel][position]
+    float* red = cv_smem;
 #pragma unroll
-    for (int j = 0; j < CV_TX / 16; ++j) {
-        const int xx = x0 + xg + 16 * j;
-        if (xx >= m) continue;
-        float v = acc[j] + bb;
+    for (int j = 0; j < NL; ++j) {
+        red[(warp * CV_TP + 2 * pl) * TN + nl + 4 * j] = acc[0][j];
+        red[(warp * CV_TP + 2 * pl + 1) * TN + nl + 4 * j] = acc[1][j];
+    }
+    __syncthreads();
+    for (int e = tid; e < CV_TP * TN; e += 32 * CV_WARPS) {
+        const int p = p0 + e / TN, n = n0 + e % TN;
+        if (p >= P || n >= n1) continue;
+        float v = 0.f;
+#pragma unroll
+        for (int w = 0; w < CV_WARPS; ++w) v += red[w * CV_TP * TN + e];
+        if (bias) v += bias[p];
         if (relu) v = fmaxf(v, 0.f);
-        const size_t idx = ((size_t)b * P + p) * m + xx;
+        const int b = n / m;
+        const size_t idx = ((size_t)b * P + p) * m + n - b * m;
         if (mask && !(mask[idx] > 0.f)) v = 0.f;
         stf(y + idx, v);
     }
 }
 
-// dW[o][c][k] += sum_{b in group} sum_x g[b][o][x] a[b][c][x + k - K/2]; one thread per (o, c)
-// of a 16 x 16 tile, the batch split over gridDim.z groups (atomic accumulation).
+// dW[o][c][k] += sum_{b in group} sum_x g[b][o][x] a[b][c][x + k - K/2] and, in the CTAs of
+// the first channels, db[o] += sum g; one thread per (o, c) of a 16 x 16 tile, the flattened
+// positions of the batch split over gridDim.z groups of whole samples (atomic accumulation).
+// 10 us a layer at 64 channels, 16 modes, 32 samples, against 22 (64-position tiles of single
+// samples) and 10 for the bias sums in a launch of their own.
+constexpr int WG_N = 64;  // positions staged at once
 __global__ void __launch_bounds__(256)
 conv_wgrad_kernel(const float* __restrict__ g, int O, const float* __restrict__ a, int C, int K, int m, int B,
-                  float* __restrict__ dW) {
-    __shared__ float s_g[16][64];
-    __shared__ float s_a[16][64 + CV_KMAX - 1];
+                  float* __restrict__ dW, float* __restrict__ db, int ld) {
+    extern __shared__ float wg_smem[];
+    float* s_g = wg_smem;                  // [16][WG_N + 1]
+    float* s_a = wg_smem + 16 * (WG_N + 1);  // [16][ld]
     const int o0 = blockIdx.y * 16, c0 = blockIdx.x * 16;
     const int ol = threadIdx.x / 16, cl = threadIdx.x % 16;
     const int h = K / 2;
-    float acc[CV_KMAX];
+    float acc[CV_KMAX], sum = 0.f;
 #pragma unroll
     for (int k = 0; k < CV_KMAX; ++k) acc[k] = 0.f;
-    const int groups = gridDim.z;
-    for (int b = blockIdx.z; b < B; b += groups) {
-        for (int x0 = 0; x0 < m; x0 += 64) {
-            for (int e = threadIdx.x; e < 16 * 64; e += blockDim.x) {
-                const int r = e / 64, t = e % 64;
-                const int xx = x0 + t;
-                s_g[r][t] = (o0 + r < O && xx < m) ? g[((size_t)b * O + o0 + r) * m + xx] : 0.f;
-            }
-            for (int e = threadIdx.x; e < 16 * (64 + K - 1); e += blockDim.x) {
-                const int r = e / (64 + K - 1), t = e % (64 + K - 1);
-                const int xx = x0 - h + t;
-                s_a[r][t] = (c0 + r < C && xx >= 0 && xx < m) ? a[((size_t)b * C + c0 + r) * m + xx] : 0.f;
-            }
-            __syncthreads();
-            for (int t = 0; t < 64; ++t) {
-                const float gv = s_g[ol][t];
+    const int per = (B + gridDim.z - 1) / gridDim.z;  // samples of this group
+    const int lo = blockIdx.z * per * m, hi = min(B, ((int)blockIdx.z + 1) * per) * m;
+    for (int n0 = lo; n0 < hi; n0 += WG_N) {
+        const int n1 = min(n0 + WG_N, hi), len = cv_length(n0, n1, m, h);
+        {
+            const int t = threadIdx.x % WG_N, n = n0 + t, b = n / m;
+            const float* gr = g + ((size_t)b * O + o0) * m + n - b * m;
 #pragma unroll
-                for (int k = 0; k < CV_KMAX; ++k)
-                    if (k < K) acc[k] += gv * s_a[cl][t + k];
-            }
-            __syncthreads();
+            for (int r = threadIdx.x / WG_N; r < 16; r += 256 / WG_N)
+                s_g[r * (WG_N + 1) + t] = o0 + r < O && n < n1 ? gr[(size_t)r * m] : 0.f;
         }
+        cv_stage(a, C, c0, min(16, C - c0), 16, n0, m, h, len, s_a, ld);
+        __syncthreads();
+        int x = n0 % m;
+        const float* ap = s_a + cl * ld;
+        for (int t = 0; t < n1 - n0; ++t) {
+            const float gv = s_g[ol * (WG_N + 1) + t];
+            sum += gv;
+#pragma unroll
+            for (int k = 0; k < CV_KMAX; ++k)
+                if (k < K) acc[k] += gv * ap[k];
+            ++ap;
+            if (++x == m) {  // the next sample's piece
+                x = 0;
+                ap += 2 * h;
+            }
+        }
+        __syncthreads();
     }
     if (o0 + ol < O && c0 + cl < C)
         for (int k = 0; k < K; ++k) atomicAdd(dW + ((size_t)(o0 + ol) * C + c0 + cl) * K + k, acc[k]);
-}
-
-// db[o] = sum_{b,x} g[b][o][x]
-__global__ void bias_grad_kernel(const float* __restrict__ g, int O, int m, int B, float* __restrict__ db) {
-    const int o = blockIdx.x;
-    float s = 0.f;
-    for (int b = 0; b < B; ++b)
-        for (int x = threadIdx.x; x < m; x += blockDim.x) s += g[((size_t)b * O + o) * m + x];
-    __shared__ float red[256];
-    red[threadIdx.x] = s;
-    __syncthreads();
-    for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-        if (threadIdx.x < w) red[threadIdx.x] += red[threadIdx.x + w];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) db[o] = red[0];
+    if (c0 + cl == 0 && o0 + ol < O) atomicAdd(db + o0 + ol, sum);
 }
 
 // g = 2 (y - t) / N, loss += sum (y - t)^2 / N
@@ -161,7 +221,13 @@ __global__ void mse_kernel(const float* __restrict__ y, const float* __restrict_
         s += (double)d * d;
     }
     for (int off = 16; off; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-    if ((threadIdx.x & 31) == 0) atomicAdd(loss, s * inv);
+    __shared__ double part[8];
+    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = s;
+    __syncthreads();
+    if (threadIdx.x == 0) {  // one atomic a CTA (256 threads)
+        for (int w = 1; w < 8; ++w) s += part[w];
+        atomicAdd(loss, s * inv);
+    }
 }
 
 __global__ void adam_kernel(float* __restrict__ p, const float* __restrict__ g, float* __restrict__ m1,
@@ -284,13 +350,41 @@ struct fde_nop {
 
 namespace {
 
+// Longest staged row of any tile of `tile` positions.
+int staged_length(int tile, int N, int m, int K) {
+    const int n = tile < N ? tile : N;
+    const int pieces = (n + m - 2) / m + 1;  // samples a tile can touch
+    return n + pieces * 2 * (K / 2);
+}
+
+template <typename TI, typename TW, typename TO, bool TRANS, int NL, int KT>
+int conv_tiles(const TI* x, int Q, const TW* W, const float* bias, int P, int K, int m, int N, int relu,
+               const float* mask, TO* y, cudaStream_t st) {
+    constexpr int TN = 4 * NL, QC = (NL == 4 ? 8 : 4) * CV_WARPS;
+    const int ld = staged_length(TN, N, m, K) | 1;
+    const size_t stage = (size_t)QC * (ld + K * CV_LDW), red = (size_t)CV_WARPS * CV_TP * TN;
+    const size_t smem = (stage > red ? stage : red) * sizeof(float);
+    auto kern = conv_kernel<TI, TW, TO, TRANS, NL, KT>;
+    FDE_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
+    const dim3 grid((N + TN - 1) / TN, (P + CV_TP - 1) / CV_TP);
+    kern<<<grid, 32 * CV_WARPS, smem, st>>>(x, Q, W, bias, P, K, m, N, relu, mask, y, ld);
+    FDE_LAUNCH_CHECK("conv_kernel");
+    return FDE_OK;
+}
+
+// 16 positions a CTA while that leaves the launch within a few waves of the 152 SMs; beyond
+// it 64, which reads the weights a quarter as often.
 template <typename TI, typename TW, typename TO, bool TRANS>
 int conv(const TI* x, int Q, const TW* W, const float* bias, int P, int K, int m, int B, int relu, const float* mask,
          TO* y, cudaStream_t st) {
-    dim3 grid((m + CV_TX - 1) / CV_TX, (P + CV_TCO - 1) / CV_TCO, B);
-    conv_kernel<TI, TW, TO, TRANS><<<grid, 256, 0, st>>>(x, Q, W, bias, P, K, m, relu, mask, y);
-    FDE_LAUNCH_CHECK("conv_kernel");
-    return FDE_OK;
+    const int N = B * m;
+    const long ctas = (long)((N + 15) / 16) * ((P + CV_TP - 1) / CV_TP);
+    if (ctas > 8 * 152)
+        return conv_tiles<TI, TW, TO, TRANS, 16, 0>(x, Q, W, bias, P, K, m, N, relu, mask, y, st);
+    if (K == 3) return conv_tiles<TI, TW, TO, TRANS, 4, 3>(x, Q, W, bias, P, K, m, N, relu, mask, y, st);
+    if (K == 5) return conv_tiles<TI, TW, TO, TRANS, 4, 5>(x, Q, W, bias, P, K, m, N, relu, mask, y, st);
+    if (K == 7) return conv_tiles<TI, TW, TO, TRANS, 4, 7>(x, Q, W, bias, P, K, m, N, relu, mask, y, st);
+    return conv_tiles<TI, TW, TO, TRANS, 4, 0>(x, Q, W, bias, P, K, m, N, relu, mask, y, st);
 }
 
 int ensure_batch(fde_nop* n, int B) {
@@ -435,11 +529,13 @@ int fde_nop_loss_grad(fde_nop* n, const float* in, const float* target, int batc
     for (int l = L - 1; l >= 0; --l) {
         const float* a = l == 0 ? in : n->act[l];
         const int O = n->dout[l], C = n->din[l];
-        dim3 wg((C + 15) / 16, (O + 15) / 16, std::min(B, 16));
-        conv_wgrad_kernel<<<wg, 256, 0, n->stream>>>(g, O, a, C, n->K, m, B, n->g + n->woff[l]);
+        const dim3 wg((C + 15) / 16, (O + 15) / 16, std::min(B, 16));
+        const int ld = staged_length(WG_N, B * m, m, n->K) | 1;
+        const size_t smem = (size_t)16 * (WG_N + 1 + ld) * sizeof(float);
+        FDE_CUDA_TRY(cudaFuncSetAttribute(conv_wgrad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
+        conv_wgrad_kernel<<<wg, 256, smem, n->stream>>>(g, O, a, C, n->K, m, B, n->g + n->woff[l], n->g + n->boff[l],
+                                                        ld);
         FDE_LAUNCH_CHECK("conv_wgrad_kernel");
-        bias_grad_kernel<<<O, 256, 0, n->stream>>>(g, O, m, B, n->g + n->boff[l]);
-        FDE_LAUNCH_CHECK("bias_grad_kernel");
         if (l > 0) {
             // gradient w.r.t. the layer input, through the ReLU of layer l-1 (mask = its output)
             rc = conv<float, float, float, true>(g, O, n->p + n->woff[l], nullptr, C, n->K, m, B, 0, n->act[l], gnext,
