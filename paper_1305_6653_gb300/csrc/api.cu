@@ -324,29 +324,13 @@ static void drop_iter_graphs(Problem& P) {
 // w = M z_j (Toeplitz part in FP32 when fp32), CGS2 against v_0..v_j, Hessenberg
 // column / Givens rotation, w /= |w|.
 static int iteration_launches(Problem& P, int j, int ldh, int reorth, bool fp32) {
-    const long n = P.n;
-    cudaStream_t st = P.stream;
-    double* V = P.d_V;
-    double* sc = P.d_scal;
-    double* vj = V + (size_t)j * n;
-    double* w = V + (size_t)(j + 1) * n;
-    double* zj = P.d_Z + (size_t)j * n;
+    const size_t n = P.n;
+    double* zj = P.d_Z + j * n;
     int rc;
-    if ((rc = apply_precond(P, vj, zj))) return rc;
-    if ((rc = matvec(P, zj, w, fp32))) return rc;
+    if ((rc = apply_precond(P, P.d_V + j * n, zj))) return rc;
+    if ((rc = matvec(P, zj, P.d_V + (j + 1) * n, fp32))) return rc;
     StageTimer kt(P, FDE_STAGE_KRYLOV);
-    // CGS2 in three passes over V: h1 = V^T w; w -= V h1 and h2 = V^T w;
-    // w -= V h2 and |w|^2 (one pass fewer without re-orthogonalisation)
-    if ((rc = launch_cgs_pass(0, V, j + 1, nullptr, w, n, sc, P.d_partial, P.d_counter, st))) return rc;
-    if (reorth) {
-        if ((rc = launch_cgs_pass(1, V, j + 1, sc, w, n, sc + 64, P.d_partial, P.d_counter, st))) return rc;
-    }
-    if ((rc = launch_cgs_pass(2, V, j + 1, reorth ? sc + 64 : sc, w, n, sc + 128, P.d_partial, P.d_counter, st)))
-        return rc;
-    if ((rc = launch_arnoldi_finish(P.d_H, ldh, j, sc, reorth ? sc + 64 : nullptr, sc + 128, P.d_cs, P.d_sn,
-                                    P.d_gv, sc + 129, st)))
-        return rc;
-    return launch_scale(w, sc + 128, w, n, st);
+    return launch_gram_schmidt(P, j, ldh, reorth, P.stream);
 }
 
 // Run iteration j: replay its CUDA graph or launch the kernels directly.  Graphs are
@@ -993,8 +977,10 @@ int pgmres_solve(fde_problem* h, const fde_pgmres_opts* opts, const double* x0_a
     auto finish = [&](int code) -> int {
         int derr = 0;  // a bounded wait of the block solves ran out
         if (cudaMemcpyAsync(&derr, P.d_err, sizeof(int), cudaMemcpyDeviceToHost, st) == cudaSuccess &&
-            cudaStreamSynchronize(st) == cudaSuccess && derr && code == FDE_OK)
-            code = set_error(FDE_ERR_TIMEOUT, "a bounded wait in the block solves ran out");
+            cudaStreamSynchronize(st) == cudaSuccess && derr) {
+            cudaMemsetAsync(P.d_counter, 0, 4 * sizeof(unsigned int), st);  // the Gram-Schmidt barriers start over
+            if (code == FDE_OK) code = set_error(FDE_ERR_TIMEOUT, "a bounded wait of the iteration ran out");
+        }
         if (host_x) {  // the solution (or last iterate) back to the caller's host array
             cudaError_t e = cudaMemcpyAsync(x_arg, x, n * sizeof(double), cudaMemcpyDeviceToHost, st);
             if (e != cudaSuccess && code == FDE_OK) code = cuda_error(e, "copy of the solution to the host");
@@ -1026,7 +1012,9 @@ int pgmres_solve(fde_problem* h, const fde_pgmres_opts* opts, const double* x0_a
         S.rel_residual = 0.0;
         return finish(FDE_OK);
     }
-    // r = b - M x -> V_0
+    // r = b - M x -> V_0; from x = 0 it is b, whose norm is known
+    int beta_slot = 131;
+    beta2 = bnorm2;
     if (x0) {
         if ((rc = matvec(P, x, P.d_work))) return finish(rc);
         if ((rc = launch_sub(P.d_b_rhs, P.d_work, V, n, st))) return finish(rc);
@@ -1034,13 +1022,17 @@ int pgmres_solve(fde_problem* h, const fde_pgmres_opts* opts, const double* x0_a
         cudaError_t e = cudaMemcpyAsync(V, P.d_b_rhs, n * sizeof(double), cudaMemcpyDeviceToDevice, st);
         if (e != cudaSuccess) return finish(cuda_error(e, "copy of b"));
     }
-    if ((rc = norm2(P, V, 132, &beta2, pin))) return finish(rc);
-    if (x0 && !(beta2 <= bnorm2)) {
-        // the initial guess is worse than zero (or not finite): start from x = 0
-        FDE_CUDA_TRY(cudaMemsetAsync(x, 0, n * sizeof(double), st));
-        FDE_CUDA_TRY(cudaMemcpyAsync(V, P.d_b_rhs, n * sizeof(double), cudaMemcpyDeviceToDevice, st));
+    if (x0) {
         if ((rc = norm2(P, V, 132, &beta2, pin))) return finish(rc);
-        S.x0_rejected = 1;
+        beta_slot = 132;
+        if (!(beta2 <= bnorm2)) {
+            // the initial guess is worse than zero (or not finite): start from x = 0
+            FDE_CUDA_TRY(cudaMemsetAsync(x, 0, n * sizeof(double), st));
+            FDE_CUDA_TRY(cudaMemcpyAsync(V, P.d_b_rhs, n * sizeof(double), cudaMemcpyDeviceToDevice, st));
+            beta_slot = 131;
+            beta2 = bnorm2;
+            S.x0_rejected = 1;
+        }
     }
     int its = 0;
     std::vector<double> g0(o.restart + 1, 0.0);
@@ -1054,7 +1046,7 @@ int pgmres_solve(fde_problem* h, const fde_pgmres_opts* opts, const double* x0_a
             status = set_error(FDE_ERR_NOT_CONVERGED, "maxit reached before the tolerance");
             break;
         }
-        if ((rc = launch_scale(V, sc + 132, V, n, st))) return finish(rc);
+        if ((rc = launch_scale(V, sc + beta_slot, V, n, st))) return finish(rc);
         g0[0] = beta;
         std::fill(g0.begin() + 1, g0.end(), 0.0);
         FDE_CUDA_TRY(cudaMemcpyAsync(P.d_gv, g0.data(), g0.size() * sizeof(double), cudaMemcpyHostToDevice, st));
@@ -1090,6 +1082,7 @@ int pgmres_solve(fde_problem* h, const fde_pgmres_opts* opts, const double* x0_a
         if ((rc = matvec(P, x, P.d_work))) return finish(rc);
         if ((rc = launch_sub(P.d_b_rhs, P.d_work, V, n, st))) return finish(rc);
         if ((rc = norm2(P, V, 132, &beta2, pin))) return finish(rc);
+        beta_slot = 132;
     }
     S.iterations = its;
     ++P.solves;

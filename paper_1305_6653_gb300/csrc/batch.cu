@@ -83,7 +83,7 @@ int gather(fde_batch* b) {
 // One restart cycle of the batched flexible GMRES for the nr instances of the current
 // round list (b->d_act): iterations j = 0..restart-1, each a fixed sequence of launches
 // over the whole round.  An instance that meets its tolerance (or maxit, a breakdown,
-// a non-finite value) has its live flag cleared by finish_batched on the device, and
+// a non-finite value) has its live flag cleared by gs_batched on the device, and
 // every later kernel of the cycle skips it; nothing returns to the host until the
 // cycle is over.
 int cycle_launches(fde_batch* b, int nr, const fde_pgmres_opts& o, cudaStream_t st) {
@@ -103,15 +103,7 @@ int cycle_launches(fde_batch* b, int nr, const fde_pgmres_opts& o, cudaStream_t 
         if (rc) return rc;
         if ((rc = launch_time_ifft_batched(b->d_inst, b->d_act, nr, b->max_mp, b->max_s, j, st))) return rc;
         if ((rc = launch_matvec_batched(b->d_inst, b->d_act, nr, b->max_s, b->max_L, b->max_m, 0, j, st))) return rc;
-        if ((rc = launch_dots_batched(b->d_inst, b->d_act, nr, 0, j, st))) return rc;
-        if ((rc = launch_update_batched(b->d_inst, b->d_act, nr, 0, j, b->d_kvec, b->max_n, st))) return rc;
-        if (o.reorth) {
-            if ((rc = launch_dots_batched(b->d_inst, b->d_act, nr, 1, j, st))) return rc;
-            if ((rc = launch_update_batched(b->d_inst, b->d_act, nr, 1, j, b->d_kvec, b->max_n, st))) return rc;
-        }
-        if ((rc = launch_dots_batched(b->d_inst, b->d_act, nr, 2, j, st))) return rc;
-        if ((rc = launch_finish_batched(b->d_inst, b->d_act, nr, j, ldh, o.reorth, o.tol, o.maxit, st))) return rc;
-        if ((rc = launch_scale_batched(b->d_inst, b->d_act, nr, 0, j, o.restart, b->max_n, st))) return rc;
+        if ((rc = launch_gs_batched(b->d_inst, b->d_act, nr, j, ldh, o.reorth, o.tol, o.maxit, b->d_err, st))) return rc;
     }
     return FDE_OK;
 }
@@ -488,8 +480,8 @@ int fde_batch_solve(fde_batch* b, const fde_pgmres_opts* opts, double* const* x_
     if ((rc = launch_ctl_set_batched(b->d_inst, b->d_act, n, 1, 2, st))) return fail(rc);
     if ((rc = launch_matvec_batched(b->d_inst, b->d_act, n, b->max_s, b->max_L, b->max_m, 1, 0, st))) return fail(rc);
     if ((rc = launch_residual_batched(b->d_inst, b->d_act, n, b->max_n, st))) return fail(rc);
-    if ((rc = launch_dots_batched(b->d_inst, b->d_act, n, 4, 0, st))) return fail(rc);
-    if ((rc = launch_dots_batched(b->d_inst, b->d_act, n, 3, 0, st))) return fail(rc);
+    if ((rc = launch_norm_batched(b->d_inst, b->d_act, n, 4, st))) return fail(rc);
+    if ((rc = launch_norm_batched(b->d_inst, b->d_act, n, 3, st))) return fail(rc);
     std::vector<double> bnorm(n), beta(n), est(n, 0.0);
     // |b|^2 sits in scal[131]; gather it through a one-off copy per instance
     for (int i = 0; i < n; ++i) {
@@ -516,7 +508,7 @@ int fde_batch_solve(fde_batch* b, const fde_pgmres_opts* opts, double* const* x_
         const int nr = (int)round.size();
         if ((rc = upload_list(b, round, b->h_act, b->d_act))) return fail(rc);
         if ((rc = launch_ctl_set_batched(b->d_inst, b->d_act, nr, 1, 1, st))) return fail(rc);
-        if ((rc = launch_scale_batched(b->d_inst, b->d_act, nr, 1, 0, o.restart, b->max_n, st))) return fail(rc);
+        if ((rc = launch_scale_batched(b->d_inst, b->d_act, nr, o.restart, b->max_n, st))) return fail(rc);
         if ((rc = run_cycle(b, nr, o, st))) return fail(rc);
         FDE_CUDA_TRY(cudaMemcpyAsync(b->h_ctl, b->d_ctl, 4 * n * sizeof(int), cudaMemcpyDeviceToHost, st));
         if ((rc = gather(b))) return fail(rc);  // synchronises
@@ -540,11 +532,11 @@ int fde_batch_solve(fde_batch* b, const fde_pgmres_opts* opts, double* const* x_
         if ((rc = upload_list(b, upd, b->h_act, b->d_act))) return fail(rc);
         if ((rc = launch_ctl_set_batched(b->d_inst, b->d_act, nu, 1, 0, st))) return fail(rc);
         if ((rc = launch_lsq_batched(b->d_inst, b->d_act, nu, b->d_kvec, ldh, st))) return fail(rc);
-        if ((rc = launch_update_batched(b->d_inst, b->d_act, nu, 2, 0, b->d_kvec, b->max_n, st))) return fail(rc);
+        if ((rc = launch_update_batched(b->d_inst, b->d_act, nu, b->d_kvec, b->max_n, st))) return fail(rc);
         if ((rc = launch_matvec_batched(b->d_inst, b->d_act, nu, b->max_s, b->max_L, b->max_m, 1, 0, st)))
             return fail(rc);
         if ((rc = launch_residual_batched(b->d_inst, b->d_act, nu, b->max_n, st))) return fail(rc);
-        if ((rc = launch_dots_batched(b->d_inst, b->d_act, nu, 3, 0, st))) return fail(rc);
+        if ((rc = launch_norm_batched(b->d_inst, b->d_act, nu, 3, st))) return fail(rc);
         if ((rc = gather(b))) return fail(rc);
         for (int i : upd) {
             ++restarts[i];
@@ -573,7 +565,11 @@ int fde_batch_solve(fde_batch* b, const fde_pgmres_opts* opts, double* const* x_
     cudaEventElapsedTime(&ms, ev0, ev1);
     cudaEventDestroy(ev0);
     cudaEventDestroy(ev1);
-    if (derr) return set_error(FDE_ERR_TIMEOUT, "a bounded wait of the block solves timed out");
+    if (derr) {
+        for (fde_problem* p : b->probs)  // the Gram-Schmidt barriers start over
+            FDE_CUDA_TRY(cudaMemsetAsync(problem_of(p)->d_counter, 0, 4 * sizeof(unsigned int), st));
+        return set_error(FDE_ERR_TIMEOUT, "a bounded wait of the iteration timed out");
+    }
     int worst = FDE_OK;
     for (int i = 0; i < n; ++i) {
         if (stats) {

@@ -142,19 +142,13 @@ int launch_tile_inverse_fp32(Problem& P, cudaStream_t st);
 int launch_block_trsv(const Problem& P, void* rhat, cudaStream_t st);
 
 // krylov.cu
-int launch_dots(const double* V, int k, const double* w, long n, double* out, double* partial,
-                unsigned int* counter, cudaStream_t st);
 int launch_update(const double* V, int k, const double* coef, double sign, double* w, long n, cudaStream_t st);
 int launch_norm(const double* w, long n, double* out, double* partial, unsigned int* counter, cudaStream_t st);
-// Fused classical Gram-Schmidt pass over V_0..V_{k-1} (V row-major [k][n], w length n):
-// mode 0: out = V^T w;  1: w -= V c, then out = V^T w;  2: w -= V c, then out[0] = |w|^2
-int launch_cgs_pass(int mode, const double* V, int k, const double* c, double* w, long n, double* out,
-                    double* partial, unsigned int* counter, cudaStream_t st);
+// Arnoldi step j after the product: V_{j+1} against V_0..V_j (CGS2, or one pass without
+// reorth), column j of H with its Givens rotation, scal[128..130], V_{j+1} / |V_{j+1}|
+int launch_gram_schmidt(Problem& P, int j, int ldh, int reorth, cudaStream_t st);
 int launch_scale(const double* src, const double* nrm_sq, double* dst, long n, cudaStream_t st);
-int launch_arnoldi_finish(double* H, int ldh, int j, const double* h1, const double* h2, const double* nrm_sq,
-                          double* cs, double* sn, double* g, double* est, cudaStream_t st);
 int launch_lsq_solve(const double* H, int ldh, int k, const double* g, double* y, cudaStream_t st);
-int launch_axpy(double a, const double* x, double* y, long n, cudaStream_t st);
 int launch_sub(const double* b, const double* ax, double* r, long n, cudaStream_t st);
 
 // ---------------------------------------------------------------------------
@@ -363,16 +357,16 @@ int launch_time_ifft_batched(const InstDev* I, const int* act, int nact, int max
                              cudaStream_t st);
 int launch_matvec_batched(const InstDev* I, const int* act, int nact, int max_s, int max_L, int max_m, int which,
                           int j, cudaStream_t st);
-int launch_dots_batched(const InstDev* I, const int* act, int nact, int mode, int j, cudaStream_t st);
-int launch_update_batched(const InstDev* I, const int* act, int nact, int mode, int j, const int* kvec, long max_n,
-                          cudaStream_t st);
-int launch_scale_batched(const InstDev* I, const int* act, int nact, int mode, int j, int restart, long max_n,
-                         cudaStream_t st);
+// mode 3: |V_0|^2, mode 4: |b|^2 of every live instance
+int launch_norm_batched(const InstDev* I, const int* act, int nact, int mode, cudaStream_t st);
+int launch_update_batched(const InstDev* I, const int* act, int nact, const int* kvec, long max_n, cudaStream_t st);
+int launch_scale_batched(const InstDev* I, const int* act, int nact, int restart, long max_n, cudaStream_t st);
+// Gram-Schmidt step j of every live instance; it also decides, on the device, whether an
+// instance leaves the cycle (estimate <= tol |b|, maxit total steps, breakdown or a
+// non-finite value).  *err: set when a bounded wait ran out
+int launch_gs_batched(const InstDev* I, const int* act, int nact, int j, int ldh, int reorth, double tol, int maxit,
+                      int* err, cudaStream_t st);
 int launch_residual_batched(const InstDev* I, const int* act, int nact, long max_n, cudaStream_t st);
-// finish_batched also decides, on the device, whether the instance leaves the cycle
-// (estimate <= tol |b|, maxit total steps, breakdown or a non-finite value)
-int launch_finish_batched(const InstDev* I, const int* act, int nact, int j, int ldh, int reorth, double tol,
-                          int maxit, cudaStream_t st);
 // ctl[0] = live for the listed instances; reset: also zero ctl[1] (and ctl[2], ctl[3] when reset > 1)
 int launch_ctl_set_batched(const InstDev* I, const int* act, int nact, int live, int reset, cudaStream_t st);
 int launch_lsq_batched(const InstDev* I, const int* act, int nact, const int* kvec, int ldh, cudaStream_t st);

@@ -1,12 +1,9 @@
 // FP64 Krylov kernels of the flexible GMRES(restart) iteration (Sec. 3.2 cites
 // Saad's GMRES; Sec. 4 runs GMRES(20)): classical Gram-Schmidt with one
-// re-orthogonalisation (CGS2) as multi-dot / multi-axpy passes over the basis V,
-// the Givens least-squares update, and small vector kernels.
+// re-orthogonalisation (CGS2), the Givens least-squares update and the
+// normalisation of the new basis vector as one kernel, and small vector kernels.
 //
-// Reductions are deterministic: every CTA writes its partial sums, and the last
-// CTA to finish (atomic ticket after a fence; nothing waits) adds them in a fixed
-// order (one warp per vector, lanes over the partials, then a shuffle tree) and
-// resets the ticket.
+// Reductions are deterministic: partial sums are added in a fixed order.
 #include <algorithm>
 
 #include "fde_internal.h"
@@ -17,144 +14,452 @@ constexpr int RED_CTAS = 304;  // 2 per SM on 152 SMs
 constexpr int RED_THREADS = 256;
 constexpr int KMAX = 64;       // max Krylov vectors per multi-dot
 
-// Per-thread partial sums acc[0..k) -> out[0..k): each CTA stores its partials,
-// and the last CTA to finish adds them in a fixed order.
-template <int KC>
-__device__ __forceinline__ void reduce_partials(const double (&acc)[KC], int k, double* __restrict__ out,
-                                                double* __restrict__ partial, unsigned int* __restrict__ counter,
-                                                int bx, int nblocks) {
-    __shared__ double red[RED_THREADS / 32][KC];
+// Sum over a warp of C values a thread (C = 8 or 16), 15 / 16 additions a lane where C
+// butterflies take 5 C: every step halves the number of values, a lane keeping one half and
+// handing over the other.  Lane l ends with the sum of value l / (32 / C).
+template <int C>
+__device__ __forceinline__ double warp_sums(double (&a)[C]) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int off = 16, h = C / 2; h >= 1; off >>= 1, h >>= 1) {
+        const bool up = lane & off;
+#pragma unroll
+        for (int i = 0; i < h; ++i) {
+            const double keep = up ? a[i + h] : a[i], give = up ? a[i] : a[i + h];
+            a[i] = keep + __shfl_xor_sync(0xffffffffu, give, off);
+        }
+    }
+#pragma unroll
+    for (int off = 16 / C; off; off >>= 1) a[0] += __shfl_xor_sync(0xffffffffu, a[0], off);
+    return a[0];
+}
+
+// |w|^2 of a vector: CTA sums to partial, the last CTA to finish (atomic ticket after a
+// fence; nothing waits) adds them.
+__device__ __forceinline__ void norm_body(const double* __restrict__ w, long n, double* __restrict__ out,
+                                          double* __restrict__ partial, unsigned int* __restrict__ counter, int bx,
+                                          int nblocks) {
+    __shared__ double red[RED_THREADS / 32];
     __shared__ bool last;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int i = 0; i < KC; ++i) {
-        double v = acc[i];
-        for (int off = 16; off; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-        if (lane == 0) red[warp][i] = v;
-    }
+    double v = 0.0;
+    const long stride = (long)nblocks * blockDim.x;
+    for (long x = (long)bx * blockDim.x + threadIdx.x; x < n; x += stride) v += w[x] * w[x];
+    for (int off = 16; off; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+    if (lane == 0) red[warp] = v;
     __syncthreads();
-    for (int i = threadIdx.x; i < k; i += blockDim.x) {
-        double v = 0.0;
-        for (int q = 0; q < RED_THREADS / 32; ++q) v += red[q][i];
-        partial[(size_t)bx * KMAX + i] = v;
-    }
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) last = (atomicAdd(counter, 1u) == (unsigned)nblocks - 1);
-    __syncthreads();
-    if (last) {
+    if (threadIdx.x == 0) {
+        for (int q = 1; q < RED_THREADS / 32; ++q) v += red[q];
+        partial[bx] = v;
         __threadfence();
-        // warp q adds vectors i = q, q + 8, ..: its lanes split the CTA partials (fixed
-        // order, independent L2 loads), then a fixed shuffle tree
-        for (int i = warp; i < k; i += RED_THREADS / 32) {
+        last = (atomicAdd(counter, 1u) == (unsigned)nblocks - 1);
+    }
+    __syncthreads();
+    if (last && warp == 0) {
+        __threadfence();
+        v = 0.0;
+        for (int c = lane; c < nblocks; c += 32) v += __ldcg(partial + c);
+        for (int off = 16; off; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+        if (lane == 0) {
+            *out = v;
+            *counter = 0u;
+        }
+    }
+}
+
+__global__ void __launch_bounds__(RED_THREADS)
+norm_kernel(const double* __restrict__ w, long n, double* __restrict__ out, double* __restrict__ partial,
+            unsigned int* __restrict__ counter) {
+    norm_body(w, n, out, partial, counter, blockIdx.x, gridDim.x);
+}
+
+// ---------------------------------------------------------------------------
+// One Gram-Schmidt step: w against V_0..V_{k-1} (k = j + 1), column j of the Hessenberg
+// matrix with its Givens rotation, w / |w|.
+//
+//   h1 = V^T w;  w -= V h1, h2 = V^T w (with re-orthogonalisation);  w -= V h, |w|^2;
+//   w /= |w|.
+//
+// All passes run in one cooperative launch of G CTAs that meet at a barrier after each
+// pass; every CTA then adds the CTAs' partial sums itself.  GB300's two FP64 lanes an SM
+// bound it at large n (4 k n multiply-adds; m = 2047, s = 256: 49 us at the mean k = 13.5
+// were the lanes never idle), so what matters there is that nothing but those runs on them:
+// the passes' reductions took 5 butterfly additions per value and warp, half as much again
+// as the dots themselves.  At small n it is bound by latency: three barriers and three
+// reductions instead of five launches, and V stays in registers (ONE).
+// Mean step of a solve at m = 2047, s = 256 (26 steps): 144 -> 101 us; at m = 255, s = 64 (15
+// steps): 49 -> 19 us.
+// ---------------------------------------------------------------------------
+constexpr int GS_CTAS = 152;                 // at most one CTA per SM; partial sums are [2][64][GS_CTAS]
+constexpr int GS_WARPS = RED_THREADS / 32;   // most warps of a CTA
+constexpr int GS_SMEM = 200 * 1024;          // for the staged V of the looping form
+constexpr unsigned GS_SPINS = 1u << 24;      // polls before a wait gives up (seconds)
+
+struct GsArgs {
+    const double* V;
+    double* w;
+    long n;
+    int k, ldh, reorth;
+    double *H, *cs, *sn, *g, *scal;  // scal: [128] |w|^2, [129] estimate, [130] H(j+1,j) before rotation
+    double* partial;
+    unsigned int* bar;  // a counter per barrier, zero before the launch
+    int* err;
+};
+
+// The CTAs of one Gram-Schmidt step meet.  CTA 0 clears the next counter before it arrives
+// (nobody can be there yet), and counter 0 once everybody has left it.
+__device__ __forceinline__ void gs_barrier(unsigned int* bar, int slot, int cta, int G, int* err) {
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        if (cta == 0) bar[slot + 1] = 0u;
+        __threadfence();
+        atomicAdd(bar + slot, 1u);
+        unsigned seen, polls = 0;
+        do {
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(bar + slot) : "memory");
+        } while (seen < (unsigned)G && ++polls < GS_SPINS);
+        if (seen < (unsigned)G) *err = 1;
+        if (cta == 0 && slot > 0) bar[0] = 0u;
+    }
+    __syncthreads();
+}
+
+// out[i] = sum over the CTAs of sum over the warps of red[warp][i], i < k
+template <int KC, int NT>
+__device__ __forceinline__ void gs_collect(const GsArgs& A, const double (*red)[KC], int k, int slot, int cta, int G,
+                                           double* out) {
+    constexpr int NW = NT / 32;
+    __syncthreads();
+    double* part = A.partial + (size_t)(slot & 1) * 64 * GS_CTAS;
+    if ((int)threadIdx.x < k) {
+        double v = 0.0;
+#pragma unroll
+        for (int q = 0; q < NW; ++q) v += red[q][threadIdx.x];
+        if (G > 1) part[(size_t)threadIdx.x * GS_CTAS + cta] = v;
+        else out[threadIdx.x] = v;
+    }
+    if (G > 1) {
+        gs_barrier(A.bar, slot, cta, G, A.err);
+        const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+        for (int i = warp; i < k; i += NW) {
             double v = 0.0;
-            for (int c = lane; c < nblocks; c += 32) v += __ldcg(partial + (size_t)c * KMAX + i);
+            for (int c = lane; c < G; c += 32) v += __ldcg(part + (size_t)i * GS_CTAS + c);
             for (int off = 16; off; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
             if (lane == 0) out[i] = v;
         }
-        if (threadIdx.x == 0) *counter = 0u;
+    }
+    __syncthreads();
+}
+
+// red[warp][i] = the warp's sum of a(i), i < k: eights, of which those beyond k are skipped by
+// a branch (as everywhere below: a predicated FP64 instruction costs what an executed one does)
+template <int KC, typename F>
+__device__ __forceinline__ void gs_warp_sums(double (*red)[KC], int k, F a) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    static_assert(KC % 8 == 0, "whole eights");
+#pragma unroll
+    for (int i0 = 0; i0 < KC; i0 += 8) {
+        if (i0 < k) {
+            double b[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) b[i] = a(i0 + i);
+            const double v = warp_sums<8>(b);
+            if ((lane & 3) == 0) red[warp][i0 + (lane >> 2)] = v;
+        }
     }
 }
 
-template <int KC>
-__device__ __forceinline__ void dots_body(const double* __restrict__ V, int k, const double* __restrict__ w, long n,
-                                          double* __restrict__ out, double* __restrict__ partial,
-                                          unsigned int* __restrict__ counter, int bx, int nblocks) {
-    double acc[KC];
-#pragma unroll
-    for (int i = 0; i < KC; ++i) acc[i] = 0.0;
-    const long stride = (long)nblocks * blockDim.x;
-    for (long x = (long)bx * blockDim.x + threadIdx.x; x < n; x += stride) {
-        const double wx = w[x];
-#pragma unroll
-        for (int i = 0; i < KC; ++i)
-            if (i < k) acc[i] += V[(size_t)i * n + x] * wx;
+// Column j of the rotated Hessenberg matrix, its rotation and the rotated right-hand side;
+// |g_{j+1}| is the residual estimate.  H is column-major.  One thread.
+struct GsColumn {
+    double est, hnext, nrm;
+};
+__device__ __forceinline__ GsColumn gs_column(const GsArgs& A, const double* h1, const double* h2, const double* c0,
+                                              const double* s0, double nrm) {
+    const int j = A.k - 1;
+    double* col = A.H + (size_t)j * A.ldh;
+    double t = h1[0] + (h2 ? h2[0] : 0.0);
+    for (int i = 0; i < j; ++i) {
+        const double c = c0[i], s = s0[i], b = h1[i + 1] + (h2 ? h2[i + 1] : 0.0);
+        col[i] = c * t + s * b;
+        t = -s * t + c * b;
     }
-    reduce_partials<KC>(acc, k, out, partial, counter, bx, nblocks);
+    const double b = sqrt(nrm), r = hypot(t, b);
+    const double c = r > 0.0 ? t / r : 1.0, s = r > 0.0 ? b / r : 0.0;
+    A.cs[j] = c;
+    A.sn[j] = s;
+    col[j] = r;
+    col[j + 1] = 0.0;
+    const double gj = A.g[j];
+    A.g[j + 1] = -s * gj;
+    A.g[j] = c * gj;
+    GsColumn out{fabs(s * gj), b, nrm};
+    A.scal[128] = nrm;
+    A.scal[129] = out.est;
+    A.scal[130] = b;
+    return out;
 }
 
-// One pass of classical Gram-Schmidt over the basis V_0..V_{k-1} (x: element):
-//   MODE 0: out[i] = sum_x V_i[x] w[x]
-//   MODE 1: w[x] -= sum_i c[i] V_i[x], then out[i] = sum_x V_i[x] w[x] of the new w
-//   MODE 2: w[x] -= sum_i c[i] V_i[x], then out[0] = sum_x w[x]^2
-// The V_i[x] of an element are loaded once and serve both the update and the
-// sums, so CGS2 (dots, update + dots, update + norm) reads V three times.
-// PAIR: two neighbouring elements per thread with 16-byte loads (n even, so every
-// V_i starts on a 16-byte boundary).
-template <int KC, int MODE, bool PAIR>
-__global__ void __launch_bounds__(RED_THREADS)
-cgs_pass_kernel(const double* __restrict__ V, int k, const double* __restrict__ c, double* __restrict__ w, long n,
-                double* __restrict__ out, double* __restrict__ partial, unsigned int* __restrict__ counter) {
-    constexpr int NA = MODE == 2 ? 1 : KC;
-    constexpr int E = PAIR ? 2 : 1;
-    __shared__ double cs[KC];
-    if (MODE > 0) {
-        for (int i = threadIdx.x; i < KC; i += blockDim.x) cs[i] = i < k ? c[i] : 0.0;
-        __syncthreads();
+__device__ __forceinline__ void cp_async_elems(double* dst, const double* src, int bytes) {
+    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+    if (bytes == 16) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
+    else asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d), "l"(src) : "memory");
+}
+
+// The end of a step: |w|^2 from the warps' sums, w's scale, and on CTA 0 the column.
+template <int KC, int NT, typename Scale, typename Done>
+__device__ __forceinline__ void gs_end(const GsArgs& A, double sq, double (*red)[KC], const double* h1,
+                                       const double* h2, const double* gc, const double* gsn, int slot, int cta,
+                                       int G, Scale scale, Done done) {
+    __shared__ double nrm[1];
+    for (int off = 16; off; off >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, off);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5][0] = sq;
+    gs_collect<KC, NT>(A, red, 1, slot, cta, G, nrm);
+    const double len = sqrt(nrm[0]);
+    scale(len > 0.0 ? 1.0 / len : 0.0);
+    if (cta == 0 && threadIdx.x == 0) done(gs_column(A, h1, A.reorth ? h2 : nullptr, gc, gsn, nrm[0]));
+}
+
+// At most one element a thread (E neighbours): V and w stay in registers.
+template <int KC, int E, int NT>
+__global__ void __launch_bounds__(NT, 1) gs_one_kernel(const __grid_constant__ GsArgs A) {
+    __shared__ double red[NT / 32][KC];
+    __shared__ double h1[KC], h2[KC], gc[KC], gsn[KC];
+    const int tid = threadIdx.x, k = A.k, cta = blockIdx.x, G = gridDim.x;
+    const long n = A.n, x = ((long)cta * NT + tid) * E;
+    if (cta == 0 && tid < k - 1) {  // earlier rotations, for the column at the end
+        gc[tid] = A.cs[tid];
+        gsn[tid] = A.sn[tid];
     }
-    double acc[NA];
+    double v[KC][E], w[E];
 #pragma unroll
-    for (int i = 0; i < NA; ++i) acc[i] = 0.0;
-    const long ne = n / E;
-    const long stride = (long)gridDim.x * blockDim.x;
-    for (long q = (long)blockIdx.x * blockDim.x + threadIdx.x; q < ne; q += stride) {
-        const long x = q * E;
-        double wx[E], v[KC][E];
-        if (PAIR) {
-            const double2 t = *reinterpret_cast<const double2*>(w + x);
-            wx[0] = t.x;
-            wx[E - 1] = t.y;
+    for (int e = 0; e < E; ++e) w[e] = 0.0;
+#pragma unroll
+    for (int i = 0; i < KC; ++i)
+#pragma unroll
+        for (int e = 0; e < E; ++e) v[i][e] = 0.0;
+    if (x < n) {
+        if constexpr (E == 2) {
+            const double2 t = *reinterpret_cast<const double2*>(A.w + x);
+            w[0] = t.x;
+            w[1] = t.y;
         } else {
-            wx[0] = w[x];
+            w[0] = A.w[x];
         }
 #pragma unroll
         for (int i = 0; i < KC; ++i) {
             if (i < k) {
-                if (PAIR) {
-                    const double2 t = *reinterpret_cast<const double2*>(V + (size_t)i * n + x);
+                if constexpr (E == 2) {
+                    const double2 t = *reinterpret_cast<const double2*>(A.V + (size_t)i * n + x);
                     v[i][0] = t.x;
-                    v[i][E - 1] = t.y;
+                    v[i][1] = t.y;
                 } else {
-                    v[i][0] = V[(size_t)i * n + x];
+                    v[i][0] = A.V[(size_t)i * n + x];
                 }
-            } else {
-#pragma unroll
-                for (int e = 0; e < E; ++e) v[i][e] = 0.0;
-            }
-        }
-        if (MODE > 0) {
-#pragma unroll
-            for (int e = 0; e < E; ++e) {
-                double a = wx[e];
-#pragma unroll
-                for (int i = 0; i < KC; ++i)
-                    if (i < k) a -= cs[i] * v[i][e];
-                wx[e] = a;
-            }
-            if (PAIR)
-                *reinterpret_cast<double2*>(w + x) = make_double2(wx[0], wx[E - 1]);
-            else
-                w[x] = wx[0];
-        }
-#pragma unroll
-        for (int e = 0; e < E; ++e) {
-            if (MODE == 2) {
-                acc[0] += wx[e] * wx[e];
-            } else {
-#pragma unroll
-                for (int i = 0; i < NA; ++i)
-                    if (i < k) acc[i] += v[i][e] * wx[e];
             }
         }
     }
-    reduce_partials<NA>(acc, MODE == 2 ? 1 : k, out, partial, counter, blockIdx.x, gridDim.x);
+    const auto dots = [&](int slot, double* out) {
+        gs_warp_sums<KC>(red, k, [&](int i) {
+            double a = v[i][0] * w[0];
+#pragma unroll
+            for (int e = 1; e < E; ++e) a += v[i][e] * w[e];
+            return a;
+        });
+        gs_collect<KC, NT>(A, red, k, slot, cta, G, out);
+    };
+    const auto update = [&](const double* c) {
+        double s0[E], s1[E];
+#pragma unroll
+        for (int e = 0; e < E; ++e) s0[e] = s1[e] = 0.0;
+#pragma unroll
+        for (int i0 = 0; i0 < KC; i0 += 4) {
+            if (i0 < k) {
+#pragma unroll
+                for (int i = i0; i < i0 + 4; i += 2) {
+                    const double c0 = i < k ? c[i] : 0.0, c1 = i + 1 < k ? c[i + 1] : 0.0;
+#pragma unroll
+                    for (int e = 0; e < E; ++e) {
+                        s0[e] += c0 * v[i][e];
+                        s1[e] += c1 * v[i + 1][e];
+                    }
+                }
+            }
+        }
+#pragma unroll
+        for (int e = 0; e < E; ++e) w[e] -= s0[e] + s1[e];
+    };
+    dots(0, h1);
+    update(h1);
+    int slot = 1;
+    if (A.reorth) {
+        dots(1, h2);
+        update(h2);
+        slot = 2;
+    }
+    double sq = w[0] * w[0];
+#pragma unroll
+    for (int e = 1; e < E; ++e) sq += w[e] * w[e];
+    gs_end<KC, NT>(A, sq, red, h1, h2, gc, gsn, slot, cta, G, [&](double inv) {
+        if (x < n) {
+#pragma unroll
+            for (int e = 0; e < E; ++e) A.w[x + e] = w[e] * inv;
+        }
+    }, [](const GsColumn&) {});
 }
 
-template <int KC>
-__global__ void __launch_bounds__(RED_THREADS)
-dots_kernel(const double* __restrict__ V, int k, const double* __restrict__ w, long n, double* __restrict__ out,
-            double* __restrict__ partial, unsigned int* __restrict__ counter) {
-    dots_body<KC>(V, k, w, n, out, partial, counter, blockIdx.x, gridDim.x);
+// Any number of elements a thread, E neighbours at a time (E = 2: n even).  A thread copies
+// its own elements of V asynchronously into shared memory, one group ahead of the one it
+// works on, so the FP64 lanes do not wait for the loads and the registers hold only the sums.
+template <int KC, int E, typename Done>
+__device__ __forceinline__ void gs_body(const GsArgs& A, int cta, int G, double* stage, Done done) {
+    __shared__ double red[GS_WARPS][KC];
+    __shared__ double h1[KC], h2[KC], gc[KC], gsn[KC];
+    constexpr int ROW = RED_THREADS * E;
+    const int tid = threadIdx.x, k = A.k, k4 = (k + 3) & ~3;
+    const int stages = 2 * k4 * ROW * (int)sizeof(double) <= GS_SMEM ? 2 : 1;
+    const long n = A.n, step = (long)G * ROW, x0 = ((long)cta * RED_THREADS + tid) * E;
+    if (cta == 0 && tid < k - 1) {  // earlier rotations, for the column at the end
+        gc[tid] = A.cs[tid];
+        gsn[tid] = A.sn[tid];
+    }
+    // rows k .. k4 - 1 stay zero, so that the loops run in fours
+    for (int s = 0; s < stages; ++s)
+        for (int i = k; i < k4; ++i)
+#pragma unroll
+            for (int e = 0; e < E; ++e) stage[(s * k4 + i) * ROW + tid * E + e] = 0.0;
+    const auto issue = [&](long x, int s) {
+        if (x < n) {
+            const double* src = A.V + x;
+            double* dst = stage + s * k4 * ROW + tid * E;
+#pragma unroll 4
+            for (int i = 0; i < k; ++i) cp_async_elems(dst + i * ROW, src + (size_t)i * n, 8 * E);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    const auto load_w = [&](long x, double (&t)[E]) {
+        if (x >= n) return;
+        if constexpr (E == 2) {
+            const double2 u = *reinterpret_cast<const double2*>(A.w + x);
+            t[0] = u.x;
+            t[1] = u.y;
+        } else {
+            t[0] = A.w[x];
+        }
+    };
+    const auto store_w = [&](long x, const double (&t)[E]) {
+        if constexpr (E == 2) *reinterpret_cast<double2*>(A.w + x) = make_double2(t[0], t[1]);
+        else A.w[x] = t[0];
+    };
+    const auto row = [&](const double* v, int i, double (&t)[E]) {
+        if constexpr (E == 2) {
+            const double2 u = *reinterpret_cast<const double2*>(v + i * ROW);
+            t[0] = u.x;
+            t[1] = u.y;
+        } else {
+            t[0] = v[i * ROW];
+        }
+    };
+    // w -= V c where c is given (stored), then work(v, w) for every group of elements
+    const auto pass = [&](const double* c, auto work) {
+        double w[E], wn[E];
+        int s = 0;
+        issue(x0, 0);
+        load_w(x0, wn);
+        for (long x = x0; x < n; x += step) {
+#pragma unroll
+            for (int e = 0; e < E; ++e) w[e] = wn[e];
+            if (stages == 2) {
+                issue(x + step, s ^ 1);
+                asm volatile("cp.async.wait_group 1;" ::: "memory");
+            } else {
+                asm volatile("cp.async.wait_group 0;" ::: "memory");
+            }
+            load_w(x + step, wn);
+            const double* v = stage + s * k4 * ROW + tid * E;
+            if (c) {
+                double p[4][E];
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+#pragma unroll
+                    for (int e = 0; e < E; ++e) p[u][e] = 0.0;
+#pragma unroll 2
+                for (int i = 0; i < k4; i += 4) {
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        double t[E];
+                        row(v, i + u, t);
+                        const double ci = c[i + u];
+#pragma unroll
+                        for (int e = 0; e < E; ++e) p[u][e] += ci * t[e];
+                    }
+                }
+#pragma unroll
+                for (int e = 0; e < E; ++e) w[e] -= (p[0][e] + p[1][e]) + (p[2][e] + p[3][e]);
+                store_w(x, w);
+            }
+            work(v, w);
+            if (stages == 2) s ^= 1;
+            else issue(x + step, 0);
+        }
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+    };
+    const auto dots = [&](const double* c, int slot, double* out) {
+        double acc[KC];
+#pragma unroll
+        for (int i = 0; i < KC; ++i) acc[i] = 0.0;
+        pass(c, [&](const double* v, const double (&w)[E]) {
+#pragma unroll
+            for (int i0 = 0; i0 < KC; i0 += 4) {
+                if (i0 < k) {
+#pragma unroll
+                    for (int i = i0; i < i0 + 4; ++i) {
+                        double t[E];
+                        row(v, i, t);
+#pragma unroll
+                        for (int e = 0; e < E; ++e) acc[i] += t[e] * w[e];
+                    }
+                }
+            }
+        });
+        gs_warp_sums<KC>(red, k, [&](int i) { return acc[i]; });
+        gs_collect<KC, RED_THREADS>(A, red, k, slot, cta, G, out);
+    };
+    if (tid >= k && tid < KC) h1[tid] = h2[tid] = 0.0;  // the coefficients of the zero rows
+    dots(nullptr, 0, h1);
+    const double* c = h1;
+    int slot = 1;
+    if (A.reorth) {
+        dots(h1, 1, h2);
+        c = h2;
+        slot = 2;
+    }
+    double sq = 0.0;
+    pass(c, [&](const double*, const double (&w)[E]) {
+#pragma unroll
+        for (int e = 0; e < E; ++e) sq += w[e] * w[e];
+    });
+    gs_end<KC, RED_THREADS>(A, sq, red, h1, h2, gc, gsn, slot, cta, G, [&](double inv) {
+        for (long x = x0; x < n; x += step) {
+            double w[E];
+            load_w(x, w);
+#pragma unroll
+            for (int e = 0; e < E; ++e) w[e] *= inv;
+            store_w(x, w);
+        }
+    }, done);
+}
+
+template <int KC, int E>
+__global__ void __launch_bounds__(RED_THREADS, 1) gs_kernel(const __grid_constant__ GsArgs A) {
+    extern __shared__ __align__(16) unsigned char gs_smem[];
+    gs_body<KC, E>(A, blockIdx.x, gridDim.x, reinterpret_cast<double*>(gs_smem), [](const GsColumn&) {});
+}
+
+// shared memory of the staged V for k vectors
+static size_t gs_stage_bytes(int k, int E) {
+    const size_t one = (size_t)((k + 3) & ~3) * RED_THREADS * E * sizeof(double);
+    return 2 * one <= (size_t)GS_SMEM ? 2 * one : one;
 }
 
 // w += sign * sum_i coef[i] V_i
@@ -179,46 +484,10 @@ __global__ void scale_kernel(const double* __restrict__ src, const double* __res
     for (long x = (long)blockIdx.x * blockDim.x + threadIdx.x; x < n; x += stride) dst[x] = src[x] * inv;
 }
 
-__global__ void axpy_kernel(double a, const double* __restrict__ x, double* __restrict__ y, long n) {
-    const long stride = (long)gridDim.x * blockDim.x;
-    for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) y[i] += a * x[i];
-}
-
 __global__ void sub_kernel(const double* __restrict__ b, const double* __restrict__ ax, double* __restrict__ r,
                            long n) {
     const long stride = (long)gridDim.x * blockDim.x;
     for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) r[i] = b[i] - ax[i];
-}
-
-// Column j of the Hessenberg matrix from the Gram-Schmidt coefficients, the
-// previous Givens rotations applied to it, a new rotation that annihilates
-// H[j+1][j], and the rotated right-hand side g; est = |g_{j+1}| is the residual
-// norm of the current cycle.  H is column-major with leading dimension ldh.
-__global__ void arnoldi_finish_kernel(double* __restrict__ H, int ldh, int j, const double* __restrict__ h1,
-                                      const double* __restrict__ h2, const double* __restrict__ nrm_sq,
-                                      double* __restrict__ cs, double* __restrict__ sn, double* __restrict__ g,
-                                      double* __restrict__ est) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    double* col = H + (size_t)j * ldh;
-    for (int i = 0; i <= j; ++i) col[i] = h1[i] + (h2 ? h2[i] : 0.0);
-    col[j + 1] = sqrt(*nrm_sq);
-    for (int i = 0; i < j; ++i) {
-        const double t = cs[i] * col[i] + sn[i] * col[i + 1];
-        col[i + 1] = -sn[i] * col[i] + cs[i] * col[i + 1];
-        col[i] = t;
-    }
-    const double a = col[j], b = col[j + 1];
-    const double r = hypot(a, b);
-    const double c = r > 0.0 ? a / r : 1.0;
-    const double s = r > 0.0 ? b / r : 0.0;
-    cs[j] = c;
-    sn[j] = s;
-    col[j] = r;
-    col[j + 1] = 0.0;
-    g[j + 1] = -s * g[j];
-    g[j] = c * g[j];
-    est[0] = fabs(g[j + 1]);
-    est[1] = b;  // H[j+1][j] before rotation (breakdown test)
 }
 
 // y = R^{-1} g with R the k x k upper-triangular part of the rotated H.
@@ -238,68 +507,122 @@ __global__ void lsq_solve_kernel(const double* __restrict__ H, int ldh, int k, c
 // ---------------------------------------------------------------------------
 constexpr int RED_CTAS_B = 32;  // reduction CTAs per instance in a batch
 
-// mode 0 / 1: h1 / h2 = V_{0..j}^T V_{j+1};  mode 2: |V_{j+1}|^2 -> scal[128];
 // mode 3: |V_0|^2 -> scal[132];  mode 4: |b|^2 -> scal[131]
-template <int KC>
 __global__ void __launch_bounds__(RED_THREADS)
-dots_batched(const InstDev* __restrict__ I, const int* __restrict__ act, int mode, int j) {
+norm_batched(const InstDev* __restrict__ I, const int* __restrict__ act, int mode) {
     const InstDev& d = I[act[blockIdx.y]];
     if (!d.ctl[0]) return;  // the instance has left the cycle: no CTA of it takes part
-    const double* w;
-    const double* V;
-    int k;
-    double* out;
-    if (mode <= 1) {
-        V = d.V; k = j + 1; w = d.V + (size_t)(j + 1) * d.n; out = d.scal + (mode == 0 ? 0 : 64);
-    } else if (mode == 2) {
-        V = w = d.V + (size_t)(j + 1) * d.n; k = 1; out = d.scal + 128;
-    } else if (mode == 3) {
-        V = w = d.V; k = 1; out = d.scal + 132;
-    } else {
-        V = w = d.b; k = 1; out = d.scal + 131;
-    }
-    dots_body<KC>(V, k, w, d.n, out, d.partial, d.counter, blockIdx.x, gridDim.x);
+    norm_body(mode == 3 ? d.V : d.b, d.n, d.scal + (mode == 3 ? 132 : 131), d.partial, d.counter, blockIdx.x,
+              gridDim.x);
 }
 
-// mode 0 / 1: V_{j+1} -= V_{0..j} h1 / h2;  mode 2: x += Z_{0..k-1} y with k = kvec[instance]
-__global__ void update_batched(const InstDev* __restrict__ I, const int* __restrict__ act, int mode, int j,
+// x += Z_{0..k-1} y with k = kvec[instance]
+__global__ void update_batched(const InstDev* __restrict__ I, const int* __restrict__ act,
                                const int* __restrict__ kvec) {
     __shared__ double c[KMAX];
     const int inst = act[blockIdx.y];
     const InstDev& d = I[inst];
     if (!d.ctl[0]) return;
-    const double* V;
-    double* w;
-    const double* coef;
-    int k;
-    double sign;
-    if (mode <= 1) {
-        V = d.V; w = d.V + (size_t)(j + 1) * d.n; coef = d.scal + (mode == 0 ? 0 : 64); k = j + 1; sign = -1.0;
-    } else {
-        V = d.Z; w = d.x; coef = d.y; k = kvec[inst]; sign = 1.0;
-    }
-    for (int i = threadIdx.x; i < k; i += blockDim.x) c[i] = sign * coef[i];
+    const int k = kvec[inst];
+    for (int i = threadIdx.x; i < k; i += blockDim.x) c[i] = d.y[i];
     __syncthreads();
     const long stride = (long)gridDim.x * blockDim.x;
     for (long x = (long)blockIdx.x * blockDim.x + threadIdx.x; x < d.n; x += stride) {
-        double acc = w[x];
-        for (int i = 0; i < k; ++i) acc += c[i] * V[(size_t)i * d.n + x];
-        w[x] = acc;
+        double acc = d.x[x];
+        for (int i = 0; i < k; ++i) acc += c[i] * d.Z[(size_t)i * d.n + x];
+        d.x[x] = acc;
     }
 }
 
-// mode 0: V_{j+1} /= sqrt(scal[128]);  mode 1: V_0 /= sqrt(scal[132]) and g = (sqrt(scal[132]), 0, ...)
-__global__ void scale_batched(const InstDev* __restrict__ I, const int* __restrict__ act, int mode, int j,
-                              int restart) {
+// V_0 /= sqrt(scal[132]) and g = (sqrt(scal[132]), 0, ...)
+__global__ void scale_batched(const InstDev* __restrict__ I, const int* __restrict__ act, int restart) {
     const InstDev& d = I[act[blockIdx.y]];
     if (!d.ctl[0]) return;
-    double* v = mode == 0 ? d.V + (size_t)(j + 1) * d.n : d.V;
-    const double nr = sqrt(d.scal[mode == 0 ? 128 : 132]);
+    const double nr = sqrt(d.scal[132]);
     const double inv = nr > 0.0 ? 1.0 / nr : 0.0;
     const long stride = (long)gridDim.x * blockDim.x;
-    for (long x = (long)blockIdx.x * blockDim.x + threadIdx.x; x < d.n; x += stride) v[x] *= inv;
-    if (mode == 1 && blockIdx.x == 0)
+    for (long x = (long)blockIdx.x * blockDim.x + threadIdx.x; x < d.n; x += stride) d.V[x] *= inv;
+    if (blockIdx.x == 0)
         for (int i = threadIdx.x; i <= restart; i += blockDim.x) d.gv[i] = i == 0 ? nr : 0.0;
+}
+
+// The Gram-Schmidt step j of every live instance in one cooperative launch.  The CTAs are
+// shared out in proportion to the instances' lengths, one at least; with more live instances
+// than CTAs each CTA takes instances of its own, alone.  Every CTA works the shares out for
+// itself: an instance takes part if it is live or has already finished this step (a CTA that
+// starts late may see the flags its step has left: ctl[1] = j + 1 is written before ctl[0]).
+// An instance leaves the cycle on the device: tolerance met (Givens estimate), maxit,
+// breakdown, or a non-finite value.
+template <int KC, int E>
+__global__ void __launch_bounds__(RED_THREADS, 1)
+gs_batched(const InstDev* __restrict__ I, const int* __restrict__ act, int nact, int j, int ldh, int reorth,
+           double tol, int maxit, int* __restrict__ err, int stage_doubles) {
+    extern __shared__ __align__(16) unsigned char gs_smem[];
+    double* stage = reinterpret_cast<double*>(gs_smem);
+    double* len = stage + stage_doubles;  // length of each listed instance, 0: not taking part
+    __shared__ int sh_inst, sh_cta, sh_G, sh_live;
+    for (int a = threadIdx.x; a < nact; a += RED_THREADS) {
+        const InstDev& d = I[act[a]];
+        volatile int* c = d.ctl;
+        bool on = c[0] != 0;
+        __threadfence();
+        if (!on) on = c[1] == j + 1;
+        len[a] = on ? (double)d.n : 0.0;
+    }
+    __syncthreads();
+    const int B = gridDim.x;
+    if (threadIdx.x == 0) {
+        double total = 0.0;
+        int live = 0;
+        for (int a = 0; a < nact; ++a) {
+            total += len[a];
+            live += len[a] > 0.0;
+        }
+        sh_live = live;
+        sh_inst = -1;
+        if (live <= B) {
+            int at = 0, rest = live;
+            for (int a = 0; a < nact; ++a) {
+                if (len[a] == 0.0) continue;
+                --rest;  // at most what leaves one for each of the rest
+                const int g = min(1 + (int)((double)(B - live) * (len[a] / total)), B - at - rest);
+                if ((int)blockIdx.x >= at && (int)blockIdx.x < at + g) {
+                    sh_inst = a;
+                    sh_cta = blockIdx.x - at;
+                    sh_G = g;
+                }
+                at += g;
+            }
+        }
+    }
+    __syncthreads();
+    const auto step = [&](int a, int cta, int G) {
+        const InstDev& d = I[act[a]];
+        GsArgs A{d.V, d.V + (size_t)(j + 1) * d.n, d.n, j + 1, ldh, reorth, d.H, d.cs, d.sn, d.gv, d.scal,
+                 d.partial, d.counter, err};
+        gs_body<KC, E>(A, cta, G, stage, [&](const GsColumn& col) {
+            volatile int* c = d.ctl;
+            const int its = c[2] + 1;
+            c[2] = its;
+            c[1] = j + 1;
+            const bool bad = !isfinite(col.est) || !isfinite(col.nrm);
+            if (bad) c[3] = 1;
+            __threadfence();
+            if (bad || col.est <= tol * sqrt(d.scal[131]) || its >= maxit || fabs(col.hnext) <= 1e-300) c[0] = 0;
+        });
+    };
+    if (sh_live <= B) {
+        if (sh_inst >= 0) step(sh_inst, sh_cta, sh_G);
+    } else {
+        int i = 0;
+        for (int a = 0; a < nact; ++a) {
+            if (len[a] == 0.0) continue;
+            if (i++ % B == (int)blockIdx.x) {
+                step(a, 0, 1);
+                __syncthreads();
+            }
+        }
+    }
 }
 
 // V_0 = b - work (work = M x)
@@ -308,48 +631,6 @@ __global__ void residual_batched(const InstDev* __restrict__ I, const int* __res
     if (!d.ctl[0]) return;
     const long stride = (long)gridDim.x * blockDim.x;
     for (long x = (long)blockIdx.x * blockDim.x + threadIdx.x; x < d.n; x += stride) d.V[x] = d.b[x] - d.work[x];
-}
-
-// one thread per active instance
-__global__ void finish_batched(const InstDev* __restrict__ I, const int* __restrict__ act, int nact, int j, int ldh,
-                               int reorth, double tol, int maxit) {
-    const int a = blockIdx.x * blockDim.x + threadIdx.x;
-    if (a >= nact) return;
-    const InstDev& d = I[act[a]];
-    if (!d.ctl[0]) return;
-    double* col = d.H + (size_t)j * ldh;
-    const double* h1 = d.scal;
-    const double* h2 = d.scal + 64;
-    for (int i = 0; i <= j; ++i) col[i] = h1[i] + (reorth ? h2[i] : 0.0);
-    col[j + 1] = sqrt(d.scal[128]);
-    for (int i = 0; i < j; ++i) {
-        const double t = d.cs[i] * col[i] + d.sn[i] * col[i + 1];
-        col[i + 1] = -d.sn[i] * col[i] + d.cs[i] * col[i + 1];
-        col[i] = t;
-    }
-    const double aa = col[j], bb = col[j + 1];
-    const double r = hypot(aa, bb);
-    const double c = r > 0.0 ? aa / r : 1.0;
-    const double sn = r > 0.0 ? bb / r : 0.0;
-    d.cs[j] = c;
-    d.sn[j] = sn;
-    col[j] = r;
-    col[j + 1] = 0.0;
-    d.gv[j + 1] = -sn * d.gv[j];
-    d.gv[j] = c * d.gv[j];
-    const double est = fabs(d.gv[j + 1]);
-    d.scal[129] = est;
-    d.scal[130] = bb;
-    // leave the cycle: tolerance met (Givens estimate), maxit, breakdown, or non-finite
-    const int its = d.ctl[2] + 1;
-    d.ctl[2] = its;
-    d.ctl[1] = j + 1;
-    if (!isfinite(est) || !isfinite(d.scal[128])) {
-        d.ctl[3] = 1;
-        d.ctl[0] = 0;
-    } else if (est <= tol * sqrt(d.scal[131]) || its >= maxit || fabs(bb) <= 1e-300) {
-        d.ctl[0] = 0;
-    }
 }
 
 __global__ void ctl_set_batched(const InstDev* __restrict__ I, const int* __restrict__ act, int nact, int live,
@@ -393,35 +674,59 @@ __global__ void gather_scalars(const InstDev* __restrict__ I, int ninst, double*
 
 static int grid_for(long n);
 
-int launch_dots_batched(const InstDev* I, const int* act, int nact, int mode, int j, cudaStream_t st) {
+int launch_norm_batched(const InstDev* I, const int* act, int nact, int mode, cudaStream_t st) {
     if (nact <= 0) return FDE_OK;
-    const int k = mode <= 1 ? j + 1 : 1;
-    const dim3 grid(RED_CTAS_B, nact);
-    if (k <= 8) dots_batched<8><<<grid, RED_THREADS, 0, st>>>(I, act, mode, j);
-    else if (k <= 16) dots_batched<16><<<grid, RED_THREADS, 0, st>>>(I, act, mode, j);
-    else if (k <= 32) dots_batched<32><<<grid, RED_THREADS, 0, st>>>(I, act, mode, j);
-    else dots_batched<64><<<grid, RED_THREADS, 0, st>>>(I, act, mode, j);
-    FDE_LAUNCH_CHECK("dots_batched");
+    norm_batched<<<dim3(RED_CTAS_B, nact), RED_THREADS, 0, st>>>(I, act, mode);
+    FDE_LAUNCH_CHECK("norm_batched");
     return FDE_OK;
 }
 
-int launch_update_batched(const InstDev* I, const int* act, int nact, int mode, int j, const int* kvec, long max_n,
-                          cudaStream_t st) {
+int launch_update_batched(const InstDev* I, const int* act, int nact, const int* kvec, long max_n, cudaStream_t st) {
     if (nact <= 0) return FDE_OK;
     int g = (int)((max_n + 255) / 256);
     if (g > 64) g = 64;
-    update_batched<<<dim3(g, nact), 256, 0, st>>>(I, act, mode, j, kvec);
+    update_batched<<<dim3(g, nact), 256, 0, st>>>(I, act, kvec);
     FDE_LAUNCH_CHECK("update_batched");
     return FDE_OK;
 }
 
-int launch_scale_batched(const InstDev* I, const int* act, int nact, int mode, int j, int restart, long max_n,
-                         cudaStream_t st) {
+int launch_scale_batched(const InstDev* I, const int* act, int nact, int restart, long max_n, cudaStream_t st) {
     if (nact <= 0) return FDE_OK;
     int g = (int)((max_n + 255) / 256);
     if (g > 64) g = 64;
-    scale_batched<<<dim3(g, nact), 256, 0, st>>>(I, act, mode, j, restart);
+    scale_batched<<<dim3(g, nact), 256, 0, st>>>(I, act, restart);
     FDE_LAUNCH_CHECK("scale_batched");
+    return FDE_OK;
+}
+
+// CTAs of a cooperative Gram-Schmidt launch: one per SM of the current device
+static int gs_ctas(int* out) {
+    int dev = 0, sms = 0;
+    FDE_CUDA_TRY(cudaGetDevice(&dev));
+    FDE_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    *out = std::min(sms, GS_CTAS);
+    return FDE_OK;
+}
+
+int launch_gs_batched(const InstDev* I, const int* act, int nact, int j, int ldh, int reorth, double tol, int maxit,
+                      int* err, cudaStream_t st) {
+    if (nact <= 0) return FDE_OK;
+    const int k = j + 1;
+    if (k > KMAX) return set_error(FDE_ERR_ARG, "too many Krylov vectors for one Gram-Schmidt step");
+    int ctas = 0, rc = gs_ctas(&ctas);
+    if (rc) return rc;
+    const void* kern = k <= 8    ? (const void*)gs_batched<8, 2>
+                       : k <= 16 ? (const void*)gs_batched<16, 2>
+                       : k <= 24 ? (const void*)gs_batched<24, 2>
+                       : k <= 32 ? (const void*)gs_batched<32, 1>
+                                 : (const void*)gs_batched<64, 1>;
+    const size_t stage = gs_stage_bytes(k, k <= 24 ? 2 : 1);
+    int stage_doubles = (int)(stage / sizeof(double));
+    const size_t smem = stage + (size_t)nact * sizeof(double);
+    FDE_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    void* args[] = {&I, &act, &nact, &j, &ldh, &reorth, &tol, &maxit, &err, &stage_doubles};
+    FDE_CUDA_TRY(cudaLaunchCooperativeKernel(kern, dim3(ctas), dim3(RED_THREADS), args, smem, st));
+    FDE_LAUNCH_CHECK("gs_batched");
     return FDE_OK;
 }
 
@@ -431,14 +736,6 @@ int launch_residual_batched(const InstDev* I, const int* act, int nact, long max
     if (g > 64) g = 64;
     residual_batched<<<dim3(g, nact), 256, 0, st>>>(I, act);
     FDE_LAUNCH_CHECK("residual_batched");
-    return FDE_OK;
-}
-
-int launch_finish_batched(const InstDev* I, const int* act, int nact, int j, int ldh, int reorth, double tol,
-                          int maxit, cudaStream_t st) {
-    if (nact <= 0) return FDE_OK;
-    finish_batched<<<(nact + 63) / 64, 64, 0, st>>>(I, act, nact, j, ldh, reorth, tol, maxit);
-    FDE_LAUNCH_CHECK("finish_batched");
     return FDE_OK;
 }
 
@@ -469,81 +766,44 @@ static int grid_for(long n) {
     return (int)g;
 }
 
-int launch_dots(const double* V, int k, const double* w, long n, double* out, double* partial, unsigned int* counter,
-                cudaStream_t st) {
-    if (k <= 0) return FDE_OK;
-    if (k > KMAX) return set_error(FDE_ERR_ARG, "too many Krylov vectors for one multi-dot");
-    if (k <= 8)
-        dots_kernel<8><<<RED_CTAS, RED_THREADS, 0, st>>>(V, k, w, n, out, partial, counter);
-    else if (k <= 16)
-        dots_kernel<16><<<RED_CTAS, RED_THREADS, 0, st>>>(V, k, w, n, out, partial, counter);
-    else if (k <= 32)
-        dots_kernel<32><<<RED_CTAS, RED_THREADS, 0, st>>>(V, k, w, n, out, partial, counter);
-    else
-        dots_kernel<64><<<RED_CTAS, RED_THREADS, 0, st>>>(V, k, w, n, out, partial, counter);
-    FDE_LAUNCH_CHECK("dots_kernel");
-    return FDE_OK;
-}
-
-// One wave: as many CTAs as fit on the device at once (the wide variants hold
-// their basis values in registers and fit one CTA per SM), at most RED_CTAS.
-template <int KC, int MODE, bool PAIR>
-static int one_wave_grid() {
-    static int grid = 0;  // per kernel instantiation
-    if (grid == 0) {
-        auto kernel = cgs_pass_kernel<KC, MODE, PAIR>;
-        int dev = 0, sms = 0, occ = 0;
-        if (cudaGetDevice(&dev) != cudaSuccess ||
-            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, RED_THREADS, 0) != cudaSuccess || occ < 1)
-            return RED_CTAS;
-        grid = std::min(RED_CTAS, sms * occ);
+// The form for n elements and k <= KC vectors: one element a thread in CTAs of 64, 128 or 256
+// threads (the fewest that need no more CTAs than SMs, so that all SMs share the FP64 work),
+// then the loop over pairs.  At n = 16,320 a step of k <= 8 takes 15.7 us with 128 threads a CTA and
+// 16.5 with 256 on half as many SMs.
+struct GsForm {
+    const void* kern;
+    int grid, threads;
+    size_t smem;
+};
+template <int KC, int E>
+static GsForm gs_form(long n, int k, int ctas) {
+    const auto fits = [&](int per) { return (n + per - 1) / per <= ctas; };
+    const auto grid = [&](int per) { return (int)((n + per - 1) / per); };
+    if constexpr (KC <= 32) {
+        if (fits(64)) return {(const void*)gs_one_kernel<KC, 1, 64>, grid(64), 64, 0};
+        if (fits(128)) return {(const void*)gs_one_kernel<KC, 1, 128>, grid(128), 128, 0};
+        if (fits(256)) return {(const void*)gs_one_kernel<KC, 1, 256>, grid(256), 256, 0};
     }
-    return grid;
+    // n = s m is even (s is a power of two), as the pairs of E = 2 need it
+    return {(const void*)gs_kernel<KC, E>, std::min(grid(RED_THREADS * E), ctas), RED_THREADS, gs_stage_bytes(k, E)};
 }
 
-template <int KC, int MODE>
-static void cgs_pass_launch(const double* V, int k, const double* c, double* w, long n, double* out, double* partial,
-                            unsigned int* counter, cudaStream_t st) {
-    if constexpr (KC <= 24) {  // wider paired variants would spill
-        if ((n & 1) == 0) {
-            auto kern = cgs_pass_kernel<KC, MODE, true>;
-            kern<<<one_wave_grid<KC, MODE, true>(), RED_THREADS, 0, st>>>(V, k, c, w, n, out, partial, counter);
-            return;
-        }
-    }
-    auto kern = cgs_pass_kernel<KC, MODE, false>;
-    kern<<<one_wave_grid<KC, MODE, false>(), RED_THREADS, 0, st>>>(V, k, c, w, n, out, partial, counter);
-}
-
-template <int MODE>
-static void cgs_pass_dispatch(const double* V, int k, const double* c, double* w, long n, double* out,
-                              double* partial, unsigned int* counter, cudaStream_t st) {
-    if (k <= 8)
-        cgs_pass_launch<8, MODE>(V, k, c, w, n, out, partial, counter, st);
-    else if (k <= 16)
-        cgs_pass_launch<16, MODE>(V, k, c, w, n, out, partial, counter, st);
-    else if (k <= 24)
-        cgs_pass_launch<24, MODE>(V, k, c, w, n, out, partial, counter, st);
-    else if (k <= 32)
-        cgs_pass_launch<32, MODE>(V, k, c, w, n, out, partial, counter, st);
-    else
-        cgs_pass_launch<64, MODE>(V, k, c, w, n, out, partial, counter, st);
-}
-
-int launch_cgs_pass(int mode, const double* V, int k, const double* c, double* w, long n, double* out,
-                    double* partial, unsigned int* counter, cudaStream_t st) {
-    if (k <= 0 || n <= 0) return set_error(FDE_ERR_ARG, "empty Gram-Schmidt pass");
-    if (k > KMAX) return set_error(FDE_ERR_ARG, "too many Krylov vectors for one Gram-Schmidt pass");
-    if (mode == 0)
-        cgs_pass_dispatch<0>(V, k, c, w, n, out, partial, counter, st);
-    else if (mode == 1)
-        cgs_pass_dispatch<1>(V, k, c, w, n, out, partial, counter, st);
-    else if (mode == 2)
-        cgs_pass_dispatch<2>(V, k, c, w, n, out, partial, counter, st);
-    else
-        return set_error(FDE_ERR_ARG, "unknown Gram-Schmidt pass mode");
-    FDE_LAUNCH_CHECK("cgs_pass_kernel");
+int launch_gram_schmidt(Problem& P, int j, int ldh, int reorth, cudaStream_t st) {
+    const int k = j + 1;
+    if (k > KMAX) return set_error(FDE_ERR_ARG, "too many Krylov vectors for one Gram-Schmidt step");
+    int ctas = 0, rc = gs_ctas(&ctas);
+    if (rc) return rc;
+    const GsForm f = k <= 8    ? gs_form<8, 2>(P.n, k, ctas)
+                     : k <= 16 ? gs_form<16, 2>(P.n, k, ctas)
+                     : k <= 24 ? gs_form<24, 2>(P.n, k, ctas)
+                     : k <= 32 ? gs_form<32, 1>(P.n, k, ctas)
+                               : gs_form<64, 1>(P.n, k, ctas);
+    if (f.smem) FDE_CUDA_TRY(cudaFuncSetAttribute(f.kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)f.smem));
+    GsArgs A{P.d_V, P.d_V + (size_t)k * P.n, P.n, k, ldh, reorth, P.d_H, P.d_cs, P.d_sn, P.d_gv, P.d_scal,
+             P.d_partial, P.d_counter, P.d_err};
+    void* args[] = {&A};
+    FDE_CUDA_TRY(cudaLaunchCooperativeKernel(f.kern, dim3(f.grid), dim3(f.threads), args, f.smem, st));
+    FDE_LAUNCH_CHECK("gs_kernel");
     return FDE_OK;
 }
 
@@ -555,8 +815,9 @@ int launch_update(const double* V, int k, const double* coef, double sign, doubl
 }
 
 int launch_norm(const double* w, long n, double* out, double* partial, unsigned int* counter, cudaStream_t st) {
-    dots_kernel<8><<<RED_CTAS, RED_THREADS, 0, st>>>(w, 1, w, n, out, partial, counter);
-    FDE_LAUNCH_CHECK("dots_kernel(norm)");
+    const int grid = (int)std::max<long>(1, std::min<long>(RED_CTAS, (n + 1023) / 1024));
+    norm_kernel<<<grid, RED_THREADS, 0, st>>>(w, n, out, partial, counter);
+    FDE_LAUNCH_CHECK("norm_kernel");
     return FDE_OK;
 }
 
@@ -566,22 +827,9 @@ int launch_scale(const double* src, const double* nrm_sq, double* dst, long n, c
     return FDE_OK;
 }
 
-int launch_arnoldi_finish(double* H, int ldh, int j, const double* h1, const double* h2, const double* nrm_sq,
-                          double* cs, double* sn, double* g, double* est, cudaStream_t st) {
-    arnoldi_finish_kernel<<<1, 32, 0, st>>>(H, ldh, j, h1, h2, nrm_sq, cs, sn, g, est);
-    FDE_LAUNCH_CHECK("arnoldi_finish_kernel");
-    return FDE_OK;
-}
-
 int launch_lsq_solve(const double* H, int ldh, int k, const double* g, double* y, cudaStream_t st) {
     lsq_solve_kernel<<<1, 32, 0, st>>>(H, ldh, k, g, y);
     FDE_LAUNCH_CHECK("lsq_solve_kernel");
-    return FDE_OK;
-}
-
-int launch_axpy(double a, const double* x, double* y, long n, cudaStream_t st) {
-    axpy_kernel<<<grid_for(n), 256, 0, st>>>(a, x, y, n);
-    FDE_LAUNCH_CHECK("axpy_kernel");
     return FDE_OK;
 }
 
