@@ -50,12 +50,17 @@ constexpr int T2_CROW = 528;        // bytes per C-tile row in shared memory (51
 constexpr int T2_C_BYTES = T2_BM * T2_CROW;  // one plane
 
 // KIND 0: TF32; 1: BF16; 2: split TF32 -- every operand as hi + lo (both TF32) and
-// the product as A_hi B_hi + A_lo B_hi + A_hi B_lo (three K' = 256 segments), which
-// restores FP32-level accuracy at three times the tensor work.
+// the product as A_hi B_hi + A_lo B_hi + A_hi B_lo, which restores FP32-level accuracy at
+// three times the tensor work.  Each part is packed and streamed once: the main loop takes
+// a hi step (A_hi, B_hi chunks: one product) and a lo step (A_lo, B_lo: the two products
+// with the hi chunks of the step before) per K chunk, 512 KB a tile.  As three K' segments
+// (hi twice) it was 768 KB: the whole LU at m_p = 4096, 65 blocks took 80 ms, now 69.  What
+// bounds the update then is shared memory (the MMAs read 28 KB per K = 8, 109 of 128 bytes a
+// clock at full rate, beside the arriving operands); the tensor pipe is active 60 %.
 template <int KIND>
 struct Tc2 {
     static constexpr int ESZ = KIND == 1 ? 2 : 4;
-    static constexpr int KP = KIND == 2 ? 3 * T2_KP : T2_KP;  // K' of the packed operands
+    static constexpr int KP = KIND == 2 ? 2 * T2_KP : T2_KP;  // K' of the packed operands (hi, then lo)
     static constexpr int PER_CORE = 16 / ESZ;   // elements per core-matrix row
     static constexpr int KCH = 64 / ESZ;        // elements per 64-byte K-chunk
     static constexpr int NCH = KP / KCH;        // chunks per tile
@@ -83,8 +88,9 @@ struct Tc2 {
     static constexpr uint32_t IDESC_H = tc::instr_desc(KIND == 1 ? 1u : 2u, T2_BM, T2_BN);
     static constexpr uint32_t IDESC_HN = IDESC_H | tc::IDESC_NEGATE_A;
     // A' chunk holding the real K part of main-loop step it (its imaginary part is HALF
-    // chunks further; the step's B' chunk is chunk it)
-    __host__ __device__ static constexpr int re_chunk(int it) { return (it / HALF) * CPS + it % HALF; }
+    // chunks further) and the step's B' chunk; split TF32: even steps hi, odd steps lo
+    __host__ __device__ static constexpr int re_chunk(int it) { return KIND == 2 ? (it & 1) * CPS + it / 2 : it; }
+    __host__ __device__ static constexpr int b_chunk(int it) { return KIND == 2 ? (it & 1) * HALF + it / 2 : it; }
 };
 
 // The MMAs of one main-loop step into the accumulator at tacc (256 columns): a_re /
@@ -113,6 +119,28 @@ __device__ __forceinline__ void cplx_mma_step(uint32_t tacc, uint32_t a_re, uint
     }
 }
 
+// The products of main-loop step c for the A' chunks at offset a of its stage and the B'
+// chunk at offset b (cur, prev: shared addresses of this step's stage and the one before).
+template <int KIND>
+__device__ __forceinline__ void tc2_mma_step(uint32_t tacc, uint32_t cur, uint32_t prev, uint32_t a, uint32_t b, int c) {
+    using Cfg = Tc2<KIND>;
+    if (KIND == 2 && (c & 1)) {  // lo hi, hi lo
+        cplx_mma_step<KIND>(tacc, cur + a, cur + a + Cfg::A_CHUNK, prev + b, false);
+        cplx_mma_step<KIND>(tacc, prev + a, prev + a + Cfg::A_CHUNK, cur + b, false);
+    } else {
+        cplx_mma_step<KIND>(tacc, cur + a, cur + a + Cfg::A_CHUNK, cur + b, c == 0);
+    }
+}
+// ... and what frees its stages: a hi step's is read again by the lo step after it.
+template <int KIND>
+__device__ __forceinline__ void tc2_release(uint64_t* cur, uint64_t* prev, int c) {
+    if (KIND == 2) {
+        if (!(c & 1)) return;
+        tc::mma_commit(prev);
+    }
+    tc::mma_commit(cur);
+}
+
 // Byte offset of element (row, kp) of a packed tile whose chunks hold `rows` rows.
 template <int KIND>
 __device__ __forceinline__ uint32_t pack2_off(int rows, int row, int kp) {
@@ -131,8 +159,8 @@ __device__ __forceinline__ void pack2_raw(unsigned char* tile, int rows, int row
 }
 
 // Store value v at K' position kp of an A' tile (b_side = false, kp < 256) or a B'
-// tile (kp < 128).  Split TF32 repeats each value per product segment (256 K' for A',
-// 128 for B').
+// tile (kp < 128).  Split TF32 stores hi and, one segment (256 K' for A', 128 for B')
+// further, lo.
 template <int KIND>
 __device__ __forceinline__ void pack2_store(unsigned char* tile, int rows, int row, int kp, float v, bool b_side) {
     if constexpr (KIND == 2) {
@@ -140,8 +168,7 @@ __device__ __forceinline__ void pack2_store(unsigned char* tile, int rows, int r
         const float lo = tc::to_tf32(v - hi);
         const int seg = b_side ? TB : T2_KP;
         pack2_raw<KIND>(tile, rows, row, kp, hi);
-        pack2_raw<KIND>(tile, rows, row, seg + kp, b_side ? hi : lo);
-        pack2_raw<KIND>(tile, rows, row, 2 * seg + kp, b_side ? lo : hi);
+        pack2_raw<KIND>(tile, rows, row, seg + kp, lo);
     } else {
         pack2_raw<KIND>(tile, rows, row, kp, v);
     }
@@ -149,7 +176,7 @@ __device__ __forceinline__ void pack2_store(unsigned char* tile, int rows, int r
 
 // Store the PER_CORE values v[0..PER_CORE) at K' positions kp0 .. kp0 + PER_CORE - 1
 // (kp0 a multiple of PER_CORE, < 256 for A', < 128 for B') of one row: one 16-byte
-// core-matrix row segment per product segment.
+// core-matrix row segment (split TF32: one of hi and one of lo).
 template <int KIND>
 __device__ __forceinline__ void pack2_seg(unsigned char* tile, int rows, int row, int kp0, const float* v,
                                           bool b_side) {
@@ -165,8 +192,7 @@ __device__ __forceinline__ void pack2_seg(unsigned char* tile, int rows, int row
             const float4 lo = make_float4(tc::to_tf32(v[0] - hi.x), tc::to_tf32(v[1] - hi.y),
                                           tc::to_tf32(v[2] - hi.z), tc::to_tf32(v[3] - hi.w));
             const int seg = b_side ? TB : T2_KP;
-            *reinterpret_cast<float4*>(tile + pack2_off<KIND>(rows, row, seg + kp0)) = b_side ? hi : lo;
-            *reinterpret_cast<float4*>(tile + pack2_off<KIND>(rows, row, 2 * seg + kp0)) = b_side ? lo : hi;
+            *reinterpret_cast<float4*>(tile + pack2_off<KIND>(rows, row, seg + kp0)) = lo;
         }
     }
 }
@@ -256,6 +282,34 @@ __device__ __forceinline__ void pack_staged_b(unsigned char* __restrict__ pk, co
     }
 }
 
+// The operand ring of a CTA in which one thread both loads and issues: load(c) fills stage
+// c mod NS, mma(c, stage, stage before) issues step c's products.  A step's stages are
+// refilled one step (split TF32: one pair of steps) after its products were issued, so
+// that the products of the next are queued behind them meanwhile.  False on a timeout.
+template <int KIND, int NS, typename Load, typename Mma>
+__device__ __forceinline__ bool tc2_main_loop(int nsteps, uint64_t* full, uint64_t* empty, Load load, Mma mma) {
+    constexpr int AHEAD = KIND == 2 ? NS : NS - 1;
+    for (int c = 0; c < AHEAD && c < nsteps; ++c) load(c);
+    const auto refill = [&](int n) {  // step n takes the stage of step n - NS
+        if (n >= nsteps) return true;
+        if (n >= NS && !tc::mbar_wait(&empty[n % NS], (n / NS - 1) & 1)) return false;
+        load(n);
+        return true;
+    };
+    for (int c = 0; c < nsteps; ++c) {
+        const int s = c % NS, sp = (c + NS - 1) % NS;
+        if (!tc::mbar_wait(&full[s], (c / NS) & 1)) return false;
+        mma(c, s, sp);
+        tc2_release<KIND>(&empty[s], &empty[sp], c);
+        if (KIND == 2) {  // after a hi step: the stages of the pair before it
+            if (c >= 2 && !(c & 1) && !(refill(c - 2 + NS) && refill(c - 1 + NS))) return false;
+        } else if (!refill(c + NS - 1)) {
+            return false;
+        }
+    }
+    return true;
+}
+
 // One 128 x 128 complex output tile at (r0, c0) of one block, D = A' B'^T from the
 // packed tiles ga (A') and gb (B'):
 //   STORE = false: C[r0.., c0..] -= D (C prefetched into L2 at the start, staged
@@ -332,32 +386,12 @@ __device__ __forceinline__ void tc2_tile_body(int mp, int r0, int c0, float* __r
             tc::mbar_arrive_expect_tx(&bar_full[s], Cfg::STAGE);
             tc::bulk_g2s(sa, a + (size_t)kc * Cfg::A_CHUNK, Cfg::A_CHUNK, &bar_full[s]);
             tc::bulk_g2s(sa + Cfg::A_CHUNK, a + (size_t)(kc + Cfg::HALF) * Cfg::A_CHUNK, Cfg::A_CHUNK, &bar_full[s]);
-            tc::bulk_g2s(sa + 2 * Cfg::A_CHUNK, b + (size_t)cl * Cfg::B_CHUNK, Cfg::B_CHUNK, &bar_full[s]);
+            tc::bulk_g2s(sa + 2 * Cfg::A_CHUNK, b + (size_t)Cfg::b_chunk(cl) * Cfg::B_CHUNK, Cfg::B_CHUNK, &bar_full[s]);
         };
-        for (int c = 0; c < NS - 1 && c < nsteps; ++c) load_chunk(c);
-        bool ok = true;
-        for (int c = 0; c < nsteps && ok; ++c) {
-            const int s = c % NS;
-            if (!tc::mbar_wait(&bar_full[s], (c / NS) & 1)) {
-                ok = false;
-                break;
-            }
-            const uint32_t a0 = tc::smem_u32(sStage + s * Cfg::STAGE);
-            cplx_mma_step<KIND>(tbase, a0, a0 + Cfg::A_CHUNK, a0 + 2 * Cfg::A_CHUNK, c == 0);
-            tc::mma_commit(&bar_empty[s]);
-            // refill the stage freed by step c-1 with step c + STAGES - 1
-            const int nxt = c + NS - 1;
-            if (nxt < nsteps) {
-                if (c >= 1) {
-                    const int sp = (c - 1) % NS;
-                    if (!tc::mbar_wait(&bar_empty[sp], ((c - 1) / NS) & 1)) {
-                        ok = false;
-                        break;
-                    }
-                }
-                load_chunk(nxt);
-            }
-        }
+        const bool ok = tc2_main_loop<KIND, NS>(nsteps, bar_full, bar_empty, load_chunk, [&](int c, int s, int sp) {
+            tc2_mma_step<KIND>(tbase, tc::smem_u32(sStage + s * Cfg::STAGE), tc::smem_u32(sStage + sp * Cfg::STAGE), 0,
+                               2 * Cfg::A_CHUNK, c);
+        });
         // bar_mma tracks every MMA this thread issued, also after a failed wait
         tc::mma_commit(&bar_mma);
         if (!ok) {
@@ -666,33 +700,13 @@ __device__ __forceinline__ void tc2_pair_body(int mp, int r0, int c0, bool two, 
                 tc::bulk_g2s(sa + 2 * Cfg::A_CHUNK, a1 + ka, Cfg::A_CHUNK, &bar_full[st]);
                 tc::bulk_g2s(sa + 3 * Cfg::A_CHUNK, a1 + kai, Cfg::A_CHUNK, &bar_full[st]);
             }
-            tc::bulk_g2s(sa + 4 * Cfg::A_CHUNK, b + (size_t)cl * Cfg::B_CHUNK, Cfg::B_CHUNK, &bar_full[st]);
+            tc::bulk_g2s(sa + 4 * Cfg::A_CHUNK, b + (size_t)Cfg::b_chunk(cl) * Cfg::B_CHUNK, Cfg::B_CHUNK, &bar_full[st]);
         };
-        for (int c = 0; c < NS - 1 && c < nsteps; ++c) load_chunk(c);
-        bool ok = true;
-        for (int c = 0; c < nsteps && ok; ++c) {
-            const int st = c % NS;
-            if (!tc::mbar_wait(&bar_full[st], (c / NS) & 1)) {
-                ok = false;
-                break;
-            }
-            const uint32_t a0 = tc::smem_u32(smem + st * Pc::STAGE);
-            const uint32_t b0 = a0 + 4 * Cfg::A_CHUNK;
-            cplx_mma_step<KIND>(tbase, a0, a0 + Cfg::A_CHUNK, b0, c == 0);
-            if (two) cplx_mma_step<KIND>(tbase + 2u * T2_BN, a0 + 2 * Cfg::A_CHUNK, a0 + 3 * Cfg::A_CHUNK, b0, c == 0);
-            tc::mma_commit(&bar_empty[st]);
-            const int nxt = c + NS - 1;
-            if (nxt < nsteps) {
-                if (c >= 1) {
-                    const int sp = (c - 1) % NS;
-                    if (!tc::mbar_wait(&bar_empty[sp], ((c - 1) / NS) & 1)) {
-                        ok = false;
-                        break;
-                    }
-                }
-                load_chunk(nxt);
-            }
-        }
+        const bool ok = tc2_main_loop<KIND, NS>(nsteps, bar_full, bar_empty, load_chunk, [&](int c, int st, int sp) {
+            const uint32_t cur = tc::smem_u32(smem + st * Pc::STAGE), prev = tc::smem_u32(smem + sp * Pc::STAGE);
+            tc2_mma_step<KIND>(tbase, cur, prev, 0, 4 * Cfg::A_CHUNK, c);
+            if (two) tc2_mma_step<KIND>(tbase + 2u * T2_BN, cur, prev, 2 * Cfg::A_CHUNK, 4 * Cfg::A_CHUNK, c);
+        });
         tc::mma_commit(&bar_mma);  // tracks every MMA issued, also after a failed wait
         if (!ok) {
             ok_flag = 0;

@@ -5,17 +5,17 @@
 // (same packed operands and the same MMAs in the same K order as the row-pair and
 // single-tile kernels of lu_tc2.cuh, so the factors are bit-identical) with 256 threads:
 //   warp 0 (lane 0)  operand producer: the A' (real and imaginary K part) and B' chunks
-//                    of each K step into a ring of S_OPS stages (bulk copies);
+//                    of each K step into a ring of operand stages (bulk copies);
 //   warp 1 (lane 0)  MMA issuer: one of two 256-column TMEM accumulators per tile,
 //                    alternating, so the MMAs of tile q + 1 run during the epilogue of q;
 //   warp 2 (lane 0)  C producer: the C tile in four chunks of 32 columns (Re and Im
 //                    planes, 128 rows each) by 128-byte-swizzled tensor-map loads into a
-//                    ring of S_C chunks;
+//                    ring of chunks;
 //   warps 4..7       epilogue, one TMEM lane quadrant each (thread = tile row): per chunk
 //                    D is read with tcgen05.ld and subtracted from the staged C, and the
 //                    chunk goes back to global memory by a tensor-map store.
 // A C chunk is two 16 KB copies each way instead of 128-row bulk copies, and the ring
-// keeps up to three chunks of C reads in flight beside the operand stream.  Every wait
+// keeps up to two or three chunks of C reads in flight beside the operand stream.  Every wait
 // is bounded: on a timeout the CTA records an error, stops issuing, lets its copies and
 // MMAs land, frees its TMEM and returns; the epilogue warps decide together (a barrier
 // reduction), so none is left at a named barrier.
@@ -27,15 +27,19 @@
 
 namespace fde {
 
-constexpr int S_OPS = 4;            // operand stages (one K step of A' re, A' im and B' each)
-constexpr int S_C = 3;              // C chunks in flight
 constexpr int S_CHUNK = 32 * 1024;  // Re and Im of 128 rows x 32 columns
 constexpr int S_WQ = 8;             // tiles per CTA
 constexpr int S_THREADS = 256;
 
+// OPS operand stages (one K step of A' re, A' im and B' each) and C chunks in flight.  Split
+// TF32 streams eight times as many operands as C and frees its stages in pairs, so it takes
+// the fifth stage (m_p = 4096, 65 blocks, whole LU: 68.6 against 69.4 ms with 4 and 3); the single
+// products stream twice as many, and C bounds them.
 template <int KIND>
 struct Tc2s {
-    static constexpr int SMEM = S_OPS * Tc2<KIND>::STAGE + S_C * S_CHUNK + 1024;  // + alignment slack
+    static constexpr int OPS = KIND == 2 ? 5 : 4;
+    static constexpr int C = KIND == 2 ? 2 : 3;
+    static constexpr int SMEM = OPS * Tc2<KIND>::STAGE + C * S_CHUNK + 1024;  // + alignment slack
     static_assert(Tc2<KIND>::STAGE % 1024 == 0, "stages keep the 1024-byte alignment of the swizzled chunks");
     static_assert(SMEM <= 227 * 1024, "rings must fit one CTA");
 };
@@ -56,6 +60,7 @@ __device__ __forceinline__ void tc2s_body(int mp, int R0, int nt, int f, int fro
                                           const unsigned char* __restrict__ bpack_old, int* __restrict__ err,
                                           const CUtensorMap* cmap) {
     using Cfg = Tc2<KIND>;
+    constexpr int S_OPS = Tc2s<KIND>::OPS, S_C = Tc2s<KIND>::C;
     const int nsteps = (apack_old ? 2 : 1) * Cfg::NIT;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     __shared__ __align__(8) uint64_t ofull[S_OPS], oempty[S_OPS], cfull[S_C], cempty[S_C], acc_full[2],
@@ -138,7 +143,8 @@ __device__ __forceinline__ void tc2s_body(int mp, int R0, int nt, int f, int fro
                     tc::bulk_g2s(dst, a + (size_t)kc * Cfg::A_CHUNK, Cfg::A_CHUNK, &ofull[s]);
                     tc::bulk_g2s(dst + Cfg::A_CHUNK, a + (size_t)(kc + Cfg::HALF) * Cfg::A_CHUNK, Cfg::A_CHUNK,
                                  &ofull[s]);
-                    tc::bulk_g2s(dst + 2 * Cfg::A_CHUNK, b + (size_t)cl * Cfg::B_CHUNK, Cfg::B_CHUNK, &ofull[s]);
+                    tc::bulk_g2s(dst + 2 * Cfg::A_CHUNK, b + (size_t)Cfg::b_chunk(cl) * Cfg::B_CHUNK, Cfg::B_CHUNK,
+                                 &ofull[s]);
                     n_oi = ++u;
                 }
                 if (!ok) break;
@@ -165,9 +171,10 @@ __device__ __forceinline__ void tc2s_body(int mp, int R0, int nt, int f, int fro
                     }
                     n_ot = ++u;
                     tc::fence_after_sync();
-                    const uint32_t a0 = tc::smem_u32(ring + s * Cfg::STAGE);
-                    cplx_mma_step<KIND>(tacc, a0, a0 + Cfg::A_CHUNK, a0 + 2 * Cfg::A_CHUNK, c == 0);
-                    tc::mma_commit(&oempty[s]);
+                    const int sp = (s + S_OPS - 1) % S_OPS;
+                    tc2_mma_step<KIND>(tacc, tc::smem_u32(ring + s * Cfg::STAGE), tc::smem_u32(ring + sp * Cfg::STAGE),
+                                       0, 2 * Cfg::A_CHUNK, c);
+                    tc2_release<KIND>(&oempty[s], &oempty[sp], c);
                 }
                 if (!ok) break;
                 tc::mma_commit(&acc_full[a]);

@@ -139,7 +139,7 @@ __device__ __forceinline__ void tc2w_body(int mp, int R0, int ni, int x0, int nq
                     tc::bulk_g2s(sa, ga + (size_t)kc * Cfg::A_CHUNK, Cfg::A_CHUNK, &full[s]);
                     tc::bulk_g2s(sa + Cfg::A_CHUNK, ga + (size_t)(kc + Cfg::HALF) * Cfg::A_CHUNK, Cfg::A_CHUNK,
                                  &full[s]);
-                    tc::bulk_g2s(sa + 2 * Cfg::A_CHUNK, gb + (size_t)c * Cfg::B_CHUNK, Cfg::B_CHUNK, &full[s]);
+                    tc::bulk_g2s(sa + 2 * Cfg::A_CHUNK, gb + (size_t)Cfg::b_chunk(c) * Cfg::B_CHUNK, Cfg::B_CHUNK, &full[s]);
                     n_issued = ++g;
                 }
             }
@@ -163,9 +163,10 @@ __device__ __forceinline__ void tc2w_body(int mp, int R0, int ni, int x0, int nq
                     }
                     n_taken = ++g;
                     tc::fence_after_sync();
-                    const uint32_t a0 = tc::smem_u32(ring + s * Wc::STAGE);
-                    cplx_mma_step<KIND>(tacc, a0, a0 + Cfg::A_CHUNK, a0 + 2 * Cfg::A_CHUNK, c == 0);
-                    tc::mma_commit(&empty[s]);
+                    const int sp = (s + NS - 1) % NS;
+                    tc2_mma_step<KIND>(tacc, tc::smem_u32(ring + s * Wc::STAGE), tc::smem_u32(ring + sp * Wc::STAGE),
+                                       0, 2 * Cfg::A_CHUNK, c);
+                    tc2_release<KIND>(&empty[s], &empty[sp], c);
                 }
                 if (abort_flag) break;
                 tc::mma_commit(&acc_full[a]);
