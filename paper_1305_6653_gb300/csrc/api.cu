@@ -1,6 +1,7 @@
 // C ABI of libfde (declared in include/fde.h): problem lifecycle, BVM coefficient
 // derivation, and the host driver of the flexible GMRES iteration.  All numerical
 // work of the path runs in the kernels of the other translation units.
+#include <algorithm>
 #include <atomic>
 #include <cmath>
 #include <cstdio>
@@ -295,15 +296,34 @@ static int matvec(Problem& P, const double* z, double* y, bool fp32 = false) {
     return fp32 ? launch_matvec32(P, z, y, P.stream) : launch_matvec64(P, z, y, P.stream);
 }
 
-// ||v||^2 on the device into d_scal[slot]; optionally returned to the host (synchronises).
-static int norm2(Problem& P, const double* v, int slot, double* host_out, double* pinned) {
-    int rc = launch_norm(v, P.n, P.d_scal + slot, P.d_partial, P.d_counter, P.stream);
-    if (rc) return rc;
-    if (host_out) {
-        FDE_CUDA_TRY(cudaMemcpyAsync(pinned, P.d_scal + slot, sizeof(double), cudaMemcpyDeviceToHost, P.stream));
-        FDE_CUDA_TRY(cudaStreamSynchronize(P.stream));
-        *host_out = *pinned;
+// Wait until a kernel on st has written *word (pinned) to a nonzero value.  The kernel writes
+// it right after its result, so the host neither copies nor waits for the stream to drain; a
+// stream that fails, or that drains without the write, ends the wait.
+template <typename T>
+static int wait_host(const volatile T* word, cudaStream_t st) {
+    for (unsigned long long polls = 1;; ++polls) {
+        if (*word != T(0)) break;
+        if (polls % 4096 == 0) {
+            const cudaError_t e = cudaStreamQuery(st);
+            if (e == cudaSuccess) {
+                if (*word != T(0)) break;
+                return set_error(FDE_ERR_CUDA, "a kernel ended without its result");
+            }
+            if (e != cudaErrorNotReady) return cuda_error(e, "iteration");
+        }
     }
+    std::atomic_thread_fence(std::memory_order_acquire);
+    return FDE_OK;
+}
+
+// ||v||^2, or with ax the norm of v = b - ax (stored), into d_scal[slot] and to the host.
+static int norm2(Problem& P, double* v, int slot, double* host_out, double* pinned, const double* ax = nullptr) {
+    pinned[1] = 0.0;
+    std::atomic_thread_fence(std::memory_order_release);
+    int rc = ax ? launch_residual_norm(P.d_b_rhs, ax, v, P.n, P.d_scal + slot, P.d_partial, P.d_counter, pinned, P.stream)
+                : launch_norm(v, P.n, P.d_scal + slot, P.d_partial, P.d_counter, pinned, P.stream);
+    if (rc || (rc = wait_host(pinned + 1, P.stream))) return rc;
+    *host_out = pinned[0];
     return FDE_OK;
 }
 
@@ -326,9 +346,11 @@ static void drop_iter_graphs(Problem& P) {
 static int iteration_launches(Problem& P, int j, int ldh, int reorth, bool fp32) {
     const size_t n = P.n;
     double* zj = P.d_Z + j * n;
-    int rc;
-    if ((rc = apply_precond(P, P.d_V + j * n, zj))) return rc;
-    if ((rc = matvec(P, zj, P.d_V + (j + 1) * n, fp32))) return rc;
+    P.live = P.d_live;
+    int rc = apply_precond(P, P.d_V + j * n, zj);
+    if (!rc) rc = matvec(P, zj, P.d_V + (j + 1) * n, fp32);
+    P.live = nullptr;
+    if (rc) return rc;
     StageTimer kt(P, FDE_STAGE_KRYLOV);
     return launch_gram_schmidt(P, j, ldh, reorth, P.stream);
 }
@@ -585,6 +607,7 @@ int fde_problem_create(const fde_problem_desc* d, void* stream, fde_problem** ou
     TRY(dalloc(&P.d_counter, 4));
     TRY(dalloc(&P.d_info, (size_t)P.nblk));
     TRY(dalloc(&P.d_err, 1));
+    TRY(dalloc(&P.d_live, 1));
     if (P.timevar) {
         TRY(dalloc(&P.d_dplus_t, (size_t)(P.s + 1) * m));
         TRY(dalloc(&P.d_dminus_t, (size_t)(P.s + 1) * m));
@@ -595,6 +618,9 @@ int fde_problem_create(const fde_problem_desc* d, void* stream, fde_problem** ou
         fde_problem_destroy(h);
         return set_error(FDE_ERR_ALLOC, "cudaMallocHost failed");
     }
+    static_assert(8 * sizeof(double) + Problem::STEP_RING * sizeof(Problem::StepOutcome) <= 64 * sizeof(double),
+                  "the outcomes share the pinned buffer");
+    P.h_step = reinterpret_cast<Problem::StepOutcome*>(h->pinned + 8);
     cudaStream_t st = P.stream;
     const cudaMemcpyKind kind = cudaMemcpyDefault;
 #define CUTRY(x)                                  \
@@ -638,7 +664,7 @@ void fde_problem_destroy(fde_problem* h) {
     free_workspace(P);
     void* bufs[] = {P.d_start, P.d_a, P.d_b, P.d_dplus, P.d_dminus, P.d_u0, P.d_f, P.d_g, P.d_twL, P.d_twL32,
                     P.d_twq, P.d_kap, P.d_sym32, P.d_tws, P.d_tws32, P.d_phi, P.d_psi, P.d_b_rhs, P.d_work, P.d_rhat,
-                    P.d_fac, P.d_dinv, P.d_info, P.d_err, P.d_pack, P.d_tinv, P.d_dtile, P.d_strips, P.d_scal, P.d_partial,
+                    P.d_fac, P.d_dinv, P.d_info, P.d_err, P.d_live, P.d_pack, P.d_tinv, P.d_dtile, P.d_strips, P.d_scal, P.d_partial,
                     P.d_counter, P.d_bccb_K64, P.d_bccb_K32, P.d_rhat_b, P.d_dplus_t, P.d_dminus_t,
                     P.d_jz, P.d_xsol};
     for (void* b : bufs) dfree(b);
@@ -1015,28 +1041,28 @@ int pgmres_solve(fde_problem* h, const fde_pgmres_opts* opts, const double* x0_a
     // r = b - M x -> V_0; from x = 0 it is b, whose norm is known
     int beta_slot = 131;
     beta2 = bnorm2;
+    const double* r = P.d_b_rhs;
     if (x0) {
         if ((rc = matvec(P, x, P.d_work))) return finish(rc);
-        if ((rc = launch_sub(P.d_b_rhs, P.d_work, V, n, st))) return finish(rc);
-    } else {
-        cudaError_t e = cudaMemcpyAsync(V, P.d_b_rhs, n * sizeof(double), cudaMemcpyDeviceToDevice, st);
-        if (e != cudaSuccess) return finish(cuda_error(e, "copy of b"));
-    }
-    if (x0) {
-        if ((rc = norm2(P, V, 132, &beta2, pin))) return finish(rc);
+        if ((rc = norm2(P, V, 132, &beta2, pin, P.d_work))) return finish(rc);
         beta_slot = 132;
+        r = V;
         if (!(beta2 <= bnorm2)) {
             // the initial guess is worse than zero (or not finite): start from x = 0
             FDE_CUDA_TRY(cudaMemsetAsync(x, 0, n * sizeof(double), st));
-            FDE_CUDA_TRY(cudaMemcpyAsync(V, P.d_b_rhs, n * sizeof(double), cudaMemcpyDeviceToDevice, st));
             beta_slot = 131;
+            r = P.d_b_rhs;
             beta2 = bnorm2;
             S.x0_rejected = 1;
         }
     }
     int its = 0;
-    std::vector<double> g0(o.restart + 1, 0.0);
     double est = 0.0;
+    bool fp32_step[64] = {};  // restart <= 63
+    // One step is queued ahead of the one whose outcome is awaited, unless its product depends
+    // on that outcome (the relaxed FP32 product) or the profiler reads events after each step.
+    const bool relaxed = o.matvec_precision == FDE_FP32 && !P.timevar;
+    const bool ahead = !P.prof && !P.prof_mask && !(relaxed && o.relax > 0.0);
     for (;;) {
         const double beta = std::sqrt(beta2);
         S.rel_residual = beta / bnorm;
@@ -1046,25 +1072,32 @@ int pgmres_solve(fde_problem* h, const fde_pgmres_opts* opts, const double* x0_a
             status = set_error(FDE_ERR_NOT_CONVERGED, "maxit reached before the tolerance");
             break;
         }
-        if ((rc = launch_scale(V, sc + beta_slot, V, n, st))) return finish(rc);
-        g0[0] = beta;
-        std::fill(g0.begin() + 1, g0.end(), 0.0);
-        FDE_CUDA_TRY(cudaMemcpyAsync(P.d_gv, g0.data(), g0.size() * sizeof(double), cudaMemcpyHostToDevice, st));
-        int j = 0;
+        if ((rc = launch_cycle_start(P, r, sc + beta_slot, o.restart, o.tol * bnorm, st))) return finish(rc);
+        int j = 0, queued = 0;
         double est_rel = beta / bnorm;  // residual estimate before iteration j
+        bool replayed = false;
+        const auto queue = [&]() -> int {
+            const bool fp32 = relaxed && (o.relax <= 0.0 || est_rel > o.relax);
+            P.h_step[queued % Problem::STEP_RING].seq = 0;
+            std::atomic_thread_fence(std::memory_order_release);
+            fp32_step[queued] = fp32;
+            return run_iteration(P, queued++, ldh, o.reorth, o.restart, fp32, &replayed);
+        };
         for (; j < o.restart; ++j) {
-            bool replayed = false;
-            const bool fp32 = o.matvec_precision == FDE_FP32 && !P.timevar && (o.relax <= 0.0 || est_rel > o.relax);
-            if ((rc = run_iteration(P, j, ldh, o.reorth, o.restart, fp32, &replayed))) return finish(rc);
+            if (queued == j && (rc = queue())) return finish(rc);
+            if (ahead && queued == j + 1 && queued < o.restart && its + 1 < o.maxit && (rc = queue())) return finish(rc);
+            const Problem::StepOutcome& h = P.h_step[j % Problem::STEP_RING];
+            if ((rc = wait_host(&h.seq, st))) return finish(rc);
             ++its;
-            if (fp32) ++S.matvecs_fp32;
-            FDE_CUDA_TRY(cudaMemcpyAsync(pin, sc + 128, 3 * sizeof(double), cudaMemcpyDeviceToHost, st));
-            FDE_CUDA_TRY(cudaStreamSynchronize(st));
-            if (replayed && P.prof_mask) harvest_graph_events(P, j + (fp32 ? o.restart : 0));
-            est = pin[1];
+            if (fp32_step[j]) ++S.matvecs_fp32;
+            if (replayed && P.prof_mask) {
+                FDE_CUDA_TRY(cudaStreamSynchronize(st));
+                harvest_graph_events(P, j + (fp32_step[j] ? o.restart : 0));
+            }
+            est = h.est;
             est_rel = est / bnorm;
-            const double hnext = std::fabs(pin[2]);
-            if (!std::isfinite(est) || !std::isfinite(pin[0])) {
+            const double hnext = std::fabs(h.hnext);
+            if (!std::isfinite(est) || !std::isfinite(h.nrm_sq)) {
                 status = set_error(FDE_ERR_NAN, "non-finite Hessenberg entry");
                 break;
             }
@@ -1073,6 +1106,7 @@ int pgmres_solve(fde_problem* h, const fde_pgmres_opts* opts, const double* x0_a
                 break;
             }
         }
+        // (a step queued behind the last one has left everything as it was)
         if (status == FDE_ERR_NAN) break;
         const int k = j < o.restart ? j : o.restart;
         if ((rc = launch_lsq_solve(P.d_H, ldh, k, P.d_gv, P.d_y, st))) return finish(rc);
@@ -1080,9 +1114,9 @@ int pgmres_solve(fde_problem* h, const fde_pgmres_opts* opts, const double* x0_a
         ++S.restarts;
         S.rel_residual_estimate = est / bnorm;
         if ((rc = matvec(P, x, P.d_work))) return finish(rc);
-        if ((rc = launch_sub(P.d_b_rhs, P.d_work, V, n, st))) return finish(rc);
-        if ((rc = norm2(P, V, 132, &beta2, pin))) return finish(rc);
+        if ((rc = norm2(P, V, 132, &beta2, pin, P.d_work))) return finish(rc);
         beta_slot = 132;
+        r = V;
     }
     S.iterations = its;
     ++P.solves;

@@ -161,7 +161,8 @@ bccb_spectrum_kernel(int m, int logL, const double2* __restrict__ cinv, const do
 template <typename T>
 __global__ void __launch_bounds__(512)
 bccb_solve_kernel(int m, int mp, int logL, cplx_t<T>* __restrict__ rhat, const cplx_t<T>* __restrict__ K,
-                  const cplx_t<T>* __restrict__ tw) {
+                  const cplx_t<T>* __restrict__ tw, const int* __restrict__ live) {
+    if (live && !*live) return;
     using C = cplx_t<T>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C* buf = reinterpret_cast<C*>(smem_raw);
@@ -211,13 +212,13 @@ int launch_bccb_solve(const Problem& P, void* rhat, int prec, cudaStream_t st) {
         FDE_CUDA_TRY(cudaFuncSetAttribute(bccb_solve_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                           (int)smem));
         bccb_solve_kernel<double><<<P.nblk, 512, smem, st>>>(P.m, P.mp, P.logL, (double2*)rhat, P.d_bccb_K64,
-                                                              P.d_twL);
+                                                              P.d_twL, P.live);
     } else {
         const size_t smem = (size_t)P.L * sizeof(float2);
         FDE_CUDA_TRY(cudaFuncSetAttribute(bccb_solve_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                           (int)smem));
         bccb_solve_kernel<float><<<P.nblk, 512, smem, st>>>(P.m, P.mp, P.logL, (float2*)rhat, P.d_bccb_K32,
-                                                             P.d_twL32);
+                                                             P.d_twL32, P.live);
     }
     FDE_LAUNCH_CHECK("bccb_solve_kernel");
     return FDE_OK;

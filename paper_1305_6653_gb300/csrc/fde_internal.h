@@ -143,13 +143,20 @@ int launch_block_trsv(const Problem& P, void* rhat, cudaStream_t st);
 
 // krylov.cu
 int launch_update(const double* V, int k, const double* coef, double sign, double* w, long n, cudaStream_t st);
-int launch_norm(const double* w, long n, double* out, double* partial, unsigned int* counter, cudaStream_t st);
+// out[0] = |w|^2; host (pinned, or NULL): {|w|^2, 1} as well
+int launch_norm(const double* w, long n, double* out, double* partial, unsigned int* counter, double* host,
+                cudaStream_t st);
+// r = b - ax and out[0] = |r|^2, as launch_norm
+int launch_residual_norm(const double* b, const double* ax, double* r, long n, double* out, double* partial,
+                         unsigned int* counter, double* host, cudaStream_t st);
+// start of a cycle: V_0 = r / sqrt(*nrm_sq), g = (sqrt(*nrm_sq), 0, ..), the cycle live until the
+// estimate is at most threshold
+int launch_cycle_start(Problem& P, const double* r, const double* nrm_sq, int restart, double threshold,
+                       cudaStream_t st);
 // Arnoldi step j after the product: V_{j+1} against V_0..V_j (CGS2, or one pass without
 // reorth), column j of H with its Givens rotation, scal[128..130], V_{j+1} / |V_{j+1}|
 int launch_gram_schmidt(Problem& P, int j, int ldh, int reorth, cudaStream_t st);
-int launch_scale(const double* src, const double* nrm_sq, double* dst, long n, cudaStream_t st);
 int launch_lsq_solve(const double* H, int ldh, int k, const double* g, double* y, cudaStream_t st);
-int launch_sub(const double* b, const double* ax, double* r, long n, cudaStream_t st);
 
 // ---------------------------------------------------------------------------
 // The problem object.
@@ -256,6 +263,20 @@ struct Problem {
     double* d_scal = nullptr;   // scalars: [0..63] dots h1, [64..127] dots h2, [128] norm^2, [129] est, ...
     double* d_partial = nullptr;
     unsigned int* d_counter = nullptr;
+
+    // The Arnoldi steps of a cycle are queued one ahead of the one whose outcome the host has
+    // seen.  d_live: nonzero until the Gram-Schmidt step ends the cycle (estimate below the
+    // threshold in scal[133], breakdown, non-finite value); it makes a step queued after that
+    // leave everything as it is.  live: d_live while a step is being queued, NULL otherwise --
+    // the costly kernels take it and return at once.  h_step: pinned, a ring of outcomes.
+    int* d_live = nullptr;
+    const int* live = nullptr;
+    struct StepOutcome {
+        double nrm_sq, est, hnext;
+        unsigned long long seq;  // written last: the step's number in the cycle, from 1
+    };
+    static constexpr int STEP_RING = 4;
+    StepOutcome* h_step = nullptr;
 
     bool assembled = false;
     bool factored = false;

@@ -36,9 +36,10 @@ __device__ __forceinline__ double warp_sums(double (&a)[C]) {
 
 // |w|^2 of a vector: CTA sums to partial, the last CTA to finish (atomic ticket after a
 // fence; nothing waits) adds them.
-__device__ __forceinline__ void norm_body(const double* __restrict__ w, long n, double* __restrict__ out,
+__device__ __forceinline__ void to_host(double* host, double v);
+__device__ __forceinline__ void norm_body(const double* w, long n, double* __restrict__ out,
                                           double* __restrict__ partial, unsigned int* __restrict__ counter, int bx,
-                                          int nblocks) {
+                                          int nblocks, double* __restrict__ host = nullptr) {
     __shared__ double red[RED_THREADS / 32];
     __shared__ bool last;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -63,14 +64,30 @@ __device__ __forceinline__ void norm_body(const double* __restrict__ w, long n, 
         if (lane == 0) {
             *out = v;
             *counter = 0u;
+            if (host) to_host(host, v);
         }
     }
 }
 
+// Results the host waits for go to pinned memory, the sequence word last.
+__device__ __forceinline__ void to_host(double* host, double v) {
+    volatile double* h = host;
+    h[0] = v;
+    __threadfence_system();
+    h[1] = 1.0;
+}
+
+// out[0] = |w|^2 (SUB: of w = b - ax, which is stored)
+template <bool SUB>
 __global__ void __launch_bounds__(RED_THREADS)
-norm_kernel(const double* __restrict__ w, long n, double* __restrict__ out, double* __restrict__ partial,
-            unsigned int* __restrict__ counter) {
-    norm_body(w, n, out, partial, counter, blockIdx.x, gridDim.x);
+norm_kernel(const double* __restrict__ b, const double* __restrict__ ax, double* __restrict__ w, long n,
+            double* __restrict__ out, double* __restrict__ partial, unsigned int* __restrict__ counter,
+            double* __restrict__ host) {
+    if (SUB) {
+        const long stride = (long)gridDim.x * blockDim.x;
+        for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) w[i] = b[i] - ax[i];
+    }
+    norm_body(w, n, out, partial, counter, blockIdx.x, gridDim.x, host);  // each thread the elements it stored
 }
 
 // ---------------------------------------------------------------------------
@@ -104,6 +121,8 @@ struct GsArgs {
     double* partial;
     unsigned int* bar;  // a counter per barrier, zero before the launch
     int* err;
+    int* live;                    // Problem::d_live, or NULL (a batch: ctl)
+    Problem::StepOutcome* host;   // where the host waits for the step, or NULL
 };
 
 // The CTAs of one Gram-Schmidt step meet.  CTA 0 clears the next counter before it arrives
@@ -140,13 +159,17 @@ __device__ __forceinline__ void gs_collect(const GsArgs& A, const double (*red)[
     }
     if (G > 1) {
         gs_barrier(A.bar, slot, cta, G, A.err);
-        const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-        for (int i = warp; i < k; i += NW) {
-            double v = 0.0;
-            for (int c = lane; c < G; c += 32) v += __ldcg(part + (size_t)i * GS_CTAS + c);
-            for (int off = 16; off; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-            if (lane == 0) out[i] = v;
+        // tpv threads a vector (as many as there are for k), so that the additions fill their warps
+        int tpv = 32;
+        while (tpv * k > NT) tpv >>= 1;
+        const int i = threadIdx.x / tpv, c0 = threadIdx.x % tpv;
+        double v = 0.0;
+        if (i < k) {
+#pragma unroll 4
+            for (int c = c0; c < G; c += tpv) v += __ldcg(part + (size_t)i * GS_CTAS + c);
         }
+        for (int off = tpv >> 1; off; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+        if (i < k && c0 == 0) out[i] = v;
     }
     __syncthreads();
 }
@@ -200,6 +223,17 @@ __device__ __forceinline__ GsColumn gs_column(const GsArgs& A, const double* h1,
     return out;
 }
 
+// The end of the cycle (the test the host makes too) and the outcome to the host.  One thread.
+__device__ __forceinline__ void gs_outcome(const GsArgs& A, const GsColumn& col) {
+    if (!isfinite(col.est) || !isfinite(col.nrm) || col.est <= A.scal[133] || fabs(col.hnext) <= 1e-300) *A.live = 0;
+    volatile Problem::StepOutcome* h = A.host;
+    h->nrm_sq = col.nrm;
+    h->est = col.est;
+    h->hnext = col.hnext;
+    __threadfence_system();
+    h->seq = (unsigned long long)A.k;
+}
+
 __device__ __forceinline__ void cp_async_elems(double* dst, const double* src, int bytes) {
     const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
     if (bytes == 16) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
@@ -225,6 +259,7 @@ template <int KC, int E, int NT>
 __global__ void __launch_bounds__(NT, 1) gs_one_kernel(const __grid_constant__ GsArgs A) {
     __shared__ double red[NT / 32][KC];
     __shared__ double h1[KC], h2[KC], gc[KC], gsn[KC];
+    if (!*A.live) return;  // cleared by this launch only after every CTA has come to its last barrier
     const int tid = threadIdx.x, k = A.k, cta = blockIdx.x, G = gridDim.x;
     const long n = A.n, x = ((long)cta * NT + tid) * E;
     if (cta == 0 && tid < k - 1) {  // earlier rotations, for the column at the end
@@ -305,7 +340,7 @@ __global__ void __launch_bounds__(NT, 1) gs_one_kernel(const __grid_constant__ G
 #pragma unroll
             for (int e = 0; e < E; ++e) A.w[x + e] = w[e] * inv;
         }
-    }, [](const GsColumn&) {});
+    }, [&](const GsColumn& col) { gs_outcome(A, col); });
 }
 
 // Any number of elements a thread, E neighbours at a time (E = 2: n even).  A thread copies
@@ -453,7 +488,9 @@ __device__ __forceinline__ void gs_body(const GsArgs& A, int cta, int G, double*
 template <int KC, int E>
 __global__ void __launch_bounds__(RED_THREADS, 1) gs_kernel(const __grid_constant__ GsArgs A) {
     extern __shared__ __align__(16) unsigned char gs_smem[];
-    gs_body<KC, E>(A, blockIdx.x, gridDim.x, reinterpret_cast<double*>(gs_smem), [](const GsColumn&) {});
+    if (!*A.live) return;  // as in gs_one_kernel
+    gs_body<KC, E>(A, blockIdx.x, gridDim.x, reinterpret_cast<double*>(gs_smem),
+                   [&](const GsColumn& col) { gs_outcome(A, col); });
 }
 
 // shared memory of the staged V for k vectors
@@ -476,29 +513,46 @@ __global__ void update_kernel(const double* __restrict__ V, int k, const double*
     }
 }
 
-__global__ void scale_kernel(const double* __restrict__ src, const double* __restrict__ nrm_sq,
-                             double* __restrict__ dst, long n) {
+__global__ void cycle_start_kernel(const double* src, const double* __restrict__ nrm_sq, double* dst, long n,
+                                   double* __restrict__ g, int restart, double threshold, double* __restrict__ thr,
+                                   int* __restrict__ live) {
     const double nr = sqrt(*nrm_sq);
     const double inv = nr > 0.0 ? 1.0 / nr : 0.0;
     const long stride = (long)gridDim.x * blockDim.x;
     for (long x = (long)blockIdx.x * blockDim.x + threadIdx.x; x < n; x += stride) dst[x] = src[x] * inv;
-}
-
-__global__ void sub_kernel(const double* __restrict__ b, const double* __restrict__ ax, double* __restrict__ r,
-                           long n) {
-    const long stride = (long)gridDim.x * blockDim.x;
-    for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) r[i] = b[i] - ax[i];
-}
-
-// y = R^{-1} g with R the k x k upper-triangular part of the rotated H.
-__global__ void lsq_solve_kernel(const double* __restrict__ H, int ldh, int k, const double* __restrict__ g,
-                                 double* __restrict__ y) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    for (int i = k - 1; i >= 0; --i) {
-        double v = g[i];
-        for (int c = i + 1; c < k; ++c) v -= H[(size_t)c * ldh + i] * y[c];
-        y[i] = v / H[(size_t)i * ldh + i];
+    if (blockIdx.x == 0) {
+        for (int i = threadIdx.x; i <= restart; i += blockDim.x) g[i] = i == 0 ? nr : 0.0;
+        if (threadIdx.x == 0) {
+            *thr = threshold;
+            *live = 1;
+        }
     }
+}
+
+// y = R^{-1} g with R the k x k upper-triangular part of the rotated H: a warp, columns
+// in registers' reach (R staged in shared memory: every step of the serial chain otherwise waited
+// for a load from global memory, 56 us at k = 27).
+__device__ __forceinline__ void lsq_body(const double* __restrict__ H, int ldh, int k, const double* __restrict__ g,
+                                         double* __restrict__ y, double* R) {
+    const int lane = threadIdx.x & 31;
+    for (int c = 0; c < k; ++c)
+        for (int i = lane; i <= c; i += 32) R[c * KMAX + i] = H[(size_t)c * ldh + i];
+    double v0 = lane < k ? g[lane] : 0.0, v1 = lane + 32 < k ? g[lane + 32] : 0.0;
+    __syncwarp();
+    for (int c = k - 1; c >= 0; --c) {
+        double yc = 0.0;
+        if (lane == (c & 31)) yc = (c < 32 ? v0 : v1) / R[c * KMAX + c];
+        yc = __shfl_sync(0xffffffffu, yc, c & 31);
+        if (lane == (c & 31)) y[c] = yc;
+        if (lane < c) v0 -= R[c * KMAX + lane] * yc;
+        if (lane + 32 < c) v1 -= R[c * KMAX + lane + 32] * yc;
+    }
+}
+
+__global__ void __launch_bounds__(32) lsq_solve_kernel(const double* __restrict__ H, int ldh, int k,
+                                                       const double* __restrict__ g, double* __restrict__ y) {
+    __shared__ double R[KMAX * KMAX];
+    lsq_body(H, ldh, k, g, y, R);
 }
 
 // ---------------------------------------------------------------------------
@@ -599,7 +653,7 @@ gs_batched(const InstDev* __restrict__ I, const int* __restrict__ act, int nact,
     const auto step = [&](int a, int cta, int G) {
         const InstDev& d = I[act[a]];
         GsArgs A{d.V, d.V + (size_t)(j + 1) * d.n, d.n, j + 1, ldh, reorth, d.H, d.cs, d.sn, d.gv, d.scal,
-                 d.partial, d.counter, err};
+                 d.partial, d.counter, err, nullptr, nullptr};
         gs_body<KC, E>(A, cta, G, stage, [&](const GsColumn& col) {
             volatile int* c = d.ctl;
             const int its = c[2] + 1;
@@ -646,19 +700,13 @@ __global__ void ctl_set_batched(const InstDev* __restrict__ I, const int* __rest
     }
 }
 
-__global__ void lsq_batched(const InstDev* __restrict__ I, const int* __restrict__ act, int nact,
-                            const int* __restrict__ kvec, int ldh) {
-    const int a = blockIdx.x * blockDim.x + threadIdx.x;
-    if (a >= nact) return;
-    const int inst = act[a];
+__global__ void __launch_bounds__(32) lsq_batched(const InstDev* __restrict__ I, const int* __restrict__ act,
+                                                  const int* __restrict__ kvec, int ldh) {
+    __shared__ double R[KMAX * KMAX];
+    const int inst = act[blockIdx.x];
     const InstDev& d = I[inst];
     if (!d.ctl[0]) return;
-    const int k = kvec[inst];
-    for (int i = k - 1; i >= 0; --i) {
-        double v = d.gv[i];
-        for (int c = i + 1; c < k; ++c) v -= d.H[(size_t)c * ldh + i] * d.y[c];
-        d.y[i] = v / d.H[(size_t)i * ldh + i];
-    }
+    lsq_body(d.H, ldh, kvec[inst], d.gv, d.y, R);
 }
 
 // out[4*i + q] = scal[128 + q] of instance i (q = 0..3), and out[4*i+3] = scal[132]
@@ -748,7 +796,7 @@ int launch_ctl_set_batched(const InstDev* I, const int* act, int nact, int live,
 
 int launch_lsq_batched(const InstDev* I, const int* act, int nact, const int* kvec, int ldh, cudaStream_t st) {
     if (nact <= 0) return FDE_OK;
-    lsq_batched<<<(nact + 63) / 64, 64, 0, st>>>(I, act, nact, kvec, ldh);
+    lsq_batched<<<nact, 32, 0, st>>>(I, act, kvec, ldh);
     FDE_LAUNCH_CHECK("lsq_batched");
     return FDE_OK;
 }
@@ -800,7 +848,7 @@ int launch_gram_schmidt(Problem& P, int j, int ldh, int reorth, cudaStream_t st)
                                : gs_form<64, 1>(P.n, k, ctas);
     if (f.smem) FDE_CUDA_TRY(cudaFuncSetAttribute(f.kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)f.smem));
     GsArgs A{P.d_V, P.d_V + (size_t)k * P.n, P.n, k, ldh, reorth, P.d_H, P.d_cs, P.d_sn, P.d_gv, P.d_scal,
-             P.d_partial, P.d_counter, P.d_err};
+             P.d_partial, P.d_counter, P.d_err, P.d_live, P.h_step + j % Problem::STEP_RING};
     void* args[] = {&A};
     FDE_CUDA_TRY(cudaLaunchCooperativeKernel(f.kern, dim3(f.grid), dim3(f.threads), args, f.smem, st));
     FDE_LAUNCH_CHECK("gs_kernel");
@@ -814,28 +862,34 @@ int launch_update(const double* V, int k, const double* coef, double sign, doubl
     return FDE_OK;
 }
 
-int launch_norm(const double* w, long n, double* out, double* partial, unsigned int* counter, cudaStream_t st) {
-    const int grid = (int)std::max<long>(1, std::min<long>(RED_CTAS, (n + 1023) / 1024));
-    norm_kernel<<<grid, RED_THREADS, 0, st>>>(w, n, out, partial, counter);
+static int norm_grid(long n) { return (int)std::max<long>(1, std::min<long>(RED_CTAS, (n + 1023) / 1024)); }
+
+int launch_norm(const double* w, long n, double* out, double* partial, unsigned int* counter, double* host,
+                cudaStream_t st) {
+    norm_kernel<false><<<norm_grid(n), RED_THREADS, 0, st>>>(nullptr, nullptr, const_cast<double*>(w), n, out, partial,
+                                                             counter, host);
     FDE_LAUNCH_CHECK("norm_kernel");
     return FDE_OK;
 }
 
-int launch_scale(const double* src, const double* nrm_sq, double* dst, long n, cudaStream_t st) {
-    scale_kernel<<<grid_for(n), 256, 0, st>>>(src, nrm_sq, dst, n);
-    FDE_LAUNCH_CHECK("scale_kernel");
+int launch_residual_norm(const double* b, const double* ax, double* r, long n, double* out, double* partial,
+                         unsigned int* counter, double* host, cudaStream_t st) {
+    norm_kernel<true><<<norm_grid(n), RED_THREADS, 0, st>>>(b, ax, r, n, out, partial, counter, host);
+    FDE_LAUNCH_CHECK("norm_kernel(residual)");
+    return FDE_OK;
+}
+
+int launch_cycle_start(Problem& P, const double* r, const double* nrm_sq, int restart, double threshold,
+                       cudaStream_t st) {
+    cycle_start_kernel<<<grid_for(P.n), 256, 0, st>>>(r, nrm_sq, P.d_V, P.n, P.d_gv, restart, threshold,
+                                                      P.d_scal + 133, P.d_live);
+    FDE_LAUNCH_CHECK("cycle_start_kernel");
     return FDE_OK;
 }
 
 int launch_lsq_solve(const double* H, int ldh, int k, const double* g, double* y, cudaStream_t st) {
     lsq_solve_kernel<<<1, 32, 0, st>>>(H, ldh, k, g, y);
     FDE_LAUNCH_CHECK("lsq_solve_kernel");
-    return FDE_OK;
-}
-
-int launch_sub(const double* b, const double* ax, double* r, long n, cudaStream_t st) {
-    sub_kernel<<<grid_for(n), 256, 0, st>>>(b, ax, r, n);
-    FDE_LAUNCH_CHECK("sub_kernel");
     return FDE_OK;
 }
 

@@ -1000,7 +1000,8 @@ template <typename T>
 __global__ void __launch_bounds__(512)
 block_trsv_ring_kernel(int mp, const T* __restrict__ fac, const cplx_t<T>* __restrict__ dinv,
                        const T* __restrict__ tinv, cplx_t<T>* __restrict__ rhat, int* __restrict__ err,
-                       const __grid_constant__ CUtensorMap fmap) {
+                       const __grid_constant__ CUtensorMap fmap, const int* __restrict__ live) {
+    if (live && !*live) return;
     using C = cplx_t<T>;
     using Cf = ring_cfg<T>;
     extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -1083,7 +1084,9 @@ __device__ __forceinline__ void trsv_body(int mp, const typename fac_store<T, LA
 template <typename T, int V = 0, int LAY = LAY_PLANES>
 __global__ void __launch_bounds__(trsv_shape<T, V>::NT)
 block_trsv_kernel(int mp, const typename fac_store<T, LAY>::elem* __restrict__ fac,
-                  const cplx_t<T>* __restrict__ dinv, const T* __restrict__ tinv, cplx_t<T>* __restrict__ rhat) {
+                  const cplx_t<T>* __restrict__ dinv, const T* __restrict__ tinv, cplx_t<T>* __restrict__ rhat,
+                  const int* __restrict__ live) {
+    if (live && !*live) return;
     const int k = blockIdx.x;
     constexpr int HS = trsv_shape<T, V>::H;
     constexpr int H = LAY != LAY_STRIPS_BF16 ? HS : HS > 7 ? 7 : HS == 2 ? 3 : HS;
@@ -2643,7 +2646,7 @@ static int launch_trsv_shape(const Problem& P, void* rhat, cudaStream_t st) {
             FDE_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
             kern<<<P.nblk, trsv_shape<T, V>::NT, smem, st>>>(P.mp, (const unsigned short*)P.d_strips,
                                                               (const cplx_t<T>*)P.d_dinv, (const T*)P.d_tinv,
-                                                              (cplx_t<T>*)rhat);
+                                                              (cplx_t<T>*)rhat, P.live);
             FDE_LAUNCH_CHECK("block_trsv_kernel");
             return FDE_OK;
         }
@@ -2654,7 +2657,7 @@ static int launch_trsv_shape(const Problem& P, void* rhat, cudaStream_t st) {
         FDE_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
         kern<<<P.nblk, trsv_shape<T, V>::NT, smem, st>>>(P.mp, (const T*)(strips ? P.d_strips : P.d_fac),
                                                           (const cplx_t<T>*)P.d_dinv, (const T*)P.d_tinv,
-                                                          (cplx_t<T>*)rhat);
+                                                          (cplx_t<T>*)rhat, P.live);
     }
     FDE_LAUNCH_CHECK("block_trsv_kernel");
     return FDE_OK;
@@ -2699,7 +2702,7 @@ static int launch_trsv_ring(const Problem& P, void* rhat, cudaStream_t st) {
     auto kern = block_trsv_ring_kernel<T>;
     FDE_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     kern<<<P.nblk, ring_cfg<T>::NT, smem, st>>>(P.mp, (const T*)P.d_fac, (const cplx_t<T>*)P.d_dinv,
-                                                 (const T*)P.d_tinv, (cplx_t<T>*)rhat, P.d_err, map);
+                                                 (const T*)P.d_tinv, (cplx_t<T>*)rhat, P.d_err, map, P.live);
     FDE_LAUNCH_CHECK("block_trsv_ring_kernel");
     return FDE_OK;
 }

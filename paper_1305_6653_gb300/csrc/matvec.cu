@@ -116,7 +116,8 @@ __global__ void __launch_bounds__(1024)
 st_matvec32_kernel(int m, int logL, int mu, double h, const int* __restrict__ start, const double* __restrict__ A,
                    const double* __restrict__ B, const double* __restrict__ dplus, const double* __restrict__ dminus,
                    const float2* __restrict__ sym, const float2* __restrict__ tw, const double* __restrict__ z,
-                   double* __restrict__ y) {
+                   double* __restrict__ y, const int* __restrict__ live) {
+    if (live && !*live) return;
     matvec_body<float, 0>(m, logL, mu, h, start, A, B, dplus, dminus, sym, tw, z, y, blockIdx.x);
 }
 
@@ -314,7 +315,8 @@ __global__ void __launch_bounds__(NT, 512 / NT)
 st_matvec_kernel(int m, int logL, int mu, double h, const int* __restrict__ start, const double* __restrict__ A,
                  const double* __restrict__ B, const double* __restrict__ dplus, const double* __restrict__ dminus,
                  const bfp::Tw* __restrict__ tw, const bfp::Q61* __restrict__ kap, double fac,
-                 const double* __restrict__ z, double* __restrict__ y, int dstride) {
+                 const double* __restrict__ z, double* __restrict__ y, int dstride, const int* __restrict__ live) {
+    if (live && !*live) return;
     bfp_row<MODE>(m, logL, mu, h, start, A, B, dplus, dminus, tw, kap, fac, z, y, blockIdx.x, dstride);
 }
 
@@ -375,7 +377,7 @@ static int launch_st(const Problem& P, const double* z, double* y, int ncols, cu
     FDE_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024));
     kern<<<ncols, row_threads(P.L, NT), smem, st>>>(P.m, P.logL, P.mu, P.h, P.d_start, P.d_a, P.d_b,
                                                     dplus ? dplus : P.d_dplus, dminus ? dminus : P.d_dminus, P.d_twq,
-                                                    P.d_kap, toeplitz_scale(P), z, y, dstride);
+                                                    P.d_kap, toeplitz_scale(P), z, y, dstride, P.live);
     FDE_LAUNCH_CHECK("st_matvec_kernel");
     return FDE_OK;
 }
@@ -386,7 +388,7 @@ int launch_matvec32(const Problem& P, const double* z, double* y, cudaStream_t s
     const int threads = P.L / 2 > 1024 ? 1024 : P.L / 2 < 64 ? 64 : P.L / 2;
     FDE_CUDA_TRY(cudaFuncSetAttribute(st_matvec32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
     st_matvec32_kernel<<<P.s, threads, smem, st>>>(P.m, P.logL, P.mu, P.h, P.d_start, P.d_a, P.d_b, P.d_dplus,
-                                                   P.d_dminus, P.d_sym32, P.d_twL32, z, y);
+                                                   P.d_dminus, P.d_sym32, P.d_twL32, z, y, P.live);
     FDE_LAUNCH_CHECK("st_matvec32_kernel");
     return FDE_OK;
 }

@@ -47,3 +47,22 @@ def test_batch_with_more_instances_than_sms():
         ref = O.direct_solve(pr)
         assert st["status"] == 0
         assert np.linalg.norm(x.numpy() - ref) <= 1e-8 * np.linalg.norm(ref), pr.name
+
+
+@pytest.mark.parametrize("m,s,restart,maxit", [(63, 32, 20, 200), (63, 32, 3, 200), (255, 64, 5, 7), (40, 16, 1, 4)])
+def test_step_queued_ahead_changes_nothing(m, s, restart, maxit):
+    """The step queued behind the last one of a cycle must leave everything as it is: solutions
+    and statistics with the profiler on (a step at a time, direct launches), without it (one step
+    ahead) and from captured graphs are the same to the bit."""
+    from paper_1305_6653_gb300 import FDEProblem
+    prob = fi.manufactured(m, s, 1.5, "GBDF3")
+    with FDEProblem.from_inputs(prob, device_inputs=True) as p:
+        p.assemble().factor("fp64")
+        out = []
+        for prof in (True, False, False):
+            p.profile(prof)
+            out.append(p.solve(tol=1e-10, restart=restart, maxit=maxit, raise_on_error=False))
+    for x, st in out[1:]:
+        assert torch.equal(x, out[0][0])
+        for key in ("status", "iterations", "restarts", "rel_residual", "rel_residual_estimate"):
+            assert st[key] == out[0][1][key], key
