@@ -6,6 +6,8 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <memory>
+#include <mutex>
 #include <new>
 #include <string>
 #include <vector>
@@ -188,6 +190,25 @@ static bool formula(int family, int mu, int ell, double* a, double* b) {
         b[i] = to_d(bv[i]);
     }
     return true;
+}
+
+// The formulae of a family for every position of the approximated point, derived once per
+// process (the exact elimination takes 5 to 10 us a position, and a problem needs s of them).
+struct FormulaTable {
+    bool ok[FDE_MAX_MU + 1];
+    double a[FDE_MAX_MU + 1][FDE_MAX_MU + 1], b[FDE_MAX_MU + 1][FDE_MAX_MU + 1];
+};
+static const FormulaTable& formulas(int family, int mu) {
+    static std::mutex mu_;
+    static std::unique_ptr<FormulaTable> table[4][FDE_MAX_MU + 1];
+    std::lock_guard<std::mutex> lock(mu_);
+    std::unique_ptr<FormulaTable>& t = table[family][mu];
+    if (!t) {
+        t.reset(new FormulaTable());
+        for (int ell = 0; ell <= mu; ++ell)  // GAM / ETR formulae need a point before ell
+            t->ok[ell] = (family == FDE_GBDF || ell > 0) && formula(family, mu, ell, t->a[ell], t->b[ell]);
+    }
+    return *t;
 }
 
 // ---------------------------------------------------------------------------
@@ -425,7 +446,6 @@ using namespace fde;
 
 struct fde_problem {
     Problem P;
-    double* pinned = nullptr;  // small pinned host buffer for device -> host scalars
 };
 
 namespace fde {
@@ -478,103 +498,13 @@ int fde_problem_create(const fde_problem_desc* d, void* stream, fde_problem** ou
     P.stream = (cudaStream_t)stream;
     P.device_ptrs = d->device_ptrs != 0;
 
-    // BVM band rows t = 1..s (eqs. (1.7)-(1.9)); row 0 is the initial condition.
-    std::vector<double> ha((size_t)(P.s + 1) * (P.mu + 1), 0.0), hb((size_t)(P.s + 1) * (P.mu + 1), 0.0);
-    std::vector<int> hst(P.s + 1, 0);
-    ha[0] = 1.0;
-    for (int t = 1; t <= P.s; ++t) {
-        int st;
-        if (t < nu) st = 0;
-        else if (t <= P.s - P.mu + nu) st = t - nu;
-        else st = P.s - P.mu;
-        hst[t] = st;
-        if (!formula(P.family, P.mu, t - st, &ha[(size_t)t * (P.mu + 1)], &hb[(size_t)t * (P.mu + 1)])) {
-            delete h;
-            return set_error(FDE_ERR_ARG, "BVM order conditions are singular");
-        }
-    }
-    if (!formula(P.family, P.mu, nu, P.h_a_main, P.h_b_main)) {
-        delete h;
-        return set_error(FDE_ERR_ARG, "BVM order conditions are singular");
-    }
-    for (int t = 0; t <= P.s; ++t) P.h_start[t] = hst[t];
-
-    // validate coefficient arrays on the host when they are host pointers
-    const size_t m = P.m;
-    std::vector<double> dp(m), dm(m);
-    auto fetch = [&](const double* src, double cval, std::vector<double>& dst) -> int {
-        if (!src) {
-            for (size_t i = 0; i < m; ++i) dst[i] = cval;
-            return FDE_OK;
-        }
-        if (d->device_ptrs) {
-            cudaError_t e = cudaMemcpy(dst.data(), src, m * sizeof(double), cudaMemcpyDefault);
-            if (e != cudaSuccess) return cuda_error(e, "copy of d+/d-");
-        } else {
-            std::memcpy(dst.data(), src, m * sizeof(double));
-        }
-        return FDE_OK;
-    };
-    int rc;
     if ((d->dplus_t == nullptr) != (d->dminus_t == nullptr)) {
         delete h;
         return set_error(FDE_ERR_ARG, "give both dplus_t and dminus_t or neither");
     }
     P.timevar = d->dplus_t != nullptr;
-    std::vector<double> dpt, dmt;  // time-dependent coefficients, (s+1) x m
-    if (P.timevar) {
-        const size_t cnt = (size_t)(P.s + 1) * m;
-        dpt.resize(cnt);
-        dmt.resize(cnt);
-        for (int w = 0; w < 2; ++w) {
-            const double* src = w == 0 ? d->dplus_t : d->dminus_t;
-            double* dst = w == 0 ? dpt.data() : dmt.data();
-            if (d->device_ptrs) {
-                cudaError_t e = cudaMemcpy(dst, src, cnt * sizeof(double), cudaMemcpyDefault);
-                if (e != cudaSuccess) {
-                    delete h;
-                    return cuda_error(e, "copy of dplus_t/dminus_t");
-                }
-            } else {
-                std::memcpy(dst, src, cnt * sizeof(double));
-            }
-        }
-        for (size_t k = 0; k < cnt; ++k) {
-            if (!(dpt[k] >= 0.0) || !(dmt[k] >= 0.0) || !(dpt[k] + dmt[k] > 0.0) || !std::isfinite(dpt[k]) ||
-                !std::isfinite(dmt[k])) {
-                delete h;
-                return set_error(FDE_ERR_ARG,
-                                 "need d+ >= 0, d- >= 0, d+ + d- != 0 and finite at every point and time level");
-            }
-        }
-        // the preconditioners use the means over the unknown time levels n = 1..s
-        for (size_t i = 0; i < m; ++i) {
-            double sp = 0.0, sm = 0.0;
-            for (int n = 1; n <= P.s; ++n) {
-                sp += dpt[(size_t)n * m + i];
-                sm += dmt[(size_t)n * m + i];
-            }
-            dp[i] = sp / P.s;
-            dm[i] = sm / P.s;
-        }
-    } else if ((rc = fetch(d->dplus, d->dplus_c, dp)) || (rc = fetch(d->dminus, d->dminus_c, dm))) {
-        delete h;
-        return rc;
-    }
-    for (size_t i = 0; i < m; ++i) {
-        if (!(dp[i] >= 0.0) || !(dm[i] >= 0.0) || !(dp[i] + dm[i] > 0.0) || !std::isfinite(dp[i]) ||
-            !std::isfinite(dm[i])) {
-            delete h;
-            return set_error(FDE_ERR_ARG, "need d+ >= 0, d- >= 0, d+ + d- != 0 and finite at every point");
-        }
-    }
-    if (!d->device_ptrs) {
-        for (size_t i = 0; i < m; ++i)
-            if (!std::isfinite(d->u0[i])) { delete h; return set_error(FDE_ERR_ARG, "u0 is not finite"); }
-        for (size_t i = 0; i < (size_t)(P.s + 1) * m; ++i)
-            if (!std::isfinite(d->f[i])) { delete h; return set_error(FDE_ERR_ARG, "f is not finite"); }
-    }
-
+    const size_t m = P.m, rows = (size_t)P.s + 1, band = rows * (P.mu + 1), nf = rows * m;
+    int rc;
 #define TRY(x)            \
     do {                  \
         rc = (x);         \
@@ -583,46 +513,6 @@ int fde_problem_create(const fde_problem_desc* d, void* stream, fde_problem** ou
             return rc;    \
         }                 \
     } while (0)
-    TRY(dalloc(&P.d_start, P.s + 1));
-    TRY(dalloc(&P.d_a, ha.size()));
-    TRY(dalloc(&P.d_b, hb.size()));
-    TRY(dalloc(&P.d_dplus, m));
-    TRY(dalloc(&P.d_dminus, m));
-    TRY(dalloc(&P.d_u0, m));
-    TRY(dalloc(&P.d_f, (size_t)(P.s + 1) * m));
-    TRY(dalloc(&P.d_g, m + 2));
-    TRY(dalloc(&P.d_twL, (size_t)P.L + 1));
-    TRY(dalloc(&P.d_twL32, (size_t)P.L + 1));
-    TRY(dalloc(&P.d_twq, (size_t)P.L + P.L / 2));
-    TRY(dalloc(&P.d_kap, (size_t)P.L));
-    TRY(dalloc(&P.d_sym32, (size_t)P.L));
-    TRY(dalloc(&P.d_tws, (size_t)P.s / 2 + 1));
-    TRY(dalloc(&P.d_tws32, (size_t)P.s / 2 + 1));
-    TRY(dalloc(&P.d_phi, (size_t)P.nblk));
-    TRY(dalloc(&P.d_psi, (size_t)P.nblk));
-    TRY(dalloc(&P.d_b_rhs, (size_t)P.n));
-    TRY(dalloc(&P.d_work, (size_t)P.n));
-    TRY(dalloc(&P.d_scal, 256));
-    TRY(dalloc(&P.d_partial, (size_t)304 * 64));
-    TRY(dalloc(&P.d_counter, 4));
-    TRY(dalloc(&P.d_info, (size_t)P.nblk));
-    TRY(dalloc(&P.d_err, 1));
-    TRY(dalloc(&P.d_live, 1));
-    if (P.timevar) {
-        TRY(dalloc(&P.d_dplus_t, (size_t)(P.s + 1) * m));
-        TRY(dalloc(&P.d_dminus_t, (size_t)(P.s + 1) * m));
-        TRY(dalloc(&P.d_jz, (size_t)P.n));
-    }
-    if (cudaMallocHost((void**)&h->pinned, 64 * sizeof(double)) != cudaSuccess) {
-        h->pinned = nullptr;
-        fde_problem_destroy(h);
-        return set_error(FDE_ERR_ALLOC, "cudaMallocHost failed");
-    }
-    static_assert(8 * sizeof(double) + Problem::STEP_RING * sizeof(Problem::StepOutcome) <= 64 * sizeof(double),
-                  "the outcomes share the pinned buffer");
-    P.h_step = reinterpret_cast<Problem::StepOutcome*>(h->pinned + 8);
-    cudaStream_t st = P.stream;
-    const cudaMemcpyKind kind = cudaMemcpyDefault;
 #define CUTRY(x)                                  \
     do {                                          \
         cudaError_t e_ = (x);                     \
@@ -632,21 +522,149 @@ int fde_problem_create(const fde_problem_desc* d, void* stream, fde_problem** ou
             return rc;                            \
         }                                         \
     } while (0)
-    CUTRY(cudaMemcpyAsync(P.d_start, hst.data(), (P.s + 1) * sizeof(int), cudaMemcpyHostToDevice, st));
-    CUTRY(cudaMemcpyAsync(P.d_a, ha.data(), ha.size() * sizeof(double), cudaMemcpyHostToDevice, st));
-    CUTRY(cudaMemcpyAsync(P.d_b, hb.data(), hb.size() * sizeof(double), cudaMemcpyHostToDevice, st));
-    CUTRY(cudaMemcpyAsync(P.d_dplus, dp.data(), m * sizeof(double), cudaMemcpyHostToDevice, st));
-    CUTRY(cudaMemcpyAsync(P.d_dminus, dm.data(), m * sizeof(double), cudaMemcpyHostToDevice, st));
-    CUTRY(cudaMemcpyAsync(P.d_u0, d->u0, m * sizeof(double), kind, st));
-    CUTRY(cudaMemcpyAsync(P.d_f, d->f, (size_t)(P.s + 1) * m * sizeof(double), kind, st));
-    if (P.timevar) {
-        CUTRY(cudaMemcpyAsync(P.d_dplus_t, dpt.data(), dpt.size() * sizeof(double), cudaMemcpyHostToDevice, st));
-        CUTRY(cudaMemcpyAsync(P.d_dminus_t, dmt.data(), dmt.size() * sizeof(double), cudaMemcpyHostToDevice, st));
+    const auto bad = [&](const char* msg) {
+        if (P.h_pin) fde_problem_destroy(h);
+        else delete h;  // nothing on the GPU yet
+        return set_error(FDE_ERR_ARG, msg);
+    };
+    // What host arrays can be refused for is found before any GPU call.
+    const FormulaTable& F = formulas(P.family, P.mu);
+    const auto valid = [](double p, double q) {
+        return p >= 0.0 && q >= 0.0 && p + q > 0.0 && std::isfinite(p) && std::isfinite(q);
+    };
+    static const char* d_msg = "need d+ >= 0, d- >= 0, d+ + d- != 0 and finite at every point";
+    static const char* dt_msg = "need d+ >= 0, d- >= 0, d+ + d- != 0 and finite at every point and time level";
+    const auto at = [](const double* v, double c, size_t i) { return v ? v[i] : c; };
+    if (!d->device_ptrs) {
+        if (P.timevar) {
+            for (size_t k = 0; k < nf; ++k)
+                if (!valid(d->dplus_t[k], d->dminus_t[k])) return bad(dt_msg);
+        } else {
+            for (size_t i = 0; i < m; ++i)
+                if (!valid(at(d->dplus, d->dplus_c, i), at(d->dminus, d->dminus_c, i))) return bad(d_msg);
+        }
+        for (size_t i = 0; i < m; ++i)
+            if (!std::isfinite(d->u0[i])) return bad("u0 is not finite");
+        for (size_t i = 0; i < nf; ++i)
+            if (!std::isfinite(d->f[i])) return bad("f is not finite");
     }
-    CUTRY(cudaMemsetAsync(P.d_counter, 0, 4 * sizeof(unsigned int), st));
-    CUTRY(cudaMemsetAsync(P.d_scal, 0, 256 * sizeof(double), st));
-    // host vectors go out of scope: wait for the copies
+
+    // Pinned block: scalars [0, 8), step outcomes [8, 24), check flag [24], status words
+    // [64, 64 + 264), then the upload: A and B bands, d+, d-, zeroed scalars and counters, and the
+    // band's row starts.
+    constexpr size_t PIN_INFO = 64, PIN_UP = PIN_INFO + 264, NSCAL = 256, NCNT = 2;
+    static_assert(8 * sizeof(double) + Problem::STEP_RING * sizeof(Problem::StepOutcome) <= 24 * sizeof(double) &&
+                      (FDE_MAX_S / 2 + 2) * sizeof(int) <= 264 * sizeof(double) &&
+                      (PIN_UP + 2 * (FDE_MAX_S + 1) * (FDE_MAX_MU + 1) + 2 * FDE_MAX_M + NSCAL + NCNT + 4) * sizeof(double) +
+                              (FDE_MAX_S + 1) * sizeof(int) <= PINNED_BYTES,
+                  "the pinned block's layout");
+    void* pin = nullptr;
+    TRY(pinned_alloc(&pin));
+    P.h_pin = static_cast<double*>(pin);
+    P.h_step = reinterpret_cast<Problem::StepOutcome*>(P.h_pin + 8);
+    P.h_info = reinterpret_cast<int*>(P.h_pin + PIN_INFO);
+    double* up = P.h_pin + PIN_UP;
+    const size_t up_doubles = 2 * band + 2 * m + NSCAL + NCNT;
+    const size_t up_bytes = up_doubles * sizeof(double) + rows * sizeof(int);
+    TRY(dalloc(&P.arena[0], up_bytes));
+    P.d_a = reinterpret_cast<double*>(P.arena[0]);
+    P.d_b = P.d_a + band;
+    P.d_dplus = P.d_b + band;
+    P.d_dminus = P.d_dplus + m;
+    P.d_scal = P.d_dminus + m;
+    P.d_counter = reinterpret_cast<unsigned int*>(P.d_scal + NSCAL);
+    P.d_start = reinterpret_cast<int*>(P.d_scal + NSCAL + NCNT);
+    double *ha = up, *hb = up + band, *hp = hb + band, *hm = hp + m;
+    int* hst = reinterpret_cast<int*>(up + up_doubles);
+    std::memset(ha, 0, 2 * band * sizeof(double));
+    std::memset(hm + m, 0, (NSCAL + NCNT) * sizeof(double));
+    // BVM band rows t = 1..s (eqs. (1.7)-(1.9)); row 0 is the initial condition.
+    ha[0] = 1.0;
+    hst[0] = 0;
+    for (int t = 1; t <= P.s; ++t) {
+        const int first = t < nu ? 0 : t <= P.s - P.mu + nu ? t - nu : P.s - P.mu;
+        const int ell = t - first;
+        hst[t] = first;
+        if (!F.ok[ell]) return bad("BVM order conditions are singular");
+        std::memcpy(ha + (size_t)t * (P.mu + 1), F.a[ell], (P.mu + 1) * sizeof(double));
+        std::memcpy(hb + (size_t)t * (P.mu + 1), F.b[ell], (P.mu + 1) * sizeof(double));
+    }
+    if (!F.ok[nu]) return bad("BVM order conditions are singular");
+    std::memcpy(P.h_a_main, F.a[nu], (P.mu + 1) * sizeof(double));
+    std::memcpy(P.h_b_main, F.b[nu], (P.mu + 1) * sizeof(double));
+    for (int t = 0; t <= P.s; ++t) P.h_start[t] = hst[t];
+
+    // the tables and vectors of the problem, one allocation
+    size_t used = 0;
+    const auto part = [&](auto** p, size_t count) {
+        using T = std::remove_pointer_t<std::remove_pointer_t<decltype(p)>>;
+        *p = reinterpret_cast<T*>(P.arena[1] ? P.arena[1] + used : nullptr);
+        used = (used + count * sizeof(T) + 255) & ~size_t(255);
+    };
+    const auto layout = [&]() {
+        used = 0;
+        part(&P.d_u0, m);
+        part(&P.d_f, nf);
+        part(&P.d_g, m + 2);
+        part(&P.d_twL, (size_t)P.L);
+        part(&P.d_twL32, (size_t)P.L);
+        part(&P.d_twq, (size_t)P.L + P.L / 2);
+        part(&P.d_kap, (size_t)P.L);
+        part(&P.d_sym32, (size_t)P.L);
+        part(&P.d_tws, (size_t)P.s / 2);
+        part(&P.d_tws32, (size_t)P.s / 2);
+        part(&P.d_phi, (size_t)P.nblk);
+        part(&P.d_psi, (size_t)P.nblk);
+        part(&P.d_b_rhs, (size_t)P.n);
+        part(&P.d_work, (size_t)P.n);
+        part(&P.d_partial, (size_t)304 * 64);
+        part(&P.d_info, (size_t)P.nblk + 1);
+        P.d_err = P.d_info ? P.d_info + P.nblk : nullptr;
+        part(&P.d_live, 1);
+        if (P.timevar) {
+            part(&P.d_dplus_t, nf);
+            part(&P.d_dminus_t, nf);
+            part(&P.d_jz, (size_t)P.n);
+        }
+    };
+    layout();
+    TRY(dalloc(&P.arena[1], used));
+    layout();
+    cudaStream_t st = P.stream;
+    const cudaMemcpyKind kind = cudaMemcpyDefault;
+    CUTRY(cudaMemcpyAsync(P.d_u0, d->u0, m * sizeof(double), kind, st));
+    CUTRY(cudaMemcpyAsync(P.d_f, d->f, nf * sizeof(double), kind, st));
+    // Everything is on the device, and the caller's arrays are done with, when the call
+    // returns (other streams may then read them): one wait at the end, after the checks'
+    // copies.
+    int* flag = reinterpret_cast<int*>(P.h_pin + 24);
+    *flag = 0;
+    const double* src[2] = {P.timevar ? nullptr : d->dplus, P.timevar ? nullptr : d->dminus};
+    const double c[2] = {d->dplus_c, d->dminus_c};
+    double *host[2] = {hp, hm}, *dev[2] = {P.d_dplus, P.d_dminus};
+    for (int w = 0; w < 2; ++w)
+        for (size_t i = 0; i < m; ++i) host[w][i] = d->device_ptrs ? c[w] : at(src[w], c[w], i);
+    CUTRY(cudaMemcpyAsync(P.arena[0], up, up_bytes, cudaMemcpyHostToDevice, st));
+    for (int w = 0; w < 2; ++w) {
+        if (!src[w] || !d->device_ptrs) continue;
+        CUTRY(cudaMemcpyAsync(dev[w], src[w], m * sizeof(double), kind, st));
+        CUTRY(cudaMemcpyAsync(host[w], src[w], m * sizeof(double), kind, st));  // over the uploaded constants
+    }
+    if (P.timevar) {  // d+, d-: the means over the unknown time levels
+        CUTRY(cudaMemcpyAsync(P.d_dplus_t, d->dplus_t, nf * sizeof(double), kind, st));
+        CUTRY(cudaMemcpyAsync(P.d_dminus_t, d->dminus_t, nf * sizeof(double), kind, st));
+        TRY(launch_timevar_check(P, flag, st));
+    }
     CUTRY(cudaStreamSynchronize(st));
+    if (P.timevar) {
+        if (*flag) return bad(dt_msg);
+    } else {
+        if (d->device_ptrs)
+            for (size_t i = 0; i < m; ++i)
+                if (!valid(hp[i], hm[i])) return bad(d_msg);
+        P.h_dplus = hp;
+        P.h_dminus = hm;
+    }
 #undef CUTRY
 #undef TRY
     *out = h;
@@ -658,23 +676,15 @@ void fde_problem_destroy(fde_problem* h) {
     Problem& P = h->P;
     if (P.stream) cudaStreamSynchronize(P.stream);
     else cudaDeviceSynchronize();
-    if (P.lu_hi) cudaStreamSynchronize(P.lu_hi);
-    if (P.lu_lo) cudaStreamSynchronize(P.lu_lo);
-    if (P.lu_x) cudaStreamSynchronize(P.lu_x);
+    for (cudaStream_t side : {P.lu.hi, P.lu.lo, P.lu.x})
+        if (side) cudaStreamSynchronize(side);
     free_workspace(P);
-    void* bufs[] = {P.d_start, P.d_a, P.d_b, P.d_dplus, P.d_dminus, P.d_u0, P.d_f, P.d_g, P.d_twL, P.d_twL32,
-                    P.d_twq, P.d_kap, P.d_sym32, P.d_tws, P.d_tws32, P.d_phi, P.d_psi, P.d_b_rhs, P.d_work, P.d_rhat,
-                    P.d_fac, P.d_dinv, P.d_info, P.d_err, P.d_live, P.d_pack, P.d_tinv, P.d_dtile, P.d_strips, P.d_scal, P.d_partial,
-                    P.d_counter, P.d_bccb_K64, P.d_bccb_K32, P.d_rhat_b, P.d_dplus_t, P.d_dminus_t,
-                    P.d_jz, P.d_xsol};
+    void* bufs[] = {P.arena[0], P.arena[1], P.d_rhat, P.d_fac, P.d_dinv, P.d_pack, P.d_tinv, P.d_dtile, P.d_strips,
+                    P.d_bccb_K64, P.d_bccb_K32, P.d_rhat_b, P.d_xsol};
     for (void* b : bufs) dfree(b);
-    if (h->pinned) cudaFreeHost(h->pinned);
+    pinned_free(P.h_pin);
     for (cudaEvent_t e : P.ev_pool) cudaEventDestroy(e);
-    for (cudaEvent_t e : P.lu_ev)
-        if (e) cudaEventDestroy(e);
-    if (P.lu_hi) cudaStreamDestroy(P.lu_hi);
-    if (P.lu_lo) cudaStreamDestroy(P.lu_lo);
-    if (P.lu_x) cudaStreamDestroy(P.lu_x);
+    lu_streams_return(&P.lu);
     drop_iter_graphs(P);
     if (P.cap_stream) cudaStreamDestroy(P.cap_stream);
     delete h;
@@ -742,31 +752,9 @@ int bvm_assemble(fde_problem* h) {
     if (!h) return set_error(FDE_ERR_ARG, "NULL problem");
     Problem& P = h->P;
     int rc;
-    double* d_main = nullptr;
     StageTimer timer(P, FDE_STAGE_ASSEMBLE);
-    if ((rc = launch_grunwald(P.alpha, P.m + 2, P.d_g, P.stream))) return rc;
-    if ((rc = launch_twiddles(P.L, P.L, P.d_twL, P.d_twL32, P.stream))) return rc;      // L + 1 allocated
-    if ((rc = launch_twiddles(P.s, P.s / 2, P.d_tws, P.d_tws32, P.stream))) return rc;  // s/2 + 1 allocated
-    if ((rc = launch_bfp_twiddles(P.L, P.d_twq, P.stream))) return rc;
+    if ((rc = launch_tables(P, P.stream))) return rc;
     if ((rc = launch_toeplitz_symbol(P.d_g, P.m, P.L, P.dxa, P.d_twq, P.d_kap, P.d_sym32, P.stream))) return rc;
-    // main-formula coefficients for the Strang symbols
-    if ((rc = dalloc(&d_main, 2 * (FDE_MAX_MU + 1)))) return rc;
-    double hm[2 * (FDE_MAX_MU + 1)];
-    for (int i = 0; i <= P.mu; ++i) {
-        hm[i] = P.h_a_main[i];
-        hm[FDE_MAX_MU + 1 + i] = P.h_b_main[i];
-    }
-    cudaError_t e = cudaMemcpyAsync(d_main, hm, sizeof(hm), cudaMemcpyHostToDevice, P.stream);
-    if (e == cudaSuccess)
-        rc = launch_strang_symbols(d_main, d_main + FDE_MAX_MU + 1, P.mu, P.nu, P.s, P.d_phi, P.d_psi, P.stream);
-    else
-        rc = cuda_error(e, "copy of BVM coefficients");
-    if (!rc) {
-        e = cudaStreamSynchronize(P.stream);  // hm is a stack buffer; d_main is freed below
-        if (e != cudaSuccess) rc = cuda_error(e, "bvm_assemble");
-    }
-    cudaFree(d_main);
-    if (rc) return rc;
     // J u0 (one Toeplitz-like apply), then b
     // J u_0 (with time-dependent coefficients: J_0, the coefficients of time level 0)
     if (P.timevar)
@@ -802,19 +790,16 @@ int strang_precond_factor(fde_problem* h, int precision) {
     if (rc) return rc;
     P.factored = false;
     P.precision = precision;
-    FDE_CUDA_TRY(cudaMemsetAsync(P.d_info, 0, P.nblk * sizeof(int), P.stream));
-    FDE_CUDA_TRY(cudaMemsetAsync(P.d_err, 0, sizeof(int), P.stream));
+    const size_t words = (size_t)P.nblk + 1;  // pivots, then the bounded waits' error
+    FDE_CUDA_TRY(cudaMemsetAsync(P.d_info, 0, words * sizeof(int), P.stream));
     if ((rc = launch_block_lu(P, precision, P.stream))) return rc;
-    std::vector<int> info(P.nblk);
-    int derr = 0;
-    FDE_CUDA_TRY(cudaMemcpyAsync(info.data(), P.d_info, P.nblk * sizeof(int), cudaMemcpyDeviceToHost, P.stream));
-    FDE_CUDA_TRY(cudaMemcpyAsync(&derr, P.d_err, sizeof(int), cudaMemcpyDeviceToHost, P.stream));
+    FDE_CUDA_TRY(cudaMemcpyAsync(P.h_info, P.d_info, words * sizeof(int), cudaMemcpyDeviceToHost, P.stream));
     FDE_CUDA_TRY(cudaStreamSynchronize(P.stream));
-    if (derr) return set_error(FDE_ERR_TIMEOUT, "a bounded wait in the tensor-core LU update ran out");
+    if (P.h_info[P.nblk]) return set_error(FDE_ERR_TIMEOUT, "a bounded wait in the tensor-core LU update ran out");
     for (int k = 0; k < P.nblk; ++k)
-        if (info[k]) {
+        if (P.h_info[k]) {
             char buf[128];
-            std::snprintf(buf, sizeof buf, "zero or non-finite pivot in Strang block %d at row %d", k, info[k] - 1);
+            std::snprintf(buf, sizeof buf, "zero or non-finite pivot in Strang block %d at row %d", k, P.h_info[k] - 1);
             return set_error(FDE_ERR_SINGULAR, buf);
         }
     P.factored = true;
@@ -970,7 +955,7 @@ int pgmres_solve(fde_problem* h, const fde_pgmres_opts* opts, const double* x0_a
     if (rc) return rc;
     cudaStream_t st = P.stream;
     const long n = P.n;
-    double* pin = h->pinned;
+    double* pin = P.h_pin;
     // Host solve vectors (desc->device_ptrs == 0): the iteration runs on the device copy
     // d_xsol; x0 is copied in first and the solution copied out at the end, on the stream.
     const bool host_x = !P.device_ptrs;
@@ -1001,9 +986,9 @@ int pgmres_solve(fde_problem* h, const fde_pgmres_opts* opts, const double* x0_a
     double bnorm2 = 0, beta2 = 0;
 
     auto finish = [&](int code) -> int {
-        int derr = 0;  // a bounded wait of the block solves ran out
-        if (cudaMemcpyAsync(&derr, P.d_err, sizeof(int), cudaMemcpyDeviceToHost, st) == cudaSuccess &&
-            cudaStreamSynchronize(st) == cudaSuccess && derr) {
+        // a bounded wait ran out
+        if (cudaMemcpyAsync(P.h_info, P.d_err, sizeof(int), cudaMemcpyDeviceToHost, st) == cudaSuccess &&
+            cudaStreamSynchronize(st) == cudaSuccess && P.h_info[0]) {
             cudaMemsetAsync(P.d_counter, 0, 4 * sizeof(unsigned int), st);  // the Gram-Schmidt barriers start over
             if (code == FDE_OK) code = set_error(FDE_ERR_TIMEOUT, "a bounded wait of the iteration ran out");
         }

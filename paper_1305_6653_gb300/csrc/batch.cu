@@ -39,6 +39,7 @@ struct fde_batch {
     int* d_kvec = nullptr;
     int* d_err = nullptr;
     double* d_gather = nullptr;
+    void* h_pin = nullptr;       // the pinned block behind the four below, when it came from the cache
     double* h_gather = nullptr;  // pinned
     int* h_act = nullptr;        // pinned
     int* h_kvec = nullptr;       // pinned
@@ -74,7 +75,7 @@ int gather(fde_batch* b) {
     const int n = (int)b->probs.size();
     int rc = launch_gather_scalars(b->d_inst, n, b->d_gather, b->stream);
     if (rc) return rc;
-    FDE_CUDA_TRY(cudaMemcpyAsync(b->h_gather, b->d_gather, 4 * n * sizeof(double), cudaMemcpyDeviceToHost,
+    FDE_CUDA_TRY(cudaMemcpyAsync(b->h_gather, b->d_gather, 5 * n * sizeof(double), cudaMemcpyDeviceToHost,
                                  b->stream));
     FDE_CUDA_TRY(cudaStreamSynchronize(b->stream));
     return FDE_OK;
@@ -150,15 +151,10 @@ void fde_batch_destroy(fde_batch* b) {
     if (b->stream) cudaStreamSynchronize(b->stream);
     else cudaDeviceSynchronize();
     for (fde_problem* p : b->probs) fde_problem_destroy(p);
-    void* dev[] = {b->d_blk, b->d_inst, b->d_act, b->d_kvec, b->d_err, b->d_gather, b->d_pack,
-                   b->d_rhat_shared};
-    for (void* d : dev)
-        if (d) cudaFree(d);
-    if (b->h_gather) cudaFreeHost(b->h_gather);
-    if (b->h_act) cudaFreeHost(b->h_act);
-    if (b->h_kvec) cudaFreeHost(b->h_kvec);
-    if (b->d_ctl) cudaFree(b->d_ctl);
-    if (b->h_ctl) cudaFreeHost(b->h_ctl);
+    void* dev[] = {b->d_blk, b->d_inst, b->d_pack, b->d_rhat_shared};
+    for (void* d : dev) dev_free(d);
+    if (b->h_pin) pinned_free(b->h_pin);
+    else if (b->h_gather) cudaFreeHost(b->h_gather);
     for (auto& kv : b->cycle_graphs) cudaGraphExecDestroy(kv.second.first);
     if (b->cap_stream) cudaStreamDestroy(b->cap_stream);
     delete b;
@@ -192,20 +188,36 @@ int fde_batch_create(const fde_problem_desc* descs, int count, void* stream, fde
         b->max_nblk = std::max(b->max_nblk, P.nblk);
         b->max_n = std::max(b->max_n, P.n);
     }
-    bool ok = cudaMalloc(&b->d_act, count * sizeof(int)) == cudaSuccess &&
-              cudaMalloc(&b->d_kvec, count * sizeof(int)) == cudaSuccess &&
-              cudaMalloc(&b->d_err, sizeof(int)) == cudaSuccess &&
-              cudaMalloc(&b->d_gather, 4 * count * sizeof(double)) == cudaSuccess &&
-              cudaMalloc(&b->d_inst, count * sizeof(InstDev)) == cudaSuccess &&
-              cudaMallocHost(&b->h_gather, 4 * count * sizeof(double)) == cudaSuccess &&
-              cudaMallocHost(&b->h_act, count * sizeof(int)) == cudaSuccess &&
-              cudaMallocHost(&b->h_kvec, count * sizeof(int)) == cudaSuccess &&
-              cudaMalloc(&b->d_ctl, 4 * count * sizeof(int)) == cudaSuccess &&
-              cudaMallocHost(&b->h_ctl, 4 * count * sizeof(int)) == cudaSuccess;
-    if (!ok) {
+    // device words: instance descriptors, gathered scalars, round list, cycle lengths, control
+    // words, error flag; pinned counterparts of the middle four, from the cache of blocks if they fit
+    const size_t c = count, words = c * sizeof(InstDev) + 5 * c * sizeof(double) + (6 * c + 1) * sizeof(int);
+    unsigned char* w = nullptr;
+    int rc = dev_alloc((void**)&w, words);
+    const size_t host = 5 * c * sizeof(double) + 6 * c * sizeof(int);
+    void* pin = nullptr;
+    if (!rc) {
+        if (host <= PINNED_BYTES) {
+            rc = pinned_alloc(&pin);
+            b->h_pin = pin;
+        } else if (cudaMallocHost(&pin, host) != cudaSuccess) {
+            pin = nullptr;
+            rc = FDE_ERR_ALLOC;
+        }
+    }
+    b->d_inst = reinterpret_cast<InstDev*>(w);
+    b->h_gather = static_cast<double*>(pin);
+    if (rc) {
         fde_batch_destroy(b);
         return set_error(FDE_ERR_ALLOC, "batch allocation failed");
     }
+    b->d_gather = reinterpret_cast<double*>(b->d_inst + c);
+    b->d_act = reinterpret_cast<int*>(b->d_gather + 5 * c);
+    b->d_kvec = b->d_act + c;
+    b->d_ctl = b->d_kvec + c;
+    b->d_err = b->d_ctl + 4 * c;
+    b->h_act = reinterpret_cast<int*>(b->h_gather + 5 * c);
+    b->h_kvec = b->h_act + c;
+    b->h_ctl = b->h_kvec + c;
     *out = b;
     return FDE_OK;
 }
@@ -214,9 +226,6 @@ int fde_batch_share_operator(fde_batch* b) {
     if (!b) return set_error(FDE_ERR_ARG, "NULL batch");
     if (b->factored) return set_error(FDE_ERR_STATE, "fde_batch_share_operator must run before fde_batch_factor");
     const Problem& P0 = *problem_of(b->probs[0]);
-    std::vector<double> d0(2 * (size_t)P0.m), di(2 * (size_t)P0.m);
-    FDE_CUDA_TRY(cudaMemcpy(d0.data(), P0.d_dplus, P0.m * sizeof(double), cudaMemcpyDeviceToHost));
-    FDE_CUDA_TRY(cudaMemcpy(d0.data() + P0.m, P0.d_dminus, P0.m * sizeof(double), cudaMemcpyDeviceToHost));
     for (size_t i = 1; i < b->probs.size(); ++i) {
         const Problem& P = *problem_of(b->probs[i]);
         const bool same = P.m == P0.m && P.s == P0.s && P.mu == P0.mu && P.family == P0.family &&
@@ -224,9 +233,8 @@ int fde_batch_share_operator(fde_batch* b) {
         if (!same)
             return set_error(FDE_ERR_ARG, "instance " + std::to_string(i) + " has another operator (m, s, alpha, "
                                           "interval or BVM scheme)");
-        FDE_CUDA_TRY(cudaMemcpy(di.data(), P.d_dplus, P.m * sizeof(double), cudaMemcpyDeviceToHost));
-        FDE_CUDA_TRY(cudaMemcpy(di.data() + P.m, P.d_dminus, P.m * sizeof(double), cudaMemcpyDeviceToHost));
-        if (di != d0)
+        if (!std::equal(P0.h_dplus, P0.h_dplus + P0.m, P.h_dplus) ||
+            !std::equal(P0.h_dminus, P0.h_dminus + P0.m, P.h_dminus))
             return set_error(FDE_ERR_ARG, "instance " + std::to_string(i) + " has other coefficients d+, d-");
     }
     b->shared = true;
@@ -287,7 +295,7 @@ int fde_batch_factor(fde_batch* b, int precision) {
         b->trsm_tc = tc && P0w.d_dtile != nullptr;
         const Problem& P0 = P0w;
         const size_t per = (size_t)P0.nblk * P0.mp * 2 * sizeof(float);
-        if (!b->d_rhat_shared) FDE_CUDA_TRY(cudaMalloc(&b->d_rhat_shared, per * b->probs.size()));
+        if (!b->d_rhat_shared && (rc = dev_alloc(&b->d_rhat_shared, per * b->probs.size()))) return rc;
         FDE_CUDA_TRY(cudaMemsetAsync(b->d_rhat_shared, 0, per * b->probs.size(), b->stream));
         for (fde_problem* p : b->probs) {
             problem_of(p)->factored = true;
@@ -356,10 +364,12 @@ int fde_batch_factor(fde_batch* b, int precision) {
         FDE_CUDA_TRY(cudaMemsetAsync(P.d_info, 0, P.nblk * sizeof(int), b->stream));
     }
     if (kind >= 0 && b->pack_bytes < pack_total) {
-        if (b->d_pack) cudaFree(b->d_pack);
+        if (b->d_pack) FDE_CUDA_TRY(cudaStreamSynchronize(b->stream));
+        dev_free(b->d_pack);
         b->d_pack = nullptr;
         b->pack_bytes = 0;
-        FDE_CUDA_TRY(cudaMalloc(&b->d_pack, pack_total));
+        int arc = dev_alloc((void**)&b->d_pack, pack_total);
+        if (arc) return arc;
         b->pack_bytes = pack_total;
         FDE_CUDA_TRY(cudaMemsetAsync(b->d_pack, 0, pack_total, b->stream));
     }
@@ -374,9 +384,10 @@ int fde_batch_factor(fde_batch* b, int precision) {
     std::stable_sort(blks.begin(), blks.end(), [](const BlkDev& a, const BlkDev& c) { return a.mp > c.mp; });
     b->blk_mp.resize(blks.size());
     for (size_t i = 0; i < blks.size(); ++i) b->blk_mp[i] = blks[i].mp;
-    if (b->d_blk) cudaFree(b->d_blk);
-    b->d_blk = nullptr;
-    FDE_CUDA_TRY(cudaMalloc(&b->d_blk, blks.size() * sizeof(BlkDev)));
+    if (!b->d_blk) {
+        int arc = dev_alloc((void**)&b->d_blk, blks.size() * sizeof(BlkDev));  // the blocks never change
+        if (arc) return arc;
+    }
     FDE_CUDA_TRY(cudaMemcpyAsync(b->d_blk, blks.data(), blks.size() * sizeof(BlkDev), cudaMemcpyHostToDevice,
                                  b->stream));
     FDE_CUDA_TRY(cudaMemsetAsync(b->d_err, 0, sizeof(int), b->stream));
@@ -483,15 +494,11 @@ int fde_batch_solve(fde_batch* b, const fde_pgmres_opts* opts, double* const* x_
     if ((rc = launch_norm_batched(b->d_inst, b->d_act, n, 4, st))) return fail(rc);
     if ((rc = launch_norm_batched(b->d_inst, b->d_act, n, 3, st))) return fail(rc);
     std::vector<double> bnorm(n), beta(n), est(n, 0.0);
-    // |b|^2 sits in scal[131]; gather it through a one-off copy per instance
-    for (int i = 0; i < n; ++i) {
-        Problem& P = *problem_of(b->probs[i]);
-        FDE_CUDA_TRY(cudaMemcpyAsync(b->h_gather + 4 * i, P.d_scal + 131, sizeof(double), cudaMemcpyDeviceToHost, st));
-    }
-    FDE_CUDA_TRY(cudaStreamSynchronize(st));
-    for (int i = 0; i < n; ++i) bnorm[i] = std::sqrt(b->h_gather[4 * i]);
     if ((rc = gather(b))) return fail(rc);
-    for (int i = 0; i < n; ++i) beta[i] = std::sqrt(b->h_gather[4 * i + 3]);
+    for (int i = 0; i < n; ++i) {
+        bnorm[i] = std::sqrt(b->h_gather[5 * i + 4]);
+        beta[i] = std::sqrt(b->h_gather[5 * i + 3]);
+    }
     std::vector<int> its(n, 0), restarts(n, 0), status(n, FDE_OK), kk(n, 0);
     std::vector<char> done(n, 0);
     for (int i = 0; i < n; ++i) {
@@ -516,7 +523,7 @@ int fde_batch_solve(fde_batch* b, const fde_pgmres_opts* opts, double* const* x_
             const int* c = b->h_ctl + 4 * i;
             kk[i] = c[1];
             its[i] = c[2];
-            est[i] = b->h_gather[4 * i + 1];
+            est[i] = b->h_gather[5 * i + 1];
             if (c[3]) status[i] = FDE_ERR_NAN;
         }
         // end of the round: x += Z y, true residual
@@ -540,7 +547,7 @@ int fde_batch_solve(fde_batch* b, const fde_pgmres_opts* opts, double* const* x_
         if ((rc = gather(b))) return fail(rc);
         for (int i : upd) {
             ++restarts[i];
-            beta[i] = std::sqrt(b->h_gather[4 * i + 3]);
+            beta[i] = std::sqrt(b->h_gather[5 * i + 3]);
             if (!std::isfinite(beta[i])) {
                 status[i] = FDE_ERR_NAN;
                 done[i] = 1;

@@ -200,7 +200,7 @@ int launch_bccb_setup(const Problem& P, int modified, double phi0_mod, double* c
                                                                 cinv, singular);
     FDE_LAUNCH_CHECK("bccb_invcol_kernel");
     const size_t smem = (size_t)L * sizeof(double2);
-    FDE_CUDA_TRY(cudaFuncSetAttribute(bccb_spectrum_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    FDE_TRY(allow_smem((const void*)bccb_spectrum_kernel, smem));
     bccb_spectrum_kernel<<<nk, 512, smem, st>>>(m, P.logL, cinv, P.d_twL, K64, K32);
     FDE_LAUNCH_CHECK("bccb_spectrum_kernel");
     return FDE_OK;
@@ -209,14 +209,12 @@ int launch_bccb_setup(const Problem& P, int modified, double phi0_mod, double* c
 int launch_bccb_solve(const Problem& P, void* rhat, int prec, cudaStream_t st) {
     if (prec == FDE_FP64) {
         const size_t smem = (size_t)P.L * sizeof(double2);
-        FDE_CUDA_TRY(cudaFuncSetAttribute(bccb_solve_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          (int)smem));
+        FDE_TRY(allow_smem((const void*)bccb_solve_kernel<double>, smem));
         bccb_solve_kernel<double><<<P.nblk, 512, smem, st>>>(P.m, P.mp, P.logL, (double2*)rhat, P.d_bccb_K64,
                                                               P.d_twL, P.live);
     } else {
         const size_t smem = (size_t)P.L * sizeof(float2);
-        FDE_CUDA_TRY(cudaFuncSetAttribute(bccb_solve_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          (int)smem));
+        FDE_TRY(allow_smem((const void*)bccb_solve_kernel<float>, smem));
         bccb_solve_kernel<float><<<P.nblk, 512, smem, st>>>(P.m, P.mp, P.logL, (float2*)rhat, P.d_bccb_K32,
                                                              P.d_twL32, P.live);
     }

@@ -16,6 +16,7 @@
 #include <deque>
 #include <mutex>
 #include <unordered_map>
+#include <vector>
 
 #include "fde_internal.h"
 
@@ -35,6 +36,11 @@ std::mutex g_mu;
 std::deque<Block> g_cache;                     // freed blocks, oldest first
 size_t g_cached = 0;                           // bytes held in g_cache
 std::unordered_map<void*, Block> g_live;       // blocks handed out
+
+constexpr size_t PINNED_CACHE_LIMIT = 64;      // blocks (16 MB)
+constexpr size_t LU_CACHE_LIMIT = 8;
+std::vector<void*> g_pinned;                   // returned pinned blocks
+std::vector<LuStreams> g_lu;                   // returned LU streams
 
 void release_cached(int dev) {  // g_mu held
     for (auto it = g_cache.begin(); it != g_cache.end();) {
@@ -103,9 +109,116 @@ void dev_free(void* p) {
     }
 }
 
+// A cache hit costs the problem that starts 150 us less than cudaMallocHost, and the one that
+// ends 190 us less than cudaFreeHost, which waits for the device.
+int pinned_alloc(void** p) {
+    {
+        std::lock_guard<std::mutex> lock(g_mu);
+        if (!g_pinned.empty()) {
+            *p = g_pinned.back();
+            g_pinned.pop_back();
+            return FDE_OK;
+        }
+    }
+    *p = nullptr;
+    const cudaError_t e = cudaHostAlloc(p, PINNED_BYTES, cudaHostAllocPortable);
+    if (e != cudaSuccess) {
+        *p = nullptr;
+        cudaGetLastError();
+        return set_error(FDE_ERR_ALLOC, std::string("cudaHostAlloc failed: ") + cudaGetErrorString(e));
+    }
+    return FDE_OK;
+}
+
+void pinned_free(void* p) {
+    if (!p) return;
+    {
+        std::lock_guard<std::mutex> lock(g_mu);
+        if (g_pinned.size() < PINNED_CACHE_LIMIT) {
+            g_pinned.push_back(p);
+            return;
+        }
+    }
+    cudaFreeHost(p);
+}
+
+static void lu_streams_destroy(LuStreams& s) {
+    for (cudaStream_t st : {s.hi, s.lo, s.x})
+        if (st) cudaStreamDestroy(st);
+    for (cudaEvent_t e : s.ev)
+        if (e) cudaEventDestroy(e);
+    s = LuStreams();
+}
+
+int lu_streams_take(LuStreams* s) {
+    int dev = 0;
+    FDE_CUDA_TRY(cudaGetDevice(&dev));
+    {
+        std::lock_guard<std::mutex> lock(g_mu);
+        for (auto it = g_lu.begin(); it != g_lu.end(); ++it)
+            if (it->dev == dev) {
+                *s = *it;
+                g_lu.erase(it);
+                return FDE_OK;
+            }
+    }
+    LuStreams n;
+    int least = 0, greatest = 0;
+    cudaError_t e = cudaDeviceGetStreamPriorityRange(&least, &greatest);
+    if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&n.hi, cudaStreamNonBlocking, greatest);
+    if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&n.lo, cudaStreamNonBlocking, least);
+    // the cross tiles one level below the panel chain (the next diagonal kernel gets the SMs
+    // first), above the interior updates
+    const int mid = greatest < least ? greatest + 1 : greatest;
+    if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&n.x, cudaStreamNonBlocking, mid);
+    for (cudaEvent_t& ev : n.ev)
+        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
+    if (e != cudaSuccess) {
+        lu_streams_destroy(n);
+        return cuda_error(e, "streams of the block LU");
+    }
+    n.dev = dev;
+    *s = n;
+    return FDE_OK;
+}
+
+void lu_streams_return(LuStreams* s) {
+    if (!s->hi) return;
+    {
+        std::lock_guard<std::mutex> lock(g_mu);
+        if (g_lu.size() < LU_CACHE_LIMIT) {
+            g_lu.push_back(*s);
+            *s = LuStreams();
+            return;
+        }
+    }
+    lu_streams_destroy(*s);
+}
+
+int allow_smem(const void* kern, size_t bytes) {
+    static std::mutex mu;
+    static std::unordered_map<const void*, std::vector<size_t>> most;  // per kernel and device
+    int dev = 0;
+    FDE_CUDA_TRY(cudaGetDevice(&dev));
+    std::lock_guard<std::mutex> lock(mu);
+    std::vector<size_t>& m = most[kern];
+    if ((int)m.size() <= dev) m.resize(dev + 1, 0);
+    if (m[dev] >= bytes) return FDE_OK;
+    FDE_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+    m[dev] = bytes;
+    return FDE_OK;
+}
+
 int dev_release_cached() {
     std::lock_guard<std::mutex> lock(g_mu);
     cudaError_t first = cudaSuccess;
+    for (void* p : g_pinned) {
+        const cudaError_t e = cudaFreeHost(p);
+        if (e != cudaSuccess && first == cudaSuccess) first = e;
+    }
+    g_pinned.clear();
+    for (LuStreams& l : g_lu) lu_streams_destroy(l);
+    g_lu.clear();
     for (const Block& b : g_cache) {
         const cudaError_t e = cudaFree(b.p);
         if (e != cudaSuccess && first == cudaSuccess) first = e;

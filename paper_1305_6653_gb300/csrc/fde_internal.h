@@ -26,6 +26,15 @@ int cuda_error(cudaError_t e, const char* what);
         if (e_ != cudaSuccess) return ::fde::cuda_error(e_, #call); \
     } while (0)
 
+#define FDE_TRY(call)          \
+    do {                       \
+        const int rc_ = (call); \
+        if (rc_) return rc_;   \
+    } while (0)
+
+// Dynamic shared memory above 48 KB for a kernel on the current device (set once).
+int allow_smem(const void* kern, size_t bytes);
+
 void note_launch();
 void note_launches(long long k);  // k kernels launched at once (a graph replay; negative: uncount)
 
@@ -110,16 +119,13 @@ struct BlkDev {
 // ---------------------------------------------------------------------------
 struct Problem;
 
-// setup.cu
-int launch_grunwald(double alpha, int count, double* g, cudaStream_t st);
-// tw[k] = exp(-2 pi i k / L) for k < count (count = the table's length)
-int launch_twiddles(int L, int count, double2* tw64, float2* tw32, cudaStream_t st);
-// twq: L + L/2 entries (Problem::d_twq)
-int launch_bfp_twiddles(int L, bfp::Tw* twq, cudaStream_t st);
+// setup.cu: Grunwald weights, every twiddle table and the Strang symbols, in one launch
+int launch_tables(const Problem& P, cudaStream_t st);
+// *bad set (pinned) unless d+, d- are valid at every point and time level; dplus / dminus: their
+// means over n = 1..s
+int launch_timevar_check(const Problem& P, int* bad, cudaStream_t st);
 int launch_toeplitz_symbol(const double* g, int m, int L, double scale, const bfp::Tw* twq, bfp::Q61* kap,
                            float2* sym32, cudaStream_t st);
-int launch_strang_symbols(const double* a_main, const double* b_main, int mu, int nu, int s, double2* phi,
-                          double2* psi, cudaStream_t st);
 int launch_rhs(const Problem& P, const double* Ju0, cudaStream_t st);
 
 // matvec.cu: y = M z (mode 0) or y = J z for ncols columns (mode 1)
@@ -158,6 +164,14 @@ int launch_cycle_start(Problem& P, const double* r, const double* nrm_sq, int re
 int launch_gram_schmidt(Problem& P, int j, int ldh, int reorth, cudaStream_t st);
 int launch_lsq_solve(const double* H, int ldh, int k, const double* g, double* y, cudaStream_t st);
 
+// The side streams and events of a tensor-core LU.
+struct LuStreams {
+    cudaStream_t hi = nullptr, lo = nullptr, x = nullptr;  // panel chain, interior, cross tiles
+    // fork / panel products done / interior done / next diagonal block updated / cross tiles done
+    cudaEvent_t ev[5] = {};
+    int dev = -1;
+};
+
 // ---------------------------------------------------------------------------
 // The problem object.
 // ---------------------------------------------------------------------------
@@ -178,7 +192,16 @@ struct Problem {
     int h_start[FDE_MAX_S + 1];
     double h_a_main[FDE_MAX_MU + 1], h_b_main[FDE_MAX_MU + 1];
 
-    // device buffers
+    // Pinned block (PINNED_BYTES): scalars and step outcomes the kernels write, the factor's
+    // status words, and the upload of the small arrays, which stays (h_dplus, h_dminus: the
+    // coefficients, when they do not vary in time)
+    double* h_pin = nullptr;
+    int* h_info = nullptr;
+    const double* h_dplus = nullptr;
+    const double* h_dminus = nullptr;
+    // device buffers: the small ones are parts of two allocations, the uploaded arrays and
+    // the tables and vectors
+    unsigned char* arena[2] = {nullptr, nullptr};
     int* d_start = nullptr;
     double* d_a = nullptr;      // (s+1)*(mu+1)
     double* d_b = nullptr;
@@ -207,7 +230,7 @@ struct Problem {
     void* d_rhat = nullptr;     // nblk * mp complex (FP64 or FP32 by precision)
     void* d_fac = nullptr;      // nblk * 2 * mp * mp (planar re/im), FP64 or FP32
     void* d_dinv = nullptr;     // nblk * mp complex: 1 / U_ii
-    int* d_info = nullptr;      // nblk: first singular pivot (+1) or 0
+    int* d_info = nullptr;      // nblk: first singular pivot (+1) or 0, followed by d_err
     int* d_err = nullptr;       // device error flag of bounded waits (0 = none)
     size_t fac_bytes = 0;
     void* d_tinv = nullptr;     // inverted 32 x 32 diagonal tiles of L and U (block solves)
@@ -245,11 +268,9 @@ struct Problem {
     long long graph_key = -1;
     int graph_gen = 0;                           // bumped whenever a buffer the graphs use changes
     int solves = 0;                              // completed pgmres_solve calls
-    // tensor-core LU look-ahead: panel chain on lu_hi, interior updates on lu_lo, the
-    // cross tiles other than the next diagonal block on lu_x
-    cudaStream_t lu_hi = nullptr, lu_lo = nullptr, lu_x = nullptr;
-    // fork / panel products done / interior done / next diagonal block updated / cross tiles done
-    cudaEvent_t lu_ev[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
+    // tensor-core LU look-ahead: panel chain on hi, interior updates on lo, the cross tiles
+    // other than the next diagonal block on x
+    LuStreams lu;
 
     // Krylov workspace
     int restart_cap = 0;
@@ -324,6 +345,14 @@ int dev_alloc(void** p, size_t bytes);
 void dev_free(void* p);
 // Frees every cached block (blocks in use are not affected).
 int dev_release_cached();
+// Pinned host blocks of PINNED_BYTES, from a bounded cache as well (the caller makes sure that
+// no queued GPU work uses a block it returns).
+constexpr size_t PINNED_BYTES = 256 * 1024;
+int pinned_alloc(void** p);
+void pinned_free(void* p);
+// The side streams and events of a tensor-core LU, from a bounded cache as well.
+int lu_streams_take(LuStreams* s);
+void lu_streams_return(LuStreams* s);  // its streams are idle
 
 // tune.cu: launch-shape autotuner.  tune_lookup returns the variant to launch for a
 // shape (forced, tabulated, or 0 = the built-in default, with *need_tuning set when

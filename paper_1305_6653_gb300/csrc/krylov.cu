@@ -709,15 +709,14 @@ __global__ void __launch_bounds__(32) lsq_batched(const InstDev* __restrict__ I,
     lsq_body(d.H, ldh, kvec[inst], d.gv, d.y, R);
 }
 
-// out[4*i + q] = scal[128 + q] of instance i (q = 0..3), and out[4*i+3] = scal[132]
+// out[5*i + q] = scal[128 + q] of instance i (q = 0..2), out[5*i+3] = scal[132], out[5*i+4] = scal[131]
 __global__ void gather_scalars(const InstDev* __restrict__ I, int ninst, double* __restrict__ out) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= ninst) return;
     const double* sc = I[i].scal;
-    out[4 * i + 0] = sc[128];
-    out[4 * i + 1] = sc[129];
-    out[4 * i + 2] = sc[130];
-    out[4 * i + 3] = sc[132];
+    for (int q = 0; q < 3; ++q) out[5 * i + q] = sc[128 + q];
+    out[5 * i + 3] = sc[132];
+    out[5 * i + 4] = sc[131];
 }
 
 static int grid_for(long n);
@@ -771,7 +770,7 @@ int launch_gs_batched(const InstDev* I, const int* act, int nact, int j, int ldh
     const size_t stage = gs_stage_bytes(k, k <= 24 ? 2 : 1);
     int stage_doubles = (int)(stage / sizeof(double));
     const size_t smem = stage + (size_t)nact * sizeof(double);
-    FDE_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    FDE_TRY(allow_smem((const void*)kern, smem));
     void* args[] = {&I, &act, &nact, &j, &ldh, &reorth, &tol, &maxit, &err, &stage_doubles};
     FDE_CUDA_TRY(cudaLaunchCooperativeKernel(kern, dim3(ctas), dim3(RED_THREADS), args, smem, st));
     FDE_LAUNCH_CHECK("gs_batched");
@@ -846,7 +845,7 @@ int launch_gram_schmidt(Problem& P, int j, int ldh, int reorth, cudaStream_t st)
                      : k <= 24 ? gs_form<24, 2>(P.n, k, ctas)
                      : k <= 32 ? gs_form<32, 1>(P.n, k, ctas)
                                : gs_form<64, 1>(P.n, k, ctas);
-    if (f.smem) FDE_CUDA_TRY(cudaFuncSetAttribute(f.kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)f.smem));
+    if (f.smem) FDE_TRY(allow_smem((const void*)f.kern, f.smem));
     GsArgs A{P.d_V, P.d_V + (size_t)k * P.n, P.n, k, ldh, reorth, P.d_H, P.d_cs, P.d_sn, P.d_gv, P.d_scal,
              P.d_partial, P.d_counter, P.d_err, P.d_live, P.h_step + j % Problem::STEP_RING};
     void* args[] = {&A};

@@ -1382,10 +1382,9 @@ static int run_lu(Problem& P, cudaStream_t st) {
         FDE_LAUNCH_CHECK("form_blocks_kernel");
     }
     const size_t panel_smem = (size_t)RC * (NB + 1) * sizeof(C);
-    FDE_CUDA_TRY(cudaFuncSetAttribute(lu_panel_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)panel_smem));
+    FDE_TRY(allow_smem((const void*)lu_panel_kernel<T>, panel_smem));
     const size_t upd_smem = (64 * (NB + 1) + NB * 65) * sizeof(C);
-    FDE_CUDA_TRY(cudaFuncSetAttribute(lu_update_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)upd_smem));
+    FDE_TRY(allow_smem((const void*)lu_update_kernel<T>, upd_smem));
     const int steps = mp / NB;
     for (int p = 0; p < steps; ++p) {
         {
@@ -1537,24 +1536,15 @@ template <int KIND>
 static int set_tc_attrs() {
     const size_t panel_smem = (size_t)RC * (NB + 1) * sizeof(float2);
     const size_t upd_smem = (64 * (NB + 1) + NB * 65) * sizeof(float2);
-    FDE_CUDA_TRY(cudaFuncSetAttribute(lu_panel_range_kernel<float, KIND>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)panel_smem));
-    FDE_CUDA_TRY(cudaFuncSetAttribute(lu_panel_range_batched<float, KIND>,
-                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)panel_smem));
-    FDE_CUDA_TRY(cudaFuncSetAttribute(lu_update_range_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)upd_smem));
-    FDE_CUDA_TRY(cudaFuncSetAttribute(lu_update_range_batched<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)upd_smem));
-    FDE_CUDA_TRY(cudaFuncSetAttribute(lu_update_tc2_kernel<KIND>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      Tc2<KIND>::SMEM));
-    FDE_CUDA_TRY(cudaFuncSetAttribute(lu_update_tc2p_kernel<KIND>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      Tc2p<KIND>::SMEM));
-    FDE_CUDA_TRY(cudaFuncSetAttribute(lu_update_tc2p_batched<KIND>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      Tc2p<KIND>::SMEM));
-    FDE_CUDA_TRY(cudaFuncSetAttribute(lu_update_tc2w_kernel<KIND>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      Tc2w<KIND>::SMEM));
-    FDE_CUDA_TRY(cudaFuncSetAttribute(lu_update_tc2s_kernel<KIND>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      Tc2s<KIND>::SMEM));
+    FDE_TRY(allow_smem((const void*)lu_panel_range_kernel<float, KIND>, panel_smem));
+    FDE_TRY(allow_smem((const void*)lu_panel_range_batched<float, KIND>, panel_smem));
+    FDE_TRY(allow_smem((const void*)lu_update_range_kernel<float>, upd_smem));
+    FDE_TRY(allow_smem((const void*)lu_update_range_batched<float>, upd_smem));
+    FDE_TRY(allow_smem((const void*)lu_update_tc2_kernel<KIND>, Tc2<KIND>::SMEM));
+    FDE_TRY(allow_smem((const void*)lu_update_tc2p_kernel<KIND>, Tc2p<KIND>::SMEM));
+    FDE_TRY(allow_smem((const void*)lu_update_tc2p_batched<KIND>, Tc2p<KIND>::SMEM));
+    FDE_TRY(allow_smem((const void*)lu_update_tc2w_kernel<KIND>, Tc2w<KIND>::SMEM));
+    FDE_TRY(allow_smem((const void*)lu_update_tc2s_kernel<KIND>, Tc2s<KIND>::SMEM));
     return FDE_OK;
 }
 
@@ -2154,20 +2144,6 @@ lu_panel_tc2_batched(const BlkDev* __restrict__ B, int o, int R0, int ntg, int* 
     }
 }
 
-static int ensure_lu_streams(Problem& P) {
-    if (P.lu_hi) return FDE_OK;
-    int least = 0, greatest = 0;
-    FDE_CUDA_TRY(cudaDeviceGetStreamPriorityRange(&least, &greatest));
-    FDE_CUDA_TRY(cudaStreamCreateWithPriority(&P.lu_hi, cudaStreamNonBlocking, greatest));
-    FDE_CUDA_TRY(cudaStreamCreateWithPriority(&P.lu_lo, cudaStreamNonBlocking, least));
-    // the cross tiles one level below the panel chain (the next diagonal kernel gets the SMs
-    // first), above the interior updates
-    const int mid = greatest < least ? greatest + 1 : greatest;
-    FDE_CUDA_TRY(cudaStreamCreateWithPriority(&P.lu_x, cudaStreamNonBlocking, mid));
-    for (cudaEvent_t& e : P.lu_ev) FDE_CUDA_TRY(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
-    return FDE_OK;
-}
-
 // Two-level tensor-core LU with look-ahead.  The panel chain (diagonal block,
 // packing, panel products) and the part of each trailing update that the next
 // panel needs (its rows and columns: the cross tiles) run on a high-priority
@@ -2214,12 +2190,10 @@ static int run_lu_tc(Problem& P, cudaStream_t st) {
     unsigned char* ipack = base ? base + (size_t)nsets * nb * (pa + pb) : nullptr;
     int rc = set_tc_attrs<KIND>();
     if (rc) return rc;
-    FDE_CUDA_TRY(cudaFuncSetAttribute(lu_diag128_kernel<KIND>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)diag128_smem()));
-    FDE_CUDA_TRY(cudaFuncSetAttribute(lu_panel_tc2_kernel<KIND>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      Cfg::SMEM_STORE_EPI));
-    if ((rc = ensure_lu_streams(P))) return rc;
-    cudaStream_t sh = P.lu_hi, sl = P.lu_lo, sx = P.lu_x;
+    FDE_TRY(allow_smem((const void*)lu_diag128_kernel<KIND>, diag128_smem()));
+    FDE_TRY(allow_smem((const void*)lu_panel_tc2_kernel<KIND>, Cfg::SMEM_STORE_EPI));
+    if (!P.lu.hi && (rc = lu_streams_take(&P.lu))) return rc;
+    cudaStream_t sh = P.lu.hi, sl = P.lu.lo, sx = P.lu.x;
     // inverted diagonal blocks kept for the tensor-core block solves (TF32, whole 128-row strips)
     const int nst = mp / TB;
     const size_t dtile_stride = (size_t)nst * 2 * Cfg::A_TILE;
@@ -2262,10 +2236,10 @@ static int run_lu_tc(Problem& P, cudaStream_t st) {
     if ((merge || strips) && (rc = factor_tensor_map_sw128(fac, mp, nb, &cmap))) return rc;
     if (strips && !sbf16 && (rc = strip_tensor_map_sw128(strips, mp, nb, &smap))) return rc;
     const int smode = strips ? (sbf16 ? 2 : 1) : 0;
-    FDE_CUDA_TRY(cudaEventRecord(P.lu_ev[0], st));  // fork after the work already queued on st
-    FDE_CUDA_TRY(cudaStreamWaitEvent(sh, P.lu_ev[0], 0));
-    FDE_CUDA_TRY(cudaStreamWaitEvent(sl, P.lu_ev[0], 0));
-    FDE_CUDA_TRY(cudaStreamWaitEvent(sx, P.lu_ev[0], 0));
+    FDE_CUDA_TRY(cudaEventRecord(P.lu.ev[0], st));  // fork after the work already queued on st
+    FDE_CUDA_TRY(cudaStreamWaitEvent(sh, P.lu.ev[0], 0));
+    FDE_CUDA_TRY(cudaStreamWaitEvent(sl, P.lu.ev[0], 0));
+    FDE_CUDA_TRY(cudaStreamWaitEvent(sx, P.lu.ev[0], 0));
 
     // diagonal block, then (if a trailing matrix follows) packing and panel products
     // after_cross: the panel products wait for the cross tiles of the previous step (on
@@ -2280,7 +2254,7 @@ static int run_lu_tc(Problem& P, cudaStream_t st) {
                 dsave ? dsave + (size_t)(o / TB) * 2 * Cfg::A_TILE : nullptr, dtile_stride, strips, sbf16 ? 1 : 0);
             FDE_LAUNCH_CHECK("lu_diag128_kernel");
         }
-        if (after_cross) FDE_CUDA_TRY(cudaStreamWaitEvent(sh, P.lu_ev[4], 0));
+        if (after_cross) FDE_CUDA_TRY(cudaStreamWaitEvent(sh, P.lu.ev[4], 0));
         if (!more) return FDE_OK;
         const int nt = cdiv(mp - R0, T2_BM);
         const long items = 2L * (mp - R0) * (TB / Cfg::PER_CORE);
@@ -2325,10 +2299,10 @@ static int run_lu_tc(Problem& P, cudaStream_t st) {
             // the interior update of step p needs this step's packed L21 / U12 (the panel
             // products just queued on sh), not the cross tiles below: it touches other tiles
             // and reads other operand buffers, so it runs beside them
-            FDE_CUDA_TRY(cudaEventRecord(P.lu_ev[1], sh));
+            FDE_CUDA_TRY(cudaEventRecord(P.lu.ev[1], sh));
             // the cross tiles update tiles the last interior update wrote and pack over a buffer
             // it may read (an even step of a merged pair touches neither)
-            if (p > 0 && !a_step) FDE_CUDA_TRY(cudaStreamWaitEvent(sh, P.lu_ev[2], 0));
+            if (p > 0 && !a_step) FDE_CUDA_TRY(cudaStreamWaitEvent(sh, P.lu.ev[2], 0));
             const bool next = R0 + TB < mp;
             {  // the next diagonal block (tile 0, 0): all the next diagonal kernel waits for
                 StageTimer t(P, FDE_STAGE_LU_TC, sh);
@@ -2336,8 +2310,8 @@ static int run_lu_tc(Problem& P, cudaStream_t st) {
                                                                               pb, P.d_err, nullptr, ao, bo);
                 FDE_LAUNCH_CHECK("lu_update_tc2_kernel");
             }
-            FDE_CUDA_TRY(cudaEventRecord(P.lu_ev[3], sh));
-            FDE_CUDA_TRY(cudaStreamWaitEvent(sx, P.lu_ev[3], 0));
+            FDE_CUDA_TRY(cudaEventRecord(P.lu.ev[3], sh));
+            FDE_CUDA_TRY(cudaStreamWaitEvent(sx, P.lu.ev[3], 0));
             {  // the rest of the next panel's rows (single tiles) and the column below them (row
                // pairs) beside the next diagonal block; when that panel has a trailing matrix, they
                // are packed as its operand tiles as well
@@ -2357,10 +2331,10 @@ static int run_lu_tc(Problem& P, cudaStream_t st) {
                     FDE_LAUNCH_CHECK("lu_update_tc2s_kernel");
                 }
             }
-            FDE_CUDA_TRY(cudaEventRecord(P.lu_ev[4], sx));
+            FDE_CUDA_TRY(cudaEventRecord(P.lu.ev[4], sx));
             const int f = b_step ? 2 : 1;  // first row / column of the interior update
             if (!a_step && nt > f) {
-                FDE_CUDA_TRY(cudaStreamWaitEvent(sl, P.lu_ev[1], 0));
+                FDE_CUDA_TRY(cudaStreamWaitEvent(sl, P.lu.ev[1], 0));
                 StageTimer t(P, FDE_STAGE_LU_TC, sl);
                 if (interior == 2) {  // warp-specialized, C through a ring of tensor-map copies
                     lu_update_tc2s_kernel<KIND>
@@ -2377,7 +2351,7 @@ static int run_lu_tc(Problem& P, cudaStream_t st) {
                                                   sl>>>(mp, R0, nt, 1, nt - 1, fac, apk(o), bpk(o), pa, pb, P.d_err);
                     FDE_LAUNCH_CHECK("lu_update_tc2p_kernel");
                 }
-                FDE_CUDA_TRY(cudaEventRecord(P.lu_ev[2], sl));
+                FDE_CUDA_TRY(cudaEventRecord(P.lu.ev[2], sl));
             }
             if ((r = panel(R0, true))) return r;
         }
@@ -2387,12 +2361,12 @@ static int run_lu_tc(Problem& P, cudaStream_t st) {
     P.strips_ok = rc == FDE_OK && strips != nullptr;
     P.strips_bf16 = sbf16;
     // join: st continues after all three streams
-    cudaEventRecord(P.lu_ev[1], sl);
-    cudaStreamWaitEvent(st, P.lu_ev[1], 0);
-    cudaEventRecord(P.lu_ev[1], sx);
-    cudaStreamWaitEvent(st, P.lu_ev[1], 0);
-    cudaEventRecord(P.lu_ev[1], sh);
-    cudaStreamWaitEvent(st, P.lu_ev[1], 0);
+    cudaEventRecord(P.lu.ev[1], sl);
+    cudaStreamWaitEvent(st, P.lu.ev[1], 0);
+    cudaEventRecord(P.lu.ev[1], sx);
+    cudaStreamWaitEvent(st, P.lu.ev[1], 0);
+    cudaEventRecord(P.lu.ev[1], sh);
+    cudaStreamWaitEvent(st, P.lu.ev[1], 0);
     return rc;
 }
 
@@ -2406,10 +2380,8 @@ static int run_lu_batched_simt(const BlkDev* d_blk, const std::vector<int>& mps,
     FDE_LAUNCH_CHECK("form_blocks_batched");
     const size_t panel_smem = (size_t)RC * (NB + 1) * sizeof(float2);
     const size_t upd_smem = (64 * (NB + 1) + NB * 65) * sizeof(float2);
-    FDE_CUDA_TRY(cudaFuncSetAttribute(lu_panel_batched<float, -1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)panel_smem));
-    FDE_CUDA_TRY(cudaFuncSetAttribute(lu_update_batched<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)upd_smem));
+    FDE_TRY(allow_smem((const void*)lu_panel_batched<float, -1>, panel_smem));
+    FDE_TRY(allow_smem((const void*)lu_update_batched<float>, upd_smem));
     for (int p = 0; p * NB < max_mp; ++p) {
         int nd = 0, nu = 0;
         while (nd < nbt && mps[nd] > p * NB) ++nd;
@@ -2437,10 +2409,8 @@ static int run_lu_batched_tc(const BlkDev* d_blk, const std::vector<int>& mps, i
     FDE_LAUNCH_CHECK("form_blocks_batched");
     int rc = set_tc_attrs<KIND>();
     if (rc) return rc;
-    FDE_CUDA_TRY(cudaFuncSetAttribute(lu_diag128_batched<KIND>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)diag128_smem()));
-    FDE_CUDA_TRY(cudaFuncSetAttribute(lu_panel_tc2_batched<KIND>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      Cfg::SMEM_STORE_EPI));
+    FDE_TRY(allow_smem((const void*)lu_diag128_batched<KIND>, diag128_smem()));
+    FDE_TRY(allow_smem((const void*)lu_panel_tc2_batched<KIND>, Cfg::SMEM_STORE_EPI));
     auto active = [&](int lim) {  // blocks with m_p > lim (a prefix of the sorted table)
         int n = 0;
         while (n < nbt && mps[n] > lim) ++n;
@@ -2507,8 +2477,7 @@ int launch_trsv_multi(const InstDev* I, const int* act, int nact, int nblk, int 
     if (nact <= 0) return FDE_OK;
     const size_t smem = trsv_multi_smem_bytes(mp);
     if (smem > 227 * 1024) return launch_trsv_batched(I, act, nact, nblk, mp, st);  // m_p > 2560: one per CTA
-    FDE_CUDA_TRY(cudaFuncSetAttribute(block_trsv_multi_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)smem));
+    FDE_TRY(allow_smem((const void*)block_trsv_multi_kernel, smem));
     block_trsv_multi_kernel<<<dim3((nact + TRSV_R - 1) / TRSV_R, nblk), TRSVM_THREADS, smem, st>>>(I, act, nact);
     FDE_LAUNCH_CHECK("block_trsv_multi_kernel");
     return FDE_OK;
@@ -2517,8 +2486,7 @@ int launch_trsv_multi(const InstDev* I, const int* act, int nact, int nblk, int 
 int launch_trsv_batched(const InstDev* I, const int* act, int nact, int max_nblk, int max_mp, cudaStream_t st) {
     if (nact <= 0) return FDE_OK;
     const size_t smem = trsv_smem_bytes(max_mp, sizeof(float));
-    FDE_CUDA_TRY(cudaFuncSetAttribute(block_trsv_batched<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)smem));
+    FDE_TRY(allow_smem((const void*)block_trsv_batched<float>, smem));
     block_trsv_batched<float><<<dim3(nact, max_nblk), TRSV_THREADS, smem, st>>>(I, act);
     FDE_LAUNCH_CHECK("block_trsv_batched");
     return FDE_OK;
@@ -2643,7 +2611,7 @@ static int launch_trsv_shape(const Problem& P, void* rhat, cudaStream_t st) {
     if constexpr (sizeof(T) == 4) {
         if (strips && P.strips_bf16) {
             auto kern = block_trsv_kernel<T, V, LAY_STRIPS_BF16>;
-            FDE_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+            FDE_TRY(allow_smem((const void*)kern, smem));
             kern<<<P.nblk, trsv_shape<T, V>::NT, smem, st>>>(P.mp, (const unsigned short*)P.d_strips,
                                                               (const cplx_t<T>*)P.d_dinv, (const T*)P.d_tinv,
                                                               (cplx_t<T>*)rhat, P.live);
@@ -2654,7 +2622,7 @@ static int launch_trsv_shape(const Problem& P, void* rhat, cudaStream_t st) {
     {
         constexpr int LS = sizeof(T) == 4 ? LAY_STRIPS : LAY_PLANES;  // FP64 factors have no copy
         auto kern = strips ? block_trsv_kernel<T, V, LS> : block_trsv_kernel<T, V, LAY_PLANES>;
-        FDE_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        FDE_TRY(allow_smem((const void*)kern, smem));
         kern<<<P.nblk, trsv_shape<T, V>::NT, smem, st>>>(P.mp, (const T*)(strips ? P.d_strips : P.d_fac),
                                                           (const cplx_t<T>*)P.d_dinv, (const T*)P.d_tinv,
                                                           (cplx_t<T>*)rhat, P.live);
@@ -2700,7 +2668,7 @@ static int launch_trsv_ring(const Problem& P, void* rhat, cudaStream_t st) {
     int rc = trsv_tensor_map<T>(P, &map);
     if (rc) return rc;
     auto kern = block_trsv_ring_kernel<T>;
-    FDE_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    FDE_TRY(allow_smem((const void*)kern, smem));
     kern<<<P.nblk, ring_cfg<T>::NT, smem, st>>>(P.mp, (const T*)P.d_fac, (const cplx_t<T>*)P.d_dinv,
                                                  (const T*)P.d_tinv, (cplx_t<T>*)rhat, P.d_err, map, P.live);
     FDE_LAUNCH_CHECK("block_trsv_ring_kernel");

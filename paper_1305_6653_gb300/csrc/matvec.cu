@@ -363,7 +363,7 @@ int launch_matvec_batched(const InstDev* I, const int* act, int nact, int max_s,
                           int j, cudaStream_t st) {
     if (nact <= 0) return FDE_OK;
     const size_t smem = (size_t)max_L * sizeof(bfp::I2) + (size_t)max_m * sizeof(double);
-    FDE_CUDA_TRY(cudaFuncSetAttribute(st_matvec_batched, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024));
+    FDE_TRY(allow_smem((const void*)st_matvec_batched, 226 * 1024));
     st_matvec_batched<<<dim3(max_s, nact), row_threads(max_L, 256), smem, st>>>(I, act, which, j);
     FDE_LAUNCH_CHECK("st_matvec_batched");
     return FDE_OK;
@@ -374,7 +374,7 @@ static int launch_st(const Problem& P, const double* z, double* y, int ncols, cu
                      const double* dplus = nullptr, const double* dminus = nullptr, int dstride = 0) {
     const size_t smem = (size_t)P.L * sizeof(bfp::I2) + (MODE == 0 ? (size_t)P.m * sizeof(double) : 0);
     auto kern = st_matvec_kernel<MODE, NT>;
-    FDE_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024));
+    FDE_TRY(allow_smem((const void*)kern, 226 * 1024));
     kern<<<ncols, row_threads(P.L, NT), smem, st>>>(P.m, P.logL, P.mu, P.h, P.d_start, P.d_a, P.d_b,
                                                     dplus ? dplus : P.d_dplus, dminus ? dminus : P.d_dminus, P.d_twq,
                                                     P.d_kap, toeplitz_scale(P), z, y, dstride, P.live);
@@ -386,7 +386,7 @@ int launch_matvec32(const Problem& P, const double* z, double* y, cudaStream_t s
     if (P.timevar) return launch_matvec64(P, z, y, st);  // the time-level products stay FP64
     const size_t smem = (size_t)P.L * sizeof(float2) + (size_t)P.m * sizeof(double);
     const int threads = P.L / 2 > 1024 ? 1024 : P.L / 2 < 64 ? 64 : P.L / 2;
-    FDE_CUDA_TRY(cudaFuncSetAttribute(st_matvec32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
+    FDE_TRY(allow_smem((const void*)st_matvec32_kernel, 227 * 1024));
     st_matvec32_kernel<<<P.s, threads, smem, st>>>(P.m, P.logL, P.mu, P.h, P.d_start, P.d_a, P.d_b, P.d_dplus,
                                                    P.d_dminus, P.d_sym32, P.d_twL32, z, y, P.live);
     FDE_LAUNCH_CHECK("st_matvec32_kernel");

@@ -365,7 +365,7 @@ int conv_tiles(const TI* x, int Q, const TW* W, const float* bias, int P, int K,
     const size_t stage = (size_t)QC * (ld + K * CV_LDW), red = (size_t)CV_WARPS * CV_TP * TN;
     const size_t smem = (stage > red ? stage : red) * sizeof(float);
     auto kern = conv_kernel<TI, TW, TO, TRANS, NL, KT>;
-    FDE_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
+    FDE_TRY(allow_smem((const void*)kern, 227 * 1024));
     const dim3 grid((N + TN - 1) / TN, (P + CV_TP - 1) / CV_TP);
     kern<<<grid, 32 * CV_WARPS, smem, st>>>(x, Q, W, bias, P, K, m, N, relu, mask, y, ld);
     FDE_LAUNCH_CHECK("conv_kernel");
@@ -532,7 +532,7 @@ int fde_nop_loss_grad(fde_nop* n, const float* in, const float* target, int batc
         const dim3 wg((C + 15) / 16, (O + 15) / 16, std::min(B, 16));
         const int ld = staged_length(WG_N, B * m, m, n->K) | 1;
         const size_t smem = (size_t)16 * (WG_N + 1 + ld) * sizeof(float);
-        FDE_CUDA_TRY(cudaFuncSetAttribute(conv_wgrad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
+        FDE_TRY(allow_smem((const void*)conv_wgrad_kernel, 227 * 1024));
         conv_wgrad_kernel<<<wg, 256, smem, n->stream>>>(g, O, a, C, n->K, m, B, n->g + n->woff[l], n->g + n->boff[l],
                                                         ld);
         FDE_LAUNCH_CHECK("conv_wgrad_kernel");

@@ -7,49 +7,120 @@
 
 namespace fde {
 
-// g_0 = 1, g_{k+1} = (1 - (alpha+1)/(k+1)) g_k (eq. (1.2)).  One warp: lane l runs
-// the recurrence over its own contiguous chunk of factors starting from 1, the
-// chunk products are scanned across lanes (multiplicative prefix), and each lane
-// rescales its chunk.  The result is the same product of the same factors as the
-// sequential recurrence, associated differently (a few ulps apart).
-__global__ void grunwald_kernel(double alpha, int count, double* __restrict__ g) {
-    const int lane = threadIdx.x;
-    const int chunk = (count + 31) / 32;
-    const int k0 = lane * chunk;  // this lane produces g[k0+1 .. k0+chunk]
+// g_0 = 1, g_{k+1} = (1 - (alpha+1)/(k+1)) g_k (eq. (1.2)).  One CTA of 256: thread t runs
+// the recurrence over its own contiguous chunk of factors starting from 1, the chunk
+// products are scanned across the threads (multiplicative prefix), and each thread rescales
+// its chunk.  The result is the same product of the same factors as the sequential
+// recurrence, associated differently (a few ulps apart).  (The chain of FP64 divisions is what
+// takes time: 58 us at m = 4095 by one warp.)
+__device__ __forceinline__ void grunwald_weights(double alpha, int count, double* __restrict__ g) {
+    __shared__ double warp_prod[8];
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int chunk = (count + 255) / 256;
+    const int k0 = t * chunk;  // this thread produces g[k0+1 .. k0+chunk]
     double prod = 1.0;
     for (int k = k0; k < k0 + chunk && k + 1 < count; ++k) {
         prod *= (1.0 - (alpha + 1.0) / (double)(k + 1));
         g[k + 1] = prod;  // partial product, rescaled below
     }
-    double pre = prod;  // inclusive scan of chunk products
+    double pre = prod;  // inclusive scan of chunk products over the warp
     for (int off = 1; off < 32; off <<= 1) {
         const double v = __shfl_up_sync(0xffffffffu, pre, off);
         if (lane >= off) pre *= v;
     }
+    if (lane == 31) warp_prod[warp] = pre;
     double excl = __shfl_up_sync(0xffffffffu, pre, 1);
     if (lane == 0) excl = 1.0;
-    __syncwarp();
+    __syncthreads();
+    for (int w = 0; w < warp; ++w) excl *= warp_prod[w];
     for (int k = k0; k < k0 + chunk && k + 1 < count; ++k) g[k + 1] *= excl;
-    if (lane == 0) g[0] = 1.0;
+    if (t == 0) g[0] = 1.0;
 }
 
-// tw[k] = exp(-2 pi i k / L) for k < count (the caller's table length: L/2 for
-// radix-2 stages, L for the radix-4 passes, which read up to 3L/4).
-__global__ void twiddle_kernel(int L, int count, double2* __restrict__ tw64, float2* __restrict__ tw32) {
-    int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= count) return;
-    double sn, cs;
-    sincospi(-2.0 * (double)k / (double)L, &sn, &cs);
-    if (tw64) tw64[k] = make_double2(cs, sn);
-    if (tw32) tw32[k] = make_float2((float)cs, (float)sn);
+// Everything that depends on (alpha, m, s, scheme) alone, in one launch (seven small ones took
+// as long as the symbol transform that follows): CTA 0 the Grunwald weights, the others one
+// table entry a thread -- exp(-2 pi i k / L) in FP64 and FP32 for k < L, exp(-2 pi i k / s) for
+// k < s/2, the block floating-point twiddles (k < L, then the first L/2 in bit-reversed
+// order), and the Strang symbols
+//   phi_k = sum_{r=-nu}^{mu-nu} a_{r+nu} exp(2 pi i r k / s), psi_k likewise with b, k = 0..s/2.
+struct TableArgs {
+    double alpha;
+    int m, logL, s, mu, nu;
+    double a[FDE_MAX_MU + 1], b[FDE_MAX_MU + 1];
+    double* g;
+    double2* twL;
+    float2* twL32;
+    double2* tws;
+    float2* tws32;
+    bfp::Tw* twq;
+    double2* phi;
+    double2* psi;
+};
+__global__ void __launch_bounds__(256) tables_kernel(const __grid_constant__ TableArgs A) {
+    if (blockIdx.x == 0) {
+        grunwald_weights(A.alpha, A.m + 2, A.g);
+        return;
+    }
+    const int L = 1 << A.logL, s = A.s;
+    int k = (blockIdx.x - 1) * blockDim.x + threadIdx.x;
+    if (k < L) {
+        double sn, cs;
+        sincospi(-2.0 * (double)k / (double)L, &sn, &cs);
+        A.twL[k] = make_double2(cs, sn);
+        A.twL32[k] = make_float2((float)cs, (float)sn);
+        return;
+    }
+    k -= L;
+    if (k < s / 2) {
+        double sn, cs;
+        sincospi(-2.0 * (double)k / (double)s, &sn, &cs);
+        A.tws[k] = make_double2(cs, sn);
+        A.tws32[k] = make_float2((float)cs, (float)sn);
+        return;
+    }
+    k -= s / 2;
+    if (k < L + L / 2) {
+        A.twq[k] = bfp::twiddle(k < L ? k : bitrev(k - L, A.logL - 1), A.logL);
+        return;
+    }
+    k -= L + L / 2;
+    if (k <= s / 2) {
+        double pr = 0, pi = 0, qr = 0, qi = 0;
+        for (int r = -A.nu; r <= A.mu - A.nu; ++r) {
+            long rk = ((long)r * k) % s;
+            double sn, cs;
+            sincospi(2.0 * (double)rk / (double)s, &sn, &cs);
+            pr += A.a[r + A.nu] * cs;
+            pi += A.a[r + A.nu] * sn;
+            qr += A.b[r + A.nu] * cs;
+            qi += A.b[r + A.nu] * sn;
+        }
+        A.phi[k] = make_double2(pr, pi);
+        A.psi[k] = make_double2(qr, qi);
+    }
 }
 
-// The block floating-point twiddles: exp(-2 pi i k / L), k < L, then the first L/2 of them
-// in bit-reversed order.
-__global__ void bfp_twiddle_kernel(int logL, bfp::Tw* __restrict__ twq) {
-    const int L = 1 << logL, k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k < L) twq[k] = bfp::twiddle(k, logL);
-    else if (k < L + L / 2) twq[k] = bfp::twiddle(bitrev(k - L, logL - 1), logL);
+// Time-dependent coefficients: a thread per point checks every time level and forms the means
+// over the unknown ones.
+__global__ void __launch_bounds__(128)
+timevar_check_kernel(int m, int s, const double* __restrict__ dpt, const double* __restrict__ dmt,
+                     double* __restrict__ dp, double* __restrict__ dm, int* __restrict__ bad) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= m) return;
+    double sp = 0.0, sm = 0.0;
+    bool ok = true;
+    for (int n = 0; n <= s; ++n) {
+        const double p = dpt[(size_t)n * m + i], q = dmt[(size_t)n * m + i];
+        ok = ok && p >= 0.0 && q >= 0.0 && p + q > 0.0 && isfinite(p) && isfinite(q);
+        if (n > 0) {
+            sp += p;
+            sm += q;
+        }
+    }
+    dp[i] = sp / s;
+    dm[i] = sm / s;
+    ok = ok && isfinite(dp[i]) && isfinite(dm[i]) && dp[i] + dm[i] > 0.0;
+    if (!ok) *bad = 1;
 }
 
 // First column of the L-periodic circulant C that embeds G (G[i][j] = g_{i-j+1}
@@ -86,25 +157,6 @@ toeplitz_symbol_kernel(const double* __restrict__ g, int m, int logL, double sca
     }
 }
 
-// phi_k = sum_{r=-nu}^{mu-nu} a_{r+nu} exp(2 pi i r k / s), psi_k likewise with b, k = 0..s/2
-__global__ void strang_symbol_kernel(const double* __restrict__ a, const double* __restrict__ b, int mu, int nu,
-                                     int s, double2* __restrict__ phi, double2* __restrict__ psi) {
-    int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k > s / 2) return;
-    double pr = 0, pi = 0, qr = 0, qi = 0;
-    for (int r = -nu; r <= mu - nu; ++r) {
-        long rk = ((long)r * k) % s;
-        double sn, cs;
-        sincospi(2.0 * (double)rk / (double)s, &sn, &cs);
-        pr += a[r + nu] * cs;
-        pi += a[r + nu] * sn;
-        qr += b[r + nu] * cs;
-        qi += b[r + nu] * sn;
-    }
-    phi[k] = make_double2(pr, pi);
-    psi[k] = make_double2(qr, qi);
-}
-
 // b_t = h sum_q B[t][start+q] f_{start+q} - A[t][0] u0 + h B[t][0] J u0, t = 1..s
 // (eq. (1.10) with the known block u_0 moved to the right-hand side).
 __global__ void rhs_kernel(int m, int s, int mu, double h, const int* __restrict__ start,
@@ -124,42 +176,33 @@ __global__ void rhs_kernel(int m, int s, int mu, double h, const int* __restrict
     b[(size_t)(t - 1) * m + i] = acc;
 }
 
-int launch_grunwald(double alpha, int count, double* g, cudaStream_t st) {
-    grunwald_kernel<<<1, 32, 0, st>>>(alpha, count, g);
-    FDE_LAUNCH_CHECK("grunwald_kernel");
+int launch_tables(const Problem& P, cudaStream_t st) {
+    TableArgs A{P.alpha, P.m, P.logL, P.s, P.mu, P.nu, {}, {}, P.d_g, P.d_twL, P.d_twL32, P.d_tws, P.d_tws32,
+                P.d_twq, P.d_phi, P.d_psi};
+    for (int i = 0; i <= P.mu; ++i) {
+        A.a[i] = P.h_a_main[i];
+        A.b[i] = P.h_b_main[i];
+    }
+    const int items = P.L + P.s / 2 + P.L + P.L / 2 + P.s / 2 + 1;
+    tables_kernel<<<1 + (items + 255) / 256, 256, 0, st>>>(A);
+    FDE_LAUNCH_CHECK("tables_kernel");
     return FDE_OK;
 }
 
-int launch_twiddles(int L, int count, double2* tw64, float2* tw32, cudaStream_t st) {
-    if (count <= 0) return FDE_OK;
-    twiddle_kernel<<<(count + 255) / 256, 256, 0, st>>>(L, count, tw64, tw32);
-    FDE_LAUNCH_CHECK("twiddle_kernel");
-    return FDE_OK;
-}
-
-int launch_bfp_twiddles(int L, bfp::Tw* twq, cudaStream_t st) {
-    const int n = L + L / 2;
-    bfp_twiddle_kernel<<<(n + 255) / 256, 256, 0, st>>>(ilog2(L), twq);
-    FDE_LAUNCH_CHECK("bfp_twiddle_kernel");
+int launch_timevar_check(const Problem& P, int* bad, cudaStream_t st) {
+    timevar_check_kernel<<<(P.m + 127) / 128, 128, 0, st>>>(P.m, P.s, P.d_dplus_t, P.d_dminus_t, P.d_dplus,
+                                                           P.d_dminus, bad);
+    FDE_LAUNCH_CHECK("timevar_check_kernel");
     return FDE_OK;
 }
 
 int launch_toeplitz_symbol(const double* g, int m, int L, double scale, const bfp::Tw* twq, bfp::Q61* kap,
                            float2* sym32, cudaStream_t st) {
     const size_t smem = (size_t)L * sizeof(bfp::I2);
-    FDE_CUDA_TRY(cudaFuncSetAttribute(toeplitz_symbol_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      226 * 1024));
+    FDE_TRY(allow_smem((const void*)toeplitz_symbol_kernel, 226 * 1024));
     const int threads = L / 8 > 512 ? 512 : L / 8 < 64 ? 64 : L / 8;
     toeplitz_symbol_kernel<<<1, threads, smem, st>>>(g, m, ilog2(L), scale, twq, kap, sym32);
     FDE_LAUNCH_CHECK("toeplitz_symbol_kernel");
-    return FDE_OK;
-}
-
-int launch_strang_symbols(const double* a_main, const double* b_main, int mu, int nu, int s, double2* phi,
-                          double2* psi, cudaStream_t st) {
-    int n = s / 2 + 1;
-    strang_symbol_kernel<<<(n + 127) / 128, 128, 0, st>>>(a_main, b_main, mu, nu, s, phi, psi);
-    FDE_LAUNCH_CHECK("strang_symbol_kernel");
     return FDE_OK;
 }
 

@@ -122,7 +122,7 @@ int launch_time_fft_batched(const InstDev* I, const int* act, int nact, int max_
     if (nact <= 0) return FDE_OK;
     const dim3 grid((max_mp + XW - 1) / XW, nact);
     const size_t smem = (size_t)NCOL * max_s * sizeof(float2);
-    FDE_CUDA_TRY(cudaFuncSetAttribute(time_fft_fwd_batched, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
+    FDE_TRY(allow_smem((const void*)time_fft_fwd_batched, 227 * 1024));
     time_fft_fwd_batched<<<grid, 256, smem, st>>>(I, act, j);
     FDE_LAUNCH_CHECK("time_fft_fwd_batched");
     return FDE_OK;
@@ -133,7 +133,7 @@ int launch_time_ifft_batched(const InstDev* I, const int* act, int nact, int max
     if (nact <= 0) return FDE_OK;
     const dim3 grid((max_mp + XW - 1) / XW, nact);
     const size_t smem = (size_t)NCOL * max_s * sizeof(float2);
-    FDE_CUDA_TRY(cudaFuncSetAttribute(time_fft_inv_batched, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024));
+    FDE_TRY(allow_smem((const void*)time_fft_inv_batched, 227 * 1024));
     time_fft_inv_batched<<<grid, 256, smem, st>>>(I, act, j);
     FDE_LAUNCH_CHECK("time_fft_inv_batched");
     return FDE_OK;
@@ -143,13 +143,11 @@ int launch_time_fft_fwd(const Problem& P, const double* r, void* rhat, int prec,
     const int grid = (P.mp + XW - 1) / XW;
     if (prec == FDE_FP64) {
         size_t smem = (size_t)NCOL * P.s * sizeof(double2);
-        FDE_CUDA_TRY(cudaFuncSetAttribute(time_fft_fwd_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          227 * 1024));
+        FDE_TRY(allow_smem((const void*)time_fft_fwd_kernel<double>, 227 * 1024));
         time_fft_fwd_kernel<double><<<grid, 256, smem, st>>>(P.m, P.mp, P.logs, r, P.d_tws, (double2*)rhat);
     } else {
         size_t smem = (size_t)NCOL * P.s * sizeof(float2);
-        FDE_CUDA_TRY(cudaFuncSetAttribute(time_fft_fwd_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          227 * 1024));
+        FDE_TRY(allow_smem((const void*)time_fft_fwd_kernel<float>, 227 * 1024));
         time_fft_fwd_kernel<float><<<grid, 256, smem, st>>>(P.m, P.mp, P.logs, r, P.d_tws32, (float2*)rhat);
     }
     FDE_LAUNCH_CHECK("time_fft_fwd_kernel");
@@ -160,13 +158,11 @@ int launch_time_fft_inv(const Problem& P, const void* xhat, double* z, int prec,
     const int grid = (P.mp + XW - 1) / XW;
     if (prec == FDE_FP64) {
         size_t smem = (size_t)NCOL * P.s * sizeof(double2);
-        FDE_CUDA_TRY(cudaFuncSetAttribute(time_fft_inv_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          227 * 1024));
+        FDE_TRY(allow_smem((const void*)time_fft_inv_kernel<double>, 227 * 1024));
         time_fft_inv_kernel<double><<<grid, 256, smem, st>>>(P.m, P.mp, P.logs, (const double2*)xhat, P.d_tws, z);
     } else {
         size_t smem = (size_t)NCOL * P.s * sizeof(float2);
-        FDE_CUDA_TRY(cudaFuncSetAttribute(time_fft_inv_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          227 * 1024));
+        FDE_TRY(allow_smem((const void*)time_fft_inv_kernel<float>, 227 * 1024));
         time_fft_inv_kernel<float><<<grid, 256, smem, st>>>(P.m, P.mp, P.logs, (const float2*)xhat, P.d_tws32, z);
     }
     FDE_LAUNCH_CHECK("time_fft_inv_kernel");

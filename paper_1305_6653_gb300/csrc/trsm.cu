@@ -416,7 +416,7 @@ int launch_trsm_tc(const InstDev* I, const int* act, int nact, const void* fac, 
     CUtensorMap map;
     int rc = factor_tensor_map_sw128(fac, mp, nblk, &map);
     if (rc) return rc;
-    FDE_CUDA_TRY(cudaFuncSetAttribute(block_trsm_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, TRSM_SMEM));
+    FDE_TRY(allow_smem((const void*)block_trsm_tc_kernel, TRSM_SMEM));
     block_trsm_tc_kernel<<<dim3((nact + TRSM_R - 1) / TRSM_R, nblk), TRSM_THREADS, TRSM_SMEM, st>>>(
         I, act, nact, mp, nblk, (const unsigned char*)dtile, err, map);
     FDE_LAUNCH_CHECK("block_trsm_tc_kernel");
