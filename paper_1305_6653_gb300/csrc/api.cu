@@ -611,8 +611,8 @@ int fde_problem_create(const fde_problem_desc* d, void* stream, fde_problem** ou
         part(&P.d_twq, (size_t)P.L + P.L / 2);
         part(&P.d_kap, (size_t)P.L);
         part(&P.d_sym32, (size_t)P.L);
-        part(&P.d_tws, (size_t)P.s / 2);
-        part(&P.d_tws32, (size_t)P.s / 2);
+        part(&P.d_tws, (size_t)P.s);
+        part(&P.d_tws32, (size_t)P.s);
         part(&P.d_phi, (size_t)P.nblk);
         part(&P.d_psi, (size_t)P.nblk);
         part(&P.d_b_rhs, (size_t)P.n);

@@ -146,6 +146,10 @@ int launch_block_lu(Problem& P, int prec, cudaStream_t st);
 // The FP32 inverses of the 32 x 32 diagonal tiles of P's factors (P.d_tinv).
 int launch_tile_inverse_fp32(Problem& P, cudaStream_t st);
 int launch_block_trsv(const Problem& P, void* rhat, cudaStream_t st);
+// lu64.cu: the FP64 blocks (formed on st before): LU, tile inverses, block solves
+int launch_lu64(Problem& P, cudaStream_t st);
+int launch_tile_inverse64(const Problem& P, cudaStream_t st);
+int launch_trsv64(const Problem& P, void* rhat, cudaStream_t st);
 
 // krylov.cu
 int launch_update(const double* V, int k, const double* coef, double sign, double* w, long n, cudaStream_t st);
@@ -221,7 +225,7 @@ struct Problem {
     bfp::Tw* d_twq = nullptr;
     bfp::Q61* d_kap = nullptr;
     float2* d_sym32 = nullptr;  // L: (lambda + i conj(lambda)) / L, lambda = FFT of the circulant embedding of G
-    double2* d_tws = nullptr;   // s/2 twiddles exp(-2 pi i k / s)
+    double2* d_tws = nullptr;   // s twiddles exp(-2 pi i k / s)
     float2* d_tws32 = nullptr;
     double2* d_phi = nullptr;   // s/2+1
     double2* d_psi = nullptr;

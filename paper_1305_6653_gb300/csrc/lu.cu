@@ -7,7 +7,7 @@
 //
 // Storage: planar complex, one m_p x m_p row-major plane for Re and one for Im per
 // block (m_p = m rounded up to 64; the padding is the identity), packed L\U in
-// place, plus 1/U_ii per row.  Precision T = double (plain method) or float.
+// place, plus 1/U_ii per row.  The FP64 blocks (plain method) are factored and solved in lu64.cu.
 //
 // Per panel step p (columns [p NB, (p+1) NB)):
 //   1. lu_diag:   factor the NB x NB diagonal block in shared memory (one CTA per block)
@@ -437,20 +437,11 @@ __global__ void __launch_bounds__(256) lu_update_batched(const BlkDev* __restric
 // previous phase has completed (the solver passes B of step d before it arrives on
 // X of step d+2; the streaming warps pass X of step d+2 before they arrive on B of
 // step d+2), so phases never mix.  All waits are hardware barriers of this CTA.
-struct dvec4 {
-    double x, y, z, w;
-};
 template <typename T> struct vec4;
 template <> struct vec4<float> { using type = float4; };
-template <> struct vec4<double> { using type = dvec4; };
 
 // Streaming loads (the factor planes are read once per solve).
 __device__ __forceinline__ float4 ld4(const float* p) { return __ldcs(reinterpret_cast<const float4*>(p)); }
-__device__ __forceinline__ dvec4 ld4(const double* p) {
-    const double2 a = __ldcs(reinterpret_cast<const double2*>(p));
-    const double2 b = __ldcs(reinterpret_cast<const double2*>(p) + 1);
-    return dvec4{a.x, a.y, b.x, b.y};
-}
 
 __device__ __forceinline__ void cp_async16(void* dst, const void* src) {
     const unsigned s = (unsigned)__cvta_generic_to_shared(dst);
@@ -471,9 +462,8 @@ __device__ __forceinline__ void named_arrive(int id, int n) {
 constexpr int TRSV_THREADS = 512;                           // the default launch shape
 constexpr int TRSV_TPR = 8;                                  // threads per row in the strip update
 constexpr int TRSV_BAR_X = 1, TRSV_BAR_B = 3;                // named barrier ids (+ d & 1)
-// Rows per group whose loads are in flight together: 8 x 2 x 16 B per thread for
-// FP32 factors; FP64 rows are twice as wide per element, 4 keep it spill-free.
-template <typename T> struct trsv_unroll { static constexpr int value = sizeof(T) == 4 ? 8 : 4; };
+// Rows per group whose loads are in flight together: 8 x 2 x 16 B per thread.
+template <typename T> struct trsv_unroll { static constexpr int value = 8; };
 // Launch shapes of the block solves (FDE_TUNE_TRSV): NT threads (warp 0 the solver,
 // NT/32 - 1 streaming warps of (NT - 32) / TRSV_TPR row groups) and H rows per
 // register buffer.  The arithmetic of every row does not depend on the shape: each
@@ -879,12 +869,12 @@ template <typename T> struct ring_cfg {
     static constexpr int NT = 512;
     static constexpr int R = (NT - 64) / TRSV_TPR;        // 56 rows per stage
     static constexpr int ROWB = 2 * 32 * (int)sizeof(T);  // bytes per stage row (Re | Im)
-    static constexpr int S = sizeof(T) == 4 ? 10 : 4;     // stages
+    static constexpr int S = 10;                          // stages
     static constexpr int CW = (NT - 64) / 32;             // consumer warps
 };
 
 static size_t trsv_ring_smem_bytes(int mp, size_t elem) {
-    const size_t s = elem == 4 ? ring_cfg<float>::S : ring_cfg<double>::S;
+    const size_t s = ring_cfg<float>::S;
     const size_t rowb = 2 * 32 * elem;
     return trsv_smem_bytes(mp, elem) + 128 + s * ((size_t)(512 - 64) / TRSV_TPR) * rowb;  // + alignment slack
 }
@@ -1368,19 +1358,22 @@ block_trsv_multi_kernel(const InstDev* __restrict__ I, const int* __restrict__ a
 }
 
 template <typename T>
+static int form_blocks(Problem& P, cudaStream_t st) {
+    StageTimer t(P, FDE_STAGE_FORM);
+    form_blocks_kernel<T><<<dim3(P.mp < 64 ? P.mp : 64, P.nblk), 256, (size_t)(P.m + 2) * sizeof(T), st>>>(
+        P.m, P.mp, P.h, P.dxa, P.d_g, P.d_dplus, P.d_dminus, P.d_phi, P.d_psi, reinterpret_cast<T*>(P.d_fac));
+    FDE_LAUNCH_CHECK("form_blocks_kernel");
+    return FDE_OK;
+}
+
 static int run_lu(Problem& P, cudaStream_t st) {
-    using C = cplx_t<T>;
+    using T = float;
+    using C = float2;
     T* fac = reinterpret_cast<T*>(P.d_fac);
     C* dinv = reinterpret_cast<C*>(P.d_dinv);
     const int mp = P.mp, nb = P.nblk;
-    {
-        dim3 grid(mp < 64 ? mp : 64, nb);
-        StageTimer t(P, FDE_STAGE_FORM);
-        const size_t gsm = (size_t)(P.m + 2) * sizeof(T);
-        form_blocks_kernel<T><<<grid, 256, gsm, st>>>(P.m, mp, P.h, P.dxa, P.d_g, P.d_dplus, P.d_dminus, P.d_phi,
-                                                      P.d_psi, fac);
-        FDE_LAUNCH_CHECK("form_blocks_kernel");
-    }
+    int rc = form_blocks<T>(P, st);
+    if (rc) return rc;
     const size_t panel_smem = (size_t)RC * (NB + 1) * sizeof(C);
     FDE_TRY(allow_smem((const void*)lu_panel_kernel<T>, panel_smem));
     const size_t upd_smem = (64 * (NB + 1) + NB * 65) * sizeof(C);
@@ -2576,11 +2569,9 @@ static int launch_tile_inverse(Problem& P, int prec, cudaStream_t st) {
         P.tinv_bytes = bytes;
     }
     StageTimer t(P, FDE_STAGE_LU_DIAG);
+    if (prec == FDE_FP64) return launch_tile_inverse64(P, st);
     const dim3 grid(P.mp / 32, P.nblk);
-    if (prec == FDE_FP64)
-        tile_inverse_kernel<double><<<grid, 64, 0, st>>>(P.mp, (const double*)P.d_fac, (double*)P.d_tinv);
-    else
-        tile_inverse_kernel<float><<<grid, 64, 0, st>>>(P.mp, (const float*)P.d_fac, (float*)P.d_tinv);
+    tile_inverse_kernel<float><<<grid, 64, 0, st>>>(P.mp, (const float*)P.d_fac, (float*)P.d_tinv);
     FDE_LAUNCH_CHECK("tile_inverse_kernel");
     return FDE_OK;
 }
@@ -2591,11 +2582,11 @@ int launch_block_lu(Problem& P, int prec, cudaStream_t st) {
     int rc;
     const bool was_ok = P.strips_ok, was_bf16 = P.strips_bf16;
     P.strips_ok = false;  // set by the tensor-core LU once it has written the strip-major copy
-    if (prec == FDE_FP64) rc = run_lu<double>(P, st);
+    if (prec == FDE_FP64) rc = (rc = form_blocks<double>(P, st)) ? rc : launch_lu64(P, st);
     else if (prec == FDE_TF32) rc = run_lu_tc<0>(P, st);
     else if (prec == FDE_BF16) rc = run_lu_tc<1>(P, st);
     else if (prec == FDE_TF32X3) rc = run_lu_tc<2>(P, st);
-    else rc = run_lu<float>(P, st);
+    else rc = run_lu(P, st);
     // the captured block solves name the layout they read: a change of it retires them
     // (a factorisation that keeps the layout keeps the graphs)
     if (P.strips_ok != was_ok || (P.strips_ok && P.strips_bf16 != was_bf16)) ++P.graph_gen;
@@ -2607,8 +2598,8 @@ template <typename T, int V>
 static int launch_trsv_shape(const Problem& P, void* rhat, cudaStream_t st) {
     const size_t smem = trsv_smem_bytes(P.mp, sizeof(T));
     // the strip-major copy of the factor (FP32 or bfloat16), where the tensor-core LU wrote one
-    const bool strips = sizeof(T) == 4 && P.strips_ok && P.d_strips;
-    if constexpr (sizeof(T) == 4) {
+    const bool strips = P.strips_ok && P.d_strips;
+    {
         if (strips && P.strips_bf16) {
             auto kern = block_trsv_kernel<T, V, LAY_STRIPS_BF16>;
             FDE_TRY(allow_smem((const void*)kern, smem));
@@ -2620,7 +2611,7 @@ static int launch_trsv_shape(const Problem& P, void* rhat, cudaStream_t st) {
         }
     }
     {
-        constexpr int LS = sizeof(T) == 4 ? LAY_STRIPS : LAY_PLANES;  // FP64 factors have no copy
+        constexpr int LS = LAY_STRIPS;
         auto kern = strips ? block_trsv_kernel<T, V, LS> : block_trsv_kernel<T, V, LAY_PLANES>;
         FDE_TRY(allow_smem((const void*)kern, smem));
         kern<<<P.nblk, trsv_shape<T, V>::NT, smem, st>>>(P.mp, (const T*)(strips ? P.d_strips : P.d_fac),
@@ -2652,8 +2643,7 @@ static int trsv_tensor_map(const Problem& P, CUtensorMap* map) {
     const cuuint64_t strides[2] = {(cuuint64_t)P.mp * sizeof(T), (cuuint64_t)P.mp * P.mp * sizeof(T)};
     const cuuint32_t box[3] = {32, (cuuint32_t)ring_cfg<T>::R, 1};
     const cuuint32_t estr[3] = {1, 1, 1};
-    const CUresult r = encode(map, sizeof(T) == 4 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_FLOAT64,
-                              3, P.d_fac, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+    const CUresult r = encode(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, P.d_fac, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
                               CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) return set_error(FDE_ERR_CUDA, "cuTensorMapEncodeTiled failed for the factor planes");
@@ -2683,17 +2673,11 @@ static int trsv_key(const Problem& P) {
 }
 
 int launch_block_trsv_variant(const Problem& P, void* rhat, int variant, cudaStream_t st) {
+    if (P.precision == FDE_FP64) return launch_trsv64(P, rhat, st);
     // the ring has no form for the bfloat16 copy: there the register shape 0 stands in for it
     if (variant == 3 && trsv_key(P) == FDE_BF16) variant = 0;
-    if (variant == 3) {  // strips streamed through a shared-memory ring by bulk copies
-        if (P.precision == FDE_FP64) return launch_trsv_ring<double>(P, rhat, st);
-        return launch_trsv_ring<float>(P, rhat, st);
-    }
-    if (P.precision == FDE_FP64) {
-        if (variant == 1) return launch_trsv_shape<double, 1>(P, rhat, st);
-        if (variant == 2) return launch_trsv_shape<double, 2>(P, rhat, st);
-        return launch_trsv_shape<double, 0>(P, rhat, st);
-    }
+    // strips streamed through a shared-memory ring by bulk copies
+    if (variant == 3) return launch_trsv_ring<float>(P, rhat, st);
     if (variant == 1) return launch_trsv_shape<float, 1>(P, rhat, st);
     if (variant == 2) return launch_trsv_shape<float, 2>(P, rhat, st);
     return launch_trsv_shape<float, 0>(P, rhat, st);
@@ -2722,8 +2706,11 @@ int autotune_trsv(Problem& P) {
     bool need = false;
     tune_lookup(FDE_TUNE_TRSV, P.mp, P.nblk, prec, &need);
     if (!need) return FDE_OK;
-    const size_t esz = P.precision == FDE_FP64 ? sizeof(double) : sizeof(float);
-    FDE_CUDA_TRY(cudaMemsetAsync(P.d_rhat, 0, (size_t)P.nblk * P.mp * 2 * esz, P.stream));
+    if (prec == FDE_FP64) {  // one form for every variant: nothing to time
+        tune_store(FDE_TUNE_TRSV, P.mp, P.nblk, prec, 0, nullptr);
+        return FDE_OK;
+    }
+    FDE_CUDA_TRY(cudaMemsetAsync(P.d_rhat, 0, (size_t)P.nblk * P.mp * 2 * sizeof(float), P.stream));
     TrsvTuneCtx ctx{&P, P.d_rhat};
     int best = 0;
     float ms[TUNE_MAX_VARIANTS] = {};

@@ -40,7 +40,7 @@ __device__ __forceinline__ void grunwald_weights(double alpha, int count, double
 // Everything that depends on (alpha, m, s, scheme) alone, in one launch (seven small ones took
 // as long as the symbol transform that follows): CTA 0 the Grunwald weights, the others one
 // table entry a thread -- exp(-2 pi i k / L) in FP64 and FP32 for k < L, exp(-2 pi i k / s) for
-// k < s/2, the block floating-point twiddles (k < L, then the first L/2 in bit-reversed
+// k < s, the block floating-point twiddles (k < L, then the first L/2 in bit-reversed
 // order), and the Strang symbols
 //   phi_k = sum_{r=-nu}^{mu-nu} a_{r+nu} exp(2 pi i r k / s), psi_k likewise with b, k = 0..s/2.
 struct TableArgs {
@@ -71,14 +71,14 @@ __global__ void __launch_bounds__(256) tables_kernel(const __grid_constant__ Tab
         return;
     }
     k -= L;
-    if (k < s / 2) {
+    if (k < s) {
         double sn, cs;
         sincospi(-2.0 * (double)k / (double)s, &sn, &cs);
         A.tws[k] = make_double2(cs, sn);
         A.tws32[k] = make_float2((float)cs, (float)sn);
         return;
     }
-    k -= s / 2;
+    k -= s;
     if (k < L + L / 2) {
         A.twq[k] = bfp::twiddle(k < L ? k : bitrev(k - L, A.logL - 1), A.logL);
         return;
@@ -183,7 +183,7 @@ int launch_tables(const Problem& P, cudaStream_t st) {
         A.a[i] = P.h_a_main[i];
         A.b[i] = P.h_b_main[i];
     }
-    const int items = P.L + P.s / 2 + P.L + P.L / 2 + P.s / 2 + 1;
+    const int items = P.L + P.s + P.L + P.L / 2 + P.s / 2 + 1;
     tables_kernel<<<1 + (items + 255) / 256, 256, 0, st>>>(A);
     FDE_LAUNCH_CHECK("tables_kernel");
     return FDE_OK;
