@@ -427,11 +427,9 @@ long long fde_launch_count(void);
  * Two kernel families have variants that compute bit-identical results and differ
  * only in how the work is spread over threads: the space-time matvec (threads per
  * time row: 1024, 512, 256, i.e. one, two or more CTAs per SM) and the block
- * triangular solves (512 threads with 4 rows per register buffer, 384 with 8, 640
- * with 2 -- reading a bfloat16 factor copy: 4, 7 and 3 -- or 512 threads fed by bulk
- * asynchronous copies through a ring of shared-memory stages, which reads the FP32
- * factors; with a bfloat16 copy that fourth setting launches the first shape, and the
- * tuner times the three register shapes; FP64 factors have one form, which every setting
+ * triangular solves (FP32 factors: 7, 14, 12 or 10 warps that apply strips streamed by tensor-map
+ * copies; a bfloat16 copy: 512 threads with 4 rows per register buffer, 384 with 7 or 640 with
+ * 3, a fourth setting launches the first; FP64 factors have one form, which every setting
  * launches).  By default the first use of a shape (the matvec in bvm_assemble, the
  * block solves at the end of strang_precond_factor) times every variant with CUDA
  * events on the problem's stream and keeps the fastest for that shape (m_p, s or
@@ -451,7 +449,7 @@ long long fde_launch_count(void);
 #define FDE_TUNE_KERNELS 3
 /* variant -1: autotune (the default); 0 .. n-1: always launch that variant.
  * Before a shape is measured the built-in default runs (block solves with FP32
- * factors: 1, the 384 x 8 shape; with the bfloat16 copy: 0, 512 threads; LU interior
+ * factors: 1, 14 warps; with the bfloat16 copy: 0, 512 threads; LU interior
  * update: 2; otherwise 0); measuring keeps the default unless
  * another variant is faster by more than 2 % (median of five interleaved rounds).
  * Process-wide.  Errors: FDE_ERR_ARG. */

@@ -410,13 +410,11 @@ int fde_batch_factor(fde_batch* b, int precision) {
             if (infos[i][k])
                 return set_error(FDE_ERR_SINGULAR, "zero or non-finite pivot in instance " + std::to_string(i) +
                                                        ", block " + std::to_string(k));
-    // the FP32 inverses of the diagonal tiles, through which the solves from a bfloat16 copy
-    // apply the diagonal tiles
+    // the FP32 inverses of the diagonal tiles, through which the solves apply them
     for (fde_problem* p : b->probs) {
         Problem& P = *problem_of(p);
-        if (!P.strips_bf16) continue;
         if ((rc = launch_tile_inverse_fp32(P, b->stream))) return rc;
-        P.strips_ok = true;
+        if (P.strips_bf16) P.strips_ok = true;
     }
     for (fde_problem* p : b->probs) problem_of(p)->factored = true;
     b->precision = precision;
@@ -451,15 +449,11 @@ int fde_batch_solve(fde_batch* b, const fde_pgmres_opts* opts, double* const* x_
         if (b->shared) {  // the factors of instance 0, frequency vectors of its own
             const Problem& P0 = *problem_of(b->probs[0]);
             d.fac = P0.d_fac;
-            d.dinv = P0.d_dinv;
             d.tinv = P0.d_tinv;
             d.rhat = (unsigned char*)b->d_rhat_shared + (size_t)i * P0.nblk * P0.mp * 2 * sizeof(float);
         } else {
-            d.rhat = P.d_rhat; d.fac = P.d_fac; d.dinv = P.d_dinv; d.tinv = nullptr;
-            if (P.strips_ok && P.strips_bf16 && P.d_strips) {  // the bfloat16 copy and the tile inverses
-                d.strips = P.d_strips;
-                d.tinv = P.d_tinv;
-            }
+            d.rhat = P.d_rhat; d.fac = P.d_fac; d.tinv = P.d_tinv;
+            if (P.strips_ok && P.strips_bf16 && P.d_strips) d.strips = P.d_strips;  // the bfloat16 copy
         }
         // host solution arrays (the instance's desc->device_ptrs == 0): solve into the
         // instance's device copy, copied out when the batch is done

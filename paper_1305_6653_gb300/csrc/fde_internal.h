@@ -75,8 +75,7 @@ struct InstDev {
     const double2* tws;
     void* rhat;
     void* fac;
-    void* dinv;
-    void* tinv;            // inverted 32 x 32 diagonal tiles of the factors, or NULL
+    void* tinv;            // inverted 32 x 32 diagonal tiles of the factors
     const void* strips;    // bfloat16 strip-major copy of the factors (with tinv), or NULL
     double* b;
     double* x;
@@ -146,9 +145,8 @@ int launch_block_lu(Problem& P, int prec, cudaStream_t st);
 // The FP32 inverses of the 32 x 32 diagonal tiles of P's factors (P.d_tinv).
 int launch_tile_inverse_fp32(Problem& P, cudaStream_t st);
 int launch_block_trsv(const Problem& P, void* rhat, cudaStream_t st);
-// lu64.cu: the FP64 blocks (formed on st before): LU, tile inverses, block solves
+// lu64.cu: the FP64 blocks (formed on st before): LU, block solves
 int launch_lu64(Problem& P, cudaStream_t st);
-int launch_tile_inverse64(const Problem& P, cudaStream_t st);
 int launch_trsv64(const Problem& P, void* rhat, cudaStream_t st);
 
 // krylov.cu
@@ -372,7 +370,8 @@ int tune_default_variant(int kernel, int prec);
 constexpr int TUNE_MAX_VARIANTS = 8;
 // the tuned kernels' variant launchers (matvec.cu, lu.cu) and the tuning passes
 int launch_matvec64_variant(const Problem& P, const double* z, double* y, int variant, cudaStream_t st);
-int launch_block_trsv_variant(const Problem& P, void* rhat, int variant, cudaStream_t st);
+// lu.cu: the block solves from the bfloat16 copy of the factors
+int launch_trsv_bf16(const Problem& P, void* rhat, int variant, cudaStream_t st);
 int autotune_matvec(Problem& P);
 int autotune_trsv(Problem& P);
 

@@ -22,6 +22,7 @@
 #include "fde_internal.h"
 #include "fft_device.cuh"
 #include "lu_tc2.cuh"
+#include "trsv.cuh"
 #include "lu_tc2w.cuh"
 #include "lu_tc2s.cuh"
 
@@ -415,8 +416,9 @@ __global__ void __launch_bounds__(256) lu_update_batched(const BlkDev* __restric
     update_body<T>(d.mp, p * NB, (p + 1) * NB + ti * 64, (p + 1) * NB + tj * 64, d.mp, d.mp, (T*)d.fac);
 }
 
-// Forward (unit lower L) then backward (U) substitution for one block per CTA, in
-// place on rhat[k] (length mp), column-oriented over 32-row tiles.  Step d of a
+// Block solves of batched instances, and of one problem from its bfloat16 copy (its FP32 and FP64
+// factors: trsv.cu, lu64.cu): forward (unit lower L) then backward (U) substitution for one block
+// per CTA, in place on rhat[k] (length mp), column-oriented over 32-row tiles.  Step d of a
 // sweep resolves tile T(d) (T(d) = d forward, nt-1-d backward) and subtracts the
 // 32-column strip of L (U) below (above) it, times the 32 new values, from the
 // remaining right-hand side.
@@ -437,131 +439,43 @@ __global__ void __launch_bounds__(256) lu_update_batched(const BlkDev* __restric
 // previous phase has completed (the solver passes B of step d before it arrives on
 // X of step d+2; the streaming warps pass X of step d+2 before they arrive on B of
 // step d+2), so phases never mix.  All waits are hardware barriers of this CTA.
-template <typename T> struct vec4;
-template <> struct vec4<float> { using type = float4; };
-
-// Streaming loads (the factor planes are read once per solve).
-__device__ __forceinline__ float4 ld4(const float* p) { return __ldcs(reinterpret_cast<const float4*>(p)); }
-
-__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
-    const unsigned s = (unsigned)__cvta_generic_to_shared(dst);
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(s), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async4(void* dst, const void* src) {
-    const uint32_t s = (uint32_t)__cvta_generic_to_shared(dst);
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(s), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait1() { asm volatile("cp.async.wait_group 1;" ::: "memory"); }
-__device__ __forceinline__ void named_sync(int id, int n) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory"); }
-__device__ __forceinline__ void named_arrive(int id, int n) {
-    asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(n) : "memory");
-}
-
 constexpr int TRSV_THREADS = 512;                           // the default launch shape
 constexpr int TRSV_TPR = 8;                                  // threads per row in the strip update
 constexpr int TRSV_BAR_X = 1, TRSV_BAR_B = 3;                // named barrier ids (+ d & 1)
-// Rows per group whose loads are in flight together: 8 x 2 x 16 B per thread.
+constexpr int TRSV_BAR_SOLVER = 6;                           // among the solver threads (groups of four)
+// Rows per group whose loads are in flight together.
 template <typename T> struct trsv_unroll { static constexpr int value = 8; };
-// Launch shapes of the block solves (FDE_TUNE_TRSV): NT threads (warp 0 the solver,
-// NT/32 - 1 streaming warps of (NT - 32) / TRSV_TPR row groups) and H rows per
-// register buffer.  The arithmetic of every row does not depend on the shape: each
-// row's strip product is the same 32-term sum, reduced by the same TRSV_TPR lanes in
-// the same order, so all shapes give bit-identical results.
-template <typename T, int V> struct trsv_shape;
-template <typename T> struct trsv_shape<T, 0> { static constexpr int NT = 512, H = trsv_unroll<T>::value / 2; };
-template <typename T> struct trsv_shape<T, 1> { static constexpr int NT = 384, H = trsv_unroll<T>::value; };
-template <typename T> struct trsv_shape<T, 2> { static constexpr int NT = 640, H = trsv_unroll<T>::value / 4; };
-// Solver tiles in shared memory: planar, rows padded by 16 bytes (16-byte aligned
-// cp.async destinations); [buffer 2][D, L][Re, Im][32][LD].
-template <typename T> struct trsv_tile { static constexpr int LD = 32 + 16 / (int)sizeof(T); };
+template <typename T> struct trsv_tile { static constexpr int LD = TRSV_LD; };
+// Launch shapes of the block solves from the bfloat16 copy (FDE_TUNE_TRSV): NT threads (warp 0 the
+// solver, NT/32 - 1 streaming warps) and H rows per register buffer.  The arithmetic of every row
+// does not depend on the shape, so all shapes give bit-identical results.
+template <int V> struct trsv_shape;
+template <> struct trsv_shape<0> { static constexpr int NT = 512, H = 4; };
+template <> struct trsv_shape<1> { static constexpr int NT = 384, H = 7; };
+template <> struct trsv_shape<2> { static constexpr int NT = 640, H = 3; };
 
-__host__ __device__ static size_t trsv_smem_bytes(int mp, size_t elem) {
-    const size_t ld = 32 + 16 / elem;
-    return (size_t)mp * 2 * elem + 8 * 32 * ld * elem;
-}
+static size_t trsv_smem_bytes(int mp, size_t elem) { return (size_t)mp * 2 * elem + 8 * 32 * TRSV_LD * elem; }
 
-// 32 x 32 tile with row pitch `pitch` (elements) -> shared tile with pitch LD.
-template <typename T>
-__device__ __forceinline__ void tile_async(T* dst, const T* src, size_t pitch, int lane) {
-    constexpr int EPC = 16 / (int)sizeof(T), CPR = 32 / EPC, LD = trsv_tile<T>::LD;
-    for (int e = lane; e < 32 * CPR; e += 32) {
-        const int r = e / CPR, ch = e % CPR;
-        cp_async16(dst + r * LD + ch * EPC, src + (size_t)r * pitch + ch * EPC);
-    }
-}
-template <typename T>
-__device__ __forceinline__ void tile_async(T* dst, const T* plane, int mp, int r0, int c0, int lane) {
-    tile_async<T>(dst, plane + (size_t)r0 * mp + c0, (size_t)mp, lane);
-}
-
-// Factor planes as the block solves read them (LAY): 0 row-major in the compute type
-// (element (r, c) at r m_p + c); 1 strip-major in the compute type (32-column strips
-// one after the other, each strip's rows contiguous: (c / 32) 32 m_p + 32 r + c mod 32),
-// so every strip of a sweep is one sequential stream; 2 strip-major in bfloat16 (FP32
-// compute).  The tensor-core LU writes the final factor row-major and, where it can,
-// in one of the strip-major forms as well.
-constexpr int LAY_PLANES = 0, LAY_STRIPS = 1, LAY_STRIPS_BF16 = 2;
-template <int LAY>
-__device__ __forceinline__ size_t fac_at(int mp, int r, int c) {
-    return LAY != LAY_PLANES ? (size_t)(c >> 5) * 32 * mp + (size_t)r * 32 + (c & 31) : (size_t)r * mp + c;
-}
 template <typename T, int LAY>
 __device__ __forceinline__ void tile_async_l(T* dst, const T* plane, int mp, int r0, int c0, int lane) {
     tile_async<T>(dst, plane + fac_at<LAY>(mp, r0, c0), LAY != LAY_PLANES ? (size_t)32 : (size_t)mp, lane);
 }
-// Element type of the factor as stored for layout LAY, and its streaming loads: four
-// consecutive entries of one row, widened to the compute type (a bfloat16 is the top
-// half of the float it came from, so the widening is exact).
-template <typename T, int LAY> struct fac_store {
-    using elem = T;
-    using raw = typename vec4<T>::type;
-    static __device__ __forceinline__ raw load(const elem* p) { return ld4(p); }
-    static __device__ __forceinline__ raw widen(const raw& v) { return v; }
-};
-template <> struct fac_store<float, LAY_STRIPS_BF16> {
-    using elem = unsigned short;
-    using raw = uint2;
-    static __device__ __forceinline__ raw load(const elem* p) { return __ldcs(reinterpret_cast<const uint2*>(p)); }
-    static __device__ __forceinline__ float4 widen(const raw& v) {
-        return make_float4(__uint_as_float(v.x << 16), __uint_as_float(v.x & 0xffff0000u),
-                           __uint_as_float(v.y << 16), __uint_as_float(v.y & 0xffff0000u));
-    }
-};
-// 32 x 32 bfloat16 tile of a strip (rows of 64 bytes, contiguous) -> shared rows of
-// TRSV_LDH elements (80 bytes: 16-byte aligned cp.async destinations).
-constexpr int TRSV_LDH = 40;
-__device__ __forceinline__ void tile_async_bf16(unsigned short* dst, const unsigned short* src, int lane) {
-    for (int e = lane; e < 32 * 4; e += 32) {
-        const int r = e >> 2, ch = e & 3;
-        cp_async16(dst + r * TRSV_LDH + ch * 8, src + r * 32 + ch * 8);
-    }
-}
 
-// Solver side of one sweep (warp 0).  INV: the inverted diagonal tiles are given
-// (tinv: per tile [L^-1 re, L^-1 im, U^-1 re, U^-1 im][32][32]) and a tile solve is
-// the product x = D^-1 a; otherwise the tile is solved by substitution.
-template <typename T, bool FWD, bool INV, int NT, int LAY = LAY_PLANES>
+// Solver side of one sweep (warp 0): a tile solve is the product x = D^-1 a with the inverted
+// diagonal tile (tinv: per tile [L^-1 re, L^-1 im, U^-1 re, U^-1 im][32][32]).
+template <typename T, bool FWD, int NT, int LAY = LAY_PLANES>
 __device__ __forceinline__ void trsv_solver(int mp, int nt, const typename fac_store<T, LAY>::elem* re,
-                                            const typename fac_store<T, LAY>::elem* im, const cplx_t<T>* dv,
-                                            const T* tinv, cplx_t<T>* y, cplx_t<T> (*xs)[32], T* tiles,
+                                            const typename fac_store<T, LAY>::elem* im, const T* tinv, cplx_t<T>* y, cplx_t<T> (*xs)[32], T* tiles,
                                             cplx_t<T>* av, int lane) {
     using C = cplx_t<T>;
-    static_assert(INV || LAY != LAY_STRIPS_BF16, "substitution reads the diagonal tiles in the compute type");
     constexpr int LD = trsv_tile<T>::LD, TS = 32 * LD;
     auto tile_of = [&](int d) { return FWD ? d : nt - 1 - d; };
     auto issue = [&](int d) {
         T* b = tiles + (d & 1) * 4 * TS;  // [D re, D im, L re, L im]
         const int j = tile_of(d);
-        if (INV) {
-            const T* ti = tinv + (size_t)j * 4096 + (FWD ? 0 : 2048);
-            tile_async<T>(b, ti, 32, lane);
-            tile_async<T>(b + TS, ti + 1024, 32, lane);
-        } else if constexpr (LAY != LAY_STRIPS_BF16) {
-            tile_async_l<T, LAY>(b, re, mp, 32 * j, 32 * j, lane);
-            tile_async_l<T, LAY>(b + TS, im, mp, 32 * j, 32 * j, lane);
-        }
+        const T* ti = tinv + (size_t)j * 4096 + (FWD ? 0 : 2048);
+        tile_async<T>(b, ti, 32, lane);
+        tile_async<T>(b + TS, ti + 1024, 32, lane);
         if (d >= 1) {
             if constexpr (LAY == LAY_STRIPS_BF16) {  // bfloat16 rows in the L slots
                 const size_t o = fac_at<LAY>(mp, 32 * j, 32 * tile_of(d - 1));
@@ -618,7 +532,7 @@ __device__ __forceinline__ void trsv_solver(int mp, int nt, const typename fac_s
             a.x -= sx0 + sx1;
             a.y -= sy0 + sy1;
         }
-        if (INV) {  // x = D^-1 a (D^-1 stored with its zeros and unit / inverted diagonal)
+        {  // x = D^-1 a (D^-1 stored with its zeros and unit / inverted diagonal)
             av[lane] = a;
             __syncwarp();
             T sx0 = 0, sy0 = 0, sx1 = 0, sy1 = 0;
@@ -634,30 +548,6 @@ __device__ __forceinline__ void trsv_solver(int mp, int nt, const typename fac_s
             }
             a.x = sx0 + sx1;
             a.y = sy0 + sy1;
-        } else if (FWD) {
-#pragma unroll 8
-            for (int c = 0; c < 32; ++c) {
-                const T yx = __shfl_sync(0xffffffffu, a.x, c);
-                const T yy = __shfl_sync(0xffffffffu, a.y, c);
-                if (lane > c) {
-                    const T lr = Dre[lane * LD + c], li = Dim[lane * LD + c];
-                    a.x = fma(li, yy, fma(-lr, yx, a.x));
-                    a.y = fma(-li, yx, fma(-lr, yy, a.y));
-                }
-            }
-        } else {
-            const C di = dv[r0 + lane];
-#pragma unroll 8
-            for (int c = 31; c >= 0; --c) {
-                if (lane == c) a = cmul(a, di);
-                const T yx = __shfl_sync(0xffffffffu, a.x, c);
-                const T yy = __shfl_sync(0xffffffffu, a.y, c);
-                if (lane < c) {
-                    const T ur = Dre[lane * LD + c], ui = Dim[lane * LD + c];
-                    a.x = fma(ui, yy, fma(-ur, yx, a.x));
-                    a.y = fma(-ui, yx, fma(-ur, yy, a.y));
-                }
-            }
         }
         y[r0 + lane] = a;
         xs[d & 1][lane] = a;
@@ -767,12 +657,6 @@ __device__ __forceinline__ void trsv_stream(int mp, int nt, const typename fac_s
 // and shuffles stay warp-uniform.  Otherwise as trsv_stream; every launch shape sums a
 // row's products in the same order, so the shapes agree bit for bit.
 constexpr int TRSV_TPR_H = 4;  // threads per row of the bfloat16 stream
-__device__ __forceinline__ void widen8(const uint4& v, float* f) {
-    f[0] = __uint_as_float(v.x << 16); f[1] = __uint_as_float(v.x & 0xffff0000u);
-    f[2] = __uint_as_float(v.y << 16); f[3] = __uint_as_float(v.y & 0xffff0000u);
-    f[4] = __uint_as_float(v.z << 16); f[5] = __uint_as_float(v.z & 0xffff0000u);
-    f[6] = __uint_as_float(v.w << 16); f[7] = __uint_as_float(v.w & 0xffff0000u);
-}
 template <bool FWD, int NT, int H>
 __device__ __forceinline__ void trsv_stream_bf16(int mp, int nt, const unsigned short* re, const unsigned short* im,
                                                  float2* y, const float2 (*xs)[32], int bt) {
@@ -849,196 +733,8 @@ __device__ __forceinline__ void trsv_stream_bf16(int mp, int nt, const unsigned 
     }
 }
 
-// ---------------------------------------------------------------------------
-// Block solves with the strips streamed by the copy engine.  Same roles and
-// hand-over as trsv_body, but warp 1 is a producer that loads every strip (32
-// columns of the Re and Im planes, R rows per stage, in sweep order) into a ring of
-// shared-memory stages with tensor-map copies (cp.async.bulk.tensor, completion
-// counted on a full[] mbarrier), running ahead of the consumers through both sweeps
-// (the factors do not depend on the solution); warps 2.. consume one stage row per
-// group of TRSV_TPR lanes with the same fused multiply-adds and the same shuffle
-// reduction as trsv_stream, so the result is bit-identical.  A stage holds
-// RING_R = (NT - 64) / TRSV_TPR rows (>= 32: the first stage of a strip covers tile
-// d+2).  The producer takes no part in the named barriers; every mbarrier wait is
-// bounded (on timeout the kernel records an error and carries on, so no thread is
-// left waiting at a barrier).
-// ---------------------------------------------------------------------------
-constexpr int TRSV_BAR_SWEEP = 5;  // solver + consumers between the two sweeps
-
-template <typename T> struct ring_cfg {
-    static constexpr int NT = 512;
-    static constexpr int R = (NT - 64) / TRSV_TPR;        // 56 rows per stage
-    static constexpr int ROWB = 2 * 32 * (int)sizeof(T);  // bytes per stage row (Re | Im)
-    static constexpr int S = 10;                          // stages
-    static constexpr int CW = (NT - 64) / 32;             // consumer warps
-};
-
-static size_t trsv_ring_smem_bytes(int mp, size_t elem) {
-    const size_t s = ring_cfg<float>::S;
-    const size_t rowb = 2 * 32 * elem;
-    return trsv_smem_bytes(mp, elem) + 128 + s * ((size_t)(512 - 64) / TRSV_TPR) * rowb;  // + alignment slack
-}
-
-template <typename T>
-__device__ __forceinline__ void ring_wait(uint64_t* bar, uint32_t parity, int* err) {
-    if (!tc::mbar_wait(bar, parity)) atomicCAS(err, 0, 3);  // recorded; carry on (no hang)
-}
-
-// Producer (lane 0 of warp 1): every stage of both sweeps, in the order the consumers
-// take them.  A stage is two tensor-map (TMA) boxes of R rows x 32 columns, one per
-// plane, landing as [Re rows][Im rows]; forward sweeps load rows lo+q0 .. upward,
-// backward sweeps the R rows that end at hi-q0 (the last boxes of a sweep may start
-// below row 0 or end past m_p: those rows are filled with zeros and never read).
-__device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* map, int x, int y, int z, uint64_t* bar) {
-    asm volatile(
-        "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], "
-        "[%5];" ::"r"(tc::smem_u32(dst)),
-        "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(z), "r"(tc::smem_u32(bar))
-        : "memory");
-}
-
-template <typename T>
-__device__ __forceinline__ void trsv_ring_producer(int mp, int nt, int k, const CUtensorMap* map, unsigned char* ring,
-                                                   uint64_t* full, uint64_t* empty, int* err) {
-    using Cf = ring_cfg<T>;
-    long g = 0;
-    for (int sweep = 0; sweep < 2; ++sweep) {
-        const bool fwd = sweep == 0;
-        for (int d = 0; d + 2 < nt; ++d) {
-            const int col = 32 * (fwd ? d : nt - 1 - d);
-            const int lo = fwd ? 32 * (d + 2) : 0;
-            const int hi = fwd ? mp : 32 * (nt - 2 - d);
-            const int len = hi - lo;
-            for (int q0 = 0; q0 < len; q0 += Cf::R, ++g) {
-                const int s = (int)(g % Cf::S);
-                if (g >= Cf::S) ring_wait<T>(&empty[s], (uint32_t)((g / Cf::S - 1) & 1), err);
-                unsigned char* st = ring + (size_t)s * Cf::R * Cf::ROWB;
-                const int y0 = fwd ? lo + q0 : hi - q0 - Cf::R;
-                tc::mbar_arrive_expect_tx(&full[s], (uint32_t)(Cf::R * Cf::ROWB));
-                tma_load_3d(st, map, col, y0, 2 * k, &full[s]);
-                tma_load_3d(st + Cf::R * Cf::ROWB / 2, map, col, y0, 2 * k + 1, &full[s]);
-            }
-        }
-    }
-}
-
-// Consumers (warps 2..): strip d of one sweep from the ring, stage by stage; g is the
-// running stage count shared with the producer's enumeration.
-template <typename T, bool FWD>
-__device__ __forceinline__ void trsv_ring_stream(int mp, int nt, cplx_t<T>* y, const cplx_t<T> (*xs)[32],
-                                                 const unsigned char* ring, uint64_t* full, uint64_t* empty,
-                                                 int* err, int bt, long& g) {
-    using C = cplx_t<T>;
-    using V = typename vec4<T>::type;
-    using Cf = ring_cfg<T>;
-    const int grp = bt / TRSV_TPR, sub = bt % TRSV_TPR, lane = bt & 31;
-    for (int d = 0; d + 2 < nt; ++d) {
-        const int lo = FWD ? 32 * (d + 2) : 0;
-        const int hi = FWD ? mp : 32 * (nt - 2 - d);
-        const int len = hi - lo;
-        named_sync(TRSV_BAR_X + (d & 1), Cf::NT - 32);
-        const C x0 = xs[d & 1][sub * 4], x1 = xs[d & 1][sub * 4 + 1];
-        const C x2 = xs[d & 1][sub * 4 + 2], x3 = xs[d & 1][sub * 4 + 3];
-        for (int q0 = 0; q0 < len; q0 += Cf::R, ++g) {
-            const int s = (int)(g % Cf::S);
-            ring_wait<T>(&full[s], (uint32_t)((g / Cf::S) & 1), err);
-            const int q = q0 + grp;
-            if (q < len) {  // uniform across a warp: an aligned quartet of groups, len a multiple of 32
-                const int br = FWD ? grp : Cf::R - 1 - grp;  // row within the stage's boxes
-                const T* pre = reinterpret_cast<const T*>(ring + (size_t)s * Cf::R * Cf::ROWB) + br * 32;
-                const T* pim = pre + Cf::R * 32;
-                const V vr = *reinterpret_cast<const V*>(pre + sub * 4);
-                const V vi = *reinterpret_cast<const V*>(pim + sub * 4);
-                T sx = vr.x * x0.x;
-                sx = fma(-vi.x, x0.y, sx);
-                sx = fma(vr.y, x1.x, sx);
-                sx = fma(-vi.y, x1.y, sx);
-                sx = fma(vr.z, x2.x, sx);
-                sx = fma(-vi.z, x2.y, sx);
-                sx = fma(vr.w, x3.x, sx);
-                sx = fma(-vi.w, x3.y, sx);
-                T sy = vr.x * x0.y;
-                sy = fma(vi.x, x0.x, sy);
-                sy = fma(vr.y, x1.y, sy);
-                sy = fma(vi.y, x1.x, sy);
-                sy = fma(vr.z, x2.y, sy);
-                sy = fma(vi.z, x2.x, sy);
-                sy = fma(vr.w, x3.y, sy);
-                sy = fma(vi.w, x3.x, sy);
-#pragma unroll
-                for (int off = 1; off < TRSV_TPR; off <<= 1) {
-                    sx += __shfl_xor_sync(0xffffffffu, sx, off);
-                    sy += __shfl_xor_sync(0xffffffffu, sy, off);
-                }
-                if (sub == 0) {
-                    const int r = FWD ? lo + q : hi - 1 - q;
-                    C v = y[r];
-                    v.x -= sx;
-                    v.y -= sy;
-                    y[r] = v;
-                }
-            }
-            __syncwarp();
-            if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tc::smem_u32(&empty[s]))
-                                        : "memory");
-            if (q0 == 0) named_arrive(TRSV_BAR_B + (d & 1), Cf::NT - 32);  // stage 0 covers tile d+2
-        }
-    }
-}
-
-template <typename T>
-__global__ void __launch_bounds__(512)
-block_trsv_ring_kernel(int mp, const T* __restrict__ fac, const cplx_t<T>* __restrict__ dinv,
-                       const T* __restrict__ tinv, cplx_t<T>* __restrict__ rhat, int* __restrict__ err,
-                       const __grid_constant__ CUtensorMap fmap, const int* __restrict__ live) {
-    if (live && !*live) return;
-    using C = cplx_t<T>;
-    using Cf = ring_cfg<T>;
-    extern __shared__ __align__(128) unsigned char smem_raw[];
-    const int k = blockIdx.x;
-    const T* re = fac + (size_t)k * 2 * mp * mp;
-    const T* im = re + (size_t)mp * mp;
-    const C* dv = dinv + (size_t)k * mp;
-    const T* ti = tinv + (size_t)k * (mp / 32) * 4096;
-    C* x = rhat + (size_t)k * mp;
-    C* y = reinterpret_cast<C*>(smem_raw);       // mp
-    T* tiles = reinterpret_cast<T*>(y + mp);     // solver tiles
-    // the ring starts at the next 128-byte boundary of the shared window (TMA destinations)
-    const uint32_t base = tc::smem_u32(smem_raw) + (uint32_t)trsv_smem_bytes(mp, sizeof(T));
-    unsigned char* ring = smem_raw + ((base + 127u) & ~127u) - tc::smem_u32(smem_raw);
-    __shared__ C xs[2][32];
-    __shared__ C av[32];
-    __shared__ __align__(8) uint64_t full[Cf::S], empty[Cf::S];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int nt = mp / 32;
-    if (threadIdx.x == 0) {
-        for (int s = 0; s < Cf::S; ++s) {
-            tc::mbar_init(&full[s], 1);
-            tc::mbar_init(&empty[s], Cf::CW);
-        }
-        tc::fence_barrier_init();
-    }
-    for (int i = threadIdx.x; i < mp; i += blockDim.x) y[i] = x[i];
-    __syncthreads();
-    if (warp == 1) {
-        if (lane == 0) trsv_ring_producer<T>(mp, nt, k, &fmap, ring, full, empty, err);
-    } else if (warp == 0) {
-        trsv_solver<T, true, true, Cf::NT - 32>(mp, nt, re, im, dv, ti, y, xs, tiles, av, lane);
-        named_sync(TRSV_BAR_SWEEP, Cf::NT - 32);
-        trsv_solver<T, false, true, Cf::NT - 32>(mp, nt, re, im, dv, ti, y, xs, tiles, av, lane);
-    } else {
-        long g = 0;
-        trsv_ring_stream<T, true>(mp, nt, y, xs, ring, full, empty, err, threadIdx.x - 64, g);
-        named_sync(TRSV_BAR_SWEEP, Cf::NT - 32);
-        trsv_ring_stream<T, false>(mp, nt, y, xs, ring, full, empty, err, threadIdx.x - 64, g);
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < mp; i += blockDim.x) x[i] = y[i];
-}
-
-template <typename T, bool INV, int NT = TRSV_THREADS, int H = trsv_unroll<T>::value / 2, int LAY = LAY_PLANES>
+template <typename T, int NT = TRSV_THREADS, int H = trsv_unroll<T>::value / 2, int LAY = LAY_PLANES>
 __device__ __forceinline__ void trsv_body(int mp, const typename fac_store<T, LAY>::elem* __restrict__ re,
-                                          const cplx_t<T>* __restrict__ dv,
                                           const T* __restrict__ tinv, cplx_t<T>* __restrict__ x) {
     using C = cplx_t<T>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1052,38 +748,30 @@ __device__ __forceinline__ void trsv_body(int mp, const typename fac_store<T, LA
     for (int i = threadIdx.x; i < mp; i += blockDim.x) y[i] = x[i];
     __syncthreads();
     if constexpr (LAY == LAY_STRIPS_BF16) {
-        if (warp == 0) trsv_solver<T, true, INV, NT, LAY>(mp, nt, re, im, dv, tinv, y, xs, tiles, av, lane);
+        if (warp == 0) trsv_solver<T, true, NT, LAY>(mp, nt, re, im, tinv, y, xs, tiles, av, lane);
         else trsv_stream_bf16<true, NT, H>(mp, nt, re, im, y, xs, threadIdx.x - 32);
         __syncthreads();
-        if (warp == 0) trsv_solver<T, false, INV, NT, LAY>(mp, nt, re, im, dv, tinv, y, xs, tiles, av, lane);
+        if (warp == 0) trsv_solver<T, false, NT, LAY>(mp, nt, re, im, tinv, y, xs, tiles, av, lane);
         else trsv_stream_bf16<false, NT, H>(mp, nt, re, im, y, xs, threadIdx.x - 32);
     } else {
-        if (warp == 0) trsv_solver<T, true, INV, NT, LAY>(mp, nt, re, im, dv, tinv, y, xs, tiles, av, lane);
+        if (warp == 0) trsv_solver<T, true, NT, LAY>(mp, nt, re, im, tinv, y, xs, tiles, av, lane);
         else trsv_stream<T, true, NT, H, LAY>(mp, nt, re, im, y, xs, threadIdx.x - 32);
         __syncthreads();
-        if (warp == 0) trsv_solver<T, false, INV, NT, LAY>(mp, nt, re, im, dv, tinv, y, xs, tiles, av, lane);
+        if (warp == 0) trsv_solver<T, false, NT, LAY>(mp, nt, re, im, tinv, y, xs, tiles, av, lane);
         else trsv_stream<T, false, NT, H, LAY>(mp, nt, re, im, y, xs, threadIdx.x - 32);
     }
     __syncthreads();
     for (int i = threadIdx.x; i < mp; i += blockDim.x) x[i] = y[i];
 }
 
-// (The bfloat16 stream loads 16 bytes per lane and plane like the FP32 one, so it keeps
-// the shape's rows per register buffer, at most 7: its eight x values per lane take the
-// registers of an eighth row; the 640-thread shape takes 3, which its registers allow.)
-template <typename T, int V = 0, int LAY = LAY_PLANES>
-__global__ void __launch_bounds__(trsv_shape<T, V>::NT)
-block_trsv_kernel(int mp, const typename fac_store<T, LAY>::elem* __restrict__ fac,
-                  const cplx_t<T>* __restrict__ dinv, const T* __restrict__ tinv, cplx_t<T>* __restrict__ rhat,
-                  const int* __restrict__ live) {
+template <int V>
+__global__ void __launch_bounds__(trsv_shape<V>::NT)
+block_trsv_bf16_kernel(int mp, const unsigned short* __restrict__ strips, const float* __restrict__ tinv,
+                       float2* __restrict__ rhat, const int* __restrict__ live) {
     if (live && !*live) return;
     const int k = blockIdx.x;
-    constexpr int HS = trsv_shape<T, V>::H;
-    constexpr int H = LAY != LAY_STRIPS_BF16 ? HS : HS > 7 ? 7 : HS == 2 ? 3 : HS;
-    trsv_body<T, true, trsv_shape<T, V>::NT, H, LAY>(mp, fac + (size_t)k * 2 * mp * mp,
-                                                                  dinv + (size_t)k * mp,
-                                                                  tinv + (size_t)k * (mp / 32) * 4096,
-                                                                  rhat + (size_t)k * mp);
+    trsv_body<float, trsv_shape<V>::NT, trsv_shape<V>::H, LAY_STRIPS_BF16>(
+        mp, strips + (size_t)k * 2 * mp * mp, tinv + (size_t)k * (mp / 32) * 4096, rhat + (size_t)k * mp);
 }
 
 // Batched over the active instances act[0..gridDim.x): block k = blockIdx.y of instance act[blockIdx.x].
@@ -1097,21 +785,13 @@ block_trsv_batched(const InstDev* __restrict__ I, const int* __restrict__ act) {
     const int k = blockIdx.y;
     if (k >= d.nblk || !d.ctl[0]) return;
     const size_t mp = d.mp;
-    const T* fac = (const T*)d.fac + (size_t)k * 2 * mp * mp;
-    const cplx_t<T>* dinv = (const cplx_t<T>*)d.dinv + (size_t)k * mp;
     cplx_t<T>* rhat = (cplx_t<T>*)d.rhat + (size_t)k * mp;
-    if constexpr (sizeof(T) == 4) {
-        if (d.strips) {  // the bfloat16 strip copy, diagonal tiles through their FP32 inverses
-            trsv_body<T, true, TRSV_THREADS, trsv_unroll<T>::value / 2, LAY_STRIPS_BF16>(
-                d.mp, (const unsigned short*)d.strips + (size_t)k * 2 * mp * mp, dinv,
-                (const T*)d.tinv + (size_t)k * (mp / 32) * 4096, rhat);
-            return;
-        }
-    }
-    if (d.tinv)  // diagonal tiles solved as products with their inverses
-        trsv_body<T, true>(d.mp, fac, dinv, (const T*)d.tinv + (size_t)k * (mp / 32) * 4096, rhat);
+    const T* tinv = (const T*)d.tinv + (size_t)k * (mp / 32) * 4096;
+    if (d.strips)  // the bfloat16 strip copy
+        trsv_body<T, TRSV_THREADS, trsv_unroll<T>::value / 2, LAY_STRIPS_BF16>(
+            d.mp, (const unsigned short*)d.strips + (size_t)k * 2 * mp * mp, tinv, rhat);
     else
-        trsv_body<T, false>(d.mp, fac, dinv, nullptr, rhat);
+        trsv_body<T>(d.mp, (const T*)d.fac + (size_t)k * 2 * mp * mp, tinv, rhat);
 }
 
 // ---------------------------------------------------------------------------
@@ -1255,8 +935,8 @@ __device__ __forceinline__ void trsv_multi_solver(int mp, int nt, const float* r
         tile_async<float>(b, ti, 32, lane);
         tile_async<float>(b + TS, ti + 1024, 32, lane);
         if (d >= 1) {
-            tile_async<float>(b + 2 * TS, re, mp, 32 * j, 32 * tile_of(d - 1), lane);
-            tile_async<float>(b + 3 * TS, im, mp, 32 * j, 32 * tile_of(d - 1), lane);
+            tile_async_l<float, LAY_PLANES>(b + 2 * TS, re, mp, 32 * j, 32 * tile_of(d - 1), lane);
+            tile_async_l<float, LAY_PLANES>(b + 3 * TS, im, mp, 32 * j, 32 * tile_of(d - 1), lane);
         }
     };
     issue(0);
@@ -1350,6 +1030,255 @@ block_trsv_multi_kernel(const InstDev* __restrict__ I, const int* __restrict__ a
     __syncthreads();
     for (int e = threadIdx.x; e < mp * TRSV_R; e += blockDim.x) {
         const int r = e / TRSV_R, j = e % TRSV_R, a = TRSV_R * blockIdx.x + j;
+        if (a < nact) {
+            const InstDev& d = I[act[a]];
+            if (d.ctl[0]) ((float2*)d.rhat)[(size_t)k * mp + r] = y[r][j];
+        }
+    }
+}
+
+// ---------------------------------------------------------------------------
+// The same in groups of R = 4, where groups of 8 would leave half the SMs idle: with 16 right-hand
+// sides and 33 blocks (m = 1023, s = 64) 66 CTAs of 8 were bound by their multiply-adds and by
+// the one solver warp.  Here four warps solve the diagonal tiles, a column each.  530 -> 331 us a
+// launch there, 90 -> 40 at m = 255, 309 -> 177 at m = 700, s = 32 with 5 right-hand sides.  With
+// more CTAs than SMs groups of 8 read the factors half as often (129 blocks, 16 right-hand sides).
+// ---------------------------------------------------------------------------
+constexpr int TRSV4_SW = 128;                    // solver threads
+constexpr int TRSV4_THREADS = TRSV4_SW + 352;    // 44 row groups
+
+__host__ __device__ static size_t trsv_multi4_smem_bytes(int mp) {
+    return (size_t)mp * 4 * sizeof(float2) + 8 * 32 * trsv_tile<float>::LD * sizeof(float);
+}
+
+// As multi_row_product for R columns, fewer than the lanes of a row: once one column is left, the
+// steps of the reduction just add; lane `sub` returns column sub R / 8's sum.
+template <int R>
+__device__ __forceinline__ float2 multi4_row_product(const float4& v, const float4& w, const float2 (&xr)[4][R],
+                                                    int sub) {
+    float pr[R], pi[R];
+#pragma unroll
+    for (int j = 0; j < R; ++j) {
+        const float2 x0 = xr[0][j], x1 = xr[1][j], x2 = xr[2][j], x3 = xr[3][j];
+        float a = v.x * x0.x;
+        a = fmaf(-w.x, x0.y, a);
+        a = fmaf(v.y, x1.x, a);
+        a = fmaf(-w.y, x1.y, a);
+        a = fmaf(v.z, x2.x, a);
+        a = fmaf(-w.z, x2.y, a);
+        a = fmaf(v.w, x3.x, a);
+        a = fmaf(-w.w, x3.y, a);
+        float b = v.x * x0.y;
+        b = fmaf(w.x, x0.x, b);
+        b = fmaf(v.y, x1.y, b);
+        b = fmaf(w.y, x1.x, b);
+        b = fmaf(v.z, x2.y, b);
+        b = fmaf(w.z, x2.x, b);
+        b = fmaf(v.w, x3.y, b);
+        b = fmaf(w.w, x3.x, b);
+        pr[j] = a;
+        pi[j] = b;
+    }
+    // lanes sub = 0..7 (xor 4, 2, 1): after the step with offset h a lane keeps the half of its
+    // columns selected by (sub & h)
+#pragma unroll
+    for (int h = 4, n = R; h >= 1; h >>= 1) {
+        if (n > 1) {
+            const bool upper = (sub & h) != 0;
+#pragma unroll
+            for (int j = 0; j < n / 2; ++j) {
+                const float sr = upper ? pr[j] : pr[j + n / 2], si = upper ? pi[j] : pi[j + n / 2];
+                const float rr = __shfl_xor_sync(0xffffffffu, sr, h), ri = __shfl_xor_sync(0xffffffffu, si, h);
+                const float kr = upper ? pr[j + n / 2] : pr[j], ki = upper ? pi[j + n / 2] : pi[j];
+                pr[j] = kr + rr;
+                pi[j] = ki + ri;
+            }
+            n >>= 1;
+        } else {
+            pr[0] += __shfl_xor_sync(0xffffffffu, pr[0], h);
+            pi[0] += __shfl_xor_sync(0xffffffffu, pi[0], h);
+        }
+    }
+    return make_float2(pr[0], pi[0]);
+}
+
+template <int R, bool FWD>
+__device__ __forceinline__ void trsv_multi4_stream(int mp, int nt, const float* re, const float* im,
+                                                  float2 (*y)[R], const float2 (*xs)[32][R], int bt) {
+    constexpr int GROUPS = (TRSV4_THREADS - TRSV4_SW) / TRSV_TPR;  // a multiple of 4
+    constexpr int H = 16 / R;                                      // rows per register buffer
+    constexpr int HG = H * GROUPS;
+    constexpr int COL = TRSV_TPR / R;                              // lanes that end up with the same column
+    static_assert(HG >= 32, "the first batch must cover tile d+2");
+    const int g = bt / TRSV_TPR, sub = bt % TRSV_TPR;
+    for (int d = 0; d + 2 < nt; ++d) {
+        const int col = 32 * (FWD ? d : nt - 1 - d) + sub * 4;
+        const int lo = FWD ? 32 * (d + 2) : 0;
+        const int hi = FWD ? mp : 32 * (nt - 2 - d);
+        const int len = hi - lo;
+        float4 ar[2][H], ai[2][H];
+        float2 xr[4][R];
+        auto load = [&](int b, int q0) {
+#pragma unroll
+            for (int u = 0; u < H; ++u) {
+                const int q = q0 + u * GROUPS;
+                if (q < len) {
+                    const int r = FWD ? lo + q : hi - 1 - q;
+                    ar[b][u] = ld4(re + (size_t)r * mp + col);
+                    ai[b][u] = ld4(im + (size_t)r * mp + col);
+                }
+            }
+        };
+        auto apply = [&](int b, int q0) {
+#pragma unroll
+            for (int u = 0; u < H; ++u) {
+                const int q = q0 + u * GROUPS;
+                if (q < len) {  // uniform across a warp (aligned quartets of groups, len a multiple of 32)
+                    const float2 s2 = multi4_row_product<R>(ar[b][u], ai[b][u], xr, sub);
+                    const int r = FWD ? lo + q : hi - 1 - q;
+                    if (sub % COL == 0) {
+                        float2 v = y[r][sub / COL];
+                        v.x -= s2.x;
+                        v.y -= s2.y;
+                        y[r][sub / COL] = v;
+                    }
+                }
+            }
+        };
+        load(0, g);
+        load(1, g + HG);
+        named_sync(TRSV_BAR_X + (d & 1), TRSV4_THREADS);
+#pragma unroll
+        for (int c = 0; c < 4; ++c)  // this lane's four columns of x_d, all right-hand sides
+#pragma unroll
+            for (int j = 0; j < R; ++j) xr[c][j] = xs[d & 1][sub * 4 + c][j];
+        apply(0, g);  // covers q < 32 (tile d+2)
+        named_arrive(TRSV_BAR_B + (d & 1), TRSV4_THREADS);
+        for (int q0 = g + HG; q0 < len; q0 += 2 * HG) {
+            load(0, q0 + HG);
+            apply(1, q0);
+            if (q0 + HG >= len) break;
+            load(1, q0 + 2 * HG);
+            apply(0, q0 + HG);
+        }
+    }
+}
+
+// v += (or -=) a row of a planar tile times the columns j0 .. j0 + W - 1 of x
+template <int R, int W, bool SUB>
+__device__ __forceinline__ void multi4_tile_row(const float* tr, const float* ti, const float2 (*x)[R], int j0,
+                                               float2 (&v)[W]) {
+#pragma unroll 2
+    for (int c = 0; c < 32; c += 4) {
+        const float4 a = *reinterpret_cast<const float4*>(tr + c), b = *reinterpret_cast<const float4*>(ti + c);
+        const float ar[4] = {a.x, a.y, a.z, a.w}, br[4] = {b.x, b.y, b.z, b.w};
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const float r = SUB ? -ar[u] : ar[u], i = SUB ? -br[u] : br[u];
+#pragma unroll
+            for (int j = 0; j < W; ++j) {
+                const float2 xv = x[c + u][j0 + j];
+                v[j].x = fmaf(-i, xv.y, fmaf(r, xv.x, v[j].x));
+                v[j].y = fmaf(i, xv.x, fmaf(r, xv.y, v[j].y));
+            }
+        }
+    }
+}
+
+// Solver warps: lane = row of the diagonal tile, W columns a warp; the inverted tiles
+// D^-1 (tinv) and the look-ahead tile L(d, d-1) arrive by cp.async two steps ahead.  A warp's
+// columns are its own from a to x, so only the tile buffers tie the warps together.
+template <int R, bool FWD>
+__device__ __forceinline__ void trsv_multi4_solver(int mp, int nt, const float* re, const float* im,
+                                                  const float* tinv, float2 (*y)[R], float2 (*xs)[32][R],
+                                                  float* tiles, float2 (*av)[R], int tid) {
+    constexpr int LD = trsv_tile<float>::LD, TS = 32 * LD, W = R * 32 / TRSV4_SW;
+    const int lane = tid & 31, j0 = W * (tid >> 5);
+    auto tile_of = [&](int d) { return FWD ? d : nt - 1 - d; };
+    auto issue = [&](int d) {
+        if (d < nt) {
+            float* b = tiles + (d & 1) * 4 * TS;
+            const int j = tile_of(d);
+            const float* ti = tinv + (size_t)j * 4096 + (FWD ? 0 : 2048);
+            tile_async<float, TRSV4_SW>(b, ti, 32, tid);
+            tile_async<float, TRSV4_SW>(b + TS, ti + 1024, 32, tid);
+            if (d >= 1) {
+                tile_async<float, TRSV4_SW>(b + 2 * TS, re + (size_t)(32 * j) * mp + 32 * tile_of(d - 1), mp, tid);
+                tile_async<float, TRSV4_SW>(b + 3 * TS, im + (size_t)(32 * j) * mp + 32 * tile_of(d - 1), mp, tid);
+            }
+        }
+        cp_async_commit();
+    };
+    issue(0);
+    issue(1);
+    for (int d = 0; d < nt; ++d) {
+        const int r0 = 32 * tile_of(d);
+        const float* Dre = tiles + (d & 1) * 4 * TS + lane * LD;
+        cp_async_wait<1>();
+        named_sync(TRSV_BAR_SOLVER, TRSV4_SW);  // everyone's copies of step d
+        if (d >= 2) named_sync(TRSV_BAR_B + (d & 1), TRSV4_THREADS);
+        float2 a[W], x[W];
+#pragma unroll
+        for (int j = 0; j < W; ++j) {
+            a[j] = y[r0 + lane][j0 + j];
+            x[j] = make_float2(0.f, 0.f);
+        }
+        if (d >= 1)  // look-ahead: strip d-1 on tile d's rows
+            multi4_tile_row<R, W, true>(Dre + 2 * TS, Dre + 3 * TS, xs[(d - 1) & 1], j0, a);
+#pragma unroll
+        for (int j = 0; j < W; ++j) av[lane][j0 + j] = a[j];
+        __syncwarp();
+        multi4_tile_row<R, W, false>(Dre, Dre + TS, av, j0, x);  // x = D^-1 a
+#pragma unroll
+        for (int j = 0; j < W; ++j) {
+            y[r0 + lane][j0 + j] = x[j];
+            xs[d & 1][lane][j0 + j] = x[j];
+        }
+        __syncwarp();
+        if (d <= nt - 3) named_arrive(TRSV_BAR_X + (d & 1), TRSV4_THREADS);
+        named_sync(TRSV_BAR_SOLVER, TRSV4_SW);  // buffer d & 1 is free again
+        issue(d + 2);
+    }
+    cp_async_wait<0>();
+}
+
+// grid (ceil(nact / R), max_nblk): CTA (x, k) solves block k for the instances
+// act[R x ..], which all use the factors of instance act[0]'s descriptor.
+template <int R>
+__global__ void __launch_bounds__(TRSV4_THREADS)
+block_trsv_multi4_kernel(const InstDev* __restrict__ I, const int* __restrict__ act, int nact) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ __align__(16) float2 xs[2][32][R];
+    __shared__ __align__(16) float2 av[32][R];
+    const InstDev& d0 = I[act[0]];
+    const int k = blockIdx.y;
+    if (k >= d0.nblk) return;
+    const int mp = d0.mp, nt = mp / 32;
+    const float* re = (const float*)d0.fac + (size_t)k * 2 * mp * mp;
+    const float* im = re + (size_t)mp * mp;
+    const float* tinv = (const float*)d0.tinv + (size_t)k * (mp / 32) * 4096;
+    float2(*y)[R] = reinterpret_cast<float2(*)[R]>(smem_raw);
+    float* tiles = reinterpret_cast<float*>(smem_raw + (size_t)mp * R * sizeof(float2));
+    const int tid = threadIdx.x;
+    // the group's right-hand sides: column j <- instance act[R blockIdx.x + j] (if live)
+    for (int e = tid; e < mp * R; e += blockDim.x) {
+        const int r = e / R, j = e % R, a = R * blockIdx.x + j;
+        float2 v = make_float2(0.f, 0.f);
+        if (a < nact) {
+            const InstDev& d = I[act[a]];
+            if (d.ctl[0]) v = ((const float2*)d.rhat)[(size_t)k * mp + r];
+        }
+        y[r][j] = v;
+    }
+    __syncthreads();
+    if (tid < TRSV4_SW) trsv_multi4_solver<R, true>(mp, nt, re, im, tinv, y, xs, tiles, av, tid);
+    else trsv_multi4_stream<R, true>(mp, nt, re, im, y, xs, tid - TRSV4_SW);
+    __syncthreads();
+    if (tid < TRSV4_SW) trsv_multi4_solver<R, false>(mp, nt, re, im, tinv, y, xs, tiles, av, tid);
+    else trsv_multi4_stream<R, false>(mp, nt, re, im, y, xs, tid - TRSV4_SW);
+    __syncthreads();
+    for (int e = tid; e < mp * R; e += blockDim.x) {
+        const int r = e / R, j = e % R, a = R * blockIdx.x + j;
         if (a < nact) {
             const InstDev& d = I[act[a]];
             if (d.ctl[0]) ((float2*)d.rhat)[(size_t)k * mp + r] = y[r][j];
@@ -2468,6 +2397,13 @@ size_t tc_pack_a_bytes_per_block(int precision, int mp) {
 
 int launch_trsv_multi(const InstDev* I, const int* act, int nact, int nblk, int mp, cudaStream_t st) {
     if (nact <= 0) return FDE_OK;
+    if ((long)nblk * ((nact + 7) / 8) <= 76) {  // groups of 8 would leave half the SMs idle
+        const size_t smem4 = trsv_multi4_smem_bytes(mp);
+        FDE_TRY(allow_smem((const void*)block_trsv_multi4_kernel<4>, smem4));
+        block_trsv_multi4_kernel<4><<<dim3((nact + 3) / 4, nblk), TRSV4_THREADS, smem4, st>>>(I, act, nact);
+        FDE_LAUNCH_CHECK("block_trsv_multi4_kernel");
+        return FDE_OK;
+    }
     const size_t smem = trsv_multi_smem_bytes(mp);
     if (smem > 227 * 1024) return launch_trsv_batched(I, act, nact, nblk, mp, st);  // m_p > 2560: one per CTA
     FDE_TRY(allow_smem((const void*)block_trsv_multi_kernel, smem));
@@ -2485,72 +2421,65 @@ int launch_trsv_batched(const InstDev* I, const int* act, int nact, int max_nblk
     return FDE_OK;
 }
 
-// Inverses of the 32 x 32 diagonal tiles of every block's factors, for the block
-// solves: warp 0 inverts the unit lower tile of L, warp 1 the upper tile of U (its
-// diagonal included), both in place column by column / row by row from the last,
-//   L^-1[i][j] = -(L[i][j] + sum_{j<k<i} L^-1[i][k] L[k][j])          (i > j)
-//   U^-1[j][c] = -(1/U[j][j]) sum_{j<k<=c} U[j][k] U^-1[k][c]         (c > j).
-// Output per block and tile: [L^-1 re, L^-1 im, U^-1 re, U^-1 im][32][32], with the
-// zeros and the unit (L) / inverted (U) diagonal written out.
+// The inverses of the 32 x 32 diagonal tiles of L (warps 0-3) and U (warps 4-7), columns by
+// substitution; U is taken from its last row and column on, which makes it lower triangular as
+// well.  Warp w has columns 8 w .. 8 w + 7, four lanes a column that share the inner sums, and
+// starts at row 8 w: the columns' zeros above are not summed.  Output per block and tile: [L^-1 re, L^-1 im, U^-1 re,
+// U^-1 im][32][32], with the zeros and the unit (L) / inverted (U) diagonal written out.
 template <typename T>
-__global__ void __launch_bounds__(64) tile_inverse_kernel(int mp, const T* __restrict__ fac, T* __restrict__ tinv) {
+__global__ void __launch_bounds__(256)
+tile_inverse_kernel(int mp, const T* __restrict__ fac, T* __restrict__ tinv) {
     using C = cplx_t<T>;
-    __shared__ C tl[2][32][33];
-    __shared__ C vb[2][32];
-    const int k = blockIdx.y, t = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const T* re = fac + (size_t)k * 2 * mp * mp;
+    __shared__ C A2[2][NB][NB + 1];  // the triangles, U reversed
+    __shared__ C X[2][NB][NB + 1];   // their inverses
+    __shared__ C di[NB];             // reciprocal diagonal of reversed U
+    const auto fms = [](C a, C b, C c) {  // a - b c
+        a.x = fma(-b.x, c.x, fma(b.y, c.y, a.x));
+        a.y = fma(-b.x, c.y, fma(-b.y, c.x, a.y));
+        return a;
+    };
+    const int k = blockIdx.y, t = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const T* re = fac + (size_t)k * 2 * mp * mp + (size_t)t * NB * mp + t * NB;
     const T* im = re + (size_t)mp * mp;
-    const int r0 = 32 * t;
-    C (*A)[33] = tl[warp];
-    C* v = vb[warp];
-    for (int r = 0; r < 32; ++r) {
-        const size_t g = (size_t)(r0 + r) * mp + r0 + lane;
-        A[r][lane] = mk(re[g], im[g]);
+    for (int r = warp; r < NB; r += 8) {
+        const C v = mk(re[(size_t)r * mp + lane], im[(size_t)r * mp + lane]);
+        A2[0][r][lane] = v;
+        A2[1][NB - 1 - r][NB - 1 - lane] = v;
+        X[0][r][lane] = X[1][r][lane] = mk(T(0), T(0));
     }
-    __syncwarp();
-    if (warp == 0) {  // lane = row
-        for (int j = 31; j >= 0; --j) {
-            v[lane] = lane > j ? A[lane][j] : mk(T(0), T(0));
-            __syncwarp();
-            C sum = mk(T(0), T(0));
-            if (lane > j) {
-                sum = v[lane];
-                for (int q = j + 1; q < lane; ++q) sum = cadd(sum, cmul(A[lane][q], v[q]));
-            }
-            __syncwarp();
-            if (lane > j) A[lane][j] = mk(-sum.x, -sum.y);
-            __syncwarp();
-        }
-    } else {  // lane = column
-        for (int j = 31; j >= 0; --j) {
-            v[lane] = lane > j ? A[j][lane] : mk(T(0), T(0));
-            const C piv = A[j][j];
-            __syncwarp();
-            const T den = piv.x * piv.x + piv.y * piv.y;
-            const C dj = den > T(0) ? mk(piv.x / den, -piv.y / den) : mk(T(0), T(0));
-            C nv = dj;
-            if (lane > j) {
-                C sum = mk(T(0), T(0));
-                for (int q = j + 1; q <= lane; ++q) sum = cadd(sum, cmul(v[q], A[q][lane]));
-                nv = cmul(dj, sum);
-                nv = mk(-nv.x, -nv.y);
-            }
-            __syncwarp();
-            if (lane >= j) A[j][lane] = nv;
-            __syncwarp();
-        }
+    __syncthreads();
+    if (warp == 0) {
+        const C p = A2[1][lane][lane];
+        const T den = p.x * p.x + p.y * p.y;
+        di[lane] = den > T(0) ? mk(p.x / den, -p.y / den) : mk(T(0), T(0));
+        X[0][lane][lane] = mk(T(1), T(0));
+        X[1][lane][lane] = di[lane];
     }
-    T* out = tinv + ((size_t)k * (mp / 32) + t) * 4096 + warp * 2048;
-    for (int r = 0; r < 32; ++r) {
-        C e = A[r][lane];
-        if (warp == 0) {
-            if (lane > r) e = mk(T(0), T(0));
-            else if (lane == r) e = mk(T(1), T(0));
-        } else if (lane < r) {
-            e = mk(T(0), T(0));
+    __syncthreads();
+    // warps q and q + 4 share a scheduler: the longest columns of L go with the shortest of U
+    const int which = warp >> 2, w = which ? 3 - (warp & 3) : warp, j = 8 * w + (lane >> 2), q = lane & 3;
+    C (*A)[NB + 1] = A2[which];
+    C (*Y)[NB + 1] = X[which];
+    for (int i = 8 * w + 1; i < NB; ++i) {
+        C sum = mk(T(0), T(0));
+        for (int c = 8 * w + q; c < i; c += 4) sum = fms(sum, A[i][c], Y[c][j]);
+#pragma unroll
+        for (int off = 1; off < 4; off <<= 1) {
+            sum.x += __shfl_xor_sync(0xffffffffu, sum.x, off);
+            sum.y += __shfl_xor_sync(0xffffffffu, sum.y, off);
         }
-        out[r * 32 + lane] = e.x;
-        out[1024 + r * 32 + lane] = e.y;
+        if (which) sum = cmul(sum, di[i]);
+        if (q == 0 && i > j) Y[i][j] = sum;
+        __syncwarp();
+    }
+    __syncthreads();
+    T* out = tinv + ((size_t)k * (mp / NB) + t) * 4096;
+    for (int r = warp; r < NB; r += 8) {
+        const C l = X[0][r][lane], u = X[1][NB - 1 - r][NB - 1 - lane];
+        out[r * NB + lane] = l.x;
+        out[1024 + r * NB + lane] = l.y;
+        out[2048 + r * NB + lane] = u.x;
+        out[3072 + r * NB + lane] = u.y;
     }
 }
 
@@ -2569,9 +2498,11 @@ static int launch_tile_inverse(Problem& P, int prec, cudaStream_t st) {
         P.tinv_bytes = bytes;
     }
     StageTimer t(P, FDE_STAGE_LU_DIAG);
-    if (prec == FDE_FP64) return launch_tile_inverse64(P, st);
     const dim3 grid(P.mp / 32, P.nblk);
-    tile_inverse_kernel<float><<<grid, 64, 0, st>>>(P.mp, (const float*)P.d_fac, (float*)P.d_tinv);
+    if (prec == FDE_FP64)
+        tile_inverse_kernel<double><<<grid, 256, 0, st>>>(P.mp, (const double*)P.d_fac, (double*)P.d_tinv);
+    else
+        tile_inverse_kernel<float><<<grid, 256, 0, st>>>(P.mp, (const float*)P.d_fac, (float*)P.d_tinv);
     FDE_LAUNCH_CHECK("tile_inverse_kernel");
     return FDE_OK;
 }
@@ -2594,132 +2525,20 @@ int launch_block_lu(Problem& P, int prec, cudaStream_t st) {
     return launch_tile_inverse(P, prec, st);
 }
 
-template <typename T, int V>
-static int launch_trsv_shape(const Problem& P, void* rhat, cudaStream_t st) {
-    const size_t smem = trsv_smem_bytes(P.mp, sizeof(T));
-    // the strip-major copy of the factor (FP32 or bfloat16), where the tensor-core LU wrote one
-    const bool strips = P.strips_ok && P.d_strips;
-    {
-        if (strips && P.strips_bf16) {
-            auto kern = block_trsv_kernel<T, V, LAY_STRIPS_BF16>;
-            FDE_TRY(allow_smem((const void*)kern, smem));
-            kern<<<P.nblk, trsv_shape<T, V>::NT, smem, st>>>(P.mp, (const unsigned short*)P.d_strips,
-                                                              (const cplx_t<T>*)P.d_dinv, (const T*)P.d_tinv,
-                                                              (cplx_t<T>*)rhat, P.live);
-            FDE_LAUNCH_CHECK("block_trsv_kernel");
-            return FDE_OK;
-        }
-    }
-    {
-        constexpr int LS = LAY_STRIPS;
-        auto kern = strips ? block_trsv_kernel<T, V, LS> : block_trsv_kernel<T, V, LAY_PLANES>;
-        FDE_TRY(allow_smem((const void*)kern, smem));
-        kern<<<P.nblk, trsv_shape<T, V>::NT, smem, st>>>(P.mp, (const T*)(strips ? P.d_strips : P.d_fac),
-                                                          (const cplx_t<T>*)P.d_dinv, (const T*)P.d_tinv,
-                                                          (cplx_t<T>*)rhat, P.live);
-    }
-    FDE_LAUNCH_CHECK("block_trsv_kernel");
+template <int V>
+static int launch_trsv_bf16_shape(const Problem& P, void* rhat, cudaStream_t st) {
+    const size_t smem = trsv_smem_bytes(P.mp, sizeof(float));
+    FDE_TRY(allow_smem((const void*)block_trsv_bf16_kernel<V>, smem));
+    block_trsv_bf16_kernel<V><<<P.nblk, trsv_shape<V>::NT, smem, st>>>(
+        P.mp, (const unsigned short*)P.d_strips, (const float*)P.d_tinv, (float2*)rhat, P.live);
+    FDE_LAUNCH_CHECK("block_trsv_bf16_kernel");
     return FDE_OK;
 }
 
-constexpr size_t TRSV_SMEM_MAX = 227 * 1024;  // dynamic shared memory of one CTA
-
-// Tensor map of the factor planes as a 3-D array [2 nblk planes][m_p rows][m_p columns],
-// boxes of R rows x 32 columns of one plane (made once per factor buffer).
-template <typename T>
-static int trsv_tensor_map(const Problem& P, CUtensorMap* map) {
-    using Fn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                            const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                            CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-    static Fn encode = nullptr;
-    if (!encode) {
-        void* fn = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        FDE_CUDA_TRY(cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &q));
-        if (q != cudaDriverEntryPointSuccess || !fn) return set_error(FDE_ERR_CUDA, "cuTensorMapEncodeTiled unavailable");
-        encode = reinterpret_cast<Fn>(fn);
-    }
-    const cuuint64_t dims[3] = {(cuuint64_t)P.mp, (cuuint64_t)P.mp, (cuuint64_t)2 * P.nblk};
-    const cuuint64_t strides[2] = {(cuuint64_t)P.mp * sizeof(T), (cuuint64_t)P.mp * P.mp * sizeof(T)};
-    const cuuint32_t box[3] = {32, (cuuint32_t)ring_cfg<T>::R, 1};
-    const cuuint32_t estr[3] = {1, 1, 1};
-    const CUresult r = encode(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, P.d_fac, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                              CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (r != CUDA_SUCCESS) return set_error(FDE_ERR_CUDA, "cuTensorMapEncodeTiled failed for the factor planes");
-    return FDE_OK;
-}
-
-template <typename T>
-static int launch_trsv_ring(const Problem& P, void* rhat, cudaStream_t st) {
-    const size_t smem = trsv_ring_smem_bytes(P.mp, sizeof(T));
-    if (smem > TRSV_SMEM_MAX) return launch_trsv_shape<T, 0>(P, rhat, st);  // the ring does not fit: default
-    CUtensorMap map;
-    int rc = trsv_tensor_map<T>(P, &map);
-    if (rc) return rc;
-    auto kern = block_trsv_ring_kernel<T>;
-    FDE_TRY(allow_smem((const void*)kern, smem));
-    kern<<<P.nblk, ring_cfg<T>::NT, smem, st>>>(P.mp, (const T*)P.d_fac, (const cplx_t<T>*)P.d_dinv,
-                                                 (const T*)P.d_tinv, (cplx_t<T>*)rhat, P.d_err, map, P.live);
-    FDE_LAUNCH_CHECK("block_trsv_ring_kernel");
-    return FDE_OK;
-}
-
-// The tuning key of the block solves: the storage of the factors they read (FP64,
-// FP32, or FDE_BF16 for the bfloat16 strip copy).
-static int trsv_key(const Problem& P) {
-    if (P.precision == FDE_FP64) return FDE_FP64;
-    return P.strips_ok && P.d_strips && P.strips_bf16 ? FDE_BF16 : FDE_FP32;
-}
-
-int launch_block_trsv_variant(const Problem& P, void* rhat, int variant, cudaStream_t st) {
-    if (P.precision == FDE_FP64) return launch_trsv64(P, rhat, st);
-    // the ring has no form for the bfloat16 copy: there the register shape 0 stands in for it
-    if (variant == 3 && trsv_key(P) == FDE_BF16) variant = 0;
-    // strips streamed through a shared-memory ring by bulk copies
-    if (variant == 3) return launch_trsv_ring<float>(P, rhat, st);
-    if (variant == 1) return launch_trsv_shape<float, 1>(P, rhat, st);
-    if (variant == 2) return launch_trsv_shape<float, 2>(P, rhat, st);
-    return launch_trsv_shape<float, 0>(P, rhat, st);
-}
-
-int launch_block_trsv(const Problem& P, void* rhat, cudaStream_t st) {
-    return launch_block_trsv_variant(P, rhat, tune_lookup(FDE_TUNE_TRSV, P.mp, P.nblk, trsv_key(P), nullptr), st);
-}
-
-namespace {
-struct TrsvTuneCtx {
-    const Problem* P;
-    void* rhat;
-};
-int trsv_trial(void* ctx, int v, cudaStream_t st) {
-    const TrsvTuneCtx& c = *static_cast<const TrsvTuneCtx*>(ctx);
-    return launch_block_trsv_variant(*c.P, c.rhat, v, st);
-}
-}  // namespace
-
-// Measure the block-solve shapes for this problem's factors, on its frequency-side
-// vector (zeroed first: the solves run in place and their timing does not depend on
-// the data), unless the table already has the shape or a variant is forced.
-int autotune_trsv(Problem& P) {
-    const int prec = trsv_key(P);
-    bool need = false;
-    tune_lookup(FDE_TUNE_TRSV, P.mp, P.nblk, prec, &need);
-    if (!need) return FDE_OK;
-    if (prec == FDE_FP64) {  // one form for every variant: nothing to time
-        tune_store(FDE_TUNE_TRSV, P.mp, P.nblk, prec, 0, nullptr);
-        return FDE_OK;
-    }
-    FDE_CUDA_TRY(cudaMemsetAsync(P.d_rhat, 0, (size_t)P.nblk * P.mp * 2 * sizeof(float), P.stream));
-    TrsvTuneCtx ctx{&P, P.d_rhat};
-    int best = 0;
-    float ms[TUNE_MAX_VARIANTS] = {};
-    // on the bfloat16 copy the three register shapes (the ring reads the FP32 planes)
-    const int rc = tune_measure(FDE_TUNE_TRSV, P.stream, trsv_trial, &ctx, &best, ms,
-                                tune_default_variant(FDE_TUNE_TRSV, prec), prec == FDE_BF16 ? 3 : 0);
-    if (rc) return rc;
-    tune_store(FDE_TUNE_TRSV, P.mp, P.nblk, prec, best, ms);
-    return FDE_OK;
+int launch_trsv_bf16(const Problem& P, void* rhat, int variant, cudaStream_t st) {
+    if (variant == 1) return launch_trsv_bf16_shape<1>(P, rhat, st);
+    if (variant == 2) return launch_trsv_bf16_shape<2>(P, rhat, st);
+    return launch_trsv_bf16_shape<0>(P, rhat, st);
 }
 
 }  // namespace fde

@@ -38,11 +38,6 @@ __device__ __forceinline__ double2 cfma(double2 a, double2 b, double2 c) {
     a.y = fma(b.x, c.y, fma(b.y, c.x, a.y));
     return a;
 }
-__device__ __forceinline__ double2 reciprocal(double2 p) {
-    const double den = p.x * p.x + p.y * p.y;
-    return den > 0.0 && isfinite(den) ? make_double2(p.x / den, -p.y / den) : make_double2(0.0, 0.0);
-}
-
 // Sums x and y over W neighbouring lanes: even lanes return sum x, odd ones sum y.  The first
 // exchange splits the pair, so a level costs one FP64 addition, not two.
 template <int W>
@@ -208,58 +203,6 @@ lu64_update_kernel(int mp, int p, int nt, double* __restrict__ fac) {
     }
 }
 
-// The inverses of the 32 x 32 diagonal tiles of L (warps 0-3) and U (warps 4-7), columns by
-// substitution; U is taken from its last row and column on, which makes it lower triangular as
-// well.  Warp w has columns 8 w .. 8 w + 7, four lanes a column that share the inner sums, and
-// starts at row 8 w: the columns' zeros above are not summed.
-__global__ void __launch_bounds__(256)
-tile_inverse64_kernel(int mp, const double* __restrict__ fac, double* __restrict__ tinv) {
-    __shared__ double2 T[2][NB][NB + 1];  // the triangles, U reversed
-    __shared__ double2 X[2][NB][NB + 1];  // their inverses
-    __shared__ double2 di[NB];            // reciprocal diagonal of reversed U
-    const int k = blockIdx.y, t = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const double* re = fac + (size_t)k * 2 * mp * mp + (size_t)t * NB * mp + t * NB;
-    const double* im = re + (size_t)mp * mp;
-    for (int r = warp; r < NB; r += 8) {
-        const double2 v = make_double2(re[(size_t)r * mp + lane], im[(size_t)r * mp + lane]);
-        T[0][r][lane] = v;
-        T[1][NB - 1 - r][NB - 1 - lane] = v;
-        X[0][r][lane] = X[1][r][lane] = make_double2(0.0, 0.0);
-    }
-    __syncthreads();
-    if (warp == 0) {
-        di[lane] = reciprocal(T[1][lane][lane]);
-        X[0][lane][lane] = make_double2(1.0, 0.0);
-        X[1][lane][lane] = di[lane];
-    }
-    __syncthreads();
-    // warps q and q + 4 share a scheduler: the longest columns of L go with the shortest of U
-    const int which = warp >> 2, w = which ? 3 - (warp & 3) : warp, j = 8 * w + (lane >> 2), q = lane & 3;
-    double2 (*A)[NB + 1] = T[which];
-    double2 (*Y)[NB + 1] = X[which];
-    for (int i = 8 * w + 1; i < NB; ++i) {
-        double2 sum = make_double2(0.0, 0.0);
-        for (int c = 8 * w + q; c < i; c += 4) sum = cfms(sum, A[i][c], Y[c][j]);
-#pragma unroll
-        for (int off = 1; off < 4; off <<= 1) {
-            sum.x += __shfl_xor_sync(0xffffffffu, sum.x, off);
-            sum.y += __shfl_xor_sync(0xffffffffu, sum.y, off);
-        }
-        if (which) sum = cmul(sum, di[i]);
-        if (q == 0 && i > j) Y[i][j] = sum;
-        __syncwarp();
-    }
-    __syncthreads();
-    double* out = tinv + ((size_t)k * (mp / NB) + t) * 4096;
-    for (int r = warp; r < NB; r += 8) {
-        const double2 l = X[0][r][lane], u = X[1][NB - 1 - r][NB - 1 - lane];
-        out[r * NB + lane] = l.x;
-        out[1024 + r * NB + lane] = l.y;
-        out[2048 + r * NB + lane] = u.x;
-        out[3072 + r * NB + lane] = u.y;
-    }
-}
-
 // Block solves in place on rhat[k], one CTA per block: per 32-row tile x = D^-1 a (eight lanes a
 // row), then the tile's strip times x from the rows that remain (four lanes a row, the loads of
 // the first rows issued before the tile is solved).  Rows from nt 32 on are padding (zero).
@@ -354,12 +297,6 @@ int launch_lu64(Problem& P, cudaStream_t st) {
         lu64_update_kernel<<<dim3(nt * nt, nb), U64_THREADS, 0, st>>>(mp, p, nt, fac);
         FDE_LAUNCH_CHECK("lu64_update_kernel");
     }
-    return FDE_OK;
-}
-
-int launch_tile_inverse64(const Problem& P, cudaStream_t st) {
-    tile_inverse64_kernel<<<dim3(P.mp / NB, P.nblk), 256, 0, st>>>(P.mp, (const double*)P.d_fac, (double*)P.d_tinv);
-    FDE_LAUNCH_CHECK("tile_inverse64_kernel");
     return FDE_OK;
 }
 

@@ -62,10 +62,8 @@ int tune_variants(int kernel) {
     return kernel == FDE_TUNE_MATVEC ? 3 : kernel == FDE_TUNE_TRSV ? 4 : kernel == FDE_TUNE_LU ? 3 : 0;
 }
 
-// The variant used before a shape is measured (or when tuning is impossible): the
-// 384 x 8 block-solve shape for FP32 factors (never slower than 512 x 4 where both were
-// timed), the first variant otherwise.
-// Built-in defaults: block solves with FP32 factors 384 x 8; the LU interior update with
+// The variant used before a shape is measured (or when tuning is impossible): block solves with
+// FP32 factors 14 warps (the fastest from m = 511 on, within 1.5 us at 255); the LU interior update with
 // C streamed by tensor-map copies (its kernel falls back to row pairs where m_p is not a
 // multiple of 128); everything else variant 0.
 static int tune_default(int kernel, int prec) {
