@@ -23,6 +23,7 @@
 #include <vector>
 
 #include "fde_internal.h"
+#include "nop_tile.cuh"
 
 namespace fde {
 
@@ -36,33 +37,14 @@ __device__ __forceinline__ float ldf(const __half* p) { return __half2float(*p);
 __device__ __forceinline__ void stf(float* p, float v) { *p = v; }
 __device__ __forceinline__ void stf(__half* p, float v) { *p = __float2half_rn(v); }
 
-// Places of a tile's positions: flattened positions n = b m + x of the batch, so that a tile
-// is full whatever the number of modes; every sample's piece of the tile is staged with a halo
-// of h zeros or neighbours on either side.
-__device__ __forceinline__ int cv_place(int n, int n0, int m, int h) { return n - n0 + (n / m - n0 / m) * 2 * h; }
-// length of a staged row for the positions [n0, n1)
-__host__ __device__ __forceinline__ int cv_length(int n0, int n1, int m, int h) {
-    return n1 - n0 + ((n1 - 1) / m - n0 / m + 1) * 2 * h;
-}
-// offset of slot t's sample row and point, (b Q) m + x for channel 0, or -1 for a zero
-__device__ __forceinline__ int cv_source(int Q, int n0, int m, int h, int t) {
-    const int b0 = n0 / m, head = m - (n0 - b0 * m) + 2 * h;  // slots of the first sample's piece
-    int b = b0, xx = n0 - b0 * m - h + t;
-    if (t >= head) {
-        const int u = t - head, w = m + 2 * h;
-        b = b0 + 1 + u / w;
-        xx = u - (u / w) * w - h;
-    }
-    return xx >= 0 && xx < m ? b * Q * m + xx : -1;
-}
 // stage channels q0 .. q0 + nq - 1 of x: one warp a channel, lanes along the slots (whose
 // sources do not depend on the channel)
 template <typename TI>
-__device__ __forceinline__ void cv_stage(const TI* __restrict__ x, int Q, int q0, int nq, int nmax, int n0, int m,
+__device__ __forceinline__ void cv_stage(const TI* __restrict__ x, int Q, int q0, int nq, int nmax, CvTile tile, int m,
                                          int h, int len, float* s, int ld) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     for (int t = lane; t < len; t += 32) {
-        const int src = cv_source(Q, n0, m, h, t);
+        const ptrdiff_t src = cv_source(tile, Q, m, h, t);
 #pragma unroll 4
         for (int c = warp; c < nmax; c += CV_WARPS)
             s[c * ld + t] = src >= 0 && c < nq ? ldf(x + src + (size_t)(q0 + c) * m) : 0.f;
@@ -83,25 +65,27 @@ __device__ __forceinline__ void cv_stage(const TI* __restrict__ x, int Q, int q0
 template <typename TI, typename TW, typename TO, bool TRANS, int NL, int KT>
 __global__ void __launch_bounds__(32 * CV_WARPS)
 conv_kernel(const TI* __restrict__ x, int Q, const TW* __restrict__ W, const float* __restrict__ bias, int P, int Kr,
-            int m, int N, int relu, const float* __restrict__ mask, TO* __restrict__ y, int ld) {
+            int m, long N, int relu, const float* __restrict__ mask, TO* __restrict__ y, int ld) {
     const int K = KT ? KT : Kr;
     constexpr int TN = 4 * NL, QW = NL == 4 ? 8 : 4, QC = QW * CV_WARPS;  // QW: channels per warp and chunk
     extern __shared__ float cv_smem[];
     float* s_in = cv_smem;            // [QC][ld]
     float* s_w = cv_smem + QC * ld;   // [QC][K][CV_LDW]
-    const int p0 = blockIdx.y * CV_TP, n0 = blockIdx.x * TN, n1 = min(n0 + TN, N);
-    const int h = K / 2, len = cv_length(n0, n1, m, h);
+    const long n0 = (long)blockIdx.x * TN;
+    const CvTile tile = cv_tile(n0, m);
+    const int p0 = blockIdx.y * CV_TP, count = (int)min((long)TN, N - n0);
+    const int h = K / 2, len = cv_length(count, tile.x0, m, h);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, pl = lane >> 2, nl = lane & 3;
     float acc[2][NL];
     int at[NL];
 #pragma unroll
     for (int j = 0; j < NL; ++j) {
         acc[0][j] = acc[1][j] = 0.f;
-        at[j] = cv_place(min(n0 + nl + 4 * j, n1 - 1), n0, m, h);
+        at[j] = cv_place(min(nl + 4 * j, count - 1), tile.x0, m, h);
     }
     for (int q0 = 0; q0 < Q; q0 += QC) {
         const int nq = min(QC, Q - q0);
-        cv_stage(x, Q, q0, nq, nq, n0, m, h, len, s_in, ld);
+        cv_stage(x, Q, q0, nq, nq, tile, m, h, len, s_in, ld);
         // 16 threads a row of weights: channel o's (TRANS = false) or input channel c's
         const int row = tid >> 4;
         if (TRANS) {
@@ -144,15 +128,14 @@ conv_kernel(const TI* __restrict__ x, int Q, const TW* __restrict__ W, const flo
     }
     __syncthreads();
     for (int e = tid; e < CV_TP * TN; e += 32 * CV_WARPS) {
-        const int p = p0 + e / TN, n = n0 + e % TN;
-        if (p >= P || n >= n1) continue;
+        const int p = p0 + e / TN, n = e % TN;
+        if (p >= P || n >= count) continue;
         float v = 0.f;
 #pragma unroll
         for (int w = 0; w < CV_WARPS; ++w) v += red[w * CV_TP * TN + e];
         if (bias) v += bias[p];
         if (relu) v = fmaxf(v, 0.f);
-        const int b = n / m;
-        const size_t idx = ((size_t)b * P + p) * m + n - b * m;
+        const size_t idx = cv_offset(tile, P, p, m, n);
         if (mask && !(mask[idx] > 0.f)) v = 0.f;
         stf(y + idx, v);
     }
@@ -177,21 +160,23 @@ conv_wgrad_kernel(const float* __restrict__ g, int O, const float* __restrict__ 
 #pragma unroll
     for (int k = 0; k < CV_KMAX; ++k) acc[k] = 0.f;
     const int per = (B + gridDim.z - 1) / gridDim.z;  // samples of this group
-    const int lo = blockIdx.z * per * m, hi = min(B, ((int)blockIdx.z + 1) * per) * m;
-    for (int n0 = lo; n0 < hi; n0 += WG_N) {
-        const int n1 = min(n0 + WG_N, hi), len = cv_length(n0, n1, m, h);
+    const int lo = blockIdx.z * per, hi = min(B, lo + per);
+    const long total = lo < hi ? (long)(hi - lo) * m : 0;
+    CvTile tile{lo, 0};
+    for (long n0 = 0; n0 < total; n0 += WG_N) {
+        const int count = (int)min((long)WG_N, total - n0), len = cv_length(count, tile.x0, m, h);
         {
-            const int t = threadIdx.x % WG_N, n = n0 + t, b = n / m;
-            const float* gr = g + ((size_t)b * O + o0) * m + n - b * m;
+            const int t = threadIdx.x % WG_N;
+            const float* gr = g + cv_offset(tile, O, o0, m, t);
 #pragma unroll
             for (int r = threadIdx.x / WG_N; r < 16; r += 256 / WG_N)
-                s_g[r * (WG_N + 1) + t] = o0 + r < O && n < n1 ? gr[(size_t)r * m] : 0.f;
+                s_g[r * (WG_N + 1) + t] = o0 + r < O && t < count ? gr[(size_t)r * m] : 0.f;
         }
-        cv_stage(a, C, c0, min(16, C - c0), 16, n0, m, h, len, s_a, ld);
+        cv_stage(a, C, c0, min(16, C - c0), 16, tile, m, h, len, s_a, ld);
         __syncthreads();
-        int x = n0 % m;
+        int x = tile.x0;
         const float* ap = s_a + cl * ld;
-        for (int t = 0; t < n1 - n0; ++t) {
+        for (int t = 0; t < count; ++t) {
             const float gv = s_g[ol * (WG_N + 1) + t];
             sum += gv;
 #pragma unroll
@@ -203,6 +188,9 @@ conv_wgrad_kernel(const float* __restrict__ g, int O, const float* __restrict__ 
                 ap += 2 * h;
             }
         }
+        const int next = tile.x0 + WG_N;
+        tile.b0 += next / m;
+        tile.x0 = next % m;
         __syncthreads();
     }
     if (o0 + ol < O && c0 + cl < C)
@@ -351,14 +339,14 @@ struct fde_nop {
 namespace {
 
 // Longest staged row of any tile of `tile` positions.
-int staged_length(int tile, int N, int m, int K) {
-    const int n = tile < N ? tile : N;
-    const int pieces = (n + m - 2) / m + 1;  // samples a tile can touch
+int staged_length(int tile, long N, int m, int K) {
+    const int n = (int)std::min<long>(tile, N);
+    const int pieces = (int)((n + (long)m - 2) / m) + 1;  // samples a tile can touch
     return n + pieces * 2 * (K / 2);
 }
 
 template <typename TI, typename TW, typename TO, bool TRANS, int NL, int KT>
-int conv_tiles(const TI* x, int Q, const TW* W, const float* bias, int P, int K, int m, int N, int relu,
+int conv_tiles(const TI* x, int Q, const TW* W, const float* bias, int P, int K, int m, long N, int relu,
                const float* mask, TO* y, cudaStream_t st) {
     constexpr int TN = 4 * NL, QC = (NL == 4 ? 8 : 4) * CV_WARPS;
     const int ld = staged_length(TN, N, m, K) | 1;
@@ -366,7 +354,7 @@ int conv_tiles(const TI* x, int Q, const TW* W, const float* bias, int P, int K,
     const size_t smem = (stage > red ? stage : red) * sizeof(float);
     auto kern = conv_kernel<TI, TW, TO, TRANS, NL, KT>;
     FDE_TRY(allow_smem((const void*)kern, 227 * 1024));
-    const dim3 grid((N + TN - 1) / TN, (P + CV_TP - 1) / CV_TP);
+    const dim3 grid((unsigned)((N + TN - 1) / TN), (P + CV_TP - 1) / CV_TP);
     kern<<<grid, 32 * CV_WARPS, smem, st>>>(x, Q, W, bias, P, K, m, N, relu, mask, y, ld);
     FDE_LAUNCH_CHECK("conv_kernel");
     return FDE_OK;
@@ -377,8 +365,8 @@ int conv_tiles(const TI* x, int Q, const TW* W, const float* bias, int P, int K,
 template <typename TI, typename TW, typename TO, bool TRANS>
 int conv(const TI* x, int Q, const TW* W, const float* bias, int P, int K, int m, int B, int relu, const float* mask,
          TO* y, cudaStream_t st) {
-    const int N = B * m;
-    const long ctas = (long)((N + 15) / 16) * ((P + CV_TP - 1) / CV_TP);
+    const long N = (long)B * m;
+    const long ctas = (N + 15) / 16 * ((P + CV_TP - 1) / CV_TP);
     if (ctas > 8 * 152)
         return conv_tiles<TI, TW, TO, TRANS, 16, 0>(x, Q, W, bias, P, K, m, N, relu, mask, y, st);
     if (K == 3) return conv_tiles<TI, TW, TO, TRANS, 4, 3>(x, Q, W, bias, P, K, m, N, relu, mask, y, st);
@@ -530,7 +518,7 @@ int fde_nop_loss_grad(fde_nop* n, const float* in, const float* target, int batc
         const float* a = l == 0 ? in : n->act[l];
         const int O = n->dout[l], C = n->din[l];
         const dim3 wg((C + 15) / 16, (O + 15) / 16, std::min(B, 16));
-        const int ld = staged_length(WG_N, B * m, m, n->K) | 1;
+        const int ld = staged_length(WG_N, (long)B * m, m, n->K) | 1;
         const size_t smem = (size_t)16 * (WG_N + 1 + ld) * sizeof(float);
         FDE_TRY(allow_smem((const void*)conv_wgrad_kernel, 227 * 1024));
         conv_wgrad_kernel<<<wg, 256, smem, n->stream>>>(g, O, a, C, n->K, m, B, n->g + n->woff[l], n->g + n->boff[l],
