@@ -141,9 +141,45 @@ conv_kernel(const TI* __restrict__ x, int Q, const TW* __restrict__ W, const flo
     }
 }
 
-// dW[o][c][k] += sum_{b in group} sum_x g[b][o][x] a[b][c][x + k - K/2] and, in the CTAs of
-// the first channels, db[o] += sum g; one thread per (o, c) of a 16 x 16 tile, the flattened
-// positions of the batch split over gridDim.z groups of whole samples (atomic accumulation).
+// db[o] = sum g of up to 16 channels o0 .., `each` of them a CTA: a channel's terms are shared
+// among the lanes of 8 / each warps (one at least) and added in fours in FP32, the rest in FP64 and in a fixed
+// order, so db repeats to the bit and its rounding does not grow with the batch.
+__device__ __forceinline__ void bias_sums(const float* __restrict__ g, int O, int m, int B, int o0, int cta, int each,
+                                          float* __restrict__ db) {
+    __shared__ double red[8];
+    const long N = (long)B * m;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int wpc = max(8 / each, 1), part = warp % wpc, last = min(min((cta + 1) * each, 16), O - o0);
+    double v = 0.0;
+    for (int c = cta * each + warp / wpc; c < last; c += 8 / wpc) {
+        v = 0.0;
+        for (long n = 32 * part + lane; n < N; n += 8 * 32 * wpc) {
+            float s[2] = {0.f, 0.f};
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                const long q = n + 32 * wpc * j;
+                if (q < N) s[j / 4] += g[cv_offset(cv_tile(q, m), O, o0 + c, m, 0)];
+            }
+            v += (double)s[0];
+            v += (double)s[1];
+        }
+        for (int off = 16; off; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+        if (wpc == 1 && lane == 0) db[o0 + c] = (float)v;
+    }
+    if (wpc == 1) return;
+    if (lane == 0) red[warp] = v;
+    __syncthreads();
+    const int c = cta * each + warp / wpc;  // every channel of the CTA was taken at once
+    if (part == 0 && lane == 0 && c < last) {
+        for (int w = 1; w < wpc; ++w) v += red[warp + w];
+        db[o0 + c] = (float)v;
+    }
+}
+
+// dW[o][c][k] += sum_{b in group} sum_x g[b][o][x] a[b][c][x + k - K/2]; one thread per (o, c)
+// of a 16 x 16 tile, the flattened positions of the batch split over gridDim.z groups of whole
+// samples (atomic accumulation).  The CTAs behind the groups form the bias gradients db: last in the
+// grid, where they join SMs that have fewer of the others.
 // 10 us a layer at 64 channels, 16 modes, 32 samples, against 22 (64-position tiles of single
 // samples) and 10 for the bias sums in a launch of their own.
 constexpr int WG_N = 64;  // positions staged at once
@@ -154,12 +190,17 @@ conv_wgrad_kernel(const float* __restrict__ g, int O, const float* __restrict__ 
     float* s_g = wg_smem;                  // [16][WG_N + 1]
     float* s_a = wg_smem + 16 * (WG_N + 1);  // [16][ld]
     const int o0 = blockIdx.y * 16, c0 = blockIdx.x * 16;
+    const int groups = gridDim.z - 1;
+    if ((int)blockIdx.z == groups) {
+        bias_sums(g, O, m, B, o0, blockIdx.x, (16 + gridDim.x - 1) / gridDim.x, db);
+        return;
+    }
     const int ol = threadIdx.x / 16, cl = threadIdx.x % 16;
     const int h = K / 2;
-    float acc[CV_KMAX], sum = 0.f;
+    float acc[CV_KMAX];
 #pragma unroll
     for (int k = 0; k < CV_KMAX; ++k) acc[k] = 0.f;
-    const int per = (B + gridDim.z - 1) / gridDim.z;  // samples of this group
+    const int per = (B + groups - 1) / groups;  // samples of this group
     const int lo = blockIdx.z * per, hi = min(B, lo + per);
     const long total = lo < hi ? (long)(hi - lo) * m : 0;
     CvTile tile{lo, 0};
@@ -178,7 +219,6 @@ conv_wgrad_kernel(const float* __restrict__ g, int O, const float* __restrict__ 
         const float* ap = s_a + cl * ld;
         for (int t = 0; t < count; ++t) {
             const float gv = s_g[ol * (WG_N + 1) + t];
-            sum += gv;
 #pragma unroll
             for (int k = 0; k < CV_KMAX; ++k)
                 if (k < K) acc[k] += gv * ap[k];
@@ -195,7 +235,6 @@ conv_wgrad_kernel(const float* __restrict__ g, int O, const float* __restrict__ 
     }
     if (o0 + ol < O && c0 + cl < C)
         for (int k = 0; k < K; ++k) atomicAdd(dW + ((size_t)(o0 + ol) * C + c0 + cl) * K + k, acc[k]);
-    if (c0 + cl == 0 && o0 + ol < O) atomicAdd(db + o0 + ol, sum);
 }
 
 // g = 2 (y - t) / N, loss += sum (y - t)^2 / N
@@ -517,10 +556,10 @@ int fde_nop_loss_grad(fde_nop* n, const float* in, const float* target, int batc
     for (int l = L - 1; l >= 0; --l) {
         const float* a = l == 0 ? in : n->act[l];
         const int O = n->dout[l], C = n->din[l];
-        const dim3 wg((C + 15) / 16, (O + 15) / 16, std::min(B, 16));
+        const dim3 wg((C + 15) / 16, (O + 15) / 16, std::min(B, 16) + 1);
         const int ld = staged_length(WG_N, (long)B * m, m, n->K) | 1;
         const size_t smem = (size_t)16 * (WG_N + 1 + ld) * sizeof(float);
-        FDE_TRY(allow_smem((const void*)conv_wgrad_kernel, 227 * 1024));
+        FDE_TRY(allow_smem((const void*)conv_wgrad_kernel, smem));
         conv_wgrad_kernel<<<wg, 256, smem, n->stream>>>(g, O, a, C, n->K, m, B, n->g + n->woff[l], n->g + n->boff[l],
                                                         ld);
         FDE_LAUNCH_CHECK("conv_wgrad_kernel");
