@@ -600,56 +600,72 @@ __global__ void scale_batched(const InstDev* __restrict__ I, const int* __restri
         for (int i = threadIdx.x; i <= restart; i += blockDim.x) d.gv[i] = i == 0 ? nr : 0.0;
 }
 
+// Sums of x and y over the CTA before this thread; x and y become the sums over the CTA.
+struct GsScan {
+    int x;
+    long y;
+};
+__device__ __forceinline__ GsScan gs_scan(int& x, long& y) {
+    __shared__ int wx[GS_WARPS];
+    __shared__ long wy[GS_WARPS];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int ix = x;
+    long iy = y;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+        const int ux = __shfl_up_sync(0xffffffffu, ix, off);
+        const long uy = __shfl_up_sync(0xffffffffu, iy, off);
+        if (lane >= off) {
+            ix += ux;
+            iy += uy;
+        }
+    }
+    __syncthreads();  // the words may still be read from the call before
+    if (lane == 31) {
+        wx[warp] = ix;
+        wy[warp] = iy;
+    }
+    __syncthreads();
+    GsScan before{ix - x, iy - y};
+    x = 0;
+    y = 0;
+    for (int w = 0; w < GS_WARPS; ++w) {
+        if (w < warp) {
+            before.x += wx[w];
+            before.y += wy[w];
+        }
+        x += wx[w];
+        y += wy[w];
+    }
+    return before;
+}
+
 // The Gram-Schmidt step j of every live instance in one cooperative launch.  The CTAs are
 // shared out in proportion to the instances' lengths, one at least; with more live instances
 // than CTAs each CTA takes instances of its own, alone.  Every CTA works the shares out for
-// itself: an instance takes part if it is live or has already finished this step (a CTA that
+// itself, by a scan over the list in pieces of a CTA's threads, so the list may have any length.  An
+// instance takes part if it is live or has already finished this step (a CTA that
 // starts late may see the flags its step has left: ctl[1] = j + 1 is written before ctl[0]).
 // An instance leaves the cycle on the device: tolerance met (Givens estimate), maxit,
 // breakdown, or a non-finite value.
 template <int KC, int E>
 __global__ void __launch_bounds__(RED_THREADS, 1)
 gs_batched(const InstDev* __restrict__ I, const int* __restrict__ act, int nact, int j, int ldh, int reorth,
-           double tol, int maxit, int* __restrict__ err, int stage_doubles) {
+           double tol, int maxit, int* __restrict__ err) {
     extern __shared__ __align__(16) unsigned char gs_smem[];
     double* stage = reinterpret_cast<double*>(gs_smem);
-    double* len = stage + stage_doubles;  // length of each listed instance, 0: not taking part
-    __shared__ int sh_inst, sh_cta, sh_G, sh_live;
-    for (int a = threadIdx.x; a < nact; a += RED_THREADS) {
+    __shared__ int sh_inst, sh_cta, sh_G;
+    __shared__ int mine[RED_THREADS];  // a piece's entries that this CTA takes alone
+    // length of entry a of the list, 0 if it takes no part
+    const auto length = [&](int a) -> long {
+        if (a >= nact) return 0;
         const InstDev& d = I[act[a]];
         volatile int* c = d.ctl;
         bool on = c[0] != 0;
         __threadfence();
         if (!on) on = c[1] == j + 1;
-        len[a] = on ? (double)d.n : 0.0;
-    }
-    __syncthreads();
-    const int B = gridDim.x;
-    if (threadIdx.x == 0) {
-        double total = 0.0;
-        int live = 0;
-        for (int a = 0; a < nact; ++a) {
-            total += len[a];
-            live += len[a] > 0.0;
-        }
-        sh_live = live;
-        sh_inst = -1;
-        if (live <= B) {
-            int at = 0, rest = live;
-            for (int a = 0; a < nact; ++a) {
-                if (len[a] == 0.0) continue;
-                --rest;  // at most what leaves one for each of the rest
-                const int g = min(1 + (int)((double)(B - live) * (len[a] / total)), B - at - rest);
-                if ((int)blockIdx.x >= at && (int)blockIdx.x < at + g) {
-                    sh_inst = a;
-                    sh_cta = blockIdx.x - at;
-                    sh_G = g;
-                }
-                at += g;
-            }
-        }
-    }
-    __syncthreads();
+        return on ? d.n : 0;
+    };
     const auto step = [&](int a, int cta, int G) {
         const InstDev& d = I[act[a]];
         GsArgs A{d.V, d.V + (size_t)(j + 1) * d.n, d.n, j + 1, ldh, reorth, d.H, d.cs, d.sn, d.gv, d.scal,
@@ -665,16 +681,57 @@ gs_batched(const InstDev* __restrict__ I, const int* __restrict__ act, int nact,
             if (bad || col.est <= tol * sqrt(d.scal[131]) || its >= maxit || fabs(col.hnext) <= 1e-300) c[0] = 0;
         });
     };
-    if (sh_live <= B) {
+    const int B = gridDim.x, me = blockIdx.x;
+    int live = 0;
+    long total = 0;
+    for (int a = threadIdx.x; a < nact; a += RED_THREADS) {
+        const long n = length(a);
+        live += n > 0;
+        total += n;
+    }
+    gs_scan(live, total);
+    if (threadIdx.x == 0) sh_inst = -1;
+    int first = 0;  // live entries before the piece, and their length
+    long cum = 0;
+    if (live > 0 && live <= B) {
+        for (int a0 = 0; a0 < nact; a0 += RED_THREADS) {
+            const int a = a0 + threadIdx.x;
+            const long n = length(a);
+            int px = n > 0;
+            long py = n;
+            const GsScan before = gs_scan(px, py);
+            if (n > 0) {  // CTAs [at, end)
+                const long i = first + before.x, c = cum + before.y;
+                const int at = (int)(i + (B - live) * c / total), end = (int)(i + 1 + (B - live) * (c + n) / total);
+                if (me >= at && me < end) {
+                    sh_inst = a;
+                    sh_cta = me - at;
+                    sh_G = end - at;
+                }
+            }
+            __syncthreads();
+            if (sh_inst >= 0) break;
+            first += px;
+            cum += py;
+        }
         if (sh_inst >= 0) step(sh_inst, sh_cta, sh_G);
-    } else {
-        int i = 0;
-        for (int a = 0; a < nact; ++a) {
-            if (len[a] == 0.0) continue;
-            if (i++ % B == (int)blockIdx.x) {
-                step(a, 0, 1);
+    } else if (live > B) {
+        for (int a0 = 0; a0 < nact; a0 += RED_THREADS) {
+            const int a = a0 + threadIdx.x;
+            const long n = length(a);
+            int px = n > 0;
+            long py = n;
+            const GsScan before = gs_scan(px, py);
+            const int i = first + before.x;
+            // entries i = me, me + B, ..: numbered within the piece
+            const int skip = (me - first % B + B) % B;  // live entries of the piece before the first of them
+            if (n > 0 && i % B == me) mine[(before.x - skip) / B] = a;
+            __syncthreads();
+            for (int q = 0; q * B + skip < px; ++q) {
+                step(mine[q], 0, 1);
                 __syncthreads();
             }
+            first += px;
         }
     }
 }
@@ -767,11 +824,9 @@ int launch_gs_batched(const InstDev* I, const int* act, int nact, int j, int ldh
                        : k <= 24 ? (const void*)gs_batched<24, 2>
                        : k <= 32 ? (const void*)gs_batched<32, 1>
                                  : (const void*)gs_batched<64, 1>;
-    const size_t stage = gs_stage_bytes(k, k <= 24 ? 2 : 1);
-    int stage_doubles = (int)(stage / sizeof(double));
-    const size_t smem = stage + (size_t)nact * sizeof(double);
+    const size_t smem = gs_stage_bytes(k, k <= 24 ? 2 : 1);
     FDE_TRY(allow_smem((const void*)kern, smem));
-    void* args[] = {&I, &act, &nact, &j, &ldh, &reorth, &tol, &maxit, &err, &stage_doubles};
+    void* args[] = {&I, &act, &nact, &j, &ldh, &reorth, &tol, &maxit, &err};
     FDE_CUDA_TRY(cudaLaunchCooperativeKernel(kern, dim3(ctas), dim3(RED_THREADS), args, smem, st));
     FDE_LAUNCH_CHECK("gs_batched");
     return FDE_OK;
