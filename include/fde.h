@@ -469,7 +469,7 @@ int fde_tune_query(int kernel, int mp, int nb, int precision, int* variant);
  * process-wide cache of at most 16 GiB, keyed by exact size, so that the next
  * problem of the same shape reuses them without cudaMalloc / cudaFree; the cache
  * is also emptied for a device when an allocation on it fails.  Pinned host blocks (at
- * most 64 of 256 KB) and the side streams of the block LU (at most 8 sets) of destroyed
+ * most 16 MB) and the side streams of the block LU (at most 8 sets) of destroyed
  * problems are kept likewise.  This call frees every cached block on every device, the
  * pinned blocks and the streams; what live problems use is not touched.
  * Thread-safe.  Makes no CUDA call when the cache is empty.  Errors: FDE_ERR_CUDA

@@ -549,35 +549,28 @@ int fde_problem_create(const fde_problem_desc* d, void* stream, fde_problem** ou
             if (!std::isfinite(d->f[i])) return bad("f is not finite");
     }
 
-    // Pinned block: scalars [0, 8), step outcomes [8, 24), check flag [24], status words
-    // [64, 64 + 264), then the upload: A and B bands, d+, d-, zeroed scalars and counters, and the
-    // band's row starts.
-    constexpr size_t PIN_INFO = 64, PIN_UP = PIN_INFO + 264, NSCAL = 256, NCNT = 2;
-    static_assert(8 * sizeof(double) + Problem::STEP_RING * sizeof(Problem::StepOutcome) <= 24 * sizeof(double) &&
-                      (FDE_MAX_S / 2 + 2) * sizeof(int) <= 264 * sizeof(double) &&
-                      (PIN_UP + 2 * (FDE_MAX_S + 1) * (FDE_MAX_MU + 1) + 2 * FDE_MAX_M + NSCAL + NCNT + 4) * sizeof(double) +
-                              (FDE_MAX_S + 1) * sizeof(int) <= PINNED_BYTES,
+    const PinnedLayout pl(P.m, P.s, P.mu);
+    static_assert(PinnedLayout::OUTCOMES * sizeof(double) + Problem::STEP_RING * sizeof(Problem::StepOutcome) <=
+                      PinnedLayout::FLAG * sizeof(double),
                   "the pinned block's layout");
     void* pin = nullptr;
-    TRY(pinned_alloc(&pin));
+    TRY(pinned_alloc(pl.bytes, &pin));
     P.h_pin = static_cast<double*>(pin);
-    P.h_step = reinterpret_cast<Problem::StepOutcome*>(P.h_pin + 8);
-    P.h_info = reinterpret_cast<int*>(P.h_pin + PIN_INFO);
-    double* up = P.h_pin + PIN_UP;
-    const size_t up_doubles = 2 * band + 2 * m + NSCAL + NCNT;
-    const size_t up_bytes = up_doubles * sizeof(double) + rows * sizeof(int);
-    TRY(dalloc(&P.arena[0], up_bytes));
-    P.d_a = reinterpret_cast<double*>(P.arena[0]);
-    P.d_b = P.d_a + band;
-    P.d_dplus = P.d_b + band;
-    P.d_dminus = P.d_dplus + m;
-    P.d_scal = P.d_dminus + m;
-    P.d_counter = reinterpret_cast<unsigned int*>(P.d_scal + NSCAL);
-    P.d_start = reinterpret_cast<int*>(P.d_scal + NSCAL + NCNT);
-    double *ha = up, *hb = up + band, *hp = hb + band, *hm = hp + m;
-    int* hst = reinterpret_cast<int*>(up + up_doubles);
+    P.h_step = reinterpret_cast<Problem::StepOutcome*>(P.h_pin + pl.OUTCOMES);
+    P.h_info = reinterpret_cast<int*>(P.h_pin + pl.INFO);
+    TRY(dalloc(&P.arena[0], pl.up_bytes));
+    const auto uploaded = [&](size_t o) { return reinterpret_cast<double*>(P.arena[0]) + (o - pl.a); };
+    P.d_a = uploaded(pl.a);
+    P.d_b = uploaded(pl.b);
+    P.d_dplus = uploaded(pl.dplus);
+    P.d_dminus = uploaded(pl.dminus);
+    P.d_scal = uploaded(pl.scal);
+    P.d_counter = reinterpret_cast<unsigned int*>(uploaded(pl.cnt));
+    P.d_start = reinterpret_cast<int*>(uploaded(pl.start));
+    double *ha = P.h_pin + pl.a, *hb = P.h_pin + pl.b, *hp = P.h_pin + pl.dplus, *hm = P.h_pin + pl.dminus;
+    int* hst = reinterpret_cast<int*>(P.h_pin + pl.start);
     std::memset(ha, 0, 2 * band * sizeof(double));
-    std::memset(hm + m, 0, (NSCAL + NCNT) * sizeof(double));
+    std::memset(P.h_pin + pl.scal, 0, (pl.NSCAL + pl.NCNT) * sizeof(double));
     // BVM band rows t = 1..s (eqs. (1.7)-(1.9)); row 0 is the initial condition.
     ha[0] = 1.0;
     hst[0] = 0;
@@ -637,14 +630,14 @@ int fde_problem_create(const fde_problem_desc* d, void* stream, fde_problem** ou
     // Everything is on the device, and the caller's arrays are done with, when the call
     // returns (other streams may then read them): one wait at the end, after the checks'
     // copies.
-    int* flag = reinterpret_cast<int*>(P.h_pin + 24);
+    int* flag = reinterpret_cast<int*>(P.h_pin + pl.FLAG);
     *flag = 0;
     const double* src[2] = {P.timevar ? nullptr : d->dplus, P.timevar ? nullptr : d->dminus};
     const double c[2] = {d->dplus_c, d->dminus_c};
     double *host[2] = {hp, hm}, *dev[2] = {P.d_dplus, P.d_dminus};
     for (int w = 0; w < 2; ++w)
         for (size_t i = 0; i < m; ++i) host[w][i] = d->device_ptrs ? c[w] : at(src[w], c[w], i);
-    CUTRY(cudaMemcpyAsync(P.arena[0], up, up_bytes, cudaMemcpyHostToDevice, st));
+    CUTRY(cudaMemcpyAsync(P.arena[0], ha, pl.up_bytes, cudaMemcpyHostToDevice, st));
     for (int w = 0; w < 2; ++w) {
         if (!src[w] || !d->device_ptrs) continue;
         CUTRY(cudaMemcpyAsync(dev[w], src[w], m * sizeof(double), kind, st));

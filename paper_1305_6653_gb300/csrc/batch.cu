@@ -39,7 +39,7 @@ struct fde_batch {
     int* d_kvec = nullptr;
     int* d_err = nullptr;
     double* d_gather = nullptr;
-    void* h_pin = nullptr;       // the pinned block behind the four below, when it came from the cache
+    void* h_pin = nullptr;       // the pinned block behind the four below
     double* h_gather = nullptr;  // pinned
     int* h_act = nullptr;        // pinned
     int* h_kvec = nullptr;       // pinned
@@ -153,8 +153,7 @@ void fde_batch_destroy(fde_batch* b) {
     for (fde_problem* p : b->probs) fde_problem_destroy(p);
     void* dev[] = {b->d_blk, b->d_inst, b->d_pack, b->d_rhat_shared};
     for (void* d : dev) dev_free(d);
-    if (b->h_pin) pinned_free(b->h_pin);
-    else if (b->h_gather) cudaFreeHost(b->h_gather);
+    pinned_free(b->h_pin);
     for (auto& kv : b->cycle_graphs) cudaGraphExecDestroy(kv.second.first);
     if (b->cap_stream) cudaStreamDestroy(b->cap_stream);
     delete b;
@@ -189,23 +188,13 @@ int fde_batch_create(const fde_problem_desc* descs, int count, void* stream, fde
         b->max_n = std::max(b->max_n, P.n);
     }
     // device words: instance descriptors, gathered scalars, round list, cycle lengths, control
-    // words, error flag; pinned counterparts of the middle four, from the cache of blocks if they fit
+    // words, error flag; pinned counterparts of the middle four
     const size_t c = count, words = c * sizeof(InstDev) + 5 * c * sizeof(double) + (6 * c + 1) * sizeof(int);
     unsigned char* w = nullptr;
     int rc = dev_alloc((void**)&w, words);
-    const size_t host = 5 * c * sizeof(double) + 6 * c * sizeof(int);
-    void* pin = nullptr;
-    if (!rc) {
-        if (host <= PINNED_BYTES) {
-            rc = pinned_alloc(&pin);
-            b->h_pin = pin;
-        } else if (cudaMallocHost(&pin, host) != cudaSuccess) {
-            pin = nullptr;
-            rc = FDE_ERR_ALLOC;
-        }
-    }
+    if (!rc) rc = pinned_alloc(5 * c * sizeof(double) + 6 * c * sizeof(int), &b->h_pin);
     b->d_inst = reinterpret_cast<InstDev*>(w);
-    b->h_gather = static_cast<double*>(pin);
+    b->h_gather = static_cast<double*>(b->h_pin);
     if (rc) {
         fde_batch_destroy(b);
         return set_error(FDE_ERR_ALLOC, "batch allocation failed");

@@ -37,9 +37,11 @@ std::deque<Block> g_cache;                     // freed blocks, oldest first
 size_t g_cached = 0;                           // bytes held in g_cache
 std::unordered_map<void*, Block> g_live;       // blocks handed out
 
-constexpr size_t PINNED_CACHE_LIMIT = 64;      // blocks (16 MB)
+constexpr size_t PINNED_CACHE_LIMIT = 16 << 20;  // bytes
 constexpr size_t LU_CACHE_LIMIT = 8;
-std::vector<void*> g_pinned;                   // returned pinned blocks
+std::vector<void*> g_pinned[PINNED_CLASSES];   // returned pinned blocks by size
+size_t g_pinned_cached = 0;                    // bytes held in g_pinned
+std::unordered_map<void*, int> g_pinned_live;  // blocks handed out: their class
 std::vector<LuStreams> g_lu;                   // returned LU streams
 
 void release_cached(int dev) {  // g_mu held
@@ -111,22 +113,28 @@ void dev_free(void* p) {
 
 // A cache hit costs the problem that starts 150 us less than cudaMallocHost, and the one that
 // ends 190 us less than cudaFreeHost, which waits for the device.
-int pinned_alloc(void** p) {
-    {
+int pinned_alloc(size_t bytes, void** p) {
+    const int c = pinned_class(bytes);
+    if (c < PINNED_CLASSES) {
+        bytes = PINNED_LEAST << c;
         std::lock_guard<std::mutex> lock(g_mu);
-        if (!g_pinned.empty()) {
-            *p = g_pinned.back();
-            g_pinned.pop_back();
+        if (!g_pinned[c].empty()) {
+            *p = g_pinned[c].back();
+            g_pinned[c].pop_back();
+            g_pinned_cached -= bytes;
+            g_pinned_live[*p] = c;
             return FDE_OK;
         }
     }
     *p = nullptr;
-    const cudaError_t e = cudaHostAlloc(p, PINNED_BYTES, cudaHostAllocPortable);
+    const cudaError_t e = cudaHostAlloc(p, bytes, cudaHostAllocPortable);
     if (e != cudaSuccess) {
         *p = nullptr;
         cudaGetLastError();
         return set_error(FDE_ERR_ALLOC, std::string("cudaHostAlloc failed: ") + cudaGetErrorString(e));
     }
+    std::lock_guard<std::mutex> lock(g_mu);
+    g_pinned_live[*p] = c;
     return FDE_OK;
 }
 
@@ -134,8 +142,12 @@ void pinned_free(void* p) {
     if (!p) return;
     {
         std::lock_guard<std::mutex> lock(g_mu);
-        if (g_pinned.size() < PINNED_CACHE_LIMIT) {
-            g_pinned.push_back(p);
+        const auto it = g_pinned_live.find(p);
+        const int c = it->second;
+        g_pinned_live.erase(it);
+        if (c < PINNED_CLASSES && g_pinned_cached + (PINNED_LEAST << c) <= PINNED_CACHE_LIMIT) {
+            g_pinned[c].push_back(p);
+            g_pinned_cached += PINNED_LEAST << c;
             return;
         }
     }
@@ -212,11 +224,14 @@ int allow_smem(const void* kern, size_t bytes) {
 int dev_release_cached() {
     std::lock_guard<std::mutex> lock(g_mu);
     cudaError_t first = cudaSuccess;
-    for (void* p : g_pinned) {
-        const cudaError_t e = cudaFreeHost(p);
-        if (e != cudaSuccess && first == cudaSuccess) first = e;
+    for (std::vector<void*>& blocks : g_pinned) {
+        for (void* p : blocks) {
+            const cudaError_t e = cudaFreeHost(p);
+            if (e != cudaSuccess && first == cudaSuccess) first = e;
+        }
+        blocks.clear();
     }
-    g_pinned.clear();
+    g_pinned_cached = 0;
     for (LuStreams& l : g_lu) lu_streams_destroy(l);
     g_lu.clear();
     for (const Block& b : g_cache) {

@@ -11,6 +11,7 @@
 
 #include "../../include/fde.h"
 #include "bfp_fft.cuh"
+#include "pinned_layout.h"
 
 namespace fde {
 
@@ -194,7 +195,7 @@ struct Problem {
     int h_start[FDE_MAX_S + 1];
     double h_a_main[FDE_MAX_MU + 1], h_b_main[FDE_MAX_MU + 1];
 
-    // Pinned block (PINNED_BYTES): scalars and step outcomes the kernels write, the factor's
+    // Pinned block (PinnedLayout): scalars and step outcomes the kernels write, the factor's
     // status words, and the upload of the small arrays, which stays (h_dplus, h_dminus: the
     // coefficients, when they do not vary in time)
     double* h_pin = nullptr;
@@ -347,10 +348,9 @@ int dev_alloc(void** p, size_t bytes);
 void dev_free(void* p);
 // Frees every cached block (blocks in use are not affected).
 int dev_release_cached();
-// Pinned host blocks of PINNED_BYTES, from a bounded cache as well (the caller makes sure that
-// no queued GPU work uses a block it returns).
-constexpr size_t PINNED_BYTES = 256 * 1024;
-int pinned_alloc(void** p);
+// Pinned host blocks of at least `bytes`, from a bounded cache as well (the caller makes sure
+// that no queued GPU work uses a block it returns).
+int pinned_alloc(size_t bytes, void** p);
 void pinned_free(void* p);
 // The side streams and events of a tensor-core LU, from a bounded cache as well.
 int lu_streams_take(LuStreams* s);
