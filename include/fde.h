@@ -426,7 +426,7 @@ long long fde_launch_count(void);
 /* ---- launch-shape autotuner ----------------------------------------------
  * Two kernel families have variants that compute bit-identical results and differ
  * only in how the work is spread over threads: the space-time matvec (threads per
- * time row: 1024, 512, 256, i.e. one, two or more CTAs per SM) and the block
+ * time row: 512, 256, 128, i.e. one, two or more CTAs per SM) and the block
  * triangular solves (FP32 factors: 7, 14, 12 or 10 warps that apply strips streamed by tensor-map
  * copies; a bfloat16 copy: 512 threads with 4 rows per register buffer, 384 with 7 or 640 with
  * 3, a fourth setting launches the first; FP64 factors have one form, which every setting
@@ -435,7 +435,9 @@ long long fde_launch_count(void);
  * events on the problem's stream and keeps the fastest for that shape (m_p, s or
  * s/2+1 blocks, precision) in a process-wide table, which is also appended to a text
  * file ($FDE_TUNE_CACHE, default $HOME/.cache/libfde_tune.txt; FDE_TUNE_CACHE=""
- * keeps it in memory) and read back by later processes. */
+ * keeps it in memory) and read back by later processes.  A measured line names the list of
+ * variants it was measured with; where the library has another list by now, the line is
+ * ignored and the shape measured again. */
 #define FDE_TUNE_MATVEC 0
 #define FDE_TUNE_TRSV 1
 /* The interior trailing update of the tensor-core block LU (FDE_TF32 / FDE_BF16 /

@@ -5,6 +5,7 @@
 // (one line per shape) and read back by later processes.
 #include <cstdio>
 #include <cstdlib>
+#include <cstring>
 #include <map>
 #include <mutex>
 #include <string>
@@ -40,6 +41,11 @@ std::string default_path() {
     return home ? std::string(home) + "/.cache/libfde_tune.txt" : std::string();
 }
 
+// Number of a family's list of variants: a line that was written after a measurement says which
+// list its variant is of, and counts only for that list (a variant's number does not say how
+// it is launched, and a list may change).  To be raised when a family's variants change.
+int list_number(int kernel) { return kernel == FDE_TUNE_LU ? 1 : 2; }
+
 void load_locked(TuneState& s) {
     if (s.loaded) return;
     s.loaded = true;
@@ -48,11 +54,15 @@ void load_locked(TuneState& s) {
     FILE* f = std::fopen(s.path.c_str(), "r");
     if (!f) return;
     char line[512], name[32];
-    int k, mp, nb, prec, v;
-    while (std::fgets(line, sizeof line, f))  // "name kernel mp nb precision variant [# measured ms ...]"
-        if (std::sscanf(line, "%31s %d %d %d %d %d", name, &k, &mp, &nb, &prec, &v) == 6 && k >= 0 &&
-            k < FDE_TUNE_KERNELS && v >= 0 && v < tune_variants(k))
-            s.table[{k, mp, nb, prec}] = v;
+    int k, mp, nb, prec, v, list;
+    while (std::fgets(line, sizeof line, f)) {  // "name kernel mp nb precision variant [# list n: measured ms ...]"
+        if (std::sscanf(line, "%31s %d %d %d %d %d", name, &k, &mp, &nb, &prec, &v) != 6 || k < 0 ||
+            k >= FDE_TUNE_KERNELS || v < 0 || v >= tune_variants(k))
+            continue;
+        const char* measured = std::strchr(line, '#');  // none: written by hand
+        if (measured && (std::sscanf(measured, "# list %d:", &list) != 1 || list != list_number(k))) continue;
+        s.table[{k, mp, nb, prec}] = v;
+    }
     std::fclose(f);
 }
 
@@ -99,9 +109,9 @@ void tune_store(int kernel, int mp, int nb, int prec, int variant, const float* 
         f = std::fopen(s.path.c_str(), "a");
         if (!f) return;  // the table stays in memory only
     }
-    std::fprintf(f, "%s %d %d %d %d %d #", kernel == FDE_TUNE_MATVEC ? "matvec" : kernel == FDE_TUNE_TRSV ? "trsv" : "lu",
-                 kernel, mp, nb, prec,
-                 variant);
+    std::fprintf(f, "%s %d %d %d %d %d # list %d:",
+                 kernel == FDE_TUNE_MATVEC ? "matvec" : kernel == FDE_TUNE_TRSV ? "trsv" : "lu", kernel, mp, nb, prec,
+                 variant, list_number(kernel));
     for (int i = 0; ms && i < tune_variants(kernel); ++i) std::fprintf(f, " %.4f", ms[i]);
     std::fprintf(f, " ms\n");
     std::fclose(f);
