@@ -131,16 +131,24 @@ BFP_FN long long to_fixed(double v, int emax) {
     long long r = s > 62 ? 0 : (long long)(s > 0 ? (sig + (1ull << (s - 1))) >> s : sig);
     return (long long)u < 0 ? -r : r;
 }
-// the double nearest to v (v an integer); integer operations only
-BFP_FN double to_double(long long v) {
+// the double nearest to v 2^e (v an integer, |e| <= 900); integer operations only
+BFP_FN double to_double(long long v, int e = 0) {
     const unsigned long long a = v < 0 ? 0ull - (unsigned long long)v : (unsigned long long)v;
     const int n = lead(a);
     if (n == 64) return 0.0;
     const unsigned long long m = a << n;  // leading bit at 63
     // significand without its leading bit, plus the rounding bit (ties upward; a carry
     // runs into the exponent, as it should)
-    const unsigned long long b = ((unsigned long long)(1023 + 63 - n - 1) << 52) + (m >> 11) + ((m >> 10) & 1);
+    const unsigned long long b = ((unsigned long long)(1023 + 63 - n - 1 + e) << 52) + (m >> 11) + ((m >> 10) & 1);
     return double_of(b | (v < 0 ? 0x8000000000000000ull : 0ull));
+}
+BFP_FN double power_of_two(int e) { return double_of((unsigned long long)(1023 + e) << 52); }  // |e| <= 1000
+// f = mantissa 2^exponent with 1 <= mantissa < 2; what is no positive normal number keeps exponent 0
+BFP_FN double mantissa(double f, int* exponent) {
+    const unsigned long long u = bits_of(f);
+    const int x = (int)(u >> 52);
+    *exponent = x > 0 && x < 0x7ff ? x - 1023 : 0;
+    return x > 0 && x < 0x7ff ? double_of((u & 0xfffffffffffffull) | 0x3ff0000000000000ull) : f;
 }
 
 // sqrt(1/2) in units of 2^-61

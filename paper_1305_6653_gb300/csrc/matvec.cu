@@ -288,20 +288,18 @@ __device__ __forceinline__ void bfp_row(int m, int logL, int mu, double h, const
 
     const double* dp = dplus + (size_t)row * dstride;  // MODE 1 with per-column coefficients
     const double* dm = dminus + (size_t)row * dstride;
-    // the row's scale, in two factors when it is extreme
-    int e = shifts - (bfp::BITS - 1 + 1023 - emax);
-    const bool extreme = e < -800 || e > 800;
-    double s2 = 1.0;
-    if (extreme) {
-        s2 = scalbn(1.0, e / 2);
-        e -= e / 2;
-    }
-    const double s1 = scalbn(MODE == 0 ? h * fac : fac, e);
+    // The row's scale: its power of two goes into the integers' conversion, so that d+, d- of any
+    // magnitude multiply numbers of the result's own; what is extreme of it is applied afterwards.
+    int ef;
+    const double f = bfp::mantissa(MODE == 0 ? h * fac : fac, &ef);
+    const int whole = shifts - (bfp::BITS - 1 + 1023 - emax) + ef;
+    const int e = min(max(whole, -900), 900), rest = whole - e;
+    const double s1 = bfp::power_of_two(rest / 2), s2 = bfp::power_of_two(rest - rest / 2);
     for (int i = tid; i < m; i += T) {
         const I2 v = buf[bfp::slot(i)];  // (imaginary, real)
-        double jz = dp[i] * bfp::to_double(v.y - v.x) + dm[i] * bfp::to_double(v.x + v.y);
-        if (extreme) jz *= s2;
-        y[(size_t)row * m + i] = MODE == 0 ? ubuf[i] - s1 * jz : s1 * jz;
+        double jz = dp[i] * bfp::to_double(v.y - v.x, e) + dm[i] * bfp::to_double(v.x + v.y, e);
+        if (rest != 0) jz = jz * s1 * s2;
+        y[(size_t)row * m + i] = MODE == 0 ? ubuf[i] - f * jz : f * jz;
     }
 }
 
