@@ -244,7 +244,11 @@ int fde_batch_factor(fde_batch* b, int precision);
  * out on the batch's stream before the call returns).  stats: host
  * array of count entries (may be NULL); ms_solve is the batch's total time.
  * Returns FDE_OK when every instance met the tolerance, else the first failing
- * code (each instance's own code is in stats[i].status). */
+ * code (each instance's own code is in stats[i].status).  The same batch gives the same bits
+ * each time; an instance's last bits depend on the other instances, though: a Gram-Schmidt step
+ * shares the SMs out by the lengths of the instances that are still live, which orders an instance's
+ * partial sums, and the CUDA-core block solves of a shared operator take 4 or 8 right-hand
+ * sides at once by their number. */
 int fde_batch_solve(fde_batch* b, const fde_pgmres_opts* opts, double* const* x_out, fde_stats* stats);
 
 /* Declare that every instance has the same operator M and preconditioner (m, s, alpha,

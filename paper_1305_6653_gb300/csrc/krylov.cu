@@ -643,7 +643,10 @@ __device__ __forceinline__ GsScan gs_scan(int& x, long& y) {
 // The Gram-Schmidt step j of every live instance in one cooperative launch.  The CTAs are
 // shared out in proportion to the instances' lengths, one at least; with more live instances
 // than CTAs each CTA takes instances of its own, alone.  Every CTA works the shares out for
-// itself, by a scan over the list in pieces of a CTA's threads, so the list may have any length.  An
+// itself, by a scan over the list in pieces of a CTA's threads, so the list may have any length.  (The
+// order of an instance's partial sums follows from the lengths of those that are live with it: the
+// same batch gives the same bits, another batch other last bits.  A fixed number of partial sums
+// an instance, 32 as there once were, would leave most SMs idle once few instances are live.)  An
 // instance takes part if it is live or has already finished this step (a CTA that
 // starts late may see the flags its step has left: ctl[1] = j + 1 is written before ctl[0]).
 // An instance leaves the cycle on the device: tolerance met (Givens estimate), maxit,
