@@ -301,7 +301,7 @@ int fde_batch_factor(fde_batch* b, int precision) {
     for (size_t i = 0; i < b->probs.size(); ++i) {
         Problem& P = *problem_of(b->probs[i]);
         int rc = ensure_factor_buffers(P, precision);
-        if (rc) return rc;
+        if (rc || (rc = ensure_tile_inverses(P, FDE_FP32, b->stream))) return rc;
         P.factored = false;
         P.precision = precision;
         // an instance set to FDE_STORAGE_BF16 (tensor-core LU, m_p a multiple of 128) gets the
@@ -343,6 +343,7 @@ int fde_batch_factor(fde_batch* b, int precision) {
             d.fac = (float*)P.d_fac + (size_t)k * 2 * P.mp * P.mp;
             d.dinv = (float2*)P.d_dinv + (size_t)k * P.mp;
             d.info = P.d_info + k;
+            d.tinv = (float*)P.d_tinv + (size_t)k * (P.mp / 32) * 4096;
             d.strips = strips ? strips + (size_t)k * 2 * P.mp * P.mp : nullptr;
             if (kind >= 0) {
                 d.apack = (unsigned char*)pack_total;  // offset, rebased below
@@ -381,6 +382,8 @@ int fde_batch_factor(fde_batch* b, int precision) {
                                  b->stream));
     FDE_CUDA_TRY(cudaMemsetAsync(b->d_err, 0, sizeof(int), b->stream));
     int rc = launch_lu_batched(b->d_blk, b->blk_mp, precision, b->d_err, b->stream);
+    // the inverses of the diagonal tiles, through which the solves apply them
+    if (!rc) rc = launch_tile_inverse_batched(b->d_blk, (int)blks.size(), b->max_mp, b->stream);
     if (rc) return rc;
     // pivots and bounded waits
     int derr = 0;
@@ -399,10 +402,8 @@ int fde_batch_factor(fde_batch* b, int precision) {
             if (infos[i][k])
                 return set_error(FDE_ERR_SINGULAR, "zero or non-finite pivot in instance " + std::to_string(i) +
                                                        ", block " + std::to_string(k));
-    // the FP32 inverses of the diagonal tiles, through which the solves apply them
     for (fde_problem* p : b->probs) {
         Problem& P = *problem_of(p);
-        if ((rc = launch_tile_inverse_fp32(P, b->stream))) return rc;
         if (P.strips_bf16) P.strips_ok = true;
     }
     for (fde_problem* p : b->probs) problem_of(p)->factored = true;

@@ -112,6 +112,7 @@ struct BlkDev {
     unsigned char* ipack;  // L11^{-1} (A') and U11^{-1} (B') tiles of the current panel
     int* info;
     unsigned short* strips;  // this block's bfloat16 strip-major copy (Re then Im), or NULL
+    float* tinv;  // this block's inverted 32 x 32 diagonal tiles
 };
 
 // ---------------------------------------------------------------------------
@@ -143,8 +144,10 @@ int launch_time_fft_inv(const Problem& P, const void* xhat, double* z, int prec,
 
 // lu.cu
 int launch_block_lu(Problem& P, int prec, cudaStream_t st);
-// The FP32 inverses of the 32 x 32 diagonal tiles of P's factors (P.d_tinv).
-int launch_tile_inverse_fp32(Problem& P, cudaStream_t st);
+// Room for the inverses of the 32 x 32 diagonal tiles of P's factors (P.d_tinv), and the inverses of
+// every block of a batch in FP32.
+int ensure_tile_inverses(Problem& P, int prec, cudaStream_t st);
+int launch_tile_inverse_batched(const BlkDev* d_blk, int nblocks, int max_mp, cudaStream_t st);
 int launch_block_trsv(const Problem& P, void* rhat, cudaStream_t st);
 // lu64.cu: the FP64 blocks (formed on st before): LU, block solves
 int launch_lu64(Problem& P, cudaStream_t st);
