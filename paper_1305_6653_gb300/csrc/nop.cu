@@ -37,17 +37,19 @@ __device__ __forceinline__ float ldf(const __half* p) { return __half2float(*p);
 __device__ __forceinline__ void stf(float* p, float v) { *p = v; }
 __device__ __forceinline__ void stf(__half* p, float v) { *p = __float2half_rn(v); }
 
-// stage channels q0 .. q0 + nq - 1 of x: one warp a channel, lanes along the slots (whose
-// sources do not depend on the channel)
+// stage nq channels of a batch of Q (nmax - nq zero rows behind them) from x, their first one in the
+// tile's first sample: one warp a channel, lanes along the slots (whose sources do not depend on
+// the channel)
 template <typename TI>
-__device__ __forceinline__ void cv_stage(const TI* __restrict__ x, int Q, int q0, int nq, int nmax, CvTile tile, int m,
+__device__ __forceinline__ void cv_stage(const TI* __restrict__ x, size_t sample, int nq, int nmax, int x0, int m,
                                          int h, int len, float* s, int ld) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     for (int t = lane; t < len; t += 32) {
-        const ptrdiff_t src = cv_source(tile, Q, m, h, t);
+        const CvPoint p = cv_slot(x0, m, h, t);
+        const TI* src = x + cv_offset(p, sample);
 #pragma unroll 4
         for (int c = warp; c < nmax; c += CV_WARPS)
-            s[c * ld + t] = src >= 0 && c < nq ? ldf(x + src + (size_t)(q0 + c) * m) : 0.f;
+            s[c * ld + t] = p.x >= 0 && c < nq ? ldf(src + (size_t)c * m) : 0.f;
     }
 }
 
@@ -85,7 +87,7 @@ conv_kernel(const TI* __restrict__ x, int Q, const TW* __restrict__ W, const flo
     }
     for (int q0 = 0; q0 < Q; q0 += QC) {
         const int nq = min(QC, Q - q0);
-        cv_stage(x, Q, q0, nq, nq, tile, m, h, len, s_in, ld);
+        cv_stage(x + ((size_t)tile.b0 * Q + q0) * m, (size_t)Q * m, nq, nq, tile.x0, m, h, len, s_in, ld);
         // 16 threads a row of weights: channel o's (TRANS = false) or input channel c's
         const int row = tid >> 4;
         if (TRANS) {
@@ -135,7 +137,7 @@ conv_kernel(const TI* __restrict__ x, int Q, const TW* __restrict__ W, const flo
         for (int w = 0; w < CV_WARPS; ++w) v += red[w * CV_TP * TN + e];
         if (bias) v += bias[p];
         if (relu) v = fmaxf(v, 0.f);
-        const size_t idx = cv_offset(tile, P, p, m, n);
+        const size_t idx = ((size_t)tile.b0 * P + p) * m + cv_offset(cv_position(tile.x0, m, n), (size_t)P * m);
         if (mask && !(mask[idx] > 0.f)) v = 0.f;
         stf(y + idx, v);
     }
@@ -148,6 +150,7 @@ __device__ __forceinline__ void bias_sums(const float* __restrict__ g, int O, in
                                           float* __restrict__ db) {
     __shared__ double red[8];
     const long N = (long)B * m;
+    const size_t sample = (size_t)O * m;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int wpc = max(8 / each, 1), part = warp % wpc, last = min(min((cta + 1) * each, 16), O - o0);
     double v = 0.0;
@@ -158,7 +161,10 @@ __device__ __forceinline__ void bias_sums(const float* __restrict__ g, int O, in
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
                 const long q = n + 32 * wpc * j;
-                if (q < N) s[j / 4] += g[cv_offset(cv_tile(q, m), O, o0 + c, m, 0)];
+                if (q < N) {
+                    const CvTile at = cv_tile(q, m);
+                    s[j / 4] += g[at.b0 * sample + (size_t)(o0 + c) * m + at.x0];
+                }
             }
             v += (double)s[0];
             v += (double)s[1];
@@ -177,22 +183,24 @@ __device__ __forceinline__ void bias_sums(const float* __restrict__ g, int O, in
 }
 
 // dW[o][c][k] += sum_{b in group} sum_x g[b][o][x] a[b][c][x + k - K/2]; one thread per (o, c)
-// of a 16 x 16 tile, the flattened positions of the batch split over gridDim.z groups of whole
-// samples (atomic accumulation).  The CTAs behind the groups form the bias gradients db: last in the
-// grid, where they join SMs that have fewer of the others.
+// of a 16 x 16 tile, the flattened positions of the batch split over `groups` of `per` (atomic
+// accumulation).  The CTAs behind the groups form the bias gradients db (before them they cost a large
+// gradient 10 %: fewer of the others start together).  Four of them a tile serve a batch of up to 1024
+// positions whose other CTAs fill the SMs; otherwise a channel gets a CTA of its own (a gradient at
+// 16 x 2047 positions, 16 channels: 640 us, 2390 with a warp a channel).
 // 10 us a layer at 64 channels, 16 modes, 32 samples, against 22 (64-position tiles of single
 // samples) and 10 for the bias sums in a launch of their own.
 constexpr int WG_N = 64;  // positions staged at once
 __global__ void __launch_bounds__(256)
 conv_wgrad_kernel(const float* __restrict__ g, int O, const float* __restrict__ a, int C, int K, int m, int B,
-                  float* __restrict__ dW, float* __restrict__ db, int ld) {
+                  int groups, long per, int bias_ctas, float* __restrict__ dW, float* __restrict__ db, int ld) {
     extern __shared__ float wg_smem[];
     float* s_g = wg_smem;                  // [16][WG_N + 1]
     float* s_a = wg_smem + 16 * (WG_N + 1);  // [16][ld]
     const int o0 = blockIdx.y * 16, c0 = blockIdx.x * 16;
-    const int groups = gridDim.z - 1;
-    if ((int)blockIdx.z == groups) {
-        bias_sums(g, O, m, B, o0, blockIdx.x, (16 + gridDim.x - 1) / gridDim.x, db);
+    if ((int)blockIdx.z >= groups) {
+        const int cta = (blockIdx.z - groups) * gridDim.x + blockIdx.x;
+        if (cta < bias_ctas) bias_sums(g, O, m, B, o0, cta, 16 / bias_ctas, db);
         return;
     }
     const int ol = threadIdx.x / 16, cl = threadIdx.x % 16;
@@ -200,20 +208,21 @@ conv_wgrad_kernel(const float* __restrict__ g, int O, const float* __restrict__ 
     float acc[CV_KMAX];
 #pragma unroll
     for (int k = 0; k < CV_KMAX; ++k) acc[k] = 0.f;
-    const int per = (B + groups - 1) / groups;  // samples of this group
-    const int lo = blockIdx.z * per, hi = min(B, lo + per);
-    const long total = lo < hi ? (long)(hi - lo) * m : 0;
-    CvTile tile{lo, 0};
+    const long lo = blockIdx.z * per, total = min((long)B * m, lo + per) - lo;
+    CvTile tile = cv_tile(lo, m);
+    const size_t sample_g = (size_t)O * m, sample_a = (size_t)C * m;
+    g += tile.b0 * sample_g + (size_t)o0 * m;  // the tile's first sample, the CTA's channels
+    a += tile.b0 * sample_a + (size_t)c0 * m;
     for (long n0 = 0; n0 < total; n0 += WG_N) {
         const int count = (int)min((long)WG_N, total - n0), len = cv_length(count, tile.x0, m, h);
         {
             const int t = threadIdx.x % WG_N;
-            const float* gr = g + cv_offset(tile, O, o0, m, t);
+            const float* gr = g + cv_offset(cv_position(tile.x0, m, t), sample_g);
 #pragma unroll
             for (int r = threadIdx.x / WG_N; r < 16; r += 256 / WG_N)
                 s_g[r * (WG_N + 1) + t] = o0 + r < O && t < count ? gr[(size_t)r * m] : 0.f;
         }
-        cv_stage(a, C, c0, min(16, C - c0), 16, tile, m, h, len, s_a, ld);
+        cv_stage(a, sample_a, min(16, C - c0), 16, tile.x0, m, h, len, s_a, ld);
         __syncthreads();
         int x = tile.x0;
         const float* ap = s_a + cl * ld;
@@ -228,9 +237,10 @@ conv_wgrad_kernel(const float* __restrict__ g, int O, const float* __restrict__ 
                 ap += 2 * h;
             }
         }
-        const int next = tile.x0 + WG_N;
-        tile.b0 += next / m;
-        tile.x0 = next % m;
+        const CvPoint next = cv_position(tile.x0, m, WG_N);
+        tile.x0 = next.x;
+        g += next.d * sample_g;
+        a += next.d * sample_a;
         __syncthreads();
     }
     if (o0 + ol < O && c0 + cl < C)
@@ -556,12 +566,15 @@ int fde_nop_loss_grad(fde_nop* n, const float* in, const float* target, int batc
     for (int l = L - 1; l >= 0; --l) {
         const float* a = l == 0 ? in : n->act[l];
         const int O = n->dout[l], C = n->din[l];
-        const dim3 wg((C + 15) / 16, (O + 15) / 16, std::min(B, 16) + 1);
+        const int groups = (int)std::min<long>(((long)B * m + 15) / 16, 16), cx = (C + 15) / 16, cy = (O + 15) / 16;
+        const long per = ((long)B * m + groups - 1) / groups;
+        const int bias_ctas = (long)B * m <= 1024 && cx * cy * groups > 152 ? 4 : 16;
+        const dim3 wg(cx, cy, groups + (bias_ctas + cx - 1) / cx);
         const int ld = staged_length(WG_N, (long)B * m, m, n->K) | 1;
         const size_t smem = (size_t)16 * (WG_N + 1 + ld) * sizeof(float);
         FDE_TRY(allow_smem((const void*)conv_wgrad_kernel, smem));
-        conv_wgrad_kernel<<<wg, 256, smem, n->stream>>>(g, O, a, C, n->K, m, B, n->g + n->woff[l], n->g + n->boff[l],
-                                                        ld);
+        conv_wgrad_kernel<<<wg, 256, smem, n->stream>>>(g, O, a, C, n->K, m, B, groups, per, bias_ctas, n->g + n->woff[l],
+                                                        n->g + n->boff[l], ld);
         FDE_LAUNCH_CHECK("conv_wgrad_kernel");
         if (l > 0) {
             // gradient w.r.t. the layer input, through the ReLU of layer l-1 (mask = its output)

@@ -23,29 +23,37 @@ struct CvTile {
     int x0;
 };
 NOP_FN CvTile cv_tile(long n, int m) {
-    const long b = n / m;
+    // (a 64-bit division takes as long as a small layer's products)
+    const long b = (n >> 32) == 0 ? (long)((unsigned)n / (unsigned)m) : n / m;
     return CvTile{b, (int)(n - b * m)};
 }
-// slot that the first tap of the tile's position t reads in a staged row (the halo's h points before its own)
+// Point x of the sample d after the tile's first one; x < 0: a zero beyond the sample's ends.
+struct CvPoint {
+    int d, x;
+};
+// the tile's position t
+NOP_FN CvPoint cv_position(int x0, int m, int t) {
+    const int d = (x0 + t) / m;
+    return CvPoint{d, x0 + t - d * m};
+}
+// slot t of a staged row
+NOP_FN CvPoint cv_slot(int x0, int m, int h, int t) {
+    const int head = m - x0 + 2 * h;  // slots of the first sample's piece
+    CvPoint p{0, x0 - h + t};
+    if (t >= head) {
+        const int u = t - head, w = m + 2 * h;
+        p.d = 1 + u / w;
+        p.x = u - (p.d - 1) * w - h;
+    }
+    if (p.x >= m) p.x = -1;
+    return p;
+}
+// slot that the first tap of the tile's position t reads in a staged row (the halo's h points
+// before its own)
 NOP_FN int cv_place(int t, int x0, int m, int h) { return t + (x0 + t) / m * 2 * h; }
 // length of a staged row of `count` positions
 NOP_FN int cv_length(int count, int x0, int m, int h) { return count + ((x0 + count - 1) / m + 1) * 2 * h; }
-// offset of slot t's point for channel 0 in a batch of Q channels, or -1 for a zero
-NOP_FN ptrdiff_t cv_source(CvTile tile, int Q, int m, int h, int t) {
-    const int head = m - tile.x0 + 2 * h;  // slots of the first sample's piece
-    long b = tile.b0;
-    int x = tile.x0 - h + t;
-    if (t >= head) {
-        const int u = t - head, w = m + 2 * h;
-        b += 1 + u / w;
-        x = u - u / w * w - h;
-    }
-    return x >= 0 && x < m ? (ptrdiff_t)b * Q * m + x : -1;
-}
-// offset of the tile's position t for channel p of a batch of P channels
-NOP_FN size_t cv_offset(CvTile tile, int P, int p, int m, int t) {
-    const int d = (tile.x0 + t) / m;
-    return ((size_t)(tile.b0 + d) * P + p) * m + (tile.x0 + t - d * m);
-}
+// offset of a point (channel 0) from the tile's first sample, `sample` entries each
+NOP_FN size_t cv_offset(CvPoint p, size_t sample) { return (size_t)p.d * sample + p.x; }
 
 }  // namespace fde

@@ -15,9 +15,13 @@ using namespace fde;
 extern "C" int places(long n0, int count, int Q, int m, int h, long* src, int* place, long* off) {
     const CvTile tile = cv_tile(n0, m);
     const int len = cv_length(count, tile.x0, m, h);
-    for (int t = 0; t < len; ++t) src[t] = cv_source(tile, Q, m, h, t);
+    const size_t sample = (size_t)Q * m, base = tile.b0 * sample;
+    for (int t = 0; t < len; ++t) {
+        const CvPoint p = cv_slot(tile.x0, m, h, t);
+        src[t] = p.x < 0 ? -1 : (long)(base + cv_offset(p, sample));
+    }
     for (int t = 0; t < count; ++t) place[t] = cv_place(t, tile.x0, m, h);
-    for (int t = 0; t < count; ++t) off[t] = cv_offset(tile, Q, Q - 1, m, t);
+    for (int t = 0; t < count; ++t) off[t] = (long)(base + cv_offset(cv_position(tile.x0, m, t), sample) + (size_t)(Q - 1) * m);
     return len;
 }
 '''
