@@ -20,6 +20,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <type_traits>
 #include <vector>
 
 #include "fde_internal.h"
@@ -53,6 +54,10 @@ __device__ __forceinline__ void cv_stage(const TI* __restrict__ x, size_t sample
     }
 }
 
+// positions of a CTA's tile and input channels of a chunk (conv_kernel)
+constexpr int cv_positions(int NL, bool pos) { return 4 * NL * (pos ? CV_WARPS : 1); }
+constexpr int cv_channels(int NL, bool pos) { return pos ? 16 : NL == 4 ? 8 * CV_WARPS : 4 * CV_WARPS; }
+
 // y[b][p][x] = bias[p] + sum_q sum_k Wacc(p,q,k) x[b][q][x + k - K/2]
 //   TRANS = false: Wacc(p,q,k) = W[p][q][k]            (W: P x Q x K)
 //   TRANS = true : Wacc(p,q,k) = W[q][p][K-1-k]        (W: Q x P x K; gradient w.r.t. the input)
@@ -64,12 +69,15 @@ __device__ __forceinline__ void cv_stage(const TI* __restrict__ x, size_t sample
 // are added in a fixed order.  Per layer at that size 9 us forward and 13 backward against 51
 // and 45 for a tile of 128 positions of one sample, seven eighths of which were padding.
 // KT: the kernel size, or 0 to take it from K (a known size makes the weights' indices cheap).
-template <typename TI, typename TW, typename TO, bool TRANS, int NL, int KT>
+// POS: the warps take positions of their own instead (32 NL a CTA), for layers of few input channels,
+// whose sums are shorter than the addition of eight partial ones.
+template <typename TI, typename TW, typename TO, bool TRANS, int NL, int KT, bool POS>
 __global__ void __launch_bounds__(32 * CV_WARPS)
 conv_kernel(const TI* __restrict__ x, int Q, const TW* __restrict__ W, const float* __restrict__ bias, int P, int Kr,
             int m, long N, int relu, const float* __restrict__ mask, TO* __restrict__ y, int ld) {
     const int K = KT ? KT : Kr;
-    constexpr int TN = 4 * NL, QW = NL == 4 ? 8 : 4, QC = QW * CV_WARPS;  // QW: channels per warp and chunk
+    constexpr int TN = cv_positions(NL, POS), QC = cv_channels(NL, POS);
+    constexpr int CW = POS ? 1 : CV_WARPS;  // warps that share a position's channels
     extern __shared__ float cv_smem[];
     float* s_in = cv_smem;            // [QC][ld]
     float* s_w = cv_smem + QC * ld;   // [QC][K][CV_LDW]
@@ -77,7 +85,8 @@ conv_kernel(const TI* __restrict__ x, int Q, const TW* __restrict__ W, const flo
     const CvTile tile = cv_tile(n0, m);
     const int p0 = blockIdx.y * CV_TP, count = (int)min((long)TN, N - n0);
     const int h = K / 2, len = cv_length(count, tile.x0, m, h);
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, pl = lane >> 2, nl = lane & 3;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, pl = lane >> 2;
+    const int cw = POS ? 0 : warp, nl = (lane & 3) + (POS ? 4 * NL * warp : 0);  // the warp's channels and positions
     float acc[2][NL];
     int at[NL];
 #pragma unroll
@@ -104,7 +113,7 @@ conv_kernel(const TI* __restrict__ x, int Q, const TW* __restrict__ W, const flo
             for (int r = tid & 15; r < nq * K; r += 16) s_w[r * CV_LDW + row] = p0 + row < P ? ldf(wr + r) : 0.f;
         }
         __syncthreads();
-        for (int c = warp; c < nq; c += CV_WARPS) {
+        for (int c = cw; c < nq; c += CW) {
             const float* in = s_in + c * ld;
             const float* w = s_w + c * K * CV_LDW + 2 * pl;
 #pragma unroll
@@ -125,8 +134,8 @@ conv_kernel(const TI* __restrict__ x, int Q, const TW* __restrict__ W, const flo
     float* red = cv_smem;
 #pragma unroll
     for (int j = 0; j < NL; ++j) {
-        red[(warp * CV_TP + 2 * pl) * TN + nl + 4 * j] = acc[0][j];
-        red[(warp * CV_TP + 2 * pl + 1) * TN + nl + 4 * j] = acc[1][j];
+        red[(cw * CV_TP + 2 * pl) * TN + nl + 4 * j] = acc[0][j];
+        red[(cw * CV_TP + 2 * pl + 1) * TN + nl + 4 * j] = acc[1][j];
     }
     __syncthreads();
     for (int e = tid; e < CV_TP * TN; e += 32 * CV_WARPS) {
@@ -134,7 +143,7 @@ conv_kernel(const TI* __restrict__ x, int Q, const TW* __restrict__ W, const flo
         if (p >= P || n >= count) continue;
         float v = 0.f;
 #pragma unroll
-        for (int w = 0; w < CV_WARPS; ++w) v += red[w * CV_TP * TN + e];
+        for (int w = 0; w < CW; ++w) v += red[w * CV_TP * TN + e];
         if (bias) v += bias[p];
         if (relu) v = fmaxf(v, 0.f);
         const size_t idx = ((size_t)tile.b0 * P + p) * m + cv_offset(cv_position(tile.x0, m, n), (size_t)P * m);
@@ -394,14 +403,14 @@ int staged_length(int tile, long N, int m, int K) {
     return n + pieces * 2 * (K / 2);
 }
 
-template <typename TI, typename TW, typename TO, bool TRANS, int NL, int KT>
+template <typename TI, typename TW, typename TO, bool TRANS, int NL, int KT, bool POS = false>
 int conv_tiles(const TI* x, int Q, const TW* W, const float* bias, int P, int K, int m, long N, int relu,
                const float* mask, TO* y, cudaStream_t st) {
-    constexpr int TN = 4 * NL, QC = (NL == 4 ? 8 : 4) * CV_WARPS;
+    constexpr int TN = cv_positions(NL, POS), QC = cv_channels(NL, POS);
     const int ld = staged_length(TN, N, m, K) | 1;
-    const size_t stage = (size_t)QC * (ld + K * CV_LDW), red = (size_t)CV_WARPS * CV_TP * TN;
+    const size_t stage = (size_t)QC * (ld + K * CV_LDW), red = (size_t)(POS ? 1 : CV_WARPS) * CV_TP * TN;
     const size_t smem = (stage > red ? stage : red) * sizeof(float);
-    auto kern = conv_kernel<TI, TW, TO, TRANS, NL, KT>;
+    auto kern = conv_kernel<TI, TW, TO, TRANS, NL, KT, POS>;
     FDE_TRY(allow_smem((const void*)kern, 227 * 1024));
     const dim3 grid((unsigned)((N + TN - 1) / TN), (P + CV_TP - 1) / CV_TP);
     kern<<<grid, 32 * CV_WARPS, smem, st>>>(x, Q, W, bias, P, K, m, N, relu, mask, y, ld);
@@ -410,18 +419,31 @@ int conv_tiles(const TI* x, int Q, const TW* W, const float* bias, int P, int K,
 }
 
 // 16 positions a CTA while that leaves the launch within a few waves of the 152 SMs; beyond
-// it 64, which reads the weights a quarter as often.
+// it 64, which reads the weights a quarter as often.  With at most 16 input channels and 128 positions
+// for every SM, 128 of them in warps of their own: three layers of 16 channels on 16 x 2047 positions, forward,
+// 48 to 59 us; 62 to 72 in tiles of 64 whose warps share the channels.
 template <typename TI, typename TW, typename TO, bool TRANS>
 int conv(const TI* x, int Q, const TW* W, const float* bias, int P, int K, int m, int B, int relu, const float* mask,
          TO* y, cudaStream_t st) {
-    const long N = (long)B * m;
-    const long ctas = (N + 15) / 16 * ((P + CV_TP - 1) / CV_TP);
-    if (ctas > 8 * 152)
-        return conv_tiles<TI, TW, TO, TRANS, 16, 0>(x, Q, W, bias, P, K, m, N, relu, mask, y, st);
-    if (K == 3) return conv_tiles<TI, TW, TO, TRANS, 4, 3>(x, Q, W, bias, P, K, m, N, relu, mask, y, st);
-    if (K == 5) return conv_tiles<TI, TW, TO, TRANS, 4, 5>(x, Q, W, bias, P, K, m, N, relu, mask, y, st);
-    if (K == 7) return conv_tiles<TI, TW, TO, TRANS, 4, 7>(x, Q, W, bias, P, K, m, N, relu, mask, y, st);
-    return conv_tiles<TI, TW, TO, TRANS, 4, 0>(x, Q, W, bias, P, K, m, N, relu, mask, y, st);
+    const long N = (long)B * m, pt = (P + CV_TP - 1) / CV_TP;
+    const auto go = [&](auto NL, auto KT, auto POS) {
+        return conv_tiles<TI, TW, TO, TRANS, NL.value, KT.value, POS.value>(x, Q, W, bias, P, K, m, N, relu, mask, y, st);
+    };
+    using std::false_type;
+    using std::true_type;
+    using N4 = std::integral_constant<int, 4>;
+    using Any = std::integral_constant<int, 0>;
+    if (Q <= 16 && (N + 127) / 128 * pt >= 152) {
+        if (K == 3) return go(N4(), std::integral_constant<int, 3>(), true_type());
+        if (K == 5) return go(N4(), std::integral_constant<int, 5>(), true_type());
+        if (K == 7) return go(N4(), std::integral_constant<int, 7>(), true_type());
+        return go(N4(), Any(), true_type());
+    }
+    if ((N + 15) / 16 * pt > 8 * 152) return go(std::integral_constant<int, 16>(), Any(), false_type());
+    if (K == 3) return go(N4(), std::integral_constant<int, 3>(), false_type());
+    if (K == 5) return go(N4(), std::integral_constant<int, 5>(), false_type());
+    if (K == 7) return go(N4(), std::integral_constant<int, 7>(), false_type());
+    return go(N4(), Any(), false_type());
 }
 
 int ensure_batch(fde_nop* n, int B) {
