@@ -435,7 +435,7 @@ int fde_batch_solve(fde_batch* b, const fde_pgmres_opts* opts, double* const* x_
         d.m = P.m; d.s = P.s; d.mp = P.mp; d.L = P.L; d.logL = P.logL; d.logs = P.logs; d.mu = P.mu;
         d.nblk = P.nblk; d.n = P.n; d.h = P.h; d.dxa = P.dxa;
         d.start = P.d_start; d.A = P.d_a; d.B = P.d_b; d.dplus = P.d_dplus; d.dminus = P.d_dminus;
-        d.twq = P.d_twq; d.kap = P.d_kap; d.jfac = toeplitz_scale(P); d.tws32 = P.d_tws32; d.tws = P.d_tws;
+        d.twq = P.d_twq; d.kap = P.d_kap; d.jfac = toeplitz_scale(P); d.tws32 = P.d_tws32;
         if (b->shared) {  // the factors of instance 0, frequency vectors of its own
             const Problem& P0 = *problem_of(b->probs[0]);
             d.fac = P0.d_fac;

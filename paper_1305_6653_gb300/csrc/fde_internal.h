@@ -73,7 +73,6 @@ struct InstDev {
     const bfp::Q61* kap;
     double jfac;           // toeplitz_scale
     const float2* tws32;
-    const double2* tws;
     void* rhat;
     void* fac;
     void* tinv;            // inverted 32 x 32 diagonal tiles of the factors

@@ -443,9 +443,7 @@ constexpr int TRSV_THREADS = 512;                           // the default launc
 constexpr int TRSV_TPR = 8;                                  // threads per row in the strip update
 constexpr int TRSV_BAR_X = 1, TRSV_BAR_B = 3;                // named barrier ids (+ d & 1)
 constexpr int TRSV_BAR_SOLVER = 6;                           // among the solver threads (groups of four)
-// Rows per group whose loads are in flight together.
-template <typename T> struct trsv_unroll { static constexpr int value = 8; };
-template <typename T> struct trsv_tile { static constexpr int LD = TRSV_LD; };
+constexpr int TRSV_ROWS = 4;                                 // rows per register buffer
 // Launch shapes of the block solves from the bfloat16 copy (FDE_TUNE_TRSV): NT threads (warp 0 the
 // solver, NT/32 - 1 streaming warps) and H rows per register buffer.  The arithmetic of every row
 // does not depend on the shape, so all shapes give bit-identical results.
@@ -468,7 +466,7 @@ __device__ __forceinline__ void trsv_solver(int mp, int nt, const typename fac_s
                                             const typename fac_store<T, LAY>::elem* im, const T* tinv, cplx_t<T>* y, cplx_t<T> (*xs)[32], T* tiles,
                                             cplx_t<T>* av, int lane) {
     using C = cplx_t<T>;
-    constexpr int LD = trsv_tile<T>::LD, TS = 32 * LD;
+    constexpr int LD = TRSV_LD, TS = 32 * LD;
     auto tile_of = [&](int d) { return FWD ? d : nt - 1 - d; };
     auto issue = [&](int d) {
         T* b = tiles + (d & 1) * 4 * TS;  // [D re, D im, L re, L im]
@@ -733,7 +731,7 @@ __device__ __forceinline__ void trsv_stream_bf16(int mp, int nt, const unsigned 
     }
 }
 
-template <typename T, int NT = TRSV_THREADS, int H = trsv_unroll<T>::value / 2, int LAY = LAY_PLANES>
+template <typename T, int NT = TRSV_THREADS, int H = TRSV_ROWS, int LAY = LAY_PLANES>
 __device__ __forceinline__ void trsv_body(int mp, const typename fac_store<T, LAY>::elem* __restrict__ re,
                                           const T* __restrict__ tinv, cplx_t<T>* __restrict__ x) {
     using C = cplx_t<T>;
@@ -788,7 +786,7 @@ block_trsv_batched(const InstDev* __restrict__ I, const int* __restrict__ act) {
     cplx_t<T>* rhat = (cplx_t<T>*)d.rhat + (size_t)k * mp;
     const T* tinv = (const T*)d.tinv + (size_t)k * (mp / 32) * 4096;
     if (d.strips)  // the bfloat16 strip copy
-        trsv_body<T, TRSV_THREADS, trsv_unroll<T>::value / 2, LAY_STRIPS_BF16>(
+        trsv_body<T, TRSV_THREADS, TRSV_ROWS, LAY_STRIPS_BF16>(
             d.mp, (const unsigned short*)d.strips + (size_t)k * 2 * mp * mp, tinv, rhat);
     else
         trsv_body<T>(d.mp, (const T*)d.fac + (size_t)k * 2 * mp * mp, tinv, rhat);
@@ -811,7 +809,7 @@ constexpr int TRSVM_THREADS = 384;  // warp 0 + 11 streaming warps (44 row group
 static_assert(TRSV_R == TRSV_TPR, "the reduce-scatter leaves one column per lane of a row group");
 
 __host__ __device__ static size_t trsv_multi_smem_bytes(int mp) {
-    return (size_t)mp * TRSV_R * sizeof(float2) + 8 * 32 * trsv_tile<float>::LD * sizeof(float);
+    return (size_t)mp * TRSV_R * sizeof(float2) + 8 * 32 * TRSV_LD * sizeof(float);
 }
 
 // One row's strip product for TRSV_R columns: lane `sub` holds factor columns
@@ -926,7 +924,7 @@ template <bool FWD>
 __device__ __forceinline__ void trsv_multi_solver(int mp, int nt, const float* re, const float* im,
                                                   const float* tinv, float2 (*y)[TRSV_R], float2 (*xs)[32][TRSV_R],
                                                   float* tiles, float2 (*av)[TRSV_R], int lane) {
-    constexpr int LD = trsv_tile<float>::LD, TS = 32 * LD;
+    constexpr int LD = TRSV_LD, TS = 32 * LD;
     auto tile_of = [&](int d) { return FWD ? d : nt - 1 - d; };
     auto issue = [&](int d) {
         float* b = tiles + (d & 1) * 4 * TS;
@@ -1048,7 +1046,7 @@ constexpr int TRSV4_SW = 128;                    // solver threads
 constexpr int TRSV4_THREADS = TRSV4_SW + 352;    // 44 row groups
 
 __host__ __device__ static size_t trsv_multi4_smem_bytes(int mp) {
-    return (size_t)mp * 4 * sizeof(float2) + 8 * 32 * trsv_tile<float>::LD * sizeof(float);
+    return (size_t)mp * 4 * sizeof(float2) + 8 * 32 * TRSV_LD * sizeof(float);
 }
 
 // As multi_row_product for R columns, fewer than the lanes of a row: once one column is left, the
@@ -1192,7 +1190,7 @@ template <int R, bool FWD>
 __device__ __forceinline__ void trsv_multi4_solver(int mp, int nt, const float* re, const float* im,
                                                   const float* tinv, float2 (*y)[R], float2 (*xs)[32][R],
                                                   float* tiles, float2 (*av)[R], int tid) {
-    constexpr int LD = trsv_tile<float>::LD, TS = 32 * LD, W = R * 32 / TRSV4_SW;
+    constexpr int LD = TRSV_LD, TS = 32 * LD, W = R * 32 / TRSV4_SW;
     const int lane = tid & 31, j0 = W * (tid >> 5);
     auto tile_of = [&](int d) { return FWD ? d : nt - 1 - d; };
     auto issue = [&](int d) {
