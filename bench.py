@@ -227,8 +227,8 @@ def matvec_flops(m: int, s: int, L: int, mu: int) -> float:
 
 
 FP64_PEAK_TFLOPS = 1.25  # GB300 nominal FP64 (no measured FP64 figure in MEASURED_PEAKS.json)
-# DRAM bytes / algorithmic bytes of the FP32 block solves (ncu, m=1023, s=256), by the
-# element size of the factor copy it streams (4: FP32, 2: bfloat16)
+# DRAM bytes / algorithmic bytes of the block solves (ncu, m=1023, s=256), by the element size of
+# the factor copy they stream (4: FP32, block_trsv_kernel; 2: bfloat16, block_trsv_bf16_kernel)
 TRSV_TRAFFIC_RATIO = {4: 1.034, 2: 1.098}
 
 

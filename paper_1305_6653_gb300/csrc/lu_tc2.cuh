@@ -57,6 +57,9 @@ constexpr int T2_C_BYTES = T2_BM * T2_CROW;  // one plane
 // (hi twice) it was 768 KB: the whole LU at m_p = 4096, 65 blocks took 80 ms, now 69.  What
 // bounds the update then is shared memory (the MMAs read 28 KB per K = 8, 109 of 128 bytes a
 // clock at full rate, beside the arriving operands); the tensor pipe is active 60 %.
+// The sums' order (a chunk's three products together, where all of A_hi B_hi came first) leaves
+// the factors' error against FP64 as it was: 0.994 of it in the geometric mean over 40 shapes (m = 137 to
+// 1940, s = 16 to 64, alpha = 1.2 to 1.9, four schemes), and 0.988 for solves from the factors.
 template <int KIND>
 struct Tc2 {
     static constexpr int ESZ = KIND == 1 ? 2 : 4;
