@@ -152,64 +152,55 @@ conv_kernel(const TI* __restrict__ x, int Q, const TW* __restrict__ W, const flo
     }
 }
 
-// db[o] = sum g of up to 16 channels o0 .., `each` of them a CTA: a channel's terms are shared
-// among the lanes of 8 / each warps (one at least) and added in fours in FP32, the rest in FP64 and in a fixed
-// order, so db repeats to the bit and its rounding does not grow with the batch.
-__device__ __forceinline__ void bias_sums(const float* __restrict__ g, int O, int m, int B, int o0, int cta, int each,
-                                          float* __restrict__ db) {
+// db[o] = sum g of one channel, by a CTA of its own: its terms are added in fours in FP32, the rest in
+// FP64 and in a fixed order, so db repeats to the bit and its rounding does not grow with the batch.
+__device__ __forceinline__ void bias_sum(const float* __restrict__ g, int O, int m, int B, int o,
+                                         float* __restrict__ db) {
     __shared__ double red[8];
     const long N = (long)B * m;
     const size_t sample = (size_t)O * m;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int wpc = max(8 / each, 1), part = warp % wpc, last = min(min((cta + 1) * each, 16), O - o0);
+    g += (size_t)o * m;
     double v = 0.0;
-    for (int c = cta * each + warp / wpc; c < last; c += 8 / wpc) {
-        v = 0.0;
-        for (long n = 32 * part + lane; n < N; n += 8 * 32 * wpc) {
-            float s[2] = {0.f, 0.f};
+    for (long n = threadIdx.x; n < N; n += 8 * 256) {
+        float s[2] = {0.f, 0.f};
 #pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                const long q = n + 32 * wpc * j;
-                if (q < N) {
-                    const CvTile at = cv_tile(q, m);
-                    s[j / 4] += g[at.b0 * sample + (size_t)(o0 + c) * m + at.x0];
-                }
+        for (int j = 0; j < 8; ++j) {
+            const long q = n + 256 * j;
+            if (q < N) {
+                const CvTile at = cv_tile(q, m);
+                s[j / 4] += g[at.b0 * sample + at.x0];
             }
-            v += (double)s[0];
-            v += (double)s[1];
         }
-        for (int off = 16; off; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-        if (wpc == 1 && lane == 0) db[o0 + c] = (float)v;
+        v += (double)s[0];
+        v += (double)s[1];
     }
-    if (wpc == 1) return;
-    if (lane == 0) red[warp] = v;
+    for (int off = 16; off; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
     __syncthreads();
-    const int c = cta * each + warp / wpc;  // every channel of the CTA was taken at once
-    if (part == 0 && lane == 0 && c < last) {
-        for (int w = 1; w < wpc; ++w) v += red[warp + w];
-        db[o0 + c] = (float)v;
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < 8; ++w) v += red[w];
+        db[o] = (float)v;
     }
 }
 
 // dW[o][c][k] += sum_{b in group} sum_x g[b][o][x] a[b][c][x + k - K/2]; one thread per (o, c)
 // of a 16 x 16 tile, the flattened positions of the batch split over `groups` of `per` (atomic
-// accumulation).  The CTAs behind the groups form the bias gradients db (before them they cost a large
-// gradient 10 %: fewer of the others start together).  Four of them a tile serve a batch of up to 1024
-// positions whose other CTAs fill the SMs; otherwise a channel gets a CTA of its own (a gradient at
-// 16 x 2047 positions, 16 channels: 640 us, 2390 with a warp a channel).
+// accumulation).  The CTAs behind the groups form the bias gradients db, a channel each (before them
+// they cost a large gradient 10 %: fewer of the others start together; with several channels a CTA they
+// are the last to finish: 2390 us a gradient at 16 x 2047 positions, 16 channels, with a warp a channel, 640 so).
 // 10 us a layer at 64 channels, 16 modes, 32 samples, against 22 (64-position tiles of single
 // samples) and 10 for the bias sums in a launch of their own.
 constexpr int WG_N = 64;  // positions staged at once
 __global__ void __launch_bounds__(256)
 conv_wgrad_kernel(const float* __restrict__ g, int O, const float* __restrict__ a, int C, int K, int m, int B,
-                  int groups, long per, int bias_ctas, float* __restrict__ dW, float* __restrict__ db, int ld) {
+                  int groups, long per, float* __restrict__ dW, float* __restrict__ db, int ld) {
     extern __shared__ float wg_smem[];
     float* s_g = wg_smem;                  // [16][WG_N + 1]
     float* s_a = wg_smem + 16 * (WG_N + 1);  // [16][ld]
     const int o0 = blockIdx.y * 16, c0 = blockIdx.x * 16;
     if ((int)blockIdx.z >= groups) {
-        const int cta = (blockIdx.z - groups) * gridDim.x + blockIdx.x;
-        if (cta < bias_ctas) bias_sums(g, O, m, B, o0, cta, 16 / bias_ctas, db);
+        const int q = (blockIdx.z - groups) * gridDim.x + blockIdx.x;
+        if (q < 16 && o0 + q < O) bias_sum(g, O, m, B, o0 + q, db);
         return;
     }
     const int ol = threadIdx.x / 16, cl = threadIdx.x % 16;
@@ -590,12 +581,11 @@ int fde_nop_loss_grad(fde_nop* n, const float* in, const float* target, int batc
         const int O = n->dout[l], C = n->din[l];
         const int groups = (int)std::min<long>(((long)B * m + 15) / 16, 16), cx = (C + 15) / 16, cy = (O + 15) / 16;
         const long per = ((long)B * m + groups - 1) / groups;
-        const int bias_ctas = (long)B * m <= 1024 && cx * cy * groups > 152 ? 4 : 16;
-        const dim3 wg(cx, cy, groups + (bias_ctas + cx - 1) / cx);
+        const dim3 wg(cx, cy, groups + (16 + cx - 1) / cx);
         const int ld = staged_length(WG_N, (long)B * m, m, n->K) | 1;
         const size_t smem = (size_t)16 * (WG_N + 1 + ld) * sizeof(float);
         FDE_TRY(allow_smem((const void*)conv_wgrad_kernel, smem));
-        conv_wgrad_kernel<<<wg, 256, smem, n->stream>>>(g, O, a, C, n->K, m, B, groups, per, bias_ctas, n->g + n->woff[l],
+        conv_wgrad_kernel<<<wg, 256, smem, n->stream>>>(g, O, a, C, n->K, m, B, groups, per, n->g + n->woff[l],
                                                         n->g + n->boff[l], ld);
         FDE_LAUNCH_CHECK("conv_wgrad_kernel");
         if (l > 0) {
