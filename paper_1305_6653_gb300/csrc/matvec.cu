@@ -289,17 +289,15 @@ __device__ __forceinline__ void bfp_row(int m, int logL, int mu, double h, const
     const double* dp = dplus + (size_t)row * dstride;  // MODE 1 with per-column coefficients
     const double* dm = dminus + (size_t)row * dstride;
     // The row's scale: its power of two goes into the integers' conversion, so that d+, d- of any
-    // magnitude multiply numbers of the result's own; what is extreme of it is applied afterwards.
+    // magnitude multiply numbers of the result's own; what is beyond 2^900 of it is left to the factor.
     int ef;
     const double f = bfp::mantissa(MODE == 0 ? h * fac : fac, &ef);
-    const int whole = shifts - (bfp::BITS - 1 + 1023 - emax) + ef;
-    const int e = min(max(whole, -900), 900), rest = whole - e;
-    const double s1 = bfp::power_of_two(rest / 2), s2 = bfp::power_of_two(rest - rest / 2);
+    const int whole = shifts - (bfp::BITS - 1 + 1023 - emax) + ef, e = min(max(whole, -900), 900);
+    const double s1 = f * bfp::power_of_two(min(max(whole - e, -1000), 1000));
     for (int i = tid; i < m; i += T) {
         const I2 v = buf[bfp::slot(i)];  // (imaginary, real)
-        double jz = dp[i] * bfp::to_double(v.y - v.x, e) + dm[i] * bfp::to_double(v.x + v.y, e);
-        if (rest != 0) jz = jz * s1 * s2;
-        y[(size_t)row * m + i] = MODE == 0 ? ubuf[i] - f * jz : f * jz;
+        const double jz = dp[i] * bfp::to_double(v.y - v.x, e) + dm[i] * bfp::to_double(v.x + v.y, e);
+        y[(size_t)row * m + i] = MODE == 0 ? ubuf[i] - s1 * jz : s1 * jz;
     }
 }
 
